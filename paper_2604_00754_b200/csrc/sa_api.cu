@@ -143,7 +143,7 @@ size_t sa_workspace_bytes(const sa_problem* p, int op) {
       return check_problem(p) == SA_OK ? branch_bytes(p) : (size_t)-1;
     case SA_OP_BACKWARD:
       if (check_problem(p) != SA_OK) return (size_t)-1;
-      return bwd_ws_bytes(p->B, p->Hq, p->n, nullptr);
+      return bwd_ws_bytes(p->B, p->Hq, p->Hkv, p->n, p->d, p->dtype, nullptr, nullptr);
     case SA_OP_FORWARD_ROPE: {
       if (check_problem(p) != SA_OK || p->d % 2 != 0) return (size_t)-1;
       FwdArgs a = fwd_args(p, p, p, p, false);      // pointers unused by the support test
@@ -335,7 +335,9 @@ sa_status sa_backward(const sa_problem* p, const void* q, const void* k, const v
   if (gate_logits && (!good_ptr(y_swa) || !good_ptr(lse_swa) || !dgate_logits))
     return SA_ERR_INVALID_ARG;
   int chunks = 0;
-  if (ws_bytes < bwd_ws_bytes(p->B, p->Hq, p->n, &chunks)) return SA_ERR_WORKSPACE;
+  size_t parts_at = 0;
+  if (ws_bytes < bwd_ws_bytes(p->B, p->Hq, p->Hkv, p->n, p->d, p->dtype, &chunks, &parts_at))
+    return SA_ERR_WORKSPACE;
   cudaStream_t st = (cudaStream_t)stream;
   if ((s = maybe_validate(p, perm, inv, st)) != SA_OK) return s;
   BwdArgs a{};
@@ -346,6 +348,7 @@ sa_status sa_backward(const sa_problem* p, const void* q, const void* k, const v
   a.delta = (float*)ws;
   const size_t delta_bytes = ((size_t)2 * p->B * p->Hq * p->n * sizeof(float) + 255) / 256 * 256;
   a.partials = (float*)((char*)ws + delta_bytes);
+  a.parts = (float*)((char*)ws + parts_at);
   a.chunks = chunks;
   a.B = p->B; a.Hq = p->Hq; a.Hkv = p->Hkv; a.n = p->n; a.d = p->d; a.w = p->w;
   a.flags = p->flags; a.scale = scale_of(p);

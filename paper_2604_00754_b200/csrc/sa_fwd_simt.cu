@@ -3,122 +3,119 @@
 // cannot hold 1e-4 max-abs error), odd shapes and strides, and is the on-device cross-check
 // of the tensor-core path.
 //
-// One warp owns one query row (Eq. 1 for one i).  Keys are taken 32 at a time in slot
-// order: each lane scores one key (gathered through perm for the SA branch), the warp
-// keeps an online softmax, then the 32 weighted value rows are accumulated with each lane
-// owning output columns lane, lane+32, ...  The finished row is scattered to its original
-// position, optionally combined with the other branch through the gate of Eq. 5.
+// A CTA of 128 threads owns 32 query rows (consecutive slots of one head) and walks the keys
+// any of them can see, 32 at a time: rows of K and V are gathered through perm with cp.async
+// into one of two shared-memory buffers while the other one is worked on.  Scores and the
+// weighted sum are register-tiled products (4 rows x 2 keys, 4 rows x 4 columns per 64 per
+// thread): a K or V row is read from memory once per 32 queries, and a shared-memory word is
+// used by 4 fused multiply-adds.  Bound: the FMA pipe and shared-memory reads in about equal
+// parts (8 wavefronts per 32 packed FMAs).  32 rows and not 64, because narrow windows pay
+// (32 + w - 1) / w of their keys, and small calls need the CTAs.
 #include "sa_common.cuh"
+#include "sa_simt_common.cuh"
 
 namespace sa {
 namespace {
 
-constexpr int kWarps = 8;
-constexpr int kMaxColsPerLane = 8;  // d <= 256
-
-template <typename T>
-__device__ __forceinline__ float dot_row(const float* __restrict__ qs, const T* __restrict__ row,
-                                         int d);
-
-template <>
-__device__ __forceinline__ float dot_row<float>(const float* __restrict__ qs,
-                                                const float* __restrict__ row, int d) {
-  float acc = 0.f;
-  for (int c = 0; c < d; c += 4) {
-    const float4 kv = *reinterpret_cast<const float4*>(row + c);
-    const float4 qv = *reinterpret_cast<const float4*>(qs + c);
-    acc = fmaf(qv.x, kv.x, acc); acc = fmaf(qv.y, kv.y, acc);
-    acc = fmaf(qv.z, kv.z, acc); acc = fmaf(qv.w, kv.w, acc);
-  }
-  return acc;
-}
-
-template <>
-__device__ __forceinline__ float dot_row<__nv_bfloat16>(const float* __restrict__ qs,
-                                                        const __nv_bfloat16* __restrict__ row,
-                                                        int d) {
-  float acc = 0.f;
-  for (int c = 0; c < d; c += 8) {
-    const uint4 raw = *reinterpret_cast<const uint4*>(row + c);
-    const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&raw);
-    const float4 q0 = *reinterpret_cast<const float4*>(qs + c);
-    const float4 q1 = *reinterpret_cast<const float4*>(qs + c + 4);
-    const float2 a = __bfloat1622float2(h[0]), b = __bfloat1622float2(h[1]);
-    const float2 e = __bfloat1622float2(h[2]), f = __bfloat1622float2(h[3]);
-    acc = fmaf(q0.x, a.x, acc); acc = fmaf(q0.y, a.y, acc);
-    acc = fmaf(q0.z, b.x, acc); acc = fmaf(q0.w, b.y, acc);
-    acc = fmaf(q1.x, e.x, acc); acc = fmaf(q1.y, e.y, acc);
-    acc = fmaf(q1.z, f.x, acc); acc = fmaf(q1.w, f.y, acc);
-  }
-  return acc;
-}
-
-template <typename T>
-__global__ void __launch_bounds__(kWarps * 32) fwd_simt_kernel(const FwdArgs a) {
-  extern __shared__ float smem[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float* qs = smem + warp * a.d;
-
-  const int slot = blockIdx.x * kWarps + warp;  // position in the order attention runs in
-  const int hq = blockIdx.y, b = blockIdx.z;
-  if (slot >= a.n) return;
-  if (a.abort_flag && *a.abort_flag) return;  // an earlier check rejected perm/inv
-  const int hk = hq / (a.Hq / a.Hkv);
+// NCG: groups of 64 output columns (d <= 64 * NCG)
+template <typename T, int NCG>
+__global__ void __launch_bounds__(kTileThreads) fwd_tile_kernel(const FwdArgs a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tx = lane & 15, half = lane >> 4;         // key / column index, row group of the warp
+  const int row0 = warp * 8 + half * 4;               // this thread's four rows
+  const int hq = blockIdx.y, b = blockIdx.z, s0 = blockIdx.x * kRows;
+  if (a.abort_flag && *a.abort_flag) return;          // an earlier check rejected perm/inv
+  const int hk = hq / (a.Hq / a.Hkv), d = a.d;
   const int32_t* perm = a.swa ? nullptr : a.perm + (size_t)b * a.n;
-  const int tok = perm ? perm[slot] : slot;
+  const TileSmem<T> sm(d);
+  float* qs = reinterpret_cast<float*>(smem_raw);
+  T* kv = reinterpret_cast<T*>(smem_raw + sm.rows_bytes());       // K0 V0 K1 V1
+  float* ps = reinterpret_cast<float*>(smem_raw + sm.rows_bytes() + 4 * sm.col_bytes());
+  float* pw = ps + warp * (kCols * 8);                // this warp's probabilities [key][8 rows]
+  __shared__ int s_slot[2][kCols], s_tok[2][kCols];
 
-  const T* q = (const T*)a.q + b * a.qs[0] + hq * a.qs[1] + tok * a.qs[2];
   const T* kbase = (const T*)a.k + b * a.ks[0] + hk * a.ks[1];
   const T* vbase = (const T*)a.v + b * a.ks[0] + hk * a.ks[1];
   const float scale2 = a.scale * kLog2e;
-  for (int c = lane; c < a.d; c += 32) qs[c] = to_f32(q[c]) * scale2;
-  __syncwarp();
+  load_rows<T>(qs, d, (const T*)a.q + b * a.qs[0] + hq * a.qs[1], a.qs[2], perm, s0, a.n, scale2);
 
-  const MaskGeom g = make_geom(a.n, a.w, a.flags, a.swa);
-  const SlotRange r = key_range(g, slot);
-
-  float acc[kMaxColsPerLane];
+  const TileMask g(a.n, a.w, a.flags, a.swa, s0, false);
+  int qslot[4], qtok[4];
 #pragma unroll
-  for (int x = 0; x < kMaxColsPerLane; ++x) acc[x] = 0.f;
-  float m = -INFINITY, l = 0.f;
+  for (int r = 0; r < 4; ++r) {
+    qslot[r] = s0 + row0 + r;
+    const int sl = min(qslot[r], a.n - 1);
+    qtok[r] = perm ? perm[sl] : sl;
+  }
+  ColLoader<T> ld(d);
+  auto fetch = [&](int t) { ld.fetch(g, perm, t); };
+  auto issue = [&](int buf) {
+    ld.issue(kv + (2 * buf) * sm.col_elems(), kbase, kv + (2 * buf + 1) * sm.col_elems(), vbase,
+             a.ks[2], s_slot[buf], s_tok[buf]);
+  };
 
-  for (int t0 = 0; t0 < r.count; t0 += 32) {
-    const int t = t0 + lane;
-    int ks = r.start + t, kt = -1;
-    bool ok = t < r.count;
-    if (ok) {
-      if (r.wrap) ks = wrap_slot(ks, a.n);
-      else ok = ks >= 0 && ks < a.n;
+  float o[4][4 * NCG];
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int c = 0; c < 4 * NCG; ++c) o[r][c] = 0.f;
+  float m[4], l[4];
+#pragma unroll
+  for (int r = 0; r < 4; ++r) { m[r] = -INFINITY; l[r] = 0.f; }
+
+  fetch(0);
+  issue(0);
+  if (g.tiles > 1) fetch(1);
+  for (int j = 0; j < g.tiles; ++j) {
+    const int buf = j & 1;
+    if (j + 1 < g.tiles) {
+      issue(buf ^ 1);
+      if (j + 2 < g.tiles) fetch(j + 2);
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
     }
-    if (ok) {
-      kt = perm ? perm[ks] : ks;
-      ok = visible(g, slot, tok, ks, kt);
-    }
-    float s = -INFINITY;
-    if (ok) s = dot_row<T>(qs, kbase + kt * a.ks[2], a.d);
-    if (!__any_sync(0xffffffffu, ok)) continue;
-    const float m_new = fmaxf(m, warp_max(s));       // finite: some lane is visible
-    const float corr = exp2f(m - m_new);              // m = -inf gives 0
-    const float p = ok ? exp2f(s - m_new) : 0.f;
-    l = l * corr + warp_sum(p);
-    m = m_new;
+    __syncthreads();
+    const T* ks_ = kv + (2 * buf) * sm.col_elems();
+    const T* vs_ = kv + (2 * buf + 1) * sm.col_elems();
+    float s[4][2];
+    tile_dot<T>(s, qs + row0 * sm.row_elems(), sm.row_elems(), ks_ + tx * sm.stride(),
+                16 * sm.stride(), d);
+    float mt[4];
 #pragma unroll
-    for (int x = 0; x < kMaxColsPerLane; ++x) acc[x] *= corr;
-    const uint32_t live = __ballot_sync(0xffffffffu, ok);
-    for (uint32_t rest = live; rest; rest &= rest - 1) {
-      const int src = __ffs(rest) - 1;
-      const float pj = __shfl_sync(0xffffffffu, p, src);
-      const int jt = __shfl_sync(0xffffffffu, kt, src);
-      const T* vr = vbase + jt * a.ks[2];
+    for (int r = 0; r < 4; ++r) mt[r] = m[r];
 #pragma unroll
-      for (int x = 0; x < kMaxColsPerLane; ++x) {
-        const int c = lane + 32 * x;
-        if (c < a.d) acc[x] = fmaf(pj, to_f32(vr[c]), acc[x]);
+    for (int c = 0; c < 2; ++c) {
+      const int sk = s_slot[buf][tx + 16 * c], jk = s_tok[buf][tx + 16 * c];
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        if (!g.sees(qslot[r], qtok[r], sk, jk)) s[r][c] = -INFINITY;
+        mt[r] = fmaxf(mt[r], s[r][c]);
       }
     }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+#pragma unroll
+      for (int x = 8; x > 0; x >>= 1) mt[r] = fmaxf(mt[r], __shfl_xor_sync(0xffffffffu, mt[r], x));
+      const float ref = mt[r] == -INFINITY ? 0.f : mt[r];
+      const float corr = exp2f(m[r] - ref);            // m = -inf gives 0
+      m[r] = mt[r];
+      s[r][0] = exp2f(s[r][0] - ref);
+      s[r][1] = exp2f(s[r][1] - ref);
+      l[r] = fmaf(l[r], corr, s[r][0] + s[r][1]);
+#pragma unroll
+      for (int c = 0; c < 4 * NCG; ++c) o[r][c] *= corr;
+    }
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+      *reinterpret_cast<float4*>(pw + (tx + 16 * c) * 8 + 4 * half) =
+          make_float4(s[0][c], s[1][c], s[2][c], s[3][c]);
+    __syncwarp();
+    tile_accumulate<T, NCG>(o, pw + 4 * half, vs_, sm.stride(), tx, d);
+    __syncthreads();                                  // the buffer may be refilled now
   }
 
-  const float inv_l = 1.f / l;
   float g_this = 1.f, g_other = 0.f;
   if (a.gate_logits) {
     const float l_sa = a.gate_logits[hq], l_swa = a.gate_logits[a.Hq + hq];
@@ -126,35 +123,60 @@ __global__ void __launch_bounds__(kWarps * 32) fwd_simt_kernel(const FwdArgs a) 
     g_this = a.swa ? s_swa : s_sa;
     g_other = a.swa ? s_sa : s_swa;
   }
-  const int64_t off = b * a.qs[0] + hq * a.qs[1] + tok * a.qs[2];
 #pragma unroll
-  for (int x = 0; x < kMaxColsPerLane; ++x) {
-    const int c = lane + 32 * x;
-    if (c < a.d) {
-      float o = acc[x] * inv_l;
-      if (a.y_branch) {
-        const T ob = from_f32<T>(o);
-        ((T*)a.y_branch)[off + c] = ob;
-        o = to_f32(ob);  // combine what was stored, as the backward pass will read it
+  for (int r = 0; r < 4; ++r) {
+#pragma unroll
+    for (int x = 8; x > 0; x >>= 1) l[r] += __shfl_xor_sync(0xffffffffu, l[r], x);
+    if (qslot[r] >= a.n) continue;
+    const float inv_l = 1.f / l[r];
+    const int64_t off = b * a.qs[0] + hq * a.qs[1] + (int64_t)qtok[r] * a.qs[2];
+#pragma unroll
+    for (int cg = 0; cg < NCG; ++cg) {
+      const int c = 64 * cg + 4 * tx;
+      if (c >= d) continue;
+      float4 v = make_float4(o[r][4 * cg] * inv_l, o[r][4 * cg + 1] * inv_l,
+                             o[r][4 * cg + 2] * inv_l, o[r][4 * cg + 3] * inv_l);
+      if (a.y_branch) {   // combine what was stored, as the backward pass will read it
+        st4((T*)a.y_branch + off + c, v);
+        v = round4<T>(v);
       }
       if (a.gate_logits) {
-        o *= g_this;
-        if (a.y_other) o = fmaf(g_other, to_f32(((const T*)a.y_other)[off + c]), o);
+        v.x *= g_this; v.y *= g_this; v.z *= g_this; v.w *= g_this;
+        if (a.y_other) {
+          const float4 w4 = ld4((const T*)a.y_other + off + c);
+          v.x = fmaf(g_other, w4.x, v.x); v.y = fmaf(g_other, w4.y, v.y);
+          v.z = fmaf(g_other, w4.z, v.z); v.w = fmaf(g_other, w4.w, v.w);
+        }
       }
-      if (a.y) ((T*)a.y)[off + c] = from_f32<T>(o);
+      if (a.y) st4((T*)a.y + off + c, v);
     }
+    if (a.lse && tx == 0)
+      a.lse[((size_t)b * a.Hq + hq) * a.n + qtok[r]] = (m[r] + log2f(l[r])) * kLn2;
   }
-  if (a.lse && lane == 0)
-    a.lse[((size_t)b * a.Hq + hq) * a.n + tok] = (m + log2f(l)) * kLn2;
+}
+
+template <typename T, int NCG>
+cudaError_t go(const FwdArgs& a, cudaStream_t st) {
+  const TileSmem<T> sm(a.d);
+  const int smem = sm.rows_bytes() + 4 * sm.col_bytes() + kTileThreads / 32 * kCols * 8 * 4;
+  cudaError_t e = allow_smem((const void*)fwd_tile_kernel<T, NCG>, smem);
+  if (e != cudaSuccess) return e;
+  fwd_tile_kernel<T, NCG>
+      <<<dim3((a.n + kRows - 1) / kRows, a.Hq, a.B), kTileThreads, smem, st>>>(a);
+  return cudaSuccess;
+}
+
+template <typename T>
+cudaError_t by_width(const FwdArgs& a, cudaStream_t st) {
+  if (a.d <= 64) return go<T, 1>(a, st);
+  return a.d <= 128 ? go<T, 2>(a, st) : go<T, 4>(a, st);
 }
 
 }  // namespace
 
 cudaError_t launch_fwd_simt(const FwdArgs& a, int dtype, cudaStream_t st) {
-  const dim3 grid((a.n + kWarps - 1) / kWarps, a.Hq, a.B);
-  const size_t smem = (size_t)kWarps * a.d * sizeof(float);
-  if (dtype == SA_F32) fwd_simt_kernel<float><<<grid, kWarps * 32, smem, st>>>(a);
-  else fwd_simt_kernel<__nv_bfloat16><<<grid, kWarps * 32, smem, st>>>(a);
+  const cudaError_t e = dtype == SA_F32 ? by_width<float>(a, st) : by_width<__nv_bfloat16>(a, st);
+  if (e != cudaSuccess) return e;
   bump_launches();
   return cudaGetLastError();
 }
