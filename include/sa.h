@@ -207,12 +207,13 @@ int32_t sa_host_forward_plan(int32_t Hq, int32_t Hkv, int32_t n_groups, int32_t 
  *   of q (kv == 0: H = Hq) or of k (kv != 0: H = Hkv); out may be x.  inverse != 0 turns by the
  *   opposite angle (the transpose: maps a gradient with respect to the rotated tensor back).
  * sa_forward_rope / sa_swa_gated_forward_rope: sa_forward / sa_swa_gated_forward on rotated Q
- *   and K without that pass: bf16 with d = 64 or 128 rotates the rows inside the kernels' row
- *   gather, where the token a row belongs to is at hand (no rotated copy of Q or K exists);
- *   every other case rotates Q and K into ws first (sa_workspace_bytes(.., SA_OP_FORWARD_ROPE)
- *   bytes; 0 when the fused path applies).  Same results as sa_rope_apply followed by the plain
- *   call.  For the backward pass rotate q and k with sa_rope_apply, call sa_backward on them, and
- *   turn dq and dk back with inverse = 1.
+ *   and K.  With a workspace of sa_workspace_bytes(.., SA_OP_FORWARD_ROPE) bytes (copies of Q and
+ *   K and one branch output, in their layouts) the rotation is a pass over Q and K in one launch.
+ *   bf16 with d = 64 or 128 also works without a workspace, and for small sa_forward_rope calls
+ *   (less than 16 MB of Q) ignores it: the rows are then rotated inside the kernels' row gather,
+ *   which is one launch less and turns each K row once per query tile that meets it.  Same
+ *   results as sa_rope_apply followed by the plain call.  For the backward pass rotate q and k with
+ *   sa_rope_apply, call sa_backward on them, and turn dq and dk back with inverse = 1.
  * Errors: as the plain calls, plus SA_ERR_INVALID_ARG for null tables or odd d. */
 sa_status sa_rope_table(int32_t n, int32_t d, double base, float* rope_cos, float* rope_sin,
                         sa_stream_t stream);

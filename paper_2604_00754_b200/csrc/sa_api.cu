@@ -67,13 +67,16 @@ size_t branch_bytes(const sa_problem* p) {
   return (size_t)elems * (p->dtype == SA_BF16 ? 2 : 4);
 }
 
-// Bytes a tensor with the given strides spans (the rotated copies of the unfused RoPE path).
+// Bytes a tensor with the given strides spans.
 size_t span_bytes(const sa_problem* p, bool kv) {
   const int64_t* s = kv ? p->kv_stride : p->q_stride;
   const int H = kv ? p->Hkv : p->Hq;
   const int64_t elems = (p->B - 1) * s[0] + (H - 1) * s[1] + (int64_t)(p->n - 1) * s[2] + p->d;
   return ((size_t)elems * (p->dtype == SA_BF16 ? 2 : 4) + 255) / 256 * 256;
 }
+
+// The rotated copies of q and k.
+size_t rope_bytes(const sa_problem* p) { return span_bytes(p, false) + span_bytes(p, true); }
 
 float scale_of(const sa_problem* p) {
   return p->softmax_scale > 0.f ? p->softmax_scale : 1.0f / std::sqrt((float)p->d);
@@ -146,9 +149,7 @@ size_t sa_workspace_bytes(const sa_problem* p, int op) {
       return bwd_ws_bytes(p->B, p->Hq, p->Hkv, p->n, p->d, p->dtype, nullptr, nullptr);
     case SA_OP_FORWARD_ROPE: {
       if (check_problem(p) != SA_OK || p->d % 2 != 0) return (size_t)-1;
-      FwdArgs a = fwd_args(p, p, p, p, false);      // pointers unused by the support test
-      if (tc_forward_supported(a, p->dtype)) return 0;
-      return span_bytes(p, false) + span_bytes(p, true);
+      return rope_bytes(p) + branch_bytes(p);
     }
     default:
       return (size_t)-1;
@@ -242,22 +243,31 @@ sa_status sa_rope_apply(const sa_problem* p, int32_t kv, const void* x, const fl
 }
 
 namespace {
-// Where the fused rotation does not apply: rotated copies of q and k in the workspace.
+// Rotated copies of q and k in the workspace, in the layout of the originals.
 sa_status rope_prepass(const sa_problem* p, const void*& q, const void*& k, const float* rope_cos,
                        const float* rope_sin, void* ws, size_t ws_bytes, cudaStream_t st) {
-  const size_t qb = span_bytes(p, false), kb = span_bytes(p, true);
   if (!ws || !aligned16(ws)) return SA_ERR_INVALID_ARG;
-  if (ws_bytes < qb + kb) return SA_ERR_WORKSPACE;
+  if (ws_bytes < rope_bytes(p)) return SA_ERR_WORKSPACE;
   void* qr = ws;
-  void* kr = (char*)ws + qb;
-  if (launch_rope_apply(q, qr, p->B, p->Hq, p->n, p->d, p->q_stride, p->dtype, rope_cos, rope_sin,
-                        false, st) != cudaSuccess ||
-      launch_rope_apply(k, kr, p->B, p->Hkv, p->n, p->d, p->kv_stride, p->dtype, rope_cos,
-                        rope_sin, false, st) != cudaSuccess)
+  void* kr = (char*)ws + span_bytes(p, false);
+  if (launch_rope_qk(q, qr, p->Hq, p->q_stride, k, kr, p->Hkv, p->kv_stride, p->B, p->n, p->d,
+                     p->dtype, rope_cos, rope_sin, st) != cudaSuccess)
     return SA_ERR_CUDA;
   q = qr;
   k = kr;
   return SA_OK;
+}
+
+// Rotation inside the gather or as a pass of its own?  A K row is gathered, and would be turned,
+// once per query tile that meets it, at ~45 instructions per 16 bytes; the pass turns it once, at
+// HBM speed (32/8 heads of 128, n = 8192, w = 1024: 840 us against 12 + 230 us).  In the gather
+// stay callers without room for the rotated copies, and the small single-branch calls, which are
+// promised to be one launch: below 16 MB of Q.
+bool rope_in_gather(const sa_problem* p, bool one_launch, const void* ws, size_t ws_bytes) {
+  FwdArgs probe = fwd_args(p, p, p, p, false);        // pointers unused by the support test
+  if (!tc_forward_supported(probe, p->dtype)) return false;
+  if (!ws || !aligned16(ws) || ws_bytes < rope_bytes(p)) return true;
+  return one_launch && (int64_t)p->B * p->Hq * p->n * p->d < (8 << 20);
 }
 }  // namespace
 
@@ -276,7 +286,7 @@ sa_status sa_forward_rope(const sa_problem* p, const void* q, const void* k, con
   if ((s = maybe_validate(p, perm, inv, st)) != SA_OK) return s;
   FwdArgs a = fwd_args(p, q, k, v, false);
   a.perm = perm; a.inv = inv; a.y = y; a.lse = lse;
-  if (tc_forward_supported(a, p->dtype)) {
+  if (rope_in_gather(p, true, ws, ws_bytes)) {
     a.rope_cos = rope_cos; a.rope_sin = rope_sin;
   } else {
     if ((s = rope_prepass(p, a.q, a.k, rope_cos, rope_sin, ws, ws_bytes, st)) != SA_OK) return s;
@@ -304,20 +314,20 @@ sa_status sa_swa_gated_forward_rope(const sa_problem* p, const void* q, const vo
     return SA_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)stream;
   if ((s = maybe_validate(p, perm, inv, st)) != SA_OK) return s;
-  FwdArgs probe = fwd_args(p, q, k, v, false);
-  const bool fused = tc_forward_supported(probe, p->dtype);
-  if (!fused && (s = rope_prepass(p, q, k, rope_cos, rope_sin, ws, ws_bytes, st)) != SA_OK)
+  const bool in_gather = rope_in_gather(p, false, ws, ws_bytes);
+  if (!in_gather && (s = rope_prepass(p, q, k, rope_cos, rope_sin, ws, ws_bytes, st)) != SA_OK)
     return s;
   // SA branch first, the local branch combines (see sa_swa_gated_forward)
-  void* sa_rows = y_sa ? y_sa : y;
+  const bool scratch = !in_gather && ws_bytes >= rope_bytes(p) + branch_bytes(p);
+  void* sa_rows = y_sa ? y_sa : (scratch ? (char*)ws + rope_bytes(p) : y);
   FwdArgs a = fwd_args(p, q, k, v, false);
   a.perm = perm; a.inv = inv; a.y = sa_rows; a.lse = lse_sa;
-  if (fused) { a.rope_cos = rope_cos; a.rope_sin = rope_sin; }
+  if (in_gather) { a.rope_cos = rope_cos; a.rope_sin = rope_sin; }
   if (run_forward(a, p->dtype, st) != cudaSuccess) return SA_ERR_CUDA;
   FwdArgs b = fwd_args(p, q, k, v, true);
   b.y = y; b.y_branch = y_swa; b.lse = lse_swa;
   b.y_other = sa_rows; b.gate_logits = gate_logits;
-  if (fused) { b.rope_cos = rope_cos; b.rope_sin = rope_sin; }
+  if (in_gather) { b.rope_cos = rope_cos; b.rope_sin = rope_sin; }
   return from_cuda(run_forward(b, p->dtype, st));
 }
 

@@ -162,6 +162,11 @@ cudaError_t launch_rope_apply(const void* x, void* out, int B, int H, int n, int
                               const int64_t s[3], int dtype, const float* cs, const float* sn,
                               bool inverse, cudaStream_t st);
 
+// Q and K in one launch where the 16-byte kernel applies.
+cudaError_t launch_rope_qk(const void* q, void* qr, int Hq, const int64_t qs[3], const void* k,
+                           void* kr, int Hkv, const int64_t ks[3], int B, int n, int d, int dtype,
+                           const float* cs, const float* sn, cudaStream_t st);
+
 bool gate_forward_wide(int64_t rows, int dm, const void* y_sa, const void* y_swa, int64_t ld_y,
                        const void* w_sa, const void* w_swa, void* out, int64_t ld_out,
                        int* status, int sms, cudaStream_t st, cudaError_t* err);
