@@ -11,6 +11,7 @@ where the C functions take device pointers.
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 from typing import Optional
 
@@ -129,6 +130,24 @@ def load_library(path: Optional[str] = None) -> ctypes.CDLL:
     return lib
 
 
+_nat = None
+
+
+def load_native():
+    """The C++ module of the per-layer calls (built first if its source is newer)."""
+    global _nat
+    if _nat is None:
+        load_library()
+        if _build.native_stale():
+            _build.build_native()
+        spec = importlib.util.spec_from_file_location(__package__ + "._native", _build.NATIVE)
+        module = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(module)
+        module.set_error_class(SaError)
+        _nat = module
+    return _nat
+
+
 def status_string(status: int) -> str:
     return load_library().sa_status_string(int(status)).decode()
 
@@ -217,15 +236,10 @@ def _same_layout(ref: torch.Tensor, *others):
 def sa_make_perm(seed: int, layer: int, B: int, n: int, device="cuda", perm=None, inv=None,
                  ws=None):
     """One uniform permutation per sequence and its inverse (int32 [B,n] each)."""
-    lib = load_library()
-    perm = torch.empty(B, n, dtype=torch.int32, device=device) if perm is None else perm
-    inv = torch.empty(B, n, dtype=torch.int32, device=device) if inv is None else inv
-    p = SaProblem(B=B, n=n)
-    nbytes = sa_workspace_bytes(p, OP_MAKE_PERM)
-    ws = _workspace(nbytes, perm.device, ws)
-    _check(lib.sa_make_perm(int(seed) & (2 ** 64 - 1), int(layer), B, n, _ptr(perm), _ptr(inv),
-                            _ptr(ws), ws.numel(), _stream()), "sa_make_perm")
-    return perm, inv
+    if device != "cuda":
+        perm = torch.empty(B, n, dtype=torch.int32, device=device) if perm is None else perm
+        inv = torch.empty(B, n, dtype=torch.int32, device=device) if inv is None else inv
+    return (_nat or load_native()).make_perm(seed, layer, B, n, perm, inv, ws)
 
 
 STATIC_SCRATCH_BYTES = 4 << 20
@@ -252,16 +266,7 @@ def sa_make_perm_static(seed: int, layer: int, B: int, n: int, perm: torch.Tenso
 def sa_forward(q, k, v, perm, inv, w, flags=CAUSAL, scale=0.0, y=None, want_lse=False,
                lse=None):
     """SA forward; returns y (and lse when asked)."""
-    lib = load_library()
-    _same_layout(k, v)
-    p = make_problem(q, k, w, flags, scale)
-    y = torch.empty_like(q) if y is None else y
-    _same_layout(q, y)
-    if want_lse and lse is None:
-        lse = torch.empty(q.shape[:3], dtype=torch.float32, device=q.device)
-    _check(lib.sa_forward(ctypes.byref(p), _ptr(q), _ptr(k), _ptr(v), _ptr(perm), _ptr(inv),
-                          _ptr(y), _ptr(lse), None, 0, _stream()), "sa_forward")
-    return (y, lse) if (want_lse or lse is not None) else y
+    return (_nat or load_native()).forward(q, k, v, perm, inv, w, flags, scale, y, want_lse, lse)
 
 
 def sa_swa_forward(q, k, v, w, flags=CAUSAL | SWA_ONE_SIDED, scale=0.0, y=None, want_lse=False,
@@ -353,53 +358,19 @@ def sa_swa_gated_forward(q, k, v, perm, inv, gate_logits, w, flags=CAUSAL | SWA_
     when neither branch output is kept: the local branch's launch then combines with its idle
     warps instead of in the row threads' epilogue.  ``fused_epilogue=True`` drops a given
     ``ws``.  Two launches either way."""
-    lib = load_library()
-    _same_layout(k, v)
-    out = dict(out or {})
-    if save_for_bwd:
-        flags |= SAVE_FOR_BWD
-        for name in ("y_sa", "y_swa"):
-            out.setdefault(name, torch.empty_like(q))
-        for name in ("lse_sa", "lse_swa"):
-            out.setdefault(name, torch.empty(q.shape[:3], dtype=torch.float32, device=q.device))
-    y = out.setdefault("y", torch.empty_like(q))
-    _same_layout(q, y, out.get("y_sa"), out.get("y_swa"))
-    p = make_problem(q, k, w, flags, scale)
-    if fused_epilogue:
-        ws = None
-    _check(lib.sa_swa_gated_forward(
-        ctypes.byref(p), _ptr(q), _ptr(k), _ptr(v), _ptr(perm), _ptr(inv), _ptr(gate_logits),
-        _ptr(y), _ptr(out.get("y_sa")), _ptr(out.get("y_swa")), _ptr(out.get("lse_sa")),
-        _ptr(out.get("lse_swa")), _ptr(ws), 0 if ws is None else ws.numel(), _stream()),
-        "sa_swa_gated_forward")
-    if save_for_bwd:
-        return y, out["y_sa"], out["y_swa"], out["lse_sa"], out["lse_swa"]
-    return y
+    o = out or {}
+    return (_nat or load_native()).gated_forward(
+        q, k, v, perm, inv, gate_logits, w, flags, scale, save_for_bwd, o.get("y"), o.get("y_sa"),
+        o.get("y_swa"), o.get("lse_sa"), o.get("lse_swa"), None if fused_epilogue else ws)
 
 
 def sa_backward(q, k, v, perm, inv, gate_logits, y_sa, y_swa, lse_sa, lse_swa, dy, w,
                 flags=CAUSAL | SWA_ONE_SIDED, scale=0.0, ws=None, out=None):
     """Backward of the (gated) forward.  Returns (dq, dk, dv, dgate_logits or None)."""
-    lib = load_library()
-    _same_layout(k, v)
-    _same_layout(q, dy, y_sa, y_swa)
-    out = dict(out or {})
-    dq = out.setdefault("dq", torch.empty_like(q))
-    dk = out.setdefault("dk", torch.empty_like(k))
-    dv = out.setdefault("dv", torch.empty_like(v))
-    _same_layout(q, dq)
-    _same_layout(k, dk, dv)
-    dgate = None
-    if gate_logits is not None:
-        dgate = out.setdefault("dgate", torch.empty(2, q.shape[1], dtype=torch.float32,
-                                                    device=q.device))
-    p = make_problem(q, k, w, flags, scale)
-    ws = _workspace(sa_workspace_bytes(p, OP_BACKWARD), q.device, ws)
-    _check(lib.sa_backward(
-        ctypes.byref(p), _ptr(q), _ptr(k), _ptr(v), _ptr(perm), _ptr(inv), _ptr(gate_logits),
-        _ptr(y_sa), _ptr(y_swa), _ptr(lse_sa), _ptr(lse_swa), _ptr(dy), _ptr(dq), _ptr(dk),
-        _ptr(dv), _ptr(dgate), _ptr(ws), ws.numel(), _stream()), "sa_backward")
-    return dq, dk, dv, dgate
+    o = out or {}
+    return (_nat or load_native()).backward(
+        q, k, v, perm, inv, gate_logits, y_sa, y_swa, lse_sa, lse_swa, dy, w, flags, scale, ws,
+        o.get("dq"), o.get("dk"), o.get("dv"), o.get("dgate"))
 
 
 def sa_coverage(perm, inv, w, flags, src, want_row_count=True, ws=None):
