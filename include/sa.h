@@ -76,7 +76,7 @@ typedef enum {
   SA_OP_GATED_FORWARD = 3,
   SA_OP_BACKWARD = 4,
   SA_OP_COVERAGE = 5,
-  SA_OP_GATED_FORWARD_SCRATCH = 6, /* optional scratch of sa_swa_gated_forward, see there */
+  SA_OP_GATED_FORWARD_SCRATCH = 6, /* accepted by sa_swa_gated_forward, see there           */
   SA_OP_FORWARD_ROPE = 7           /* sa_forward_rope / sa_swa_gated_forward_rope           */
 } sa_op;
 
@@ -150,14 +150,10 @@ sa_status sa_swa_forward(const sa_problem* p, const void* q, const void* k, cons
  * y = sigmoid(gate_logits[0,hq]) * y_sa + sigmoid(gate_logits[1,hq]) * y_swa.
  * y: out.  y_sa, y_swa, lse_sa, lse_swa: out, nullable unless SA_SAVE_FOR_BWD; the
  * branch outputs are stored in the run dtype before they are combined.
- * Two launches: the SA branch writes its ungated rows (to y_sa, else to ws, else to y itself),
- * then the local branch, whose rows are consecutive tokens, reads them back, applies both
- * gates and writes y.  ws is optional (sa_workspace_bytes(.., SA_OP_GATED_FORWARD) is 0): with
- * at least sa_workspace_bytes(.., SA_OP_GATED_FORWARD_SCRATCH) bytes (one branch output in
- * q's layout) a caller that keeps neither branch output still gets the faster form of the
- * combination, in which the local branch stores its rows (rounded to the run dtype) and two
- * otherwise idle warps of the same launch combine them; without any such buffer the row
- * threads combine in their epilogue, from unrounded local rows. */
+ * Two launches: the SA branch writes its ungated rows (to y_sa, else to y itself), then the local
+ * branch, whose rows are consecutive tokens, reads them back in its epilogue, applies both gates
+ * and writes y.  ws is not needed (sa_workspace_bytes(.., SA_OP_GATED_FORWARD) is 0); scratch of
+ * SA_OP_GATED_FORWARD_SCRATCH bytes is accepted and left alone. */
 sa_status sa_swa_gated_forward(const sa_problem* p, const void* q, const void* k,
                                const void* v, const int32_t* perm, const int32_t* inv,
                                const float* gate_logits, void* y, void* y_sa, void* y_swa,
@@ -208,7 +204,7 @@ int32_t sa_host_forward_plan(int32_t Hq, int32_t Hkv, int32_t n_groups, int32_t 
  *   opposite angle (the transpose: maps a gradient with respect to the rotated tensor back).
  * sa_forward_rope / sa_swa_gated_forward_rope: sa_forward / sa_swa_gated_forward on rotated Q
  *   and K.  With a workspace of sa_workspace_bytes(.., SA_OP_FORWARD_ROPE) bytes (copies of Q and
- *   K and one branch output, in their layouts) the rotation is a pass over Q and K in one launch.
+ *   K in their layouts) the rotation is a pass over Q and K in one launch.
  *   bf16 with d = 64 or 128 also works without a workspace, and for small sa_forward_rope calls
  *   (less than 16 MB of Q) ignores it: the rows are then rotated inside the kernels' row gather,
  *   which is one launch less and turns each K row once per query tile that meets it.  Same

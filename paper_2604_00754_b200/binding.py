@@ -354,10 +354,8 @@ def sa_swa_gated_forward(q, k, v, perm, inv, gate_logits, w, flags=CAUSAL | SWA_
     """Gated SA + SWA forward.  Returns y, or (y, y_sa, y_swa, lse_sa, lse_swa) when saving.
 
     ``out`` may hold preallocated tensors under the keys y, y_sa, y_swa, lse_sa, lse_swa.
-    ``ws``: optional scratch (uint8, OP_GATED_FORWARD_SCRATCH bytes) for the SA branch's rows
-    when neither branch output is kept: the local branch's launch then combines with its idle
-    warps instead of in the row threads' epilogue.  ``fused_epilogue=True`` drops a given
-    ``ws``.  Two launches either way."""
+    ``ws`` (scratch of OP_GATED_FORWARD_SCRATCH bytes) and ``fused_epilogue`` are accepted and
+    change nothing: the gates are applied in the local branch's epilogue.  Two launches."""
     o = out or {}
     return (_nat or load_native()).gated_forward(
         q, k, v, perm, inv, gate_logits, w, flags, scale, save_for_bwd, o.get("y"), o.get("y_sa"),

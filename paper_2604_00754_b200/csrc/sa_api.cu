@@ -149,7 +149,7 @@ size_t sa_workspace_bytes(const sa_problem* p, int op) {
       return bwd_ws_bytes(p->B, p->Hq, p->Hkv, p->n, p->d, p->dtype, nullptr, nullptr);
     case SA_OP_FORWARD_ROPE: {
       if (check_problem(p) != SA_OK || p->d % 2 != 0) return (size_t)-1;
-      return rope_bytes(p) + branch_bytes(p);
+      return rope_bytes(p);
     }
     default:
       return (size_t)-1;
@@ -211,16 +211,13 @@ sa_status sa_swa_gated_forward(const sa_problem* p, const void* q, const void* k
     return SA_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)stream;
   if ((s = maybe_validate(p, perm, inv, st)) != SA_OK) return s;
-  // Two launches.  The SA branch first: its ungated rows land in y_sa, else in the scratch,
-  // else in y itself.  The local branch then owns each output row exactly once and its rows
-  // are consecutive tokens, so the matching SA rows are read back as contiguous runs, both
-  // gates are applied and y is written: by the two warps that have nothing to load when the
-  // local branch's tiles come by TMA (this needs a home for the local rows other than the
-  // buffer the SA rows sit in: y_swa, or y when the SA rows are elsewhere), otherwise in the
-  // row threads' epilogue.  (Reading the scattered rows of the local branch from the SA
-  // branch's epilogue, the other possible order, costs more than a third launch would.)
-  const bool scratch = ws && ws_bytes >= branch_bytes(p);
-  void* sa_rows = y_sa ? y_sa : (scratch ? ws : y);
+  // Two launches.  The SA branch first: its ungated rows land in y_sa, else in y itself.  The
+  // local branch then owns each output row exactly once: its epilogue reads the matching SA row
+  // (the tensor-core kernel in coalesced pieces), applies both gates and writes y.  (Reading the
+  // scattered rows of the local branch from the SA branch's epilogue, the other possible order,
+  // costs more than a third launch would.)
+  (void)ws_bytes;
+  void* sa_rows = y_sa ? y_sa : y;
   FwdArgs a = fwd_args(p, q, k, v, false);
   a.perm = perm; a.inv = inv; a.y = sa_rows; a.lse = lse_sa;
   cudaError_t e = run_forward(a, p->dtype, st);
@@ -318,8 +315,7 @@ sa_status sa_swa_gated_forward_rope(const sa_problem* p, const void* q, const vo
   if (!in_gather && (s = rope_prepass(p, q, k, rope_cos, rope_sin, ws, ws_bytes, st)) != SA_OK)
     return s;
   // SA branch first, the local branch combines (see sa_swa_gated_forward)
-  const bool scratch = !in_gather && ws_bytes >= rope_bytes(p) + branch_bytes(p);
-  void* sa_rows = y_sa ? y_sa : (scratch ? (char*)ws + rope_bytes(p) : y);
+  void* sa_rows = y_sa ? y_sa : y;
   FwdArgs a = fwd_args(p, q, k, v, false);
   a.perm = perm; a.inv = inv; a.y = sa_rows; a.lse = lse_sa;
   if (in_gather) { a.rope_cos = rope_cos; a.rope_sin = rope_sin; }
