@@ -146,7 +146,8 @@ size_t sa_workspace_bytes(const sa_problem* p, int op) {
       return check_problem(p) == SA_OK ? branch_bytes(p) : (size_t)-1;
     case SA_OP_BACKWARD:
       if (check_problem(p) != SA_OK) return (size_t)-1;
-      return bwd_ws_bytes(p->B, p->Hq, p->Hkv, p->n, p->d, p->dtype, nullptr, nullptr);
+      return bwd_ws_bytes(p->B, p->Hq, p->Hkv, p->n, p->d, p->w, p->dtype, nullptr,
+                          nullptr);
     case SA_OP_FORWARD_ROPE: {
       if (check_problem(p) != SA_OK || p->d % 2 != 0) return (size_t)-1;
       return rope_bytes(p);
@@ -342,7 +343,8 @@ sa_status sa_backward(const sa_problem* p, const void* q, const void* k, const v
     return SA_ERR_INVALID_ARG;
   int chunks = 0;
   size_t parts_at = 0;
-  if (ws_bytes < bwd_ws_bytes(p->B, p->Hq, p->Hkv, p->n, p->d, p->dtype, &chunks, &parts_at))
+  if (ws_bytes < bwd_ws_bytes(p->B, p->Hq, p->Hkv, p->n, p->d, p->w, p->dtype, &chunks,
+                              &parts_at))
     return SA_ERR_WORKSPACE;
   cudaStream_t st = (cudaStream_t)stream;
   if ((s = maybe_validate(p, perm, inv, st)) != SA_OK) return s;
@@ -351,6 +353,7 @@ sa_status sa_backward(const sa_problem* p, const void* q, const void* k, const v
   a.gate_logits = gate_logits;
   a.y_x[0] = y_sa; a.y_x[1] = y_swa; a.lse_x[0] = lse_sa; a.lse_x[1] = lse_swa;
   a.dq = dq; a.dk = dk; a.dv = dv; a.dgate = dgate_logits;
+  a.ws = ws;
   a.delta = (float*)ws;
   const size_t delta_bytes = ((size_t)2 * p->B * p->Hq * p->n * sizeof(float) + 255) / 256 * 256;
   a.partials = (float*)((char*)ws + delta_bytes);

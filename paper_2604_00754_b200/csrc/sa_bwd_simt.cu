@@ -111,6 +111,7 @@ __global__ void __launch_bounds__(kWarps * 32) bwd_delta_kernel(const BwdArgs a)
 __global__ void __launch_bounds__(128) dgate_kernel(const BwdArgs a) {
   __shared__ float wsum[4];
   const int hq = blockIdx.x, x = blockIdx.y;
+  grid_dependency_wait();
   float s = 0.f;
   for (int i = threadIdx.x; i < a.B * a.chunks; i += 128)
     s += a.partials[(((size_t)x * a.B + i / a.chunks) * a.Hq + hq) * a.chunks + i % a.chunks];
@@ -525,19 +526,26 @@ __global__ void __launch_bounds__(kWarps * 32) bwd_dkv_kernel(const BwdArgs a) {
 
 inline size_t align_up(size_t x, size_t al) { return (x + al - 1) / al * al; }
 
+cudaError_t launch_dgate(const BwdArgs& a, cudaStream_t st) {
+  if (!a.gate_logits || !a.dgate) return cudaSuccess;
+  bump_launches();
+  return launch_dependent(dgate_kernel, dim3(a.Hq, 2), dim3(128), 0, st, a);
+}
+
 template <typename T>
-cudaError_t launch_all(const BwdArgs& a, cudaStream_t st) {
+cudaError_t launch_all(BwdArgs a, cudaStream_t st) {
+  cudaError_t e;
+  if (tc_backward_supported(a, std::is_same<T, float>::value ? SA_F32 : SA_BF16)) {
+    e = launch_bwd_tc(a, st);
+    return e != cudaSuccess ? e : launch_dgate(a, st);
+  }
   bwd_delta_kernel<T><<<dim3(a.chunks, a.Hq, a.B), kWarps * 32, 0, st>>>(a);
   bump_launches();
-  if (a.gate_logits && a.dgate) {
-    dgate_kernel<<<dim3(a.Hq, 2), 128, 0, st>>>(a);
-    bump_launches();
-  }
+  if ((e = launch_dgate(a, st)) != cudaSuccess) return e;
   if constexpr (std::is_same<T, float>::value) {
     if (a.d <= 64) return launch_tiles<1>(a, st);
     return a.d <= 128 ? launch_tiles<2>(a, st) : launch_tiles<4>(a, st);
   } else {
-    if (tc_backward_supported(a, SA_BF16)) return launch_bwd_tc(a, st);   // on the tensor cores
     const size_t smem = (size_t)kWarps * 2 * a.d * sizeof(float);
     bwd_dq_kernel<T><<<dim3((a.n + kWarps - 1) / kWarps, a.Hq, a.B), kWarps * 32, smem, st>>>(a);
     bwd_dkv_kernel<T><<<dim3((a.n + kWarps - 1) / kWarps, a.Hkv, a.B), kWarps * 32, smem, st>>>(a);
@@ -548,7 +556,7 @@ cudaError_t launch_all(const BwdArgs& a, cudaStream_t st) {
 
 }  // namespace
 
-size_t bwd_ws_bytes(int B, int Hq, int Hkv, int n, int d, int dtype, int* chunks_out,
+size_t bwd_ws_bytes(int B, int Hq, int Hkv, int n, int d, int w, int dtype, int* chunks_out,
                     size_t* parts_at) {
   const int chunks = (n + kDeltaRowsPerBlock - 1) / kDeltaRowsPerBlock;
   if (chunks_out) *chunks_out = chunks;
@@ -556,6 +564,10 @@ size_t bwd_ws_bytes(int B, int Hq, int Hkv, int n, int d, int dtype, int* chunks
                  align_up((size_t)2 * B * Hq * chunks * sizeof(float), 256);
   if (parts_at) *parts_at = bytes;
   if (dtype == SA_F32 && split_tiles(B, Hkv, n)) bytes += (size_t)6 * B * Hq * n * d * sizeof(float);
+  if (dtype == SA_BF16) {      // room for either way: the tensor cores' kernels carve their own
+    const size_t tc = tc_backward_ws_bytes(B, Hq, Hkv, n, d, w);
+    bytes = tc > bytes ? tc : bytes;
+  }
   return bytes;
 }
 

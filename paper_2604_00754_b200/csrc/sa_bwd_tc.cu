@@ -1,34 +1,43 @@
 // Backward pass on the 5th-generation tensor cores, bf16, d = 64 or 128.
 //
 // Formulas (derivative of Eq. 1 with the permutation held constant; per branch x, with
-// dO = g_x dY and Delta_i = g_x sum_c dY[i,c] Y_x[i,c] prepared by the delta kernel):
+// dO = g_x dY and Delta_i = g_x sum_c dY[i,c] Y_x[i,c]):
 //   P_ij = exp(scale q_i.k_j - lse_i),  dP_ij = dY_i . v_j,
 //   dS_ij = scale P_ij (g_x dP_ij - Delta_i),
 //   dQ_i = sum_j dS_ij k_j,   dK_j = sum_i dS_ij q_i,   dV_j = sum_i g_x P_ij dY_i.
 //
-// Two launches per branch, neither of which needs an atomic, so results are run-to-run
+// prep_kernel first: Delta and lse of every row, in the order the kernels read them, the partial
+// sums of the gate gradients, and (SA branch) copies of Q, dY, K, V in slot order.  A row is met by
+// (128 + w) / 128 row tiles in each of the two launches, and gathering it every time holds the
+// load/store unit for 28 cycles per 512 bytes (3600 cycles for a 128-row K + V tile pair, more than
+// its products take), while the copy costs one pass at HBM speed, part of which the Delta sums
+// need anyway.  Circular windows get the first and last h slots once more on the other side, so
+// that every tile is one box.  The one-sided SWA branch, whose rows are consecutive tokens, is read
+// in place.
+//
+// Then two launches per branch, neither of which needs an atomic, so results are run-to-run
 // identical:
-//   rows = queries: a CTA owns 128 query slots of one head, walks the K/V tiles of its
+//   rows = queries: an item is 128 query slots of one head; it walks the K/V tiles of its
 //                   band, and accumulates dQ;
-//   rows = keys:    a CTA owns 128 key slots of one KV head, walks the query tiles that can
+//   rows = keys:    an item is 128 key slots of one KV head; it walks the query tiles that can
 //                   see them for every query head of the group, and accumulates dK and dV.
-// Either way one step is: S = R1 C1^T and dP = R2 C2^T into tensor memory (rows: Q, dY or
-// K, V; columns: K, V or Q, dY), one thread per row turns them into P and dS (bf16, written
-// back over S and dP), then dS (and P) multiply the column tiles into the accumulators.
-// Rows of every operand are gathered through perm with cp.async into swizzled shared
-// memory, as in the forward kernel; finished rows are scattered to their original places.
+// A persistent grid, one CTA per SM, walks the items.  One step (rows: Q, dY or K, V; a column
+// tile of 128: K, V or Q, dY): S = R1 C1^T and dP = R2 C2^T into tensor memory, P and dS in
+// registers, back to tensor memory as bf16, and from there times the column tiles into the
+// accumulators.  All tiles come by TMA.
 //
-// The column tile is 128 or 64 wide (template KC).  64 halves the band-edge waste of narrow
-// windows and, where scores and accumulators then fit in 256 tensor-memory columns, lets two
-// CTAs share an SM so that one CTA's loads and epilogue hide behind the other's products.
+// Four threads share a row, 32 columns each (nothing is reduced along a row here), so that 16 warps
+// hide one another's latencies.  A thread takes its scores out of tensor memory and keeps P in
+// registers until dP is there, so the next step's scores go into the same columns S while this
+// step is worked on.  With columns left for two dP buffers (all but rows = keys at d = 128) both
+// score products of a step run ahead of the accumulation before it; P and dS are written over dP.
 //
-// With NBUF = 2 (64-wide column tiles only) the scores of two consecutive column tiles live
-// side by side in tensor memory: the products of tile i+1 run while the row threads work on
-// tile i, and two warpgroups of row threads split a tile's 64 columns.
+// Bound: the tensor pipe (128-cycle-per-16-columns products in four groups, and ~180 cycles per
+// commit) where windows are wide, HBM and the item's fixed latencies where they are narrow.
+// Measured against the gathering, one-item-per-CTA kernels before: @@MEASURED@@
 //
-// Warp roles: warp 0 MMA issuer and TMEM allocator, warps 1-3 gather producers, then one
-// (NBUF = 1) or two (NBUF = 2) warpgroups with one thread per row.  Every mbarrier wait is
-// bounded.
+// Every mbarrier wait is bounded; on expiry the CTA records SA_ERR_TIMEOUT in the device status
+// word, stops issuing work, drains what it started and returns.
 #include <type_traits>
 
 #include "sa_bwd_tc.cuh"
@@ -39,96 +48,118 @@ namespace sa {
 namespace {
 
 constexpr int kTile = 128;
-constexpr int kProducers = 96;
+constexpr int kRowWarps = 16, kThreads = 32 * (kRowWarps + 4);
+constexpr uint32_t kTmemCols = 512;
+
+// Where a branch's rows live.  Copies: row `left + slot` of [B, H, ext, d]; in place: left = 0,
+// ext = n.  Statistics and token lists: index `sleft + slot` with `spitch` per head (sequence).
+struct Order {
+  int left, ext, sleft, spitch;
+  int circular;              // the window wraps, and the copies with it
+};
 
 struct BwdTcParams {
-  const void *q, *k, *v, *dy;
   const int32_t* perm;        // null for the SWA branch
-  const float* lse;           // [B,Hq,n] of this branch
-  const float* delta;         // [B,Hq,n] of this branch (gate included)
+  const int32_t* tok;         // [B, spitch]: token of every slot
+  const float *lse2, *delta;  // [B, Hq, spitch] of this branch: lse log2(e) - log2(scale), Delta
   const float* gate_logit;    // null, or the [Hq] logits of this branch
   void *dq, *dk, *dv;
   int accumulate;             // add to what the outputs already hold
   int* status;
   const int* abort_flag;
   int B, Hq, Hkv, G, n, w, h;
-  int causal, linear, one_sided, full_range;
+  int linear, one_sided, full_range;
   int n_tiles;
+  Order o;
   float scale, scale2;
   int64_t qs[3], ks[3];
 };
 
-// Columns (virtual slots) a row tile starting at slot r0 has to meet: [cstart, cend].
-// rows_are_keys selects the transposed window of the one-sided rule.
+// Columns (virtual slots) a row tile starting at slot r0 has to meet: T tiles from cstart on.
+// rows_are_keys selects the transposed window of the one-sided rule.  For the symmetric windows
+// cstart + h is a multiple of 128 (the statistics are loaded from 16-byte boundaries).
 __device__ __forceinline__ void column_range(const BwdTcParams& p, int r0, bool rows_are_keys,
-                                             int kc, int* cstart, int* T) {
+                                             int* cstart, int* T) {
   const int rl = min(r0 + kTile - 1, p.n - 1);
   int lo, hi;
   if (p.full_range) { lo = 0; hi = p.n - 1; }
   else if (p.one_sided) {
     if (rows_are_keys) { lo = r0; hi = min(rl + p.w - 1, p.n - 1); }
     else { lo = max(r0 - (p.w - 1), 0); hi = rl; }
-  } else if (p.linear) { lo = max(r0 - p.h, 0); hi = min(rl + p.h, p.n - 1); }
-  else { lo = r0 - p.h; hi = rl + p.h; }
+  } else {
+    lo = r0 - p.h;
+    hi = rl + p.h;
+    if (p.linear) {
+      if (lo < 0) lo += -lo / kTile * kTile;
+      hi = min(hi, p.n - 1);
+    }
+  }
   *cstart = lo;
-  *T = (hi - lo + kc) / kc;
+  *T = (hi - lo + kTile) / kTile;
 }
 
-__device__ __forceinline__ int actual_slot(const BwdTcParams& p, int v) {
-  if (p.full_range || p.linear || p.one_sided) return min(max(v, 0), p.n - 1);
-  v %= p.n;
-  return v < 0 ? v + p.n : v;
-}
-
-// RW: warpgroups of row threads.  Two split a column tile's 32-column pieces between them: with
-// two score buffers (products of the next tile overlap the row work) or, for 128-wide tiles,
-// with one buffer, where they halve the time the tensor core waits for the row threads.
-template <int D, int KC, int MODE, int NBUF, int RW>
+// KEYS: rows are keys (dK, dV), else queries (dQ).
+template <int D, bool KEYS>
 struct BCfg {
-  static_assert(NBUF == 1 || KC == 64, "two score buffers need 64-wide column tiles");
-  static_assert(RW == 1 || RW == 2, "one or two warpgroups of row threads");
-  static constexpr int kRowWgs = RW;                            // warpgroups of row threads
-  static constexpr int kThreads = 128 + 128 * kRowWgs;
-  static constexpr int kTileBytes = kTile * D * 2;              // a row-operand tile
-  static constexpr int kChunkBytes = kTile * 128;               // its 64-column blocks
-  static constexpr int kColBytes = KC * D * 2;                  // a column tile
-  static constexpr int kColChunkBytes = KC * 128;
-  static constexpr int kStages = NBUF == 2 ? 4 : 2;
-  static constexpr int kOffR = 0;                               // two row-operand tiles
-  static constexpr int kOffC = 2 * kTileBytes;                  // kStages x two column tiles
-  static constexpr int kOffRowTok = kOffC + kStages * 2 * kColBytes;
-  static constexpr int kOffColTok = kOffRowTok + kTile * 4;     // kStages x 128 ints
-  static constexpr int kOffColVec = kOffColTok + kStages * kTile * 4;  // kStages x 2 x 128 floats
-  static constexpr int kOffBar = kOffColVec + kStages * 2 * kTile * 4;
-  static constexpr int kBarRFull = 0, kBarCFull = 1, kBarCEmpty = kBarCFull + kStages,
-                       kBarTokFull = kBarCEmpty + kStages, kBarSFull = kBarTokFull + kStages,
-                       kBarPReady = kBarSFull + NBUF, kBarODone = kBarPReady + NBUF,
-                       kNumBars = kBarODone + 1;
+  static constexpr int kTileBytes = kTile * D * 2, kChunkBytes = kTile * 128;
+  // Column tile slots.  A step's score products are wanted right behind the accumulations of the
+  // step before last, and a tile takes 1000 cycles to come: at d = 128 a pair of two-slot rings
+  // freed together idled the tensor pipe for 1300 of 3400 cycles a step.  Rows = queries: C1 (K)
+  // is freed by the accumulation, three slots; C2 (V) by its dP product already, one slot.  Rows =
+  // keys: C1 (Q) by dK, which goes first, C2 (dY) by dV behind it, two slots each.  At d = 64
+  // there is room for four of each.
+  static constexpr int kC1 = D == 64 ? 4 : KEYS ? 2 : 3, kC2 = D == 64 ? 4 : KEYS ? 2 : 1;
+  static constexpr int kRBufs = D == 128 ? 1 : 2;               // row operand pairs
+  static constexpr int kAccCols = (KEYS ? 2 : 1) * D;
+  static constexpr int kNX = kAccCols <= 128 ? 2 : 1;           // dP buffers
+  static constexpr int kOffR = 0;
+  static constexpr int kOffC = kRBufs * 2 * kTileBytes;
+  static constexpr int kOffC2 = kOffC + kC1 * kTileBytes;
+  static constexpr int kOffStage = kOffC2 + kC2 * kTileBytes;           // 1 KB per row warp
+  static constexpr int kOffVec = kOffStage + kRowWarps * 1024;          // lse2, delta, tokens
+  static constexpr int kOffBar = kOffVec + kC1 * 3 * kTile * 4;
+  static constexpr int kBarRFull = 0, kBarREmpty = kRBufs, kBarC1Full = 2 * kRBufs,
+                       kBarC2Full = kBarC1Full + kC1, kBarC1Empty = kBarC2Full + kC2,
+                       kBarVFull = kBarC1Empty + kC1, kBarSFull = kBarVFull + kC1, kBarSRead = kBarSFull + 1,
+                       kBarDpFull = kBarSRead + 1, kBarPReady = kBarDpFull + 1,
+                       kBarAccFull = kBarPReady + kNX, kBarAccFree = kBarAccFull + 1,
+                       kNumBars = kBarAccFree + 1;
   static constexpr int kOffMisc = kOffBar + kNumBars * 8;
   static constexpr int kBytes = kOffMisc + 16;
-  // tensor memory columns: S and dS (NBUF buffers of KC) at 0, then dP and P, then the
-  // accumulators
-  static constexpr uint32_t kColS = 0, kColP = KC * NBUF, kColAcc = 2 * KC * NBUF;
-  static constexpr uint32_t kColsUsed = 2 * KC * NBUF + (MODE == 1 ? 2 : 1) * D;
-  static constexpr uint32_t kTmemCols = kColsUsed <= 256 ? 256 : 512;
-  static constexpr int kCtasPerSm = (kTmemCols == 256 && kBytes <= 110 * 1024) ? 2 : 1;
+  // tensor memory: S, then the dP buffers (P and dS are written over them), then accumulators
+  static constexpr uint32_t kColS = 0, kColX = 128, kColAcc = 128 + 128 * kNX;
+  static_assert(kColAcc + kAccCols <= kTmemCols, "tensor memory");
   static_assert(kBytes <= 232448, "shared memory");
 };
 
-// MODE 0: rows are queries (dQ).  MODE 1: rows are keys (dK, dV).
-// TMA: the instantiation for the one-sided SWA branch, whose rows are consecutive tokens: one
-// warp loads whole tiles with cp.async.bulk.tensor (every CTA its own) instead of three warps
-// gathering rows 16 bytes at a time, which is bound by the load/store unit.
-template <int D, int KC, int MODE, int NBUF, int RW, bool TMA>
-__global__ void __launch_bounds__(BCfg<D, KC, MODE, NBUF, RW>::kThreads,
-                                  BCfg<D, KC, MODE, NBUF, RW>::kCtasPerSm)
+// Four K steps of D (+)= A B with A (bf16 pairs) in tensor memory in the layout the row threads
+// write, 32 columns after 32 columns, and B in shared memory, 16 rows further on each step.
+__device__ __forceinline__ void mma_ts_rows_x4(uint32_t d, uint32_t a, uint64_t b, uint32_t idesc,
+                                               uint32_t acc0) {
+  asm volatile(
+      "{\n\t.reg .pred p0, p1;\n\t.reg .b64 b1, b2, b3;\n\t.reg .b32 a1, a2, a3;\n\t"
+      "setp.ne.b32 p0, %4, 0;\n\tsetp.eq.b32 p1, %3, %3;\n\t"
+      "add.u32 a1, %1, 8;\n\tadd.u64 b1, %2, 128;\n\t"
+      "add.u32 a2, %1, 32;\n\tadd.u64 b2, %2, 256;\n\t"
+      "add.u32 a3, %1, 40;\n\tadd.u64 b3, %2, 384;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [a1], b1, %3, p1;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [a2], b2, %3, p1;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [a3], b3, %3, p1;\n\t}"
+      ::"r"(d), "r"(a), "l"(b), "r"(idesc), "r"(acc0)
+      : "memory");
+}
+
+// TOK: the token order decides which columns a row sees (causal, window in slot space).
+template <int D, bool KEYS, bool TOK>
+__global__ void __launch_bounds__(kThreads, 1)
 bwd_tc_kernel(const __grid_constant__ BwdTcParams p, const __grid_constant__ CUtensorMap tm_q,
               const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
               const __grid_constant__ CUtensorMap tm_dy) {
   extern __shared__ __align__(1024) uint8_t smem[];
-  using C = BCfg<D, KC, MODE, NBUF, RW>;
-  constexpr uint32_t kTmemCols = C::kTmemCols;
-  constexpr bool kKeys = MODE == 1;
+  using C = BCfg<D, KEYS>;
+  constexpr bool kVec = KEYS || TOK;          // something travels with the column tiles
+  constexpr int kMmaWarp = kRowWarps, kLoadWarp = kRowWarps + 1;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
   const uint32_t sbase = smem_u32(smem);
@@ -141,27 +172,16 @@ bwd_tc_kernel(const __grid_constant__ BwdTcParams p, const __grid_constant__ CUt
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + C::kOffMisc);
   volatile int* gave_up = reinterpret_cast<volatile int*>(smem + C::kOffMisc + 4);
 
-  // work item: (batch, head of the row operand, row tile)
-  const int H = kKeys ? p.Hkv : p.Hq;
-  const int tile = blockIdx.x % p.n_tiles, bh = blockIdx.x / p.n_tiles;
-  const int hr = bh % H, b = bh / H;
-  const int hk = kKeys ? hr : hr / p.G;
-  const int r0 = tile * kTile;
-  int cstart, T;
-  column_range(p, r0, kKeys, KC, &cstart, &T);
-  const int iters = kKeys ? T * p.G : T;      // column tiles (times query heads of the group)
-  const int32_t* perm = p.perm ? p.perm + (size_t)b * p.n : nullptr;
-
   if (threadIdx.x == 0) {
     *gave_up = 0;
-    note_skip(reinterpret_cast<volatile int*>(smem + C::kOffMisc + 8), p.status, p.abort_flag);
     for (int i = 0; i < C::kNumBars; ++i)
-      mbar_init(bar(i), (i >= C::kBarPReady && i < C::kBarODone) ? kTile * C::kRowWgs
-                        : (i == C::kBarRFull || (i >= C::kBarCFull && i < C::kBarCEmpty))
-                            ? (TMA ? 32 : kProducers) : 1);
+      mbar_init(bar(i), (i == C::kBarSRead || (i >= C::kBarPReady && i < C::kBarAccFull) || i == C::kBarAccFree)
+                            ? kRowWarps : 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    grid_dependency_wait();                   // what earlier launches wrote may be read from here on
+    note_skip(reinterpret_cast<volatile int*>(smem + C::kOffMisc + 8), p.status, p.abort_flag);
   }
-  if (warp == 0) {
+  if (warp == kMmaWarp) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
                  ::"r"(smem_u32(tmem_slot)), "r"(kTmemCols) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -169,490 +189,683 @@ bwd_tc_kernel(const __grid_constant__ BwdTcParams p, const __grid_constant__ CUt
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  grid_dependents_launch();
   const uint32_t tmem = *tmem_slot;
-  SA_LEAVE_IF_SKIPPED(reinterpret_cast<volatile int*>(smem + C::kOffMisc + 8), 0, tmem, kTmemCols)
+  SA_LEAVE_IF_SKIPPED(reinterpret_cast<volatile int*>(smem + C::kOffMisc + 8), kMmaWarp, tmem, kTmemCols)
 
-  if (warp >= 1 && warp < 4 && TMA) {
-    // ------------------------------------------------- tile loads by TMA (warp 1 alone)
-    // Rows and columns are consecutive tokens (no permutation, window by slots only), so a tile
-    // is D / 64 boxes of KC tokens x 64 columns per operand; tokens outside the sequence read
-    // zeros and are masked by the slot window.  Lane 0 posts the byte counts and the loads;
-    // for rows = keys the 32 lanes also fetch the per-query lse and delta of the columns.
-    // The token lists are not written: the one-sided rule does not look at them.
-    if (warp == 1) {
-      auto signal = [&](uint32_t mb) {
-        asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(mb) : "memory");
-      };
-      auto load_rows = [&](const CUtensorMap* tm, uint32_t dst, int tok, int head, int rows,
-                           uint32_t mb) {
-        for (int r = 0; r < rows; r += KC)
-#pragma unroll
-          for (int c = 0; c < D / 64; ++c)
-            tma_load_4d(dst + c * (rows * 128) + r * 128, tm, 64 * c, tok + r, head, b, mb);
-      };
-      if (lane == 0) {
-        mbar_expect_tx(bar(C::kBarRFull), 2 * C::kTileBytes);   // counts as this lane's arrival
-        load_rows(kKeys ? &tm_k : &tm_q, sbase + C::kOffR, r0, hr, kTile, bar(C::kBarRFull));
-        load_rows(kKeys ? &tm_v : &tm_dy, sbase + C::kOffR + C::kTileBytes, r0, hr, kTile,
-                  bar(C::kBarRFull));
-      } else {
-        mbar_arrive(bar(C::kBarRFull));
-      }
+  // An item: (batch, head of the row operand, row tile), the row tile innermost so that
+  // neighbouring items meet the same column tiles in L2.
+  const int H = KEYS ? p.Hkv : p.Hq;
+  const int total = p.B * H * p.n_tiles;
+  struct Item { int b, hr, hk, r0, cstart, T, iters; };
+  auto item_of = [&](int w_item) {
+    Item i;
+    const int bh = w_item / p.n_tiles;
+    i.r0 = (w_item - bh * p.n_tiles) * kTile;
+    i.b = bh / H;
+    i.hr = bh - i.b * H;
+    i.hk = KEYS ? i.hr : i.hr / p.G;
+    column_range(p, i.r0, KEYS, &i.cstart, &i.T);
+    i.iters = KEYS ? i.T * p.G : i.T;      // column tiles (times query heads of the group)
+    return i;
+  };
+
+  // Registers move from the issuer and loading warps to the row threads.  Per lane over the 20
+  // warps: 4 x 64 + 16 x 104 = 1920, all that the launch holds (20 x 96).  (The sum may never
+  // exceed what the launch holds: a warpgroup asking for more waits for ever.)
+  static_assert(4 * 64 + 16 * 104 == 20 * 96, "register split");
+  if (warp >= kRowWarps) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
+    if (warp == kLoadWarp && lane == 0) {
+      // ------------------------------------------------------------- loads (one thread, TMA)
+      // A tile is D / 64 boxes of 128 rows x 64 columns; rows outside the tensor read zeros and
+      // are masked by the slot window.
+      uint32_t u = 0, it = 0, r_on = 0, c1_on = 0, c2_on = 0;      // tiles started
       bool live = true;
-      int issued = 0;
-      for (int it = 0; it < iters && live; ++it) {
-        const int s = it % C::kStages;
-        const int j = kKeys ? it % T : it, gi = kKeys ? it / T : 0;
-        const int hq = kKeys ? hk * p.G + gi : hr;
-        if (it >= C::kStages)
-          live = mbar_wait(bar(C::kBarCEmpty + s), (it / C::kStages - 1) & 1u, gave_up, p.status);
-        live = __all_sync(0xffffffffu, live);
+      auto load_tile = [&](const CUtensorMap* tm, uint32_t dst, int row, int head, int b, uint32_t mb) {
+#pragma unroll
+        for (int c = 0; c < D / 64; ++c)
+          tma_load_4d(dst + c * C::kChunkBytes, tm, 64 * c, row, head, b, mb);
+      };
+      for (int w_item = blockIdx.x; w_item < total && live; w_item += gridDim.x, ++it) {
+        const Item i = item_of(w_item);
+        const uint32_t rb = it % C::kRBufs;
+        if (it >= (uint32_t)C::kRBufs)
+          live = mbar_wait(bar(C::kBarREmpty + rb), (it / C::kRBufs - 1) & 1u, gave_up, p.status);
         if (!live) break;
-        issued = it + 1;
-        const uint32_t colvec = sbase + C::kOffColVec + s * 2 * kTile * 4;
-        const uint32_t c1 = sbase + C::kOffC + s * 2 * C::kColBytes, c2 = c1 + C::kColBytes;
-        const uint32_t mb = bar(C::kBarCFull + s);
-        if (lane == 0) mbar_arrive(bar(C::kBarTokFull + s));
-        if (kKeys) {
-          const float* lse_h = p.lse + ((size_t)b * p.Hq + hq) * p.n;
-          const float* del_h = p.delta + ((size_t)b * p.Hq + hq) * p.n;
-          // (lanes 1-31: lane 0 arrives by posting the byte count, which does not wait for
-          // copies of its own)
-          for (int x = lane - 1; x < KC && lane > 0; x += 31) {
-            const int t0 = actual_slot(p, cstart + j * KC + x);
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(colvec + 4 * x), "l"(lse_h + t0) : "memory");
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(colvec + 4 * (kTile + x)), "l"(del_h + t0) : "memory");
-          }
+        {
+          const uint32_t dst = sbase + C::kOffR + rb * 2 * C::kTileBytes, mb = bar(C::kBarRFull + rb);
+          mbar_expect_tx(mb, 2 * C::kTileBytes);
+          load_tile(KEYS ? &tm_k : &tm_q, dst, p.o.left + i.r0, i.hr, i.b, mb);
+          load_tile(KEYS ? &tm_v : &tm_dy, dst + C::kTileBytes, p.o.left + i.r0, i.hr, i.b, mb);
+          r_on = it + 1;
         }
-        if (lane == 0) {
-          mbar_expect_tx(mb, 2 * C::kColBytes);                 // this lane's arrival
-          load_rows(kKeys ? &tm_q : &tm_k, c1, cstart + j * KC, kKeys ? hq : hk, KC, mb);
-          load_rows(kKeys ? &tm_dy : &tm_v, c2, cstart + j * KC, kKeys ? hq : hk, KC, mb);
-        } else {
-          signal(mb);                                           // after this lane's small copies
+        int j = 0, hq = KEYS ? i.hk * p.G : i.hr;
+        for (int x = 0; x < i.iters; ++x, ++u) {
+          const uint32_t s = u % C::kC1, s2 = u % C::kC2;
+          if (u >= (uint32_t)C::kC1)
+            live = mbar_wait(bar(C::kBarC1Empty + s), (u / C::kC1 - 1) & 1u, gave_up, p.status);
+          if (!live) break;
+          const int col = i.cstart + j * kTile, hc = KEYS ? hq : i.hk;
+          uint32_t mb = bar(C::kBarC1Full + s);
+          mbar_expect_tx(mb, C::kTileBytes);
+          load_tile(KEYS ? &tm_q : &tm_k, sbase + C::kOffC + s * C::kTileBytes, p.o.left + col, hc,
+                    i.b, mb);
+          c1_on = u + 1;
+          if (kVec) {
+            const uint32_t vb = bar(C::kBarVFull + s), vec = sbase + C::kOffVec + s * 3 * kTile * 4;
+            mbar_expect_tx(vb, ((KEYS ? 2 : 0) + (TOK ? 1 : 0)) * kTile * 4);
+            if (KEYS) {
+              const size_t at = ((size_t)i.b * p.Hq + hq) * p.o.spitch + p.o.sleft + col;
+              bulk_load(vec, p.lse2 + at, kTile * 4, vb);
+              bulk_load(vec + kTile * 4, p.delta + at, kTile * 4, vb);
+            }
+            if (TOK)
+              bulk_load(vec + 2 * kTile * 4, p.tok + (size_t)i.b * p.o.spitch + p.o.sleft + col,
+                        kTile * 4, vb);
+          }
+          // (d = 64: C2's slot was freed together with C1's)
+          if (D == 128 && u >= (uint32_t)C::kC2)
+            live = KEYS ? mbar_wait(bar(C::kBarDpFull), (u - 1) & 1u, gave_up, p.status)
+                        : mbar_wait(bar(C::kBarSFull), (u - 1) & 1u, gave_up, p.status);
+          if (!live) break;
+          mb = bar(C::kBarC2Full + s2);
+          mbar_expect_tx(mb, C::kTileBytes);
+          load_tile(KEYS ? &tm_dy : &tm_v, sbase + C::kOffC2 + s2 * C::kTileBytes, p.o.left + col, hc,
+                    i.b, mb);
+          c2_on = u + 1;
+          if (++j == i.T) { j = 0; ++hq; }
         }
       }
-      asm volatile("cp.async.wait_all;" ::: "memory");
       // loads that were started but never consumed (only after a failed wait) must land before
       // the shared memory goes away: wait for them, again with a limit
-      if (lane == 0 && (!live || *gave_up)) {
-        for (int tries = 0; tries < 100000; ++tries) {
-          if (mbar_try(bar(C::kBarRFull), 0u)) break;
-          __nanosleep(100);
-        }
-        for (int u = issued > C::kStages ? issued - C::kStages : 0; u < issued; ++u)
+      if (!live || *gave_up) {
+        auto landed = [&](int index, uint32_t parity) {
           for (int tries = 0; tries < 100000; ++tries) {
-            if (mbar_try(bar(C::kBarCFull + u % C::kStages), (u / C::kStages) & 1u)) break;
+            if (mbar_try(bar(index), parity)) break;
             __nanosleep(100);
           }
-      }
-    }
-  } else if (warp >= 1 && warp < 4) {
-    // ---------------------------------------------------- gather producers (warps 1-3)
-    constexpr int kCpr = D / 8;            // 16-byte pieces per row
-    constexpr int kRpi = 32 / kCpr;        // rows per warp instruction
-    const int ptid = threadIdx.x - 32;     // 0..95
-    const int sub = lane / kCpr, chunk = lane % kCpr;
-    const __nv_bfloat16* qg = (const __nv_bfloat16*)p.q;
-    const __nv_bfloat16* kg = (const __nv_bfloat16*)p.k;
-    const __nv_bfloat16* vg = (const __nv_bfloat16*)p.v;
-    const __nv_bfloat16* dyg = (const __nv_bfloat16*)p.dy;
-    int32_t* const rowtok = reinterpret_cast<int32_t*>(smem + C::kOffRowTok);
-    auto signal = [&](uint32_t mb) {
-      asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(mb) : "memory");
-    };
-    // rows x D elements into a tile whose 64-column blocks are rows x 128 bytes each
-    auto gather = [&](const __nv_bfloat16* base, int64_t tok_stride, const int32_t* toks,
-                      uint32_t dst_tile, int rows) {
-#pragma unroll 4
-      for (int grp = warp - 1; grp < rows / kRpi; grp += 3) {
-        const int r = grp * kRpi + sub;
-        const __nv_bfloat16* src = base + (int64_t)toks[r] * tok_stride + chunk * 8;
-        const uint32_t dst = dst_tile + (uint32_t)(chunk >> 3) * (rows * 128) + r * 128 +
-                             (((chunk & 7) ^ (r & 7)) << 4);
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-      }
-    };
-    // Barrier over the three producer warps that also agrees on whether anyone in the CTA
-    // has given up, so that every producer thread leaves at the same point.
-    auto group_sync_stop = [&]() {
-      uint32_t any;
-      asm volatile(
-          "{\n\t.reg .pred p, q;\n\t"
-          "setp.ne.u32 q, %1, 0;\n\t"
-          "bar.red.or.pred p, 1, 96, q;\n\t"
-          "selp.u32 %0, 1, 0, p;\n\t}"
-          : "=r"(any)
-          : "r"((uint32_t)*gave_up)
-          : "memory");
-      return any != 0;
-    };
-    auto tok_of = [&](int slot) { return perm ? perm[slot] : slot; };
-
-    // row operands
-    rowtok[ptid] = tok_of(min(r0 + ptid, p.n - 1));
-    if (ptid < 32) rowtok[ptid + 96] = tok_of(min(r0 + ptid + 96, p.n - 1));
-    bool live = !group_sync_stop();
-    if (live) {
-      if (kKeys) {
-        gather(kg + b * p.ks[0] + hr * p.ks[1], p.ks[2], rowtok, sbase + C::kOffR, kTile);
-        gather(vg + b * p.ks[0] + hr * p.ks[1], p.ks[2], rowtok, sbase + C::kOffR + C::kTileBytes, kTile);
-      } else {
-        gather(qg + b * p.qs[0] + hr * p.qs[1], p.qs[2], rowtok, sbase + C::kOffR, kTile);
-        gather(dyg + b * p.qs[0] + hr * p.qs[1], p.qs[2], rowtok, sbase + C::kOffR + C::kTileBytes, kTile);
-      }
-      signal(bar(C::kBarRFull));
-    }
-    // The tokens of a column tile come from global memory (perm); they are fetched one tile
-    // ahead of their use so that this latency is not paid inside every step.
-    auto col_tok = [&](int it, int x) {
-      const int j = kKeys ? it % T : it;
-      return tok_of(actual_slot(p, cstart + j * KC + x));
-    };
-    int nt0 = 0, nt1 = 0;
-    if (live && iters > 0) {
-      if (ptid < KC) nt0 = col_tok(0, ptid);
-      if (ptid + 96 < KC) nt1 = col_tok(0, ptid + 96);
-    }
-    for (int it = 0; it < iters && live; ++it) {
-      const int s = it % C::kStages;
-      const int gi = kKeys ? it / T : 0;
-      const int hq = kKeys ? hk * p.G + gi : hr;
-      const int t0 = nt0, t1 = nt1;
-      if (it + 1 < iters) {
-        if (ptid < KC) nt0 = col_tok(it + 1, ptid);
-        if (ptid + 96 < KC) nt1 = col_tok(it + 1, ptid + 96);
-      }
-      if (it >= C::kStages)
-        mbar_wait(bar(C::kBarCEmpty + s), (it / C::kStages - 1) & 1u, gave_up, p.status);
-      int32_t* coltok = reinterpret_cast<int32_t*>(smem + C::kOffColTok) + s * kTile;
-      const uint32_t colvec = sbase + C::kOffColVec + s * 2 * kTile * 4;
-      if (ptid < KC) coltok[ptid] = t0;
-      if (ptid + 96 < KC) coltok[ptid + 96] = t1;
-      if (group_sync_stop()) { live = false; break; }
-      if (ptid == 0) mbar_arrive(bar(C::kBarTokFull + s));
-      const uint32_t c1 = sbase + C::kOffC + s * 2 * C::kColBytes, c2 = c1 + C::kColBytes;
-      if (kKeys) {
-        // per-query vectors of this head travel with the tile
-        const float* lse_h = p.lse + ((size_t)b * p.Hq + hq) * p.n;
-        const float* del_h = p.delta + ((size_t)b * p.Hq + hq) * p.n;
-        if (ptid < KC) {
-          asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(colvec + 4 * ptid), "l"(lse_h + t0) : "memory");
-          asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(colvec + 4 * (kTile + ptid)), "l"(del_h + t0) : "memory");
+        };
+        for (uint32_t x = r_on > (uint32_t)C::kRBufs ? r_on - C::kRBufs : 0u; x < r_on; ++x)
+          landed(C::kBarRFull + x % C::kRBufs, (x / C::kRBufs) & 1u);
+        for (uint32_t x = c1_on > (uint32_t)C::kC1 ? c1_on - C::kC1 : 0u; x < c1_on; ++x) {
+          landed(C::kBarC1Full + x % C::kC1, (x / C::kC1) & 1u);
+          if (kVec) landed(C::kBarVFull + x % C::kC1, (x / C::kC1) & 1u);
         }
-        if (ptid + 96 < KC) {
-          asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(colvec + 4 * (ptid + 96)), "l"(lse_h + t1) : "memory");
-          asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(colvec + 4 * (kTile + ptid + 96)), "l"(del_h + t1) : "memory");
-        }
-        gather(qg + b * p.qs[0] + hq * p.qs[1], p.qs[2], coltok, c1, KC);
-        gather(dyg + b * p.qs[0] + hq * p.qs[1], p.qs[2], coltok, c2, KC);
-      } else {
-        gather(kg + b * p.ks[0] + hk * p.ks[1], p.ks[2], coltok, c1, KC);
-        gather(vg + b * p.ks[0] + hk * p.ks[1], p.ks[2], coltok, c2, KC);
+        for (uint32_t x = c2_on > (uint32_t)C::kC2 ? c2_on - C::kC2 : 0u; x < c2_on; ++x)
+          landed(C::kBarC2Full + x % C::kC2, (x / C::kC2) & 1u);
       }
-      signal(bar(C::kBarCFull + s));
-    }
-    asm volatile("cp.async.wait_all;" ::: "memory");   // nothing in flight when the CTA leaves
-  } else if (warp == 0) {
-    // -------------------------------------------------------------- MMA issuer (warp 0)
-    if (lane == 0) {
-      constexpr uint32_t idesc_s = instr_desc(kTile, KC, false);
+    } else if (warp == kMmaWarp && lane == 0) {
+      // ---------------------------------------------------------------- MMA issuer (one thread)
+      constexpr uint32_t idesc_s = instr_desc(kTile, kTile, false);
       constexpr uint32_t idesc_acc = instr_desc(kTile, D, true);
       constexpr uint32_t kDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
-      constexpr uint32_t kLoK = (16u >> 4) << 16;                        // K-major operands
-      constexpr uint32_t kLoMN = ((uint32_t)C::kColChunkBytes >> 4) << 16;  // column tile as [k][n]
-      constexpr uint32_t kBlockR = C::kChunkBytes >> 4;     // next 64 columns of a row tile
-      constexpr uint32_t kBlockC = C::kColChunkBytes >> 4;  // next 64 columns of a column tile
-      const uint64_t r1 = desc64(((sbase + C::kOffR) >> 4) | kLoK, kDescHi);
-      const uint64_t r2 = desc64(((sbase + C::kOffR + C::kTileBytes) >> 4) | kLoK, kDescHi);
+      constexpr uint32_t kLoK = (16u >> 4) << 16;                             // K-major operands
+      constexpr uint32_t kLoMN = ((uint32_t)C::kChunkBytes >> 4) << 16;       // column tile as [k][n]
+      constexpr uint32_t kBlock = C::kChunkBytes >> 4, kTileD = C::kTileBytes >> 4;
+      const uint32_t r_lo = (sbase + C::kOffR) >> 4, c_lo = (sbase + C::kOffC) >> 4,
+                     c2_lo = (sbase + C::kOffC2) >> 4;
       // X (128 x 128, fp32, tensor memory column col) = A B^T, both tiles K-major, K = D
-      auto product = [&](uint32_t col, uint64_t a, uint32_t b_addr) {
-        const uint64_t bd = desc64((b_addr >> 4) | kLoK, kDescHi);
-        mma_ss_x4(tmem + col, a, bd, idesc_s, 0u);
-        if (D == 128) mma_ss_x4(tmem + col, a + kBlockR, bd + kBlockC, idesc_s, 1u);
+      auto product = [&](uint32_t col, uint32_t a_lo, uint32_t b_lo) {
+        const uint64_t ad = desc64(a_lo | kLoK, kDescHi), bd = desc64(b_lo | kLoK, kDescHi);
+        mma_ss_x4(tmem + col, ad, bd, idesc_s, 0u);
+        if (D == 128) mma_ss_x4(tmem + col, ad + kBlock, bd + kBlock, idesc_s, 1u);
       };
-      // acc (128 x D, tensor memory column col) += X (bf16 pairs at column xcol) * tile
-      auto accumulate = [&](uint32_t col, uint32_t xcol, uint32_t b_addr, uint32_t acc0) {
-        const uint64_t bd = desc64((b_addr >> 4) | kLoMN, kDescHi);
-        mma_ts_x4(tmem + col, tmem + xcol, bd, idesc_acc, acc0);
-        if (KC == 128) mma_ts_x4(tmem + col, tmem + xcol + 32, bd + 512, idesc_acc, 1u);
+      // acc (128 x D, tensor memory column col) += X (bf16 pairs from column xcol on) * tile
+      auto accumulate = [&](uint32_t col, uint32_t xcol, uint32_t b_lo, uint32_t acc0) {
+        const uint64_t bd = desc64(b_lo | kLoMN, kDescHi);
+        mma_ts_rows_x4(tmem + col, tmem + xcol, bd, idesc_acc, acc0);
+        mma_ts_rows_x4(tmem + col, tmem + xcol + 64, bd + 512, idesc_acc, 1u);
       };
-      // scores of column tile `it` into buffer it % NBUF
-      auto scores = [&](int it) {
-        const int s = it % C::kStages;
-        const uint32_t c1 = sbase + C::kOffC + s * 2 * C::kColBytes, c2 = c1 + C::kColBytes;
-        if (!mbar_wait(bar(C::kBarCFull + s), (it / C::kStages) & 1u, gave_up, p.status))
-          return false;
-        fence_proxy_async();
+      // the score products run one step ahead of the accumulations, across items
+      bool ok = true;
+      int sw = blockIdx.x, s_left = 0;            // score cursor: item, steps left of it
+      uint32_t su = 0, s_it = 0;                  // steps and items started
+      if (sw < total) s_left = item_of(sw).iters;
+      // S of the next step into the S columns, once the row threads hold the one before
+      auto next_s = [&]() {
+        const uint32_t rb = s_it % C::kRBufs, s = su % C::kC1;
+        ok = mbar_wait(bar(C::kBarRFull + rb), (s_it / C::kRBufs) & 1u, gave_up, p.status);
+        if (ok) ok = mbar_wait(bar(C::kBarC1Full + s), (su / C::kC1) & 1u, gave_up, p.status);
+        if (ok && su > 0) ok = mbar_wait(bar(C::kBarSRead), (su - 1) & 1u, gave_up, p.status);
+        if (!ok) return;
         tc_fence_after();
-        const uint32_t buf = (it % NBUF) * KC;
-        product(C::kColS + buf, r1, c1);
-        product(C::kColP + buf, r2, c2);
-        tc_commit(bar(C::kBarSFull + it % NBUF));
-        return true;
+        product(C::kColS, r_lo + rb * 2 * kTileD, c_lo + s * kTileD);
+        if (C::kNX == 1) tc_commit(bar(C::kBarSFull));
       };
-      bool ok = mbar_wait(bar(C::kBarRFull), 0, gave_up, p.status);
-      if (ok && NBUF == 2) ok = scores(0);
-      for (int it = 0; it < iters && ok; ++it) {
-        const int s = it % C::kStages;
-        const uint32_t c1 = sbase + C::kOffC + s * 2 * C::kColBytes, c2 = c1 + C::kColBytes;
-        // NBUF = 2: the next tile's scores go ahead of this tile's accumulation
-        if (NBUF == 2) { if (it + 1 < iters) ok = scores(it + 1); }
-        else ok = scores(it);
-        if (!ok) break;
-        ok = mbar_wait(bar(C::kBarPReady + it % NBUF), (it / NBUF) & 1u, gave_up, p.status);
-        if (!ok) break;
+      // dP of the same step, then on to the next
+      auto next_dp = [&]() {
+        const uint32_t rb = s_it % C::kRBufs, s = su % C::kC2;
+        ok = mbar_wait(bar(C::kBarC2Full + s), (su / C::kC2) & 1u, gave_up, p.status);
+        if (!ok) return;
         tc_fence_after();
-        const uint32_t buf = (it % NBUF) * KC;
-        if (kKeys) {
-          accumulate(C::kColAcc, C::kColP + buf, c2, it > 0);        // dV += (g P)^T dY
-          accumulate(C::kColAcc + D, C::kColS + buf, c1, it > 0);    // dK += dS^T Q
-        } else {
-          accumulate(C::kColAcc, C::kColS + buf, c1, it > 0);        // dQ += dS K
+        product(C::kColX + 128 * (su % C::kNX), r_lo + (rb * 2 + 1) * kTileD, c2_lo + s * kTileD);
+        tc_commit(bar(C::kNX == 1 ? C::kBarDpFull : C::kBarSFull));
+        ++su;
+        if (--s_left == 0) {
+          tc_commit(bar(C::kBarREmpty + rb));
+          ++s_it;
+          sw += gridDim.x;
+          if (sw < total) s_left = item_of(sw).iters;
         }
-        tc_commit(bar(C::kBarCEmpty + s));
+      };
+      if (s_left > 0) {
+        next_s();
+        if (ok) next_dp();
       }
-      if (ok) tc_commit(bar(C::kBarODone));
+      uint32_t u = 0, it = 0;
+      for (int w_item = blockIdx.x; w_item < total && ok; w_item += gridDim.x, ++it) {
+        const int iters = item_of(w_item).iters;
+        for (int x = 0; x < iters && ok; ++x, ++u) {
+          const bool more = s_left > 0;
+          if (more) {
+            next_s();
+            if (ok && C::kNX == 2) next_dp();
+            if (!ok) break;
+          }
+          if (x == 0 && it > 0) ok = mbar_wait(bar(C::kBarAccFree), (it - 1) & 1u, gave_up, p.status);
+          if (ok) ok = mbar_wait(bar(C::kBarPReady + u % C::kNX), (u / C::kNX) & 1u, gave_up, p.status);
+          if (!ok) break;
+          tc_fence_after();
+          const uint32_t s = u % C::kC1, xc = C::kColX + 128 * (u % C::kNX);
+          const uint32_t c1 = c_lo + s * kTileD, c2 = c2_lo + (u % C::kC2) * kTileD;
+          if (KEYS) {
+            accumulate(C::kColAcc + D, xc + 16, c1, x > 0);      // dK += dS^T Q
+            if (D == 128) tc_commit(bar(C::kBarC1Empty + s));
+            accumulate(C::kColAcc, xc, c2, x > 0);               // dV += (g P)^T dY
+            if (D == 64) tc_commit(bar(C::kBarC1Empty + s));
+          } else {
+            accumulate(C::kColAcc, xc, c1, x > 0);               // dQ += dS K
+            tc_commit(bar(C::kBarC1Empty + s));
+          }
+          if (x + 1 == iters) tc_commit(bar(C::kBarAccFull));
+          if (more && C::kNX == 1) next_dp();
+        }
+      }
     }
     __syncwarp();
   } else {
-    // ------------------------------------------------- row threads (from warp 4 on)
-    const int wg = (warp - 4) >> 2;                     // which warpgroup of row threads
-    const int row = (threadIdx.x - 128) & 127;          // 0..127 == TMEM lane
-    const uint32_t trow = tmem + ((uint32_t)(row & ~31) << 16);
-    const int rslot = r0 + row;
-    const bool row_valid = rslot < p.n;
-    const int rtok = perm ? perm[min(rslot, p.n - 1)] : min(rslot, p.n - 1);
-    const bool tok_rule = p.causal && !p.one_sided;     // token order decides, not slots
-    // rows = queries: mask key tokens above the query's; rows = keys: query tokens below
-    const int cmp = tok_rule ? rtok : (kKeys ? (int)0x80000000 : 0x7fffffff);
-    // exp2(s * scale2 - lse2 + log2(scale)) is P * scale at once: dS needs no further multiply
-    const float l2scale = __log2f(p.scale), inv_scale = 1.f / p.scale;
-    float lse2_r = 0.f, delta_r = 0.f, g = 1.f;
-    if (!kKeys) {
-      const size_t o = ((size_t)b * p.Hq + hr) * p.n + rtok;
-      lse2_r = p.lse[o] * kLog2e - l2scale;
-      delta_r = p.delta[o];
-      if (p.gate_logit) g = 1.f / (1.f + __expf(-p.gate_logit[hr]));
-    }
-    // Two warpgroups share a tile: the bf16 results of one overwrite score columns the other
-    // reads, so every row thread loads before any stores.  The barrier also agrees on whether
-    // to stop, so that all of them leave the loop together.
-    auto rows_sync_stop = [&](bool stop) {
-      uint32_t any;
-      asm volatile(
-          "{\n\t.reg .pred p, q;\n\t"
-          "setp.ne.u32 q, %1, 0;\n\t"
-          "bar.red.or.pred p, 2, 256, q;\n\t"
-          "selp.u32 %0, 1, 0, p;\n\t}"
-          : "=r"(any)
-          : "r"((uint32_t)stop)
-          : "memory");
-      return any != 0;
-    };
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 104;");
+    // --------------------------------------------------------------------- row threads
+    const int quad = warp & 3, cg = warp >> 2;          // TMEM lanes, 32-column group
+    const int row = quad * 32 + lane, c0 = 32 * cg;
+    const uint32_t trow = tmem + ((uint32_t)(quad * 32) << 16);
+    const uint32_t stage = sbase + C::kOffStage + warp * 1024;
+    const float inv_scale = 1.f / p.scale;
+    uint32_t u = 0, it = 0;
     bool ok = true;
-    for (int it = 0; it < iters; ++it) {
-      const int s = it % C::kStages;
-      const uint32_t buf = (it % NBUF) * KC;
-      const int j = kKeys ? it % T : it;
-      if (kKeys && p.gate_logit) g = 1.f / (1.f + __expf(-p.gate_logit[hk * p.G + it / T]));
-      ok = mbar_wait(bar(C::kBarTokFull + s), (it / C::kStages) & 1u, gave_up, p.status);
-      if (ok) ok = mbar_wait(bar(C::kBarSFull + it % NBUF), (it / NBUF) & 1u, gave_up, p.status);
-      ok = __all_sync(0xffffffffu, ok);   // the tensor-memory accesses below are warp-collective
-      if (C::kRowWgs == 1 && !ok) break;
-      if (ok) tc_fence_after();
-      // visible columns of this row: one interval [lo, lo + span], cut by the token order
-      const int cb = cstart + j * KC;
-      const bool clamp = p.linear || p.full_range || p.one_sided;
-      int lo, hi;
-      if (p.one_sided) {
-        if (kKeys) { lo = rslot - cb; hi = p.full_range ? p.n - 1 - cb : rslot + (p.w - 1) - cb; }
-        else { lo = p.full_range ? -cb : rslot - (p.w - 1) - cb; hi = rslot - cb; }
-      } else if (p.full_range && !p.linear) { lo = -cb; hi = p.n - 1 - cb; }
-      else { lo = rslot - p.h - cb; hi = rslot + p.h - cb; }
-      // Every row of the tile sees every column of this tile (up to the token order) when the
-      // last row's interval starts at or before column 0, the first row's ends at or after the
-      // last column and no clamp cuts in: then the per-element interval test is left out.
-      // (The interval moves with the row's slot, one column per row.)
-      const bool interior = !p.full_range && lo + (kTile - 1 - row) <= 0 && hi - row >= KC - 1 &&
-                            (!clamp || (cb >= 0 && cb + KC <= p.n)) && r0 + kTile - 1 < p.n;
-      if (clamp) {
-        lo = max(lo, -cb);
-        hi = min(hi, p.n - 1 - cb);
+    auto arrive = [&](int i) {            // one arrival per warp, behind its tensor-memory accesses
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar(i));
+    };
+    auto gate = [&](int hq) {
+      return p.gate_logit ? 1.f / (1.f + __expf(-p.gate_logit[hq])) : 1.f;
+    };
+    for (int w_item = blockIdx.x; w_item < total && ok; w_item += gridDim.x, ++it) {
+      const Item i = item_of(w_item);
+      const int rslot = i.r0 + row;
+      const bool row_valid = rslot < p.n;
+      const int rtok = row_valid ? (p.perm ? p.perm[(size_t)i.b * p.n + rslot] : rslot) : 0;
+      int hq = KEYS ? i.hk * p.G : i.hr;
+      float g = gate(hq), lse_r = 0.f, delta_r = 0.f;
+      if (!KEYS) {
+        const size_t at = ((size_t)i.b * p.Hq + hq) * p.o.spitch + p.o.sleft + min(rslot, p.n - 1);
+        lse_r = p.lse2[at];
+        delta_r = p.delta[at];
       }
-      if (hi < lo) { lo = 1 << 30; hi = lo; }
-      const uint32_t span = (uint32_t)(hi - lo);
-      const int32_t* coltok = reinterpret_cast<const int32_t*>(smem + C::kOffColTok) + s * kTile;
-      const float* colvec = reinterpret_cast<const float*>(smem + C::kOffColVec) + s * 2 * kTile;
-#pragma unroll 1
-      for (int c = wg; c < KC / 32; c += C::kRowWgs) {
-        uint32_t sv[32], dv[32];
-        if (ok) {
-          tmem_ld32(trow + C::kColS + buf + 32 * c, sv);
-          tmem_ld32(trow + C::kColP + buf + 32 * c, dv);
+      int j = 0;
+      for (int x = 0; x < i.iters; ++x, ++u) {
+        const uint32_t s = u % C::kC1;
+        const float* vec = reinterpret_cast<const float*>(smem + C::kOffVec) + s * 3 * kTile + c0;
+        const int cb = i.cstart + j * kTile;
+        if (kVec) ok = mbar_wait(bar(C::kBarVFull + s), (u / C::kC1) & 1u, gave_up, p.status);
+        if (ok) ok = mbar_wait(bar(C::kBarSFull), u & 1u, gave_up, p.status);
+        ok = __all_sync(0xffffffffu, ok);   // the tensor-memory accesses below are warp-collective
+        if (!ok) break;
+        tc_fence_after();
+        // P times scale: exp2(s scale2 - lse2), kept in registers
+        uint32_t sv[32];
+        tmem_ld32(trow + C::kColS + c0, sv);
+        tmem_wait_ld();
+        arrive(C::kBarSRead);
+        const float2 sc2 = make_float2(p.scale2, p.scale2);
+#pragma unroll
+        for (int y = 0; y < 32; y += 4) {
+          float4 l4 = make_float4(lse_r, lse_r, lse_r, lse_r);
+          if (KEYS) l4 = *reinterpret_cast<const float4*>(vec + y);
+          const float2 a = __ffma2_rn(make_float2(__uint_as_float(sv[y]), __uint_as_float(sv[y + 1])),
+                                      sc2, make_float2(-l4.x, -l4.y));
+          const float2 b = __ffma2_rn(make_float2(__uint_as_float(sv[y + 2]), __uint_as_float(sv[y + 3])),
+                                      sc2, make_float2(-l4.z, -l4.w));
+          sv[y] = __float_as_uint(exp2f(a.x));
+          sv[y + 1] = __float_as_uint(exp2f(a.y));
+          sv[y + 2] = __float_as_uint(exp2f(b.x));
+          sv[y + 3] = __float_as_uint(exp2f(b.y));
+        }
+        if (TOK) {
+          // rows = queries: hide later key tokens; rows = keys: earlier query tokens
+          const int32_t* ct = reinterpret_cast<const int32_t*>(vec + 2 * kTile);
+#pragma unroll
+          for (int y = 0; y < 32; y += 4) {
+            const int4 c4 = *reinterpret_cast<const int4*>(ct + y);
+            if (KEYS ? c4.x < rtok : c4.x > rtok) sv[y] = 0u;
+            if (KEYS ? c4.y < rtok : c4.y > rtok) sv[y + 1] = 0u;
+            if (KEYS ? c4.z < rtok : c4.z > rtok) sv[y + 2] = 0u;
+            if (KEYS ? c4.w < rtok : c4.w > rtok) sv[y + 3] = 0u;
+          }
+        }
+        // Is every column of the tile in the window of every row of it?  (The window moves with the
+        // row's slot, one column per row.)  If not: the columns [lo, hi] of this row.
+        bool inside;
+        if (p.full_range) inside = false;
+        else if (p.one_sided)
+          inside = KEYS ? cb >= i.r0 + kTile - 1 && cb + kTile <= min(i.r0 + p.w, p.n)
+                        : cb >= max(i.r0 + kTile - p.w, 0) && cb + kTile - 1 <= i.r0;
+        else
+          inside = cb >= i.r0 + kTile - 1 - p.h && cb + kTile - 1 <= i.r0 + p.h &&
+                   (!p.linear || (cb >= 0 && cb + kTile <= p.n));
+        if (!inside) {
+          int lo = -cb, hi = p.n - 1 - cb;                 // inside the sequence
+          if (p.one_sided) {
+            if (KEYS) {
+              lo = rslot - cb;
+              if (!p.full_range) hi = min(hi, rslot + p.w - 1 - cb);
+            } else {
+              if (!p.full_range) lo = max(lo, rslot - (p.w - 1) - cb);
+              hi = min(hi, rslot - cb);
+            }
+          } else if (!p.full_range || p.linear) {
+            const int a = rslot - p.h - cb, e = rslot + p.h - cb;
+            lo = p.linear ? max(lo, a) : a;
+            hi = p.linear ? min(hi, e) : e;
+          }
+          lo -= c0;
+          hi -= c0;
+          const uint32_t span = hi < lo ? 0u : (uint32_t)(hi - lo);
+          if (hi < lo) lo = 1 << 30;
+#pragma unroll
+          for (int y = 0; y < 32; ++y)
+            if ((uint32_t)(y - lo) > span) sv[y] = 0u;
+        }
+        // dP, dS; P (times the gate, for dV) and dS go back as bf16 pairs over dP
+        const uint32_t xa = trow + C::kColX + 128 * (u % C::kNX) + c0;
+        if (C::kNX == 1) {
+          ok = mbar_wait(bar(C::kBarDpFull), u & 1u, gave_up, p.status);
+          ok = __all_sync(0xffffffffu, ok);
+          if (!ok) break;
+          tc_fence_after();
+        }
+        const float2 g2 = make_float2(g, g);
+        const float gp = g * inv_scale;
+        uint32_t ds[16];
+#pragma unroll
+        for (int hf = 0; hf < 2; ++hf) {
+          uint32_t dv[16];
+          tmem_ld16(xa + 16 * hf, dv);
           tmem_wait_ld();
-        }
-        if (C::kRowWgs == 2 && rows_sync_stop(!ok)) { ok = false; break; }
-        uint32_t ds_pk[16], p_pk[16];
-        auto chunk = [&](auto inter_c) {
-        constexpr bool kInter = decltype(inter_c)::value;
-        // TMA tiles are the one-sided local branch: slots decide, the token lists are not even
-        // written, and their loads would only take shared-memory bandwidth from the products
-        constexpr bool kTok = !TMA;
 #pragma unroll
-        for (int x = 0; x < 32; x += 4) {
-          const int col = 32 * c + x;
-          int4 ct = make_int4(0, 0, 0, 0);
-          if (kTok) ct = *reinterpret_cast<const int4*>(coltok + col);
-          float4 l4 = make_float4(lse2_r, lse2_r, lse2_r, lse2_r);
-          float4 d4 = make_float4(delta_r, delta_r, delta_r, delta_r);
-          if (kKeys) {
-            l4 = *reinterpret_cast<const float4*>(colvec + col);
-            l4.x = fmaf(l4.x, kLog2e, -l2scale); l4.y = fmaf(l4.y, kLog2e, -l2scale);
-            l4.z = fmaf(l4.z, kLog2e, -l2scale); l4.w = fmaf(l4.w, kLog2e, -l2scale);
-            d4 = *reinterpret_cast<const float4*>(colvec + kTile + col);
-          }
-          const int ctk[4] = {ct.x, ct.y, ct.z, ct.w};
-          const float lv[4] = {l4.x, l4.y, l4.z, l4.w}, dl[4] = {d4.x, d4.y, d4.z, d4.w};
-          float pv[4], dsv[4];
-          const float gp = g * inv_scale;
-          // two elements per instruction where the operation has a packed form
-          const float2 sc2 = make_float2(p.scale2, p.scale2), g2 = make_float2(g, g);
-#pragma unroll
-          for (int y = 0; y < 4; y += 2) {
-            const bool vis0 = (kInter || (uint32_t)(col + y - lo) <= span) &&
-                              (!kTok || (kKeys ? ctk[y] >= cmp : ctk[y] <= cmp));
-            const bool vis1 = (kInter || (uint32_t)(col + y + 1 - lo) <= span) &&
-                              (!kTok || (kKeys ? ctk[y + 1] >= cmp : ctk[y + 1] <= cmp));
-            const float2 a = __ffma2_rn(make_float2(__uint_as_float(sv[x + y]), __uint_as_float(sv[x + y + 1])),
-                                        sc2, make_float2(-lv[y], -lv[y + 1]));
-            const float2 ps = make_float2(vis0 ? exp2f(a.x) : 0.f, vis1 ? exp2f(a.y) : 0.f);   // P * scale
-            const float2 in = __ffma2_rn(g2, make_float2(__uint_as_float(dv[x + y]), __uint_as_float(dv[x + y + 1])),
-                                         make_float2(-dl[y], -dl[y + 1]));
-            const float2 ds = __fmul2_rn(ps, in);
-            dsv[y] = ds.x;
-            dsv[y + 1] = ds.y;
-            pv[y] = ps.x * gp;                                      // g P, for dV
-            pv[y + 1] = ps.y * gp;
-          }
-          const __nv_bfloat162 a0 = __floats2bfloat162_rn(dsv[0], dsv[1]);
-          const __nv_bfloat162 a1 = __floats2bfloat162_rn(dsv[2], dsv[3]);
-          ds_pk[x / 2] = *reinterpret_cast<const uint32_t*>(&a0);
-          ds_pk[x / 2 + 1] = *reinterpret_cast<const uint32_t*>(&a1);
-          if (kKeys) {
-            const __nv_bfloat162 b0 = __floats2bfloat162_rn(pv[0], pv[1]);
-            const __nv_bfloat162 b1 = __floats2bfloat162_rn(pv[2], pv[3]);
-            p_pk[x / 2] = *reinterpret_cast<const uint32_t*>(&b0);
-            p_pk[x / 2 + 1] = *reinterpret_cast<const uint32_t*>(&b1);
+          for (int y = 0; y < 16; y += 4) {
+            const int e = 16 * hf + y;
+            float4 d4 = make_float4(delta_r, delta_r, delta_r, delta_r);
+            if (KEYS) d4 = *reinterpret_cast<const float4*>(vec + kTile + e);
+            const float2 a = __ffma2_rn(g2, make_float2(__uint_as_float(dv[y]), __uint_as_float(dv[y + 1])),
+                                        make_float2(-d4.x, -d4.y));
+            const float2 b = __ffma2_rn(g2, make_float2(__uint_as_float(dv[y + 2]), __uint_as_float(dv[y + 3])),
+                                        make_float2(-d4.z, -d4.w));
+            const float2 sa = __fmul2_rn(make_float2(__uint_as_float(sv[e]), __uint_as_float(sv[e + 1])), a);
+            const float2 sb = __fmul2_rn(make_float2(__uint_as_float(sv[e + 2]), __uint_as_float(sv[e + 3])), b);
+            const __nv_bfloat162 ha = __floats2bfloat162_rn(sa.x, sa.y), hb = __floats2bfloat162_rn(sb.x, sb.y);
+            ds[e / 2] = *reinterpret_cast<const uint32_t*>(&ha);
+            ds[e / 2 + 1] = *reinterpret_cast<const uint32_t*>(&hb);
+            if (KEYS) {     // P of these four, packed into the registers they leave
+              const __nv_bfloat162 pa = __floats2bfloat162_rn(__uint_as_float(sv[e]) * gp, __uint_as_float(sv[e + 1]) * gp);
+              const __nv_bfloat162 pb = __floats2bfloat162_rn(__uint_as_float(sv[e + 2]) * gp, __uint_as_float(sv[e + 3]) * gp);
+              sv[e / 2] = *reinterpret_cast<const uint32_t*>(&pa);
+              sv[e / 2 + 1] = *reinterpret_cast<const uint32_t*>(&pb);
+            }
           }
         }
-        };
-        if (interior) chunk(std::true_type{});
-        else chunk(std::false_type{});
-        // bf16 results go back over the columns already consumed (16 c .. 16 c + 15)
-        tmem_st16(trow + C::kColS + buf + 16 * c, ds_pk);
-        if (kKeys) tmem_st16(trow + C::kColP + buf + 16 * c, p_pk);
+        if (KEYS) {
+          tmem_st16(xa, reinterpret_cast<const uint32_t(&)[16]>(sv[0]));
+          tmem_st16(xa + 16, ds);
+        } else {
+          tmem_st16(xa, ds);
+        }
+        tmem_wait_st();
+        // (with two dP buffers a quick warp may be here for step u + 1 before a slow one for step u)
+        arrive(C::kBarPReady + u % C::kNX);
+        if (++j == i.T) {
+          j = 0;
+          ++hq;
+          if (KEYS && x + 1 < i.iters) g = gate(hq);
+        }
       }
       if (!ok) break;
-      tmem_wait_st();
-      tc_fence_before();
-      mbar_arrive(bar(C::kBarPReady + it % NBUF));
-    }
 
-    if (ok) ok = mbar_wait(bar(C::kBarODone), 0, gave_up, p.status);
-    ok = __all_sync(0xffffffffu, ok);
-    if (ok) {
+      // ------------------------------------------------------------------------ epilogue
+      // Accumulator columns 32 at a time (rows = keys: dV, then dK), the pieces dealt to the column
+      // groups.  A thread holds 64 bytes of a row; 16 rows at a time are turned in the warp's
+      // kilobyte, so that 4 lanes store 64 consecutive bytes.  What the first branch left in the
+      // rows comes in the same way, and is added before the one rounding.
+      constexpr int kPieces = C::kAccCols / 32;
+      const int prow = lane >> 2, pc = lane & 3;
+      auto turned = [&](int r) { return stage + r * 64 + ((pc ^ ((r >> 1) & 3)) << 4); };
+      auto own = [&](int x8) { return stage + (lane & 15) * 64 + ((x8 ^ ((lane >> 1) & 3)) << 4); };
+      auto out_of = [&](int piece, __nv_bfloat16** out, int64_t* tok_stride) {
+        const int o = piece / (D / 32);
+        const int64_t* st = KEYS ? p.ks : p.qs;
+        *out = (__nv_bfloat16*)(KEYS ? (o == 0 ? p.dv : p.dk) : p.dq) + i.b * st[0] + i.hr * st[1] +
+               32 * (piece % (D / 32)) + 8 * pc;
+        *tok_stride = st[2];
+      };
+      uint4 old[4];
+      auto load_old = [&](int piece) {
+        __nv_bfloat16* out;
+        int64_t ts;
+        out_of(piece, &out, &ts);
+#pragma unroll
+        for (int y = 0; y < 4; ++y) {
+          const int64_t tk = __shfl_sync(0xffffffffu, rtok, 8 * y + prow);
+          old[y] = make_uint4(0u, 0u, 0u, 0u);
+          if (i.r0 + quad * 32 + 8 * y + prow < p.n) old[y] = *reinterpret_cast<const uint4*>(out + tk * ts);
+        }
+      };
+      if (cg < kPieces && p.accumulate) load_old(cg);
+      ok = mbar_wait(bar(C::kBarAccFull), it & 1u, gave_up, p.status);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
       tc_fence_after();
-      // 32-column pieces of the accumulators (rows = keys: dV first, then dK), dealt to the
-      // warpgroups in turn
-      constexpr int kPieces = (kKeys ? 2 : 1) * (D / 32);
 #pragma unroll 1
-      for (int piece = wg; piece < kPieces; piece += C::kRowWgs) {
-        const int o = piece / (D / 32), c = piece % (D / 32);
-        __nv_bfloat16* out = (__nv_bfloat16*)(kKeys ? (o == 0 ? p.dv : p.dk) : p.dq);
-        const int64_t* st = kKeys ? p.ks : p.qs;
-        const int64_t off = b * st[0] + hr * st[1] + (int64_t)rtok * st[2];
-        uint32_t raw[32];
-        tmem_ld32(trow + C::kColAcc + o * D + 32 * c, raw);   // warp-collective
+      for (int piece = cg; piece < kPieces; piece += 4) {
+        __nv_bfloat16* out;
+        int64_t ts;
+        out_of(piece, &out, &ts);
+        uint32_t acc[32];
+        tmem_ld32(trow + C::kColAcc + 32 * piece, acc);
         tmem_wait_ld();
-        if (row_valid) {
+        if (piece + 4 >= kPieces) arrive(C::kBarAccFree);
+        if (p.accumulate) {
+          if (piece != cg) load_old(piece);
 #pragma unroll
-          for (int x8 = 0; x8 < 4; ++x8) {
-            float v8[8];
+          for (int hf = 0; hf < 2; ++hf) {
+            __syncwarp();
 #pragma unroll
-            for (int x = 0; x < 8; ++x) v8[x] = __uint_as_float(raw[8 * x8 + x]);
-            uint4* dst = reinterpret_cast<uint4*>(out + off + 32 * c + 8 * x8);
-            if (p.accumulate) {
-              const uint4 old = *dst;
-              const __nv_bfloat162* h2 = reinterpret_cast<const __nv_bfloat162*>(&old);
+            for (int y = 0; y < 2; ++y)
+              sts128(turned(8 * y + prow), reinterpret_cast<const uint32_t(&)[4]>(old[2 * hf + y]));
+            __syncwarp();
+            if ((lane >> 4) == hf) {
 #pragma unroll
-              for (int x = 0; x < 4; ++x) {
-                v8[2 * x] += __low2float(h2[x]);
-                v8[2 * x + 1] += __high2float(h2[x]);
+              for (int x8 = 0; x8 < 4; ++x8) {
+                uint32_t v[4];
+                lds128(v, own(x8));
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                  const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&v[c]));
+                  acc[8 * x8 + 2 * c] = __float_as_uint(__uint_as_float(acc[8 * x8 + 2 * c]) + f.x);
+                  acc[8 * x8 + 2 * c + 1] = __float_as_uint(__uint_as_float(acc[8 * x8 + 2 * c + 1]) + f.y);
+                }
               }
             }
-            uint4 pk;
-            __nv_bfloat162* h2 = reinterpret_cast<__nv_bfloat162*>(&pk);
+          }
+        }
 #pragma unroll
-            for (int x = 0; x < 4; ++x) h2[x] = __floats2bfloat162_rn(v8[2 * x], v8[2 * x + 1]);
-            *dst = pk;
+        for (int hf = 0; hf < 2; ++hf) {
+          __syncwarp();
+          if ((lane >> 4) == hf) {
+#pragma unroll
+            for (int x8 = 0; x8 < 4; ++x8) {
+              uint32_t v[4];
+#pragma unroll
+              for (int c = 0; c < 4; ++c) {
+                const __nv_bfloat162 h2 = __floats2bfloat162_rn(__uint_as_float(acc[8 * x8 + 2 * c]),
+                                                                __uint_as_float(acc[8 * x8 + 2 * c + 1]));
+                v[c] = *reinterpret_cast<const uint32_t*>(&h2);
+              }
+              sts128(own(x8), v);
+            }
+          }
+          __syncwarp();
+#pragma unroll
+          for (int y = 0; y < 2; ++y) {
+            const int r = 16 * hf + 8 * y + prow;
+            const int64_t tk = __shfl_sync(0xffffffffu, rtok, r);
+            uint32_t v[4];
+            lds128(v, turned(8 * y + prow));
+            if (i.r0 + quad * 32 + r < p.n)
+              *reinterpret_cast<uint4*>(out + tk * ts) = make_uint4(v[0], v[1], v[2], v[3]);
           }
         }
       }
+      if (cg >= kPieces) arrive(C::kBarAccFree);
     }
   }
 
   // ----------------------------------------------------------------------- teardown
   tc_fence_before();
   __syncthreads();
-  if (warp == 0) {
+  if (warp == kMmaWarp) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols)
                  : "memory");
   }
 }
 
+// ---------------------------------------------------------------------------- preparation
+
+struct PrepParams {
+  const __nv_bfloat16 *q, *k, *v, *dy, *y[2];
+  const int32_t *perm, *inv;          // of the branch the copies are for; null: token order
+  const float *lse[2], *gate_logits;
+  __nv_bfloat16 *cq, *cdy, *ck, *cv;  // copies; cq null: none
+  int32_t* tok;                       // [B, spitch] of that branch, null: not needed
+  float *lse2[2], *delta[2];          // per branch; null: this launch makes no statistics
+  float* partials;                    // [2, B, Hq, chunks]
+  const int* abort_flag;
+  int B, Hq, Hkv, n, nbranch, chunks, copy_branch;
+  float log2_scale;
+  Order o[2];
+  int64_t qs[3], ks[3];
+};
+
+constexpr int kPrepRows = 64;
+
+// blockIdx.y: the Hq query heads (Delta, lse, copies of dY and Q), then the Hkv KV heads (copies of K and
+// V; the first of them also writes the token list).  D / 8 lanes per row, 16 bytes each; rows are read
+// in token order and stored at their slot.  HBM-bound: every tensor read once and written once.
+template <int D>
+__global__ void __launch_bounds__(256) prep_kernel(const __grid_constant__ PrepParams p) {
+  __shared__ float wsum[2][8];
+  constexpr int kCpr = D / 8, kRpp = 256 / kCpr;      // lanes per row, rows per pass
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int sub = tid / kCpr, c = tid % kCpr;
+  const int b = blockIdx.z, i0 = blockIdx.x * kPrepRows;
+  const bool qside = (int)blockIdx.y < p.Hq, copies = p.cq != nullptr, stats = p.lse2[0] != nullptr;
+  const int h = qside ? blockIdx.y : blockIdx.y - p.Hq;
+  grid_dependency_wait();
+  grid_dependents_launch();
+  if (p.abort_flag && *p.abort_flag) return;          // an earlier check rejected perm/inv
+  const Order& oc = p.o[p.copy_branch];
+  // a row goes to its slot, and on to the other side where the circular window reaches over the end
+  auto places = [&](int slot, int left, int (&at)[3], const Order& o) {
+    at[0] = left + slot;
+    const int reach = o.circular ? o.sleft : 0;
+    at[1] = slot >= p.n - reach ? left + slot - p.n : -1;
+    at[2] = slot < reach ? left + p.n + slot : -1;
+  };
+  auto store = [&](__nv_bfloat16* base, const int (&at)[3], const uint4& v) {
+#pragma unroll
+    for (int x = 0; x < 3; ++x)
+      if (at[x] >= 0) *reinterpret_cast<uint4*>(base + (int64_t)at[x] * D + 8 * c) = v;
+  };
+  if (!qside) {
+    if (!copies) return;
+    const int64_t src = b * p.ks[0] + h * p.ks[1] + 8 * c;
+    const int64_t dst = ((int64_t)b * p.Hkv + h) * oc.ext * D;
+#pragma unroll
+    for (int r = 0; r < kPrepRows / kRpp; ++r) {
+      const int i = i0 + r * kRpp + sub;
+      if (i >= p.n) break;
+      const int slot = p.inv ? p.inv[(size_t)b * p.n + i] : i;
+      const uint4 kk = __ldg(reinterpret_cast<const uint4*>(p.k + src + (int64_t)i * p.ks[2]));
+      const uint4 vv = __ldg(reinterpret_cast<const uint4*>(p.v + src + (int64_t)i * p.ks[2]));
+      int at[3];
+      places(slot, oc.left, at, oc);
+      store(p.ck + dst, at, kk);
+      store(p.cv + dst, at, vv);
+    }
+    if (h == 0 && p.tok) {            // this block's share of the list, in slot order
+      const int per = (oc.spitch + gridDim.x - 1) / gridDim.x;
+      for (int e = blockIdx.x * per + tid; e < min((int)(blockIdx.x + 1) * per, oc.spitch); e += 256) {
+        int slot = e - oc.sleft;
+        if (oc.circular) { slot %= p.n; slot = slot < 0 ? slot + p.n : slot; }
+        int t = 0;
+        if (slot >= 0 && slot < p.n) t = p.perm ? p.perm[(size_t)b * p.n + slot] : slot;
+        p.tok[(size_t)b * oc.spitch + e] = t;
+      }
+    }
+    return;
+  }
+  const int64_t src = b * p.qs[0] + h * p.qs[1] + 8 * c;
+  const int64_t dst = ((int64_t)b * p.Hq + h) * oc.ext * D;
+  const size_t bh = (size_t)b * p.Hq + h;
+  float g[2], part[2] = {0.f, 0.f};
+  for (int x = 0; x < 2; ++x)
+    g[x] = p.gate_logits ? 1.f / (1.f + __expf(-p.gate_logits[x * p.Hq + h])) : 1.f;
+#pragma unroll
+  for (int r = 0; r < kPrepRows / kRpp; ++r) {
+    const int i = i0 + r * kRpp + sub;
+    const bool have = i < p.n;
+    const int64_t off = src + (int64_t)min(i, p.n - 1) * p.qs[2];
+    int slot = i;
+    if (have && p.inv) slot = p.inv[(size_t)b * p.n + i];
+    const uint4 dy = __ldg(reinterpret_cast<const uint4*>(p.dy + off));
+    if (stats) {
+      const __nv_bfloat162* hd = reinterpret_cast<const __nv_bfloat162*>(&dy);
+      for (int x = 0; x < p.nbranch; ++x) {
+        const uint4 y = __ldg(reinterpret_cast<const uint4*>((x ? p.y[1] : p.y[0]) + off));
+        const __nv_bfloat162* hy = reinterpret_cast<const __nv_bfloat162*>(&y);
+        float dot = 0.f;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const float2 u = __bfloat1622float2(hd[e]), w = __bfloat1622float2(hy[e]);
+          dot = fmaf(u.x, w.x, dot);
+          dot = fmaf(u.y, w.y, dot);
+        }
+#pragma unroll
+        for (int o = kCpr / 2; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
+        if (!have) dot = 0.f;
+        if (c == 0) part[x] += dot;
+        if (c == 0 && have) {
+          const Order& o = p.o[x];
+          int at[3];
+          places(x == 0 ? slot : i, o.sleft, at, o);
+          const float l2 = p.lse[x][bh * p.n + i] * kLog2e - p.log2_scale;
+#pragma unroll
+          for (int y3 = 0; y3 < 3; ++y3)
+            if (at[y3] >= 0) {
+              p.lse2[x][bh * o.spitch + at[y3]] = l2;
+              p.delta[x][bh * o.spitch + at[y3]] = g[x] * dot;
+            }
+        }
+      }
+    }
+    if (copies && have) {
+      const uint4 qq = __ldg(reinterpret_cast<const uint4*>(p.q + off));
+      int at[3];
+      places(slot, oc.left, at, oc);
+      store(p.cdy + dst, at, dy);
+      store(p.cq + dst, at, qq);
+    }
+  }
+  if (!stats) return;
+  for (int x = 0; x < p.nbranch; ++x) {
+    // what lies outside the sequence is read with the last tiles: it has to be finite
+    const Order& o = p.o[x];
+    const int end = o.sleft + p.n + (o.circular ? o.sleft : 0), lead = o.circular ? 0 : o.sleft;
+    if (blockIdx.x == 0)
+      for (int e = tid; e < lead + o.spitch - end; e += 256) {
+        const size_t at = bh * o.spitch + (e < lead ? e : end + e - lead);
+        p.lse2[x][at] = 0.f;
+        p.delta[x][at] = 0.f;
+      }
+    const float s = warp_sum(part[x]);
+    if (lane == 0) wsum[x][warp] = s;
+  }
+  __syncthreads();
+  if (tid < p.nbranch) {
+    float s = 0.f;
+    for (int wv = 0; wv < 8; ++wv) s += wsum[tid][wv];
+    p.partials[((size_t)tid * p.B * p.Hq + bh) * p.chunks + blockIdx.x] = s;
+  }
+}
+
 // ---------------------------------------------------------------------------- host
 
-template <int D, int KC, int NBUF, int RW, bool TMA>
-cudaError_t launch_branch_as(const BwdTcParams& p, const CUtensorMap* tm, cudaStream_t st) {
-  using C0 = BCfg<D, KC, 0, NBUF, RW>;
-  using C1 = BCfg<D, KC, 1, NBUF, RW>;
-  cudaError_t e = cudaFuncSetAttribute(bwd_tc_kernel<D, KC, 0, NBUF, RW, TMA>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, C0::kBytes);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(bwd_tc_kernel<D, KC, 1, NBUF, RW, TMA>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, C1::kBytes);
-  if (e != cudaSuccess) return e;
-  bwd_tc_kernel<D, KC, 0, NBUF, RW, TMA><<<(unsigned)(p.B * p.Hq * p.n_tiles), C0::kThreads, C0::kBytes, st>>>(
-      p, tm[0], tm[1], tm[2], tm[3]);
-  bwd_tc_kernel<D, KC, 1, NBUF, RW, TMA><<<(unsigned)(p.B * p.Hkv * p.n_tiles), C1::kThreads, C1::kBytes, st>>>(
-      p, tm[0], tm[1], tm[2], tm[3]);
-  bump_launches(2);
-  return cudaGetLastError();
+Order order_of(int n, int w, uint32_t flags, bool swa) {
+  const MaskGeom g = make_geom(n, w, flags, swa);
+  const bool full = g.one_sided ? false : 2ll * g.h + 1 >= n;
+  Order o;
+  o.circular = !g.one_sided && !g.linear && !full;
+  o.left = o.circular ? g.h : 0;
+  o.ext = n + 2 * o.left;
+  o.sleft = g.one_sided || full ? 0 : g.h;
+  o.spitch = (o.sleft + n + (o.circular ? g.h : 0) + 256 + 3) / 4 * 4;   // the last tiles read on
+  return o;
 }
 
-// tm: tensor maps of q, k, v, dy with boxes of KC tokens when the branch's tiles come by TMA,
-// else null.
-template <int D, int KC, int NBUF, int RW>
-cudaError_t launch_branch(const BwdTcParams& p, const CUtensorMap* tm, cudaStream_t st) {
-  if (tm) return launch_branch_as<D, KC, NBUF, RW, true>(p, tm, st);
-  const CUtensorMap none[4] = {};
-  return launch_branch_as<D, KC, NBUF, RW, false>(p, none, st);
+struct BwdCarve {
+  size_t partials, lse2[2], delta[2], tok, q, dy, k, v, total;
+};
+
+// Sized for circular windows, the largest case: the flags do not matter.
+BwdCarve carve(int B, int Hq, int Hkv, int n, int d, int w) {
+  const Order o[2] = {order_of(n, w, 0, false), order_of(n, w, 0, true)};
+  BwdCarve c;
+  size_t at = 0;
+  auto take = [&](size_t bytes) {
+    const size_t r = at;
+    at += (bytes + 255) / 256 * 256;
+    return r;
+  };
+  c.partials = take((size_t)2 * B * Hq * ((n + kPrepRows - 1) / kPrepRows) * 4);
+  int spitch = 0, ext = 0;
+  for (int x = 0; x < 2; ++x) {
+    c.lse2[x] = take((size_t)B * Hq * o[x].spitch * 4);
+    c.delta[x] = take((size_t)B * Hq * o[x].spitch * 4);
+    spitch = o[x].spitch > spitch ? o[x].spitch : spitch;
+    ext = o[x].ext > ext ? o[x].ext : ext;
+  }
+  c.tok = take((size_t)B * spitch * 4);
+  c.q = take((size_t)B * Hq * ext * d * 2);
+  c.dy = take((size_t)B * Hq * ext * d * 2);
+  c.k = take((size_t)B * Hkv * ext * d * 2);
+  c.v = take((size_t)B * Hkv * ext * d * 2);
+  c.total = at;
+  return c;
 }
 
-constexpr int kWideDefault = 1;   // shape for w > 128
+template <int D, bool KEYS, bool TOK>
+cudaError_t launch_side(const BwdTcParams& p, const CUtensorMap* tm, int sms, cudaStream_t st) {
+  using C = BCfg<D, KEYS>;
+  auto kernel = bwd_tc_kernel<D, KEYS, TOK>;
+  const cudaError_t e =
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kBytes);
+  if (e != cudaSuccess) return e;
+  const int total = p.B * (KEYS ? p.Hkv : p.Hq) * p.n_tiles;
+  return launch_dependent(kernel, dim3(total < sms ? total : sms), dim3(kThreads), C::kBytes, st, p,
+                          tm[0], tm[1], tm[2], tm[3]);
+}
 
-// Kernel shape: 0 = 64-wide column tiles, one score buffer (narrow windows: least band-edge
-// waste, two CTAs per SM at d = 64); 1 = 64-wide tiles, two score buffers and two row
-// warpgroups (products of the next tile overlap the row work of this one); 2 = 128-wide
-// tiles, one buffer, two row warpgroups (a third fewer tensor-pipe cycles per column than
-// 64-wide tiles, and half the wait for the row threads).
-// sa_debug_set(SA_DEBUG_SCORE_BLOCK, 64 | 128) forces shape 0 or 2.
-int bwd_shape(int w) {
-  const int forced = debug_option(SA_DEBUG_SCORE_BLOCK);
-  if (forced) return forced == 64 ? 0 : 2;
-  return w <= 128 ? 0 : kWideDefault;
+template <int D>
+cudaError_t launch_branch(const BwdTcParams& p, bool tok, const CUtensorMap* tm, int sms,
+                          cudaStream_t st) {
+  cudaError_t e = tok ? launch_side<D, false, true>(p, tm, sms, st)
+                      : launch_side<D, false, false>(p, tm, sms, st);
+  if (e == cudaSuccess)
+    e = tok ? launch_side<D, true, true>(p, tm, sms, st) : launch_side<D, true, false>(p, tm, sms, st);
+  if (e == cudaSuccess) bump_launches(2);
+  return e;
 }
 
 bool bwd_tc_disabled() { return debug_option(SA_DEBUG_TENSOR_CORES) == 0; }
@@ -661,55 +874,102 @@ bool bwd_tc_disabled() { return debug_option(SA_DEBUG_TENSOR_CORES) == 0; }
 
 bool tc_backward_supported(const BwdArgs& a, int dtype) {
   if (bwd_tc_disabled() || dtype != SA_BF16 || (a.d != 128 && a.d != 64)) return false;
-  return a.n >= 1 && (int64_t)a.B * a.Hq * ((a.n + kTile - 1) / kTile) <= 0x3fffffff;
+  return a.n >= 1 && a.Hq + a.Hkv <= 65535 &&
+         (int64_t)a.B * a.Hq * ((a.n + kTile - 1) / kTile) <= 0x3fffffff;
 }
 
-cudaError_t launch_bwd_tc(const BwdArgs& a, cudaStream_t st) {
+size_t tc_backward_ws_bytes(int B, int Hq, int Hkv, int n, int d, int w) {
+  return d == 64 || d == 128 ? carve(B, Hq, Hkv, n, d, w).total : 0;
+}
+
+cudaError_t launch_bwd_tc(BwdArgs& a, cudaStream_t st) {
+  const BwdCarve c = carve(a.B, a.Hq, a.Hkv, a.n, a.d, a.w);
+  char* ws = (char*)a.ws;
+  int* status = status_ptr();
+  if (!status) return cudaErrorUnknown;
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  a.partials = (float*)(ws + c.partials);
+  a.chunks = (a.n + kPrepRows - 1) / kPrepRows;
+
+  PrepParams pp{};
+  pp.q = (const __nv_bfloat16*)a.q; pp.k = (const __nv_bfloat16*)a.k;
+  pp.v = (const __nv_bfloat16*)a.v; pp.dy = (const __nv_bfloat16*)a.dy;
+  pp.gate_logits = a.gate_logits;
+  pp.partials = a.partials;
+  pp.abort_flag = a.abort_flag;
+  pp.B = a.B; pp.Hq = a.Hq; pp.Hkv = a.Hkv; pp.n = a.n; pp.nbranch = a.nbranch; pp.chunks = a.chunks;
+  pp.log2_scale = log2f(a.scale);
+  pp.cq = (__nv_bfloat16*)(ws + c.q); pp.cdy = (__nv_bfloat16*)(ws + c.dy);
+  pp.ck = (__nv_bfloat16*)(ws + c.k); pp.cv = (__nv_bfloat16*)(ws + c.v);
+  pp.tok = (int32_t*)(ws + c.tok);
+  for (int i = 0; i < 3; ++i) { pp.qs[i] = a.qs[i]; pp.ks[i] = a.ks[i]; }
   for (int x = 0; x < a.nbranch; ++x) {
+    pp.y[x] = (const __nv_bfloat16*)a.y_x[x];
+    pp.lse[x] = a.lse_x[x];
+    pp.o[x] = order_of(a.n, a.w, a.flags, x == 1);
+  }
+  auto prepare = [&](int branch, bool stats) {
+    pp.copy_branch = branch;
+    pp.perm = branch == 0 ? a.perm : nullptr;
+    pp.inv = branch == 0 ? a.inv : nullptr;
+    for (int x = 0; x < 2; ++x) {
+      pp.lse2[x] = stats ? (float*)(ws + c.lse2[x]) : nullptr;
+      pp.delta[x] = stats ? (float*)(ws + c.delta[x]) : nullptr;
+    }
+    const dim3 grid(a.chunks, a.Hq + a.Hkv, a.B);
+    bump_launches();
+    return launch_dependent(a.d == 128 ? prep_kernel<128> : prep_kernel<64>, grid, dim3(256), 0, st, pp);
+  };
+
+  for (int x = 0; x < a.nbranch; ++x) {
+    const MaskGeom mg = make_geom(a.n, a.w, a.flags, x == 1);
     BwdTcParams p{};
-    p.q = a.q; p.k = a.k; p.v = a.v; p.dy = a.dy;
     p.perm = x == 0 ? a.perm : nullptr;
-    p.lse = a.lse_x[x];
-    p.delta = a.delta + (size_t)x * a.B * a.Hq * a.n;
+    p.tok = pp.tok;
+    p.lse2 = (const float*)(ws + c.lse2[x]);
+    p.delta = (const float*)(ws + c.delta[x]);
     p.gate_logit = a.gate_logits ? a.gate_logits + (size_t)x * a.Hq : nullptr;
     p.dq = a.dq; p.dk = a.dk; p.dv = a.dv;
     p.accumulate = x > 0;
-    p.status = status_ptr();
-    if (!p.status) return cudaErrorUnknown;
+    p.status = status;
     p.abort_flag = a.abort_flag;
     p.B = a.B; p.Hq = a.Hq; p.Hkv = a.Hkv; p.G = a.Hq / a.Hkv; p.n = a.n; p.w = a.w;
-    const MaskGeom mg = make_geom(a.n, a.w, a.flags, x == 1);
     p.h = mg.h;
-    p.causal = mg.causal; p.linear = mg.linear; p.one_sided = mg.one_sided;
+    p.linear = mg.linear; p.one_sided = mg.one_sided;
     p.full_range = mg.one_sided ? (a.w - 1 >= a.n) : (2ll * mg.h + 1 >= a.n);
     p.n_tiles = (a.n + kTile - 1) / kTile;
+    p.o = pp.o[x];
     p.scale = a.scale;
     p.scale2 = a.scale * kLog2e;
     for (int i = 0; i < 3; ++i) { p.qs[i] = a.qs[i]; p.ks[i] = a.ks[i]; }
-    const int shape = bwd_shape(a.w);
-    // whole-tile TMA loads for the one-sided SWA branch (otherwise the gather serves it too)
-    CUtensorMap maps[4];
-    const CUtensorMap* tm = nullptr;
-    const int kc = shape == 2 ? 128 : 64;
-    if (x == 1 && mg.one_sided && debug_option(SA_DEBUG_SWA_TILE_LOADS) != 0 && aligned16(a.q) &&
+    // The one-sided SWA branch is read in place where the maps can express the strides;
+    // sa_debug_set(SA_DEBUG_SWA_TILE_LOADS, 0) makes it use copies too.
+    CUtensorMap tm[4];
+    const bool in_place =
+        x == 1 && mg.one_sided && debug_option(SA_DEBUG_SWA_TILE_LOADS) != 0 && aligned16(a.q) &&
         aligned16(a.k) && aligned16(a.v) && aligned16(a.dy) &&
-        make_map_bhnd(&maps[0], a.q, a.B, a.Hq, a.n, a.d, a.qs, kc) &&
-        make_map_bhnd(&maps[1], a.k, a.B, a.Hkv, a.n, a.d, a.ks, kc) &&
-        make_map_bhnd(&maps[2], a.v, a.B, a.Hkv, a.n, a.d, a.ks, kc) &&
-        make_map_bhnd(&maps[3], a.dy, a.B, a.Hq, a.n, a.d, a.qs, kc))
-      tm = maps;
-    cudaError_t e;
-    if (a.d == 128)
-      e = shape == 0 ? launch_branch<128, 64, 1, 1>(p, tm, st)
-          : shape == 1 ? launch_branch<128, 64, 2, 2>(p, tm, st)
-                       : launch_branch<128, 128, 1, 2>(p, tm, st);
-    else
-      e = shape == 0 ? launch_branch<64, 64, 1, 1>(p, tm, st)
-          : shape == 1 ? launch_branch<64, 64, 2, 2>(p, tm, st)
-                       : launch_branch<64, 128, 1, 2>(p, tm, st);
+        make_map_bhnd(&tm[0], a.q, a.B, a.Hq, a.n, a.d, a.qs) &&
+        make_map_bhnd(&tm[1], a.k, a.B, a.Hkv, a.n, a.d, a.ks) &&
+        make_map_bhnd(&tm[2], a.v, a.B, a.Hkv, a.n, a.d, a.ks) &&
+        make_map_bhnd(&tm[3], a.dy, a.B, a.Hq, a.n, a.d, a.qs);
+    if (!in_place) {
+      if ((e = prepare(x, x == 0)) != cudaSuccess) return e;
+      const int64_t ext = p.o.ext;
+      const int64_t cqs[3] = {a.Hq * ext * a.d, ext * a.d, a.d}, cks[3] = {a.Hkv * ext * a.d, ext * a.d, a.d};
+      if (!make_map_bhnd(&tm[0], pp.cq, a.B, a.Hq, p.o.ext, a.d, cqs) ||
+          !make_map_bhnd(&tm[1], pp.ck, a.B, a.Hkv, p.o.ext, a.d, cks) ||
+          !make_map_bhnd(&tm[2], pp.cv, a.B, a.Hkv, p.o.ext, a.d, cks) ||
+          !make_map_bhnd(&tm[3], pp.cdy, a.B, a.Hq, p.o.ext, a.d, cqs))
+        return cudaErrorInvalidValue;
+    }
+    const bool tok = mg.causal && !mg.one_sided;        // the token order decides, not the slots
+    e = a.d == 128 ? launch_branch<128>(p, tok, tm, sms, st) : launch_branch<64>(p, tok, tm, sms, st);
     if (e != cudaSuccess) return e;
   }
-  return cudaSuccess;
+  return cudaGetLastError();
 }
 
 }  // namespace sa

@@ -6,7 +6,9 @@ namespace sa {
 
 // True when the bf16 tensor-core kernels can run this backward problem.
 bool tc_backward_supported(const BwdArgs& a, int dtype);
-// dq, dk, dv of every branch; expects a.delta to be filled (bwd_delta_kernel) already.
-cudaError_t launch_bwd_tc(const BwdArgs& a, cudaStream_t st);
+// Workspace of launch_bwd_tc (0: it does not serve this head dimension).
+size_t tc_backward_ws_bytes(int B, int Hq, int Hkv, int n, int d, int w);
+// dq, dk, dv of every branch, and the partial sums of the gate gradients (a.partials, a.chunks).
+cudaError_t launch_bwd_tc(BwdArgs& a, cudaStream_t st);
 
 }  // namespace sa

@@ -166,6 +166,7 @@ struct BwdArgs {
   float* delta;     // ws: [2,B,Hq,n]
   float* partials;  // ws: [2,B,Hq,chunks]
   float* parts;     // ws: partial gradients of the split fp32 form
+  void* ws;         // all of the workspace (the tensor-core path carves its own)
   int chunks;
   int B, Hq, Hkv, n, d, w;
   uint32_t flags;
@@ -198,7 +199,7 @@ bool gate_forward_wide(int64_t rows, int dm, const void* y_sa, const void* y_swa
                        int* status, int sms, cudaStream_t st, cudaError_t* err);
 
 cudaError_t launch_bwd_simt(const BwdArgs& a, int dtype, cudaStream_t st);
-size_t bwd_ws_bytes(int B, int Hq, int Hkv, int n, int d, int dtype, int* chunks_out,
+size_t bwd_ws_bytes(int B, int Hq, int Hkv, int n, int d, int w, int dtype, int* chunks_out,
                     size_t* parts_at);
 
 cudaError_t launch_coverage(int L, int n, int w, uint32_t flags, const int32_t* perm,
