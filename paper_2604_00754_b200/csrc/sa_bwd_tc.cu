@@ -111,7 +111,8 @@ struct BCfg {
   static constexpr int kC1 = D == 64 ? 4 : KEYS ? 2 : 3, kC2 = D == 64 ? 4 : KEYS ? 2 : 1;
   static constexpr int kRBufs = D == 128 ? 1 : 2;               // row operand pairs
   static constexpr int kAccCols = (KEYS ? 2 : 1) * D;
-  static constexpr int kNX = kAccCols <= 128 ? 2 : 1;           // dP buffers
+  static constexpr int kNX = KEYS ? 1 : 2;                      // dP buffers
+  static constexpr int kAccBufs = D == 64 ? 2 : 1;
   static constexpr int kOffR = 0;
   static constexpr int kOffC = kRBufs * 2 * kTileBytes;
   static constexpr int kOffC2 = kOffC + kC1 * kTileBytes;
@@ -122,26 +123,26 @@ struct BCfg {
                        kBarC2Full = kBarC1Full + kC1, kBarC1Empty = kBarC2Full + kC2,
                        kBarVFull = kBarC1Empty + kC1, kBarSFull = kBarVFull + kC1, kBarSRead = kBarSFull + 1,
                        kBarDpFull = kBarSRead + 1, kBarPReady = kBarDpFull + 1,
-                       kBarAccFull = kBarPReady + kNX, kBarAccFree = kBarAccFull + 1,
-                       kNumBars = kBarAccFree + 1;
+                       kBarAccFull = kBarPReady + kNX,
+                       kBarAccFree = kBarAccFull + kAccBufs, kNumBars = kBarAccFree + kAccBufs;
   static constexpr int kOffMisc = kOffBar + kNumBars * 8;
   static constexpr int kBytes = kOffMisc + 16;
   // tensor memory: S, then the dP buffers (P and dS are written over them), then accumulators
   static constexpr uint32_t kColS = 0, kColX = 128, kColAcc = 128 + 128 * kNX;
-  static_assert(kColAcc + kAccCols <= kTmemCols, "tensor memory");
+  static_assert(kColAcc + kAccBufs * kAccCols <= kTmemCols, "tensor memory");
   static_assert(kBytes <= 232448, "shared memory");
 };
 
-// Four K steps of D (+)= A B with A (bf16 pairs) in tensor memory in the layout the row threads
-// write, 32 columns after 32 columns, and B in shared memory, 16 rows further on each step.
+// Four K steps of D (+)= A B with A (bf16 pairs) in tensor memory, 16 columns further on each step
+// (8 of dS, then 8 of P), and B in shared memory, 16 rows further on each step.
 __device__ __forceinline__ void mma_ts_rows_x4(uint32_t d, uint32_t a, uint64_t b, uint32_t idesc,
                                                uint32_t acc0) {
   asm volatile(
       "{\n\t.reg .pred p0, p1;\n\t.reg .b64 b1, b2, b3;\n\t.reg .b32 a1, a2, a3;\n\t"
       "setp.ne.b32 p0, %4, 0;\n\tsetp.eq.b32 p1, %3, %3;\n\t"
-      "add.u32 a1, %1, 8;\n\tadd.u64 b1, %2, 128;\n\t"
+      "add.u32 a1, %1, 16;\n\tadd.u64 b1, %2, 128;\n\t"
       "add.u32 a2, %1, 32;\n\tadd.u64 b2, %2, 256;\n\t"
-      "add.u32 a3, %1, 40;\n\tadd.u64 b3, %2, 384;\n\t"
+      "add.u32 a3, %1, 48;\n\tadd.u64 b3, %2, 384;\n\t"
       "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p0;\n\t"
       "tcgen05.mma.cta_group::1.kind::f16 [%0], [a1], b1, %3, p1;\n\t"
       "tcgen05.mma.cta_group::1.kind::f16 [%0], [a2], b2, %3, p1;\n\t"
@@ -159,7 +160,7 @@ bwd_tc_kernel(const __grid_constant__ BwdTcParams p, const __grid_constant__ CUt
   extern __shared__ __align__(1024) uint8_t smem[];
   using C = BCfg<D, KEYS>;
   constexpr bool kVec = KEYS || TOK;          // something travels with the column tiles
-  constexpr int kMmaWarp = kRowWarps, kLoadWarp = kRowWarps + 1;
+  constexpr int kMmaWarp = kRowWarps, kLoadWarp = kRowWarps + 2;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
   const uint32_t sbase = smem_u32(smem);
@@ -175,7 +176,7 @@ bwd_tc_kernel(const __grid_constant__ BwdTcParams p, const __grid_constant__ CUt
   if (threadIdx.x == 0) {
     *gave_up = 0;
     for (int i = 0; i < C::kNumBars; ++i)
-      mbar_init(bar(i), (i == C::kBarSRead || (i >= C::kBarPReady && i < C::kBarAccFull) || i == C::kBarAccFree)
+      mbar_init(bar(i), (i == C::kBarSRead || (i >= C::kBarPReady && i < C::kBarAccFull) || i >= C::kBarAccFree)
                             ? kRowWarps : 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     grid_dependency_wait();                   // what earlier launches wrote may be read from here on
@@ -295,8 +296,14 @@ bwd_tc_kernel(const __grid_constant__ BwdTcParams p, const __grid_constant__ CUt
         for (uint32_t x = c2_on > (uint32_t)C::kC2 ? c2_on - C::kC2 : 0u; x < c2_on; ++x)
           landed(C::kBarC2Full + x % C::kC2, (x / C::kC2) & 1u);
       }
-    } else if (warp == kMmaWarp && lane == 0) {
-      // ---------------------------------------------------------------- MMA issuer (one thread)
+    } else if (warp < kLoadWarp && lane == 0) {
+      // ------------------------------------------------------------ MMA issuers (two threads)
+      // Issuing runs at the pace of the products, and between two groups of products the issuing
+      // thread spends some 300 cycles on waits and commits: one thread's fall into the other's
+      // products.  Thread 0: the score products, one step ahead of the accumulations, across items
+      // (rows = keys: S alone, whose columns are free once the row threads hold it).  Thread 1: the
+      // accumulations (rows = keys: and dP of the next step behind them, over the P and dS that
+      // they have read).
       constexpr uint32_t idesc_s = instr_desc(kTile, kTile, false);
       constexpr uint32_t idesc_acc = instr_desc(kTile, D, true);
       constexpr uint32_t kDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
@@ -317,69 +324,85 @@ bwd_tc_kernel(const __grid_constant__ BwdTcParams p, const __grid_constant__ CUt
         mma_ts_rows_x4(tmem + col, tmem + xcol, bd, idesc_acc, acc0);
         mma_ts_rows_x4(tmem + col, tmem + xcol + 64, bd + 512, idesc_acc, 1u);
       };
-      // the score products run one step ahead of the accumulations, across items
       bool ok = true;
-      int sw = blockIdx.x, s_left = 0;            // score cursor: item, steps left of it
-      uint32_t su = 0, s_it = 0;                  // steps and items started
-      if (sw < total) s_left = item_of(sw).iters;
-      // S of the next step into the S columns, once the row threads hold the one before
-      auto next_s = [&]() {
-        const uint32_t rb = s_it % C::kRBufs, s = su % C::kC1;
-        ok = mbar_wait(bar(C::kBarRFull + rb), (s_it / C::kRBufs) & 1u, gave_up, p.status);
-        if (ok) ok = mbar_wait(bar(C::kBarC1Full + s), (su / C::kC1) & 1u, gave_up, p.status);
-        if (ok && su > 0) ok = mbar_wait(bar(C::kBarSRead), (su - 1) & 1u, gave_up, p.status);
+      uint32_t u = 0, it = 0;                     // steps and items of this thread
+      // dP of step v (of item j) of the score stream
+      auto issue_dp = [&](uint32_t v, uint32_t j) {
+        const uint32_t rb = j % C::kRBufs, s = v % C::kC2;
+        ok = mbar_wait(bar(C::kBarC2Full + s), (v / C::kC2) & 1u, gave_up, p.status);
         if (!ok) return;
-        tc_fence_after();
-        product(C::kColS, r_lo + rb * 2 * kTileD, c_lo + s * kTileD);
-        if (C::kNX == 1) tc_commit(bar(C::kBarSFull));
+        product(C::kColX + 128 * (v % C::kNX), r_lo + (rb * 2 + 1) * kTileD, c2_lo + s * kTileD);
+        tc_commit(bar(KEYS ? C::kBarDpFull : C::kBarSFull));
       };
-      // dP of the same step, then on to the next
-      auto next_dp = [&]() {
-        const uint32_t rb = s_it % C::kRBufs, s = su % C::kC2;
-        ok = mbar_wait(bar(C::kBarC2Full + s), (su / C::kC2) & 1u, gave_up, p.status);
-        if (!ok) return;
-        tc_fence_after();
-        product(C::kColX + 128 * (su % C::kNX), r_lo + (rb * 2 + 1) * kTileD, c2_lo + s * kTileD);
-        tc_commit(bar(C::kNX == 1 ? C::kBarDpFull : C::kBarSFull));
-        ++su;
-        if (--s_left == 0) {
-          tc_commit(bar(C::kBarREmpty + rb));
-          ++s_it;
-          sw += gridDim.x;
-          if (sw < total) s_left = item_of(sw).iters;
-        }
-      };
-      if (s_left > 0) {
-        next_s();
-        if (ok) next_dp();
-      }
-      uint32_t u = 0, it = 0;
-      for (int w_item = blockIdx.x; w_item < total && ok; w_item += gridDim.x, ++it) {
-        const int iters = item_of(w_item).iters;
-        for (int x = 0; x < iters && ok; ++x, ++u) {
-          const bool more = s_left > 0;
-          if (more) {
-            next_s();
-            if (ok && C::kNX == 2) next_dp();
+      if (warp == kMmaWarp) {
+        for (int w_item = blockIdx.x; w_item < total && ok; w_item += gridDim.x, ++it) {
+          const int iters = item_of(w_item).iters;
+          const uint32_t rb = it % C::kRBufs;
+          ok = mbar_wait(bar(C::kBarRFull + rb), (it / C::kRBufs) & 1u, gave_up, p.status);
+          for (int x = 0; x < iters && ok; ++x, ++u) {
+            const uint32_t s = u % C::kC1;
+            ok = mbar_wait(bar(C::kBarC1Full + s), (u / C::kC1) & 1u, gave_up, p.status);
+            if (ok && u > 0) ok = mbar_wait(bar(C::kBarSRead), (u - 1) & 1u, gave_up, p.status);
             if (!ok) break;
+            tc_fence_after();
+            product(C::kColS, r_lo + rb * 2 * kTileD, c_lo + s * kTileD);
+            if (KEYS) {
+              tc_commit(bar(C::kBarSFull));
+            } else {
+              // the dP buffer was read by the accumulation two steps ago, which freed C1
+              if (u > 1)
+                ok = mbar_wait(bar(C::kBarC1Empty + (u - 2) % C::kC1), ((u - 2) / C::kC1) & 1u, gave_up,
+                               p.status);
+              if (ok) {
+                tc_fence_after();
+                issue_dp(u, it);
+              }
+            }
           }
-          if (x == 0 && it > 0) ok = mbar_wait(bar(C::kBarAccFree), (it - 1) & 1u, gave_up, p.status);
-          if (ok) ok = mbar_wait(bar(C::kBarPReady + u % C::kNX), (u / C::kNX) & 1u, gave_up, p.status);
-          if (!ok) break;
-          tc_fence_after();
-          const uint32_t s = u % C::kC1, xc = C::kColX + 128 * (u % C::kNX);
-          const uint32_t c1 = c_lo + s * kTileD, c2 = c2_lo + (u % C::kC2) * kTileD;
-          if (KEYS) {
-            accumulate(C::kColAcc + D, xc + 16, c1, x > 0);      // dK += dS^T Q
-            if (D == 128) tc_commit(bar(C::kBarC1Empty + s));
-            accumulate(C::kColAcc, xc, c2, x > 0);               // dV += (g P)^T dY
-            if (D == 64) tc_commit(bar(C::kBarC1Empty + s));
-          } else {
-            accumulate(C::kColAcc, xc, c1, x > 0);               // dQ += dS K
-            tc_commit(bar(C::kBarC1Empty + s));
+          // rows = keys: dP still reads the row operands, the other thread says when it is done
+          if (!KEYS && ok) tc_commit(bar(C::kBarREmpty + rb));
+        }
+      } else {
+        if (KEYS && (int)blockIdx.x < total) {
+          ok = mbar_wait(bar(C::kBarRFull), 0u, gave_up, p.status);
+          if (ok) issue_dp(0, 0);
+        }
+        for (int w_item = blockIdx.x; w_item < total && ok; w_item += gridDim.x, ++it) {
+          const int iters = item_of(w_item).iters;
+          const uint32_t ab = it % C::kAccBufs, acc = C::kColAcc + ab * C::kAccCols;
+          for (int x = 0; x < iters && ok; ++x, ++u) {
+            const uint32_t s = u % C::kC1, s2 = u % C::kC2, xc = C::kColX + 128 * (u % C::kNX);
+            if (x == 0 && it >= (uint32_t)C::kAccBufs)
+              ok = mbar_wait(bar(C::kBarAccFree + ab), (it / C::kAccBufs - 1) & 1u, gave_up, p.status);
+            if (ok) ok = mbar_wait(bar(C::kBarC1Full + s), (u / C::kC1) & 1u, gave_up, p.status);
+            if (ok) ok = mbar_wait(bar(C::kBarPReady + u % C::kNX), (u / C::kNX) & 1u, gave_up, p.status);
+            if (!ok) break;
+            tc_fence_after();
+            if (KEYS) {
+              accumulate(acc + D, xc, c_lo + s * kTileD, x > 0);          // dK += dS^T Q
+              if (D == 128) tc_commit(bar(C::kBarC1Empty + s));
+              accumulate(acc, xc + 8, c2_lo + s2 * kTileD, x > 0);        // dV += (g P)^T dY
+              if (D == 64) tc_commit(bar(C::kBarC1Empty + s));
+            } else {
+              accumulate(acc, xc, c_lo + s * kTileD, x > 0);              // dQ += dS K
+              tc_commit(bar(C::kBarC1Empty + s));
+            }
+            const bool last = x + 1 == iters;
+            if (last) tc_commit(bar(C::kBarAccFull + ab));
+            if (KEYS) {
+              if (!last) {
+                issue_dp(u + 1, it);
+              } else {
+                // (S and dP of this item are over: dP by this thread, S long before)
+                tc_commit(bar(C::kBarREmpty + it % C::kRBufs));
+                if (w_item + (int)gridDim.x < total) {
+                  const uint32_t nr = (it + 1) % C::kRBufs;
+                  ok = mbar_wait(bar(C::kBarRFull + nr), ((it + 1) / C::kRBufs) & 1u, gave_up, p.status);
+                  if (ok) issue_dp(u + 1, it + 1);
+                }
+              }
+            }
           }
-          if (x + 1 == iters) tc_commit(bar(C::kBarAccFull));
-          if (more && C::kNX == 1) next_dp();
         }
       }
     }
@@ -402,20 +425,131 @@ bwd_tc_kernel(const __grid_constant__ BwdTcParams p, const __grid_constant__ CUt
     auto gate = [&](int hq) {
       return p.gate_logit ? 1.f / (1.f + __expf(-p.gate_logit[hq])) : 1.f;
     };
-    for (int w_item = blockIdx.x; w_item < total && ok; w_item += gridDim.x, ++it) {
-      const Item i = item_of(w_item);
-      const int rslot = i.r0 + row;
-      const bool row_valid = rslot < p.n;
-      const int rtok = row_valid ? (p.perm ? p.perm[(size_t)i.b * p.n + rslot] : rslot) : 0;
-      int hq = KEYS ? i.hk * p.G : i.hr;
-      float g = gate(hq), lse_r = 0.f, delta_r = 0.f;
+    // an item and what its rows need from memory, fetched one item ahead
+    struct RowItem { Item i; int tok; float lse, delta, g; };
+    auto fetch = [&](int w_item) {
+      RowItem r;
+      r.i = item_of(w_item);
+      const int slot = min(r.i.r0 + row, p.n - 1);
+      r.tok = p.perm ? p.perm[(size_t)r.i.b * p.n + slot] : slot;
+      r.g = gate(KEYS ? r.i.hk * p.G : r.i.hr);
+      r.lse = r.delta = 0.f;
       if (!KEYS) {
-        const size_t at = ((size_t)i.b * p.Hq + hq) * p.o.spitch + p.o.sleft + min(rslot, p.n - 1);
-        lse_r = p.lse2[at];
-        delta_r = p.delta[at];
+        const size_t at = ((size_t)r.i.b * p.Hq + r.i.hr) * p.o.spitch + p.o.sleft + slot;
+        r.lse = p.lse2[at];
+        r.delta = p.delta[at];
       }
-      int j = 0;
-      for (int x = 0; x < i.iters; ++x, ++u) {
+      return r;
+    };
+    int done_tok = 0, done_b = 0, done_hr = 0, done_r0 = 0;     // the item before
+    // Epilogue of the item before: it runs behind the first step of the next one, so that neither the
+    // last accumulation's latency nor the row threads' stores leave the pipes idle.
+    auto finish = [&]() {
+      // Accumulator columns 32 at a time (rows = keys: dV, then dK), the pieces dealt to the column
+      // groups.  A thread holds 64 bytes of a row; 16 rows at a time are turned in the warp's
+      // kilobyte, so that 4 lanes store 64 consecutive bytes.  What the first branch left in the
+      // rows comes in the same way, and is added before the one rounding.
+      constexpr int kPieces = C::kAccCols / 32;
+      const int prow = lane >> 2, pc = lane & 3;
+      auto turned = [&](int r) { return stage + r * 64 + ((pc ^ ((r >> 1) & 3)) << 4); };
+      auto own = [&](int x8) { return stage + (lane & 15) * 64 + ((x8 ^ ((lane >> 1) & 3)) << 4); };
+      auto out_of = [&](int piece, __nv_bfloat16** out, int64_t* tok_stride) {
+        const int o = piece / (D / 32);
+        const int64_t* st = KEYS ? p.ks : p.qs;
+        *out = (__nv_bfloat16*)(KEYS ? (o == 0 ? p.dv : p.dk) : p.dq) + done_b * st[0] + done_hr * st[1] +
+               32 * (piece % (D / 32)) + 8 * pc;
+        *tok_stride = st[2];
+      };
+      uint4 old[4];
+      auto load_old = [&](int piece) {
+        __nv_bfloat16* out;
+        int64_t ts;
+        out_of(piece, &out, &ts);
+#pragma unroll
+        for (int y = 0; y < 4; ++y) {
+          const int64_t tk = __shfl_sync(0xffffffffu, done_tok, 8 * y + prow);
+          old[y] = make_uint4(0u, 0u, 0u, 0u);
+          if (done_r0 + quad * 32 + 8 * y + prow < p.n) old[y] = *reinterpret_cast<const uint4*>(out + tk * ts);
+        }
+      };
+      if (cg < kPieces && p.accumulate) load_old(cg);
+      const uint32_t ab = (it - 1) % C::kAccBufs;
+      ok = mbar_wait(bar(C::kBarAccFull + ab), ((it - 1) / C::kAccBufs) & 1u, gave_up, p.status);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) return;
+      tc_fence_after();
+#pragma unroll 1
+      for (int piece = cg; piece < kPieces; piece += 4) {
+        __nv_bfloat16* out;
+        int64_t ts;
+        out_of(piece, &out, &ts);
+        uint32_t acc[32];
+        tmem_ld32(trow + C::kColAcc + ab * C::kAccCols + 32 * piece, acc);
+        tmem_wait_ld();
+        if (piece + 4 >= kPieces) arrive(C::kBarAccFree + ab);
+        if (p.accumulate) {
+          if (piece != cg) load_old(piece);
+#pragma unroll
+          for (int hf = 0; hf < 2; ++hf) {
+            __syncwarp();
+#pragma unroll
+            for (int y = 0; y < 2; ++y)
+              sts128(turned(8 * y + prow), reinterpret_cast<const uint32_t(&)[4]>(old[2 * hf + y]));
+            __syncwarp();
+            if ((lane >> 4) == hf) {
+#pragma unroll
+              for (int x8 = 0; x8 < 4; ++x8) {
+                uint32_t v[4];
+                lds128(v, own(x8));
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                  const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&v[c]));
+                  acc[8 * x8 + 2 * c] = __float_as_uint(__uint_as_float(acc[8 * x8 + 2 * c]) + f.x);
+                  acc[8 * x8 + 2 * c + 1] = __float_as_uint(__uint_as_float(acc[8 * x8 + 2 * c + 1]) + f.y);
+                }
+              }
+            }
+          }
+        }
+#pragma unroll
+        for (int hf = 0; hf < 2; ++hf) {
+          __syncwarp();
+          if ((lane >> 4) == hf) {
+#pragma unroll
+            for (int x8 = 0; x8 < 4; ++x8) {
+              uint32_t v[4];
+#pragma unroll
+              for (int c = 0; c < 4; ++c) {
+                const __nv_bfloat162 h2 = __floats2bfloat162_rn(__uint_as_float(acc[8 * x8 + 2 * c]),
+                                                                __uint_as_float(acc[8 * x8 + 2 * c + 1]));
+                v[c] = *reinterpret_cast<const uint32_t*>(&h2);
+              }
+              sts128(own(x8), v);
+            }
+          }
+          __syncwarp();
+#pragma unroll
+          for (int y = 0; y < 2; ++y) {
+            const int r = 16 * hf + 8 * y + prow;
+            const int64_t tk = __shfl_sync(0xffffffffu, done_tok, r);
+            uint32_t v[4];
+            lds128(v, turned(8 * y + prow));
+            if (done_r0 + quad * 32 + r < p.n)
+              *reinterpret_cast<uint4*>(out + tk * ts) = make_uint4(v[0], v[1], v[2], v[3]);
+          }
+        }
+      }
+      if (cg >= kPieces) arrive(C::kBarAccFree + ab);
+    };
+    RowItem nxt{};
+    int w_item = blockIdx.x;
+    if (w_item < total) nxt = fetch(w_item);
+    Item i = nxt.i;
+    int rtok = nxt.tok, hq = KEYS ? i.hk * p.G : i.hr, x = 0, j = 0;
+    float lse_r = nxt.lse, delta_r = nxt.delta, g = nxt.g;
+    while (true) {
+      if (w_item < total) {
+        const int rslot = i.r0 + row;
         const uint32_t s = u % C::kC1;
         const float* vec = reinterpret_cast<const float*>(smem + C::kOffVec) + s * 3 * kTile + c0;
         const int cb = i.cstart + j * kTile;
@@ -480,28 +614,36 @@ bwd_tc_kernel(const __grid_constant__ BwdTcParams p, const __grid_constant__ CUt
             lo = p.linear ? max(lo, a) : a;
             hi = p.linear ? min(hi, e) : e;
           }
-          lo -= c0;
-          hi -= c0;
-          const uint32_t span = hi < lo ? 0u : (uint32_t)(hi - lo);
-          if (hi < lo) lo = 1 << 30;
+          // as one bit per column: a bit test per element is cheaper than a comparison
+          lo = max(lo - c0, 0);
+          hi = min(hi - c0, 31);
+          const uint32_t seen = hi < lo ? 0u : (0xffffffffu >> (31 - hi)) & (0xffffffffu << lo);
 #pragma unroll
           for (int y = 0; y < 32; ++y)
-            if ((uint32_t)(y - lo) > span) sv[y] = 0u;
+            if (!(seen & (1u << y))) sv[y] = 0u;
         }
-        // dP, dS; P (times the gate, for dV) and dS go back as bf16 pairs over dP
+        // what the next item's rows need is on its way while this one's last step is worked on
+        if (x + 1 == i.iters && w_item + (int)gridDim.x < total) nxt = fetch(w_item + gridDim.x);
+        // P times the gate for dV, then dP and dS; both go back as bf16 pairs over dP
         const uint32_t xa = trow + C::kColX + 128 * (u % C::kNX) + c0;
-        if (C::kNX == 1) {
+        uint32_t pk[KEYS ? 16 : 1];
+        if constexpr (KEYS) {
+          const float gp = g * inv_scale;
+#pragma unroll
+          for (int y = 0; y < 16; ++y) {
+            const __nv_bfloat162 h2 = __floats2bfloat162_rn(__uint_as_float(sv[2 * y]) * gp,
+                                                            __uint_as_float(sv[2 * y + 1]) * gp);
+            pk[y] = *reinterpret_cast<const uint32_t*>(&h2);
+          }
           ok = mbar_wait(bar(C::kBarDpFull), u & 1u, gave_up, p.status);
           ok = __all_sync(0xffffffffu, ok);
           if (!ok) break;
           tc_fence_after();
         }
         const float2 g2 = make_float2(g, g);
-        const float gp = g * inv_scale;
-        uint32_t ds[16];
 #pragma unroll
         for (int hf = 0; hf < 2; ++hf) {
-          uint32_t dv[16];
+          uint32_t dv[16], ds[8];
           tmem_ld16(xa + 16 * hf, dv);
           tmem_wait_ld();
 #pragma unroll
@@ -516,128 +658,41 @@ bwd_tc_kernel(const __grid_constant__ BwdTcParams p, const __grid_constant__ CUt
             const float2 sa = __fmul2_rn(make_float2(__uint_as_float(sv[e]), __uint_as_float(sv[e + 1])), a);
             const float2 sb = __fmul2_rn(make_float2(__uint_as_float(sv[e + 2]), __uint_as_float(sv[e + 3])), b);
             const __nv_bfloat162 ha = __floats2bfloat162_rn(sa.x, sa.y), hb = __floats2bfloat162_rn(sb.x, sb.y);
-            ds[e / 2] = *reinterpret_cast<const uint32_t*>(&ha);
-            ds[e / 2 + 1] = *reinterpret_cast<const uint32_t*>(&hb);
-            if (KEYS) {     // P of these four, packed into the registers they leave
-              const __nv_bfloat162 pa = __floats2bfloat162_rn(__uint_as_float(sv[e]) * gp, __uint_as_float(sv[e + 1]) * gp);
-              const __nv_bfloat162 pb = __floats2bfloat162_rn(__uint_as_float(sv[e + 2]) * gp, __uint_as_float(sv[e + 3]) * gp);
-              sv[e / 2] = *reinterpret_cast<const uint32_t*>(&pa);
-              sv[e / 2 + 1] = *reinterpret_cast<const uint32_t*>(&pb);
-            }
+            ds[y / 2] = *reinterpret_cast<const uint32_t*>(&ha);
+            ds[y / 2 + 1] = *reinterpret_cast<const uint32_t*>(&hb);
           }
-        }
-        if (KEYS) {
-          tmem_st16(xa, reinterpret_cast<const uint32_t(&)[16]>(sv[0]));
-          tmem_st16(xa + 16, ds);
-        } else {
-          tmem_st16(xa, ds);
+          // over the 16 columns of dP just read: dS, then P
+          tmem_st8(xa + 16 * hf, ds);
+          if (KEYS) tmem_st8(xa + 16 * hf + 8, reinterpret_cast<const uint32_t(&)[8]>(pk[KEYS ? 8 * hf : 0]));
         }
         tmem_wait_st();
         // (with two dP buffers a quick warp may be here for step u + 1 before a slow one for step u)
         arrive(C::kBarPReady + u % C::kNX);
-        if (++j == i.T) {
-          j = 0;
-          ++hq;
-          if (KEYS && x + 1 < i.iters) g = gate(hq);
-        }
+        ++u;
       }
-      if (!ok) break;
-
-      // ------------------------------------------------------------------------ epilogue
-      // Accumulator columns 32 at a time (rows = keys: dV, then dK), the pieces dealt to the column
-      // groups.  A thread holds 64 bytes of a row; 16 rows at a time are turned in the warp's
-      // kilobyte, so that 4 lanes store 64 consecutive bytes.  What the first branch left in the
-      // rows comes in the same way, and is added before the one rounding.
-      constexpr int kPieces = C::kAccCols / 32;
-      const int prow = lane >> 2, pc = lane & 3;
-      auto turned = [&](int r) { return stage + r * 64 + ((pc ^ ((r >> 1) & 3)) << 4); };
-      auto own = [&](int x8) { return stage + (lane & 15) * 64 + ((x8 ^ ((lane >> 1) & 3)) << 4); };
-      auto out_of = [&](int piece, __nv_bfloat16** out, int64_t* tok_stride) {
-        const int o = piece / (D / 32);
-        const int64_t* st = KEYS ? p.ks : p.qs;
-        *out = (__nv_bfloat16*)(KEYS ? (o == 0 ? p.dv : p.dk) : p.dq) + i.b * st[0] + i.hr * st[1] +
-               32 * (piece % (D / 32)) + 8 * pc;
-        *tok_stride = st[2];
-      };
-      uint4 old[4];
-      auto load_old = [&](int piece) {
-        __nv_bfloat16* out;
-        int64_t ts;
-        out_of(piece, &out, &ts);
-#pragma unroll
-        for (int y = 0; y < 4; ++y) {
-          const int64_t tk = __shfl_sync(0xffffffffu, rtok, 8 * y + prow);
-          old[y] = make_uint4(0u, 0u, 0u, 0u);
-          if (i.r0 + quad * 32 + 8 * y + prow < p.n) old[y] = *reinterpret_cast<const uint4*>(out + tk * ts);
-        }
-      };
-      if (cg < kPieces && p.accumulate) load_old(cg);
-      ok = mbar_wait(bar(C::kBarAccFull), it & 1u, gave_up, p.status);
-      ok = __all_sync(0xffffffffu, ok);
-      if (!ok) break;
-      tc_fence_after();
-#pragma unroll 1
-      for (int piece = cg; piece < kPieces; piece += 4) {
-        __nv_bfloat16* out;
-        int64_t ts;
-        out_of(piece, &out, &ts);
-        uint32_t acc[32];
-        tmem_ld32(trow + C::kColAcc + 32 * piece, acc);
-        tmem_wait_ld();
-        if (piece + 4 >= kPieces) arrive(C::kBarAccFree);
-        if (p.accumulate) {
-          if (piece != cg) load_old(piece);
-#pragma unroll
-          for (int hf = 0; hf < 2; ++hf) {
-            __syncwarp();
-#pragma unroll
-            for (int y = 0; y < 2; ++y)
-              sts128(turned(8 * y + prow), reinterpret_cast<const uint32_t(&)[4]>(old[2 * hf + y]));
-            __syncwarp();
-            if ((lane >> 4) == hf) {
-#pragma unroll
-              for (int x8 = 0; x8 < 4; ++x8) {
-                uint32_t v[4];
-                lds128(v, own(x8));
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                  const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&v[c]));
-                  acc[8 * x8 + 2 * c] = __float_as_uint(__uint_as_float(acc[8 * x8 + 2 * c]) + f.x);
-                  acc[8 * x8 + 2 * c + 1] = __float_as_uint(__uint_as_float(acc[8 * x8 + 2 * c + 1]) + f.y);
-                }
-              }
-            }
-          }
-        }
-#pragma unroll
-        for (int hf = 0; hf < 2; ++hf) {
-          __syncwarp();
-          if ((lane >> 4) == hf) {
-#pragma unroll
-            for (int x8 = 0; x8 < 4; ++x8) {
-              uint32_t v[4];
-#pragma unroll
-              for (int c = 0; c < 4; ++c) {
-                const __nv_bfloat162 h2 = __floats2bfloat162_rn(__uint_as_float(acc[8 * x8 + 2 * c]),
-                                                                __uint_as_float(acc[8 * x8 + 2 * c + 1]));
-                v[c] = *reinterpret_cast<const uint32_t*>(&h2);
-              }
-              sts128(own(x8), v);
-            }
-          }
-          __syncwarp();
-#pragma unroll
-          for (int y = 0; y < 2; ++y) {
-            const int r = 16 * hf + 8 * y + prow;
-            const int64_t tk = __shfl_sync(0xffffffffu, rtok, r);
-            uint32_t v[4];
-            lds128(v, turned(8 * y + prow));
-            if (i.r0 + quad * 32 + r < p.n)
-              *reinterpret_cast<uint4*>(out + tk * ts) = make_uint4(v[0], v[1], v[2], v[3]);
-          }
-        }
+      if (x == 0 && it > 0) finish();
+      if (!ok || w_item >= total) break;
+      ++x;
+      if (++j == i.T) {
+        j = 0;
+        ++hq;
+        if (KEYS && x < i.iters) g = gate(hq);
       }
-      if (cg >= kPieces) arrive(C::kBarAccFree);
+      if (x == i.iters) {                   // on to the next item
+        done_tok = rtok;
+        done_b = i.b;
+        done_hr = i.hr;
+        done_r0 = i.r0;
+        ++it;
+        w_item += gridDim.x;
+        i = nxt.i;
+        rtok = nxt.tok;
+        lse_r = nxt.lse;
+        delta_r = nxt.delta;
+        g = nxt.g;
+        hq = KEYS ? i.hk * p.G : i.hr;
+        x = j = 0;
+      }
     }
   }
 
