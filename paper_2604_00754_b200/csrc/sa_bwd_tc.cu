@@ -70,6 +70,8 @@ struct BwdTcParams {
   int B, Hq, Hkv, G, n, w, h;
   int linear, one_sided, full_range;
   int n_tiles;
+  int step_r0, step_h, step_b;   // from an item to the one gridDim.x later
+  uint32_t magic_g;              // hr / G == umulhi(hr, magic_g)
   Order o;
   float scale, scale2;
   int64_t qs[3], ks[3];
@@ -107,23 +109,30 @@ struct BCfg {
   // freed together idled the tensor pipe for 1300 of 3400 cycles a step.  Rows = queries: C1 (K)
   // is freed by the accumulation, three slots; C2 (V) by its dP product already, one slot.  Rows =
   // keys: C1 (Q) by dK, which goes first, C2 (dY) by dV behind it, two slots each.  At d = 64
-  // there is room for four of each.
-  static constexpr int kC1 = D == 64 ? 4 : KEYS ? 2 : 3, kC2 = D == 64 ? 4 : KEYS ? 2 : 1;
+  // three of each.
+  static constexpr int kC1 = D == 64 ? 3 : KEYS ? 2 : 3, kC2 = D == 64 ? 3 : KEYS ? 2 : 1;
   static constexpr int kRBufs = D == 128 ? 1 : 2;               // row operand pairs
   static constexpr int kAccCols = (KEYS ? 2 : 1) * D;
-  static constexpr int kNX = KEYS ? 1 : 2;                      // dP buffers
+  // dP buffers.  Rows = keys has room for one (at d = 128): it is worked on in two halves of 64
+  // columns, so that the products of one half run while the row threads have the other.
+  static constexpr int kNX = KEYS ? 1 : 2;
+  static constexpr int kPArrivals = KEYS ? kRowWarps / 2 : kRowWarps;
   static constexpr int kAccBufs = D == 64 ? 2 : 1;
   static constexpr int kOffR = 0;
   static constexpr int kOffC = kRBufs * 2 * kTileBytes;
   static constexpr int kOffC2 = kOffC + kC1 * kTileBytes;
-  static constexpr int kOffStage = kOffC2 + kC2 * kTileBytes;           // 1 KB per row warp
-  static constexpr int kOffVec = kOffStage + kRowWarps * 1024;          // lse2, delta, tokens
-  static constexpr int kOffBar = kOffVec + kC1 * 3 * kTile * 4;
+  // staging of the epilogue: rows of 64 bytes per row warp (half a warp's at a time where only
+  // 16 KB are left)
+  static constexpr int kStageRows = D == 128 && KEYS ? 16 : 32;
+  static constexpr int kOffStage = kOffC2 + kC2 * kTileBytes;
+  static constexpr int kOffVec = kOffStage + kRowWarps * kStageRows * 64;
+  static constexpr int kVecTok = KEYS ? 2 * kTile : 0, kVec = kVecTok + kTile;  // (lse2, delta,) tokens
+  static constexpr int kOffBar = kOffVec + kC1 * kVec * 4;
   static constexpr int kBarRFull = 0, kBarREmpty = kRBufs, kBarC1Full = 2 * kRBufs,
                        kBarC2Full = kBarC1Full + kC1, kBarC1Empty = kBarC2Full + kC2,
                        kBarVFull = kBarC1Empty + kC1, kBarSFull = kBarVFull + kC1, kBarSRead = kBarSFull + 1,
-                       kBarDpFull = kBarSRead + 1, kBarPReady = kBarDpFull + 1,
-                       kBarAccFull = kBarPReady + kNX,
+                       kBarDpFull = kBarSRead + 1, kBarPReady = kBarDpFull + 2,
+                       kBarAccFull = kBarPReady + 2,
                        kBarAccFree = kBarAccFull + kAccBufs, kNumBars = kBarAccFree + kAccBufs;
   static constexpr int kOffMisc = kOffBar + kNumBars * 8;
   static constexpr int kBytes = kOffMisc + 16;
@@ -176,8 +185,8 @@ bwd_tc_kernel(const __grid_constant__ BwdTcParams p, const __grid_constant__ CUt
   if (threadIdx.x == 0) {
     *gave_up = 0;
     for (int i = 0; i < C::kNumBars; ++i)
-      mbar_init(bar(i), (i == C::kBarSRead || (i >= C::kBarPReady && i < C::kBarAccFull) || i >= C::kBarAccFree)
-                            ? kRowWarps : 1);
+      mbar_init(bar(i), i >= C::kBarPReady && i < C::kBarAccFull ? C::kPArrivals
+                        : i == C::kBarSRead || i >= C::kBarAccFree ? kRowWarps : 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     grid_dependency_wait();                   // what earlier launches wrote may be read from here on
     note_skip(reinterpret_cast<volatile int*>(smem + C::kOffMisc + 8), p.status, p.abort_flag);
@@ -199,15 +208,28 @@ bwd_tc_kernel(const __grid_constant__ BwdTcParams p, const __grid_constant__ CUt
   const int H = KEYS ? p.Hkv : p.Hq;
   const int total = p.B * H * p.n_tiles;
   struct Item { int b, hr, hk, r0, cstart, T, iters; };
-  auto item_of = [&](int w_item) {
-    Item i;
-    const int bh = w_item / p.n_tiles;
-    i.r0 = (w_item - bh * p.n_tiles) * kTile;
-    i.b = bh / H;
-    i.hr = bh - i.b * H;
-    i.hk = KEYS ? i.hr : i.hr / p.G;
+  auto span_of = [&](Item& i) {
+    i.hk = KEYS || p.G == 1 ? i.hr : (int)__umulhi((uint32_t)i.hr, p.magic_g);
     column_range(p, i.r0, KEYS, &i.cstart, &i.T);
     i.iters = KEYS ? i.T * p.G : i.T;      // column tiles (times query heads of the group)
+  };
+  auto first_item = [&]() {
+    Item i;
+    const int bh = blockIdx.x / p.n_tiles;
+    i.r0 = (blockIdx.x - bh * p.n_tiles) * kTile;
+    i.b = bh / H;
+    i.hr = bh - i.b * H;
+    span_of(i);
+    return i;
+  };
+  // gridDim.x items on (sixteen row warps would spend a thousand issue slots on the divisions)
+  auto next_item = [&](Item i) {
+    i.r0 += p.step_r0;
+    i.hr += p.step_h;
+    i.b += p.step_b;
+    if (i.r0 >= p.n_tiles * kTile) { i.r0 -= p.n_tiles * kTile; ++i.hr; }
+    if (i.hr >= H) { i.hr -= H; ++i.b; }
+    span_of(i);
     return i;
   };
 
@@ -228,8 +250,8 @@ bwd_tc_kernel(const __grid_constant__ BwdTcParams p, const __grid_constant__ CUt
         for (int c = 0; c < D / 64; ++c)
           tma_load_4d(dst + c * C::kChunkBytes, tm, 64 * c, row, head, b, mb);
       };
-      for (int w_item = blockIdx.x; w_item < total && live; w_item += gridDim.x, ++it) {
-        const Item i = item_of(w_item);
+      Item i = first_item();
+      for (int w_item = blockIdx.x; w_item < total && live; w_item += gridDim.x, ++it, i = next_item(i)) {
         const uint32_t rb = it % C::kRBufs;
         if (it >= (uint32_t)C::kRBufs)
           live = mbar_wait(bar(C::kBarREmpty + rb), (it / C::kRBufs - 1) & 1u, gave_up, p.status);
@@ -254,7 +276,7 @@ bwd_tc_kernel(const __grid_constant__ BwdTcParams p, const __grid_constant__ CUt
                     i.b, mb);
           c1_on = u + 1;
           if (kVec) {
-            const uint32_t vb = bar(C::kBarVFull + s), vec = sbase + C::kOffVec + s * 3 * kTile * 4;
+            const uint32_t vb = bar(C::kBarVFull + s), vec = sbase + C::kOffVec + s * C::kVec * 4;
             mbar_expect_tx(vb, ((KEYS ? 2 : 0) + (TOK ? 1 : 0)) * kTile * 4);
             if (KEYS) {
               const size_t at = ((size_t)i.b * p.Hq + hq) * p.o.spitch + p.o.sleft + col;
@@ -262,12 +284,12 @@ bwd_tc_kernel(const __grid_constant__ BwdTcParams p, const __grid_constant__ CUt
               bulk_load(vec + kTile * 4, p.delta + at, kTile * 4, vb);
             }
             if (TOK)
-              bulk_load(vec + 2 * kTile * 4, p.tok + (size_t)i.b * p.o.spitch + p.o.sleft + col,
+              bulk_load(vec + C::kVecTok * 4, p.tok + (size_t)i.b * p.o.spitch + p.o.sleft + col,
                         kTile * 4, vb);
           }
           // (d = 64: C2's slot was freed together with C1's)
           if (D == 128 && u >= (uint32_t)C::kC2)
-            live = KEYS ? mbar_wait(bar(C::kBarDpFull), (u - 1) & 1u, gave_up, p.status)
+            live = KEYS ? mbar_wait(bar(C::kBarDpFull + 1), (u - 1) & 1u, gave_up, p.status)
                         : mbar_wait(bar(C::kBarSFull), (u - 1) & 1u, gave_up, p.status);
           if (!live) break;
           mb = bar(C::kBarC2Full + s2);
@@ -304,7 +326,7 @@ bwd_tc_kernel(const __grid_constant__ BwdTcParams p, const __grid_constant__ CUt
       // (rows = keys: S alone, whose columns are free once the row threads hold it).  Thread 1: the
       // accumulations (rows = keys: and dP of the next step behind them, over the P and dS that
       // they have read).
-      constexpr uint32_t idesc_s = instr_desc(kTile, kTile, false);
+      constexpr uint32_t idesc_s = instr_desc(kTile, kTile, false), idesc_h = instr_desc(kTile, 64, false);
       constexpr uint32_t idesc_acc = instr_desc(kTile, D, true);
       constexpr uint32_t kDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
       constexpr uint32_t kLoK = (16u >> 4) << 16;                             // K-major operands
@@ -312,96 +334,108 @@ bwd_tc_kernel(const __grid_constant__ BwdTcParams p, const __grid_constant__ CUt
       constexpr uint32_t kBlock = C::kChunkBytes >> 4, kTileD = C::kTileBytes >> 4;
       const uint32_t r_lo = (sbase + C::kOffR) >> 4, c_lo = (sbase + C::kOffC) >> 4,
                      c2_lo = (sbase + C::kOffC2) >> 4;
-      // X (128 x 128, fp32, tensor memory column col) = A B^T, both tiles K-major, K = D
-      auto product = [&](uint32_t col, uint32_t a_lo, uint32_t b_lo) {
+      // X (128 x 128 or 64, fp32, tensor memory column col) = A B^T, both tiles K-major, K = D
+      auto product = [&](uint32_t col, uint32_t a_lo, uint32_t b_lo, uint32_t idesc) {
         const uint64_t ad = desc64(a_lo | kLoK, kDescHi), bd = desc64(b_lo | kLoK, kDescHi);
-        mma_ss_x4(tmem + col, ad, bd, idesc_s, 0u);
-        if (D == 128) mma_ss_x4(tmem + col, ad + kBlock, bd + kBlock, idesc_s, 1u);
+        mma_ss_x4(tmem + col, ad, bd, idesc, 0u);
+        if (D == 128) mma_ss_x4(tmem + col, ad + kBlock, bd + kBlock, idesc, 1u);
       };
-      // acc (128 x D, tensor memory column col) += X (bf16 pairs from column xcol on) * tile
+      // acc (128 x D, tensor memory column col) += X (64 columns, from column xcol on) * 64 rows
       auto accumulate = [&](uint32_t col, uint32_t xcol, uint32_t b_lo, uint32_t acc0) {
-        const uint64_t bd = desc64(b_lo | kLoMN, kDescHi);
-        mma_ts_rows_x4(tmem + col, tmem + xcol, bd, idesc_acc, acc0);
-        mma_ts_rows_x4(tmem + col, tmem + xcol + 64, bd + 512, idesc_acc, 1u);
+        mma_ts_rows_x4(tmem + col, tmem + xcol, desc64(b_lo | kLoMN, kDescHi), idesc_acc, acc0);
       };
       bool ok = true;
       uint32_t u = 0, it = 0;                     // steps and items of this thread
-      // dP of step v (of item j) of the score stream
-      auto issue_dp = [&](uint32_t v, uint32_t j) {
-        const uint32_t rb = j % C::kRBufs, s = v % C::kC2;
-        ok = mbar_wait(bar(C::kBarC2Full + s), (v / C::kC2) & 1u, gave_up, p.status);
-        if (!ok) return;
-        product(C::kColX + 128 * (v % C::kNX), r_lo + (rb * 2 + 1) * kTileD, c2_lo + s * kTileD);
-        tc_commit(bar(KEYS ? C::kBarDpFull : C::kBarSFull));
-      };
+      Item i = first_item();
       if (warp == kMmaWarp) {
-        for (int w_item = blockIdx.x; w_item < total && ok; w_item += gridDim.x, ++it) {
-          const int iters = item_of(w_item).iters;
+        for (int w_item = blockIdx.x; w_item < total && ok; w_item += gridDim.x, ++it, i = next_item(i)) {
           const uint32_t rb = it % C::kRBufs;
           ok = mbar_wait(bar(C::kBarRFull + rb), (it / C::kRBufs) & 1u, gave_up, p.status);
-          for (int x = 0; x < iters && ok; ++x, ++u) {
-            const uint32_t s = u % C::kC1;
+          for (int x = 0; x < i.iters && ok; ++x, ++u) {
+            const uint32_t s = u % C::kC1, s2 = u % C::kC2;
             ok = mbar_wait(bar(C::kBarC1Full + s), (u / C::kC1) & 1u, gave_up, p.status);
             if (ok && u > 0) ok = mbar_wait(bar(C::kBarSRead), (u - 1) & 1u, gave_up, p.status);
             if (!ok) break;
             tc_fence_after();
-            product(C::kColS, r_lo + rb * 2 * kTileD, c_lo + s * kTileD);
-            if (KEYS) {
-              tc_commit(bar(C::kBarSFull));
-            } else {
+            product(C::kColS, r_lo + rb * 2 * kTileD, c_lo + s * kTileD, idesc_s);
+            if (!KEYS) {
               // the dP buffer was read by the accumulation two steps ago, which freed C1
               if (u > 1)
                 ok = mbar_wait(bar(C::kBarC1Empty + (u - 2) % C::kC1), ((u - 2) / C::kC1) & 1u, gave_up,
                                p.status);
-              if (ok) {
-                tc_fence_after();
-                issue_dp(u, it);
-              }
+              if (ok) ok = mbar_wait(bar(C::kBarC2Full + s2), (u / C::kC2) & 1u, gave_up, p.status);
+              if (!ok) break;
+              tc_fence_after();
+              product(C::kColX + 128 * (u % 2), r_lo + (rb * 2 + 1) * kTileD, c2_lo + s2 * kTileD, idesc_s);
             }
+            tc_commit(bar(C::kBarSFull));
           }
           // rows = keys: dP still reads the row operands, the other thread says when it is done
           if (!KEYS && ok) tc_commit(bar(C::kBarREmpty + rb));
         }
-      } else {
-        if (KEYS && (int)blockIdx.x < total) {
-          ok = mbar_wait(bar(C::kBarRFull), 0u, gave_up, p.status);
-          if (ok) issue_dp(0, 0);
-        }
-        for (int w_item = blockIdx.x; w_item < total && ok; w_item += gridDim.x, ++it) {
-          const int iters = item_of(w_item).iters;
+      } else if (!KEYS) {
+        for (int w_item = blockIdx.x; w_item < total && ok; w_item += gridDim.x, ++it, i = next_item(i)) {
           const uint32_t ab = it % C::kAccBufs, acc = C::kColAcc + ab * C::kAccCols;
-          for (int x = 0; x < iters && ok; ++x, ++u) {
-            const uint32_t s = u % C::kC1, s2 = u % C::kC2, xc = C::kColX + 128 * (u % C::kNX);
-            if (x == 0 && it >= (uint32_t)C::kAccBufs)
-              ok = mbar_wait(bar(C::kBarAccFree + ab), (it / C::kAccBufs - 1) & 1u, gave_up, p.status);
-            if (ok) ok = mbar_wait(bar(C::kBarC1Full + s), (u / C::kC1) & 1u, gave_up, p.status);
-            if (ok) ok = mbar_wait(bar(C::kBarPReady + u % C::kNX), (u / C::kNX) & 1u, gave_up, p.status);
+          if (it >= (uint32_t)C::kAccBufs)
+            ok = mbar_wait(bar(C::kBarAccFree + ab), (it / C::kAccBufs - 1) & 1u, gave_up, p.status);
+          for (int x = 0; x < i.iters && ok; ++x, ++u) {
+            const uint32_t s = u % C::kC1, xc = C::kColX + 128 * (u % 2);
+            ok = mbar_wait(bar(C::kBarC1Full + s), (u / C::kC1) & 1u, gave_up, p.status);
+            if (ok) ok = mbar_wait(bar(C::kBarPReady + u % 2), (u / 2) & 1u, gave_up, p.status);
             if (!ok) break;
             tc_fence_after();
-            if (KEYS) {
-              accumulate(acc + D, xc, c_lo + s * kTileD, x > 0);          // dK += dS^T Q
-              if (D == 128) tc_commit(bar(C::kBarC1Empty + s));
-              accumulate(acc, xc + 8, c2_lo + s2 * kTileD, x > 0);        // dV += (g P)^T dY
-              if (D == 64) tc_commit(bar(C::kBarC1Empty + s));
-            } else {
-              accumulate(acc, xc, c_lo + s * kTileD, x > 0);              // dQ += dS K
-              tc_commit(bar(C::kBarC1Empty + s));
-            }
-            const bool last = x + 1 == iters;
-            if (last) tc_commit(bar(C::kBarAccFull + ab));
-            if (KEYS) {
+            accumulate(acc, xc, c_lo + s * kTileD, x > 0);                // dQ += dS K
+            accumulate(acc, xc + 64, c_lo + s * kTileD + 512, 1u);
+            tc_commit(bar(C::kBarC1Empty + s));
+          }
+          if (ok) tc_commit(bar(C::kBarAccFull + ab));
+        }
+      } else {
+        // half hf of dP of step v, whose row operands are in buffer rb
+        auto issue_dp = [&](uint32_t v, uint32_t rb, int hf) {
+          product(C::kColX + 64 * hf, r_lo + (rb * 2 + 1) * kTileD, c2_lo + (v % C::kC2) * kTileD + 512 * hf,
+                  idesc_h);
+          tc_commit(bar(C::kBarDpFull + hf));
+        };
+        auto c2_wait = [&](uint32_t v) {
+          ok = mbar_wait(bar(C::kBarC2Full + v % C::kC2), (v / C::kC2) & 1u, gave_up, p.status);
+        };
+        if ((int)blockIdx.x < total) {
+          ok = mbar_wait(bar(C::kBarRFull), 0u, gave_up, p.status);
+          if (ok) c2_wait(0);
+          for (int hf = 0; hf < 2 && ok; ++hf) issue_dp(0, 0, hf);
+        }
+        for (int w_item = blockIdx.x; w_item < total && ok; w_item += gridDim.x, ++it, i = next_item(i)) {
+          const uint32_t ab = it % C::kAccBufs, acc = C::kColAcc + ab * C::kAccCols;
+          if (it >= (uint32_t)C::kAccBufs)
+            ok = mbar_wait(bar(C::kBarAccFree + ab), (it / C::kAccBufs - 1) & 1u, gave_up, p.status);
+          for (int x = 0; x < i.iters && ok; ++x, ++u) {
+            const uint32_t s = u % C::kC1, c1 = c_lo + s * kTileD, c2 = c2_lo + (u % C::kC2) * kTileD;
+            const bool last = x + 1 == i.iters;
+            ok = mbar_wait(bar(C::kBarC1Full + s), (u / C::kC1) & 1u, gave_up, p.status);
+#pragma unroll
+            for (int hf = 0; hf < 2; ++hf) {
+              if (ok) ok = mbar_wait(bar(C::kBarPReady + hf), u & 1u, gave_up, p.status);
+              if (!ok) break;
+              tc_fence_after();
+              accumulate(acc + D, C::kColX + 64 * hf, c1 + 512 * hf, x > 0 || hf);       // dK += dS^T Q
+              if (D == 128 && hf) tc_commit(bar(C::kBarC1Empty + s));
+              accumulate(acc, C::kColX + 64 * hf + 8, c2 + 512 * hf, x > 0 || hf);       // dV += (g P)^T dY
+              if (D == 64 && hf) tc_commit(bar(C::kBarC1Empty + s));
               if (!last) {
-                issue_dp(u + 1, it);
-              } else {
-                // (S and dP of this item are over: dP by this thread, S long before)
-                tc_commit(bar(C::kBarREmpty + it % C::kRBufs));
-                if (w_item + (int)gridDim.x < total) {
-                  const uint32_t nr = (it + 1) % C::kRBufs;
-                  ok = mbar_wait(bar(C::kBarRFull + nr), ((it + 1) / C::kRBufs) & 1u, gave_up, p.status);
-                  if (ok) issue_dp(u + 1, it + 1);
-                }
+                if (hf == 0) c2_wait(u + 1);
+                if (ok) issue_dp(u + 1, it % C::kRBufs, hf);
               }
             }
+          }
+          if (!ok) break;
+          tc_commit(bar(C::kBarAccFull + ab));
+          tc_commit(bar(C::kBarREmpty + it % C::kRBufs));     // S and dP of this item are over
+          if (w_item + (int)gridDim.x < total) {
+            const uint32_t nr = (it + 1) % C::kRBufs;
+            ok = mbar_wait(bar(C::kBarRFull + nr), ((it + 1) / C::kRBufs) & 1u, gave_up, p.status);
+            if (ok) c2_wait(u);
+            for (int hf = 0; hf < 2 && ok; ++hf) issue_dp(u, nr, hf);
           }
         }
       }
@@ -413,7 +447,7 @@ bwd_tc_kernel(const __grid_constant__ BwdTcParams p, const __grid_constant__ CUt
     const int quad = warp & 3, cg = warp >> 2;          // TMEM lanes, 32-column group
     const int row = quad * 32 + lane, c0 = 32 * cg;
     const uint32_t trow = tmem + ((uint32_t)(quad * 32) << 16);
-    const uint32_t stage = sbase + C::kOffStage + warp * 1024;
+    const uint32_t stage = sbase + C::kOffStage + warp * (C::kStageRows * 64);
     const float inv_scale = 1.f / p.scale;
     uint32_t u = 0, it = 0;
     bool ok = true;
@@ -427,9 +461,9 @@ bwd_tc_kernel(const __grid_constant__ BwdTcParams p, const __grid_constant__ CUt
     };
     // an item and what its rows need from memory, fetched one item ahead
     struct RowItem { Item i; int tok; float lse, delta, g; };
-    auto fetch = [&](int w_item) {
+    auto fetch = [&](const Item& item) {
       RowItem r;
-      r.i = item_of(w_item);
+      r.i = item;
       const int slot = min(r.i.r0 + row, p.n - 1);
       r.tok = p.perm ? p.perm[(size_t)r.i.b * p.n + slot] : slot;
       r.g = gate(KEYS ? r.i.hk * p.G : r.i.hr);
@@ -446,30 +480,34 @@ bwd_tc_kernel(const __grid_constant__ BwdTcParams p, const __grid_constant__ CUt
     // last accumulation's latency nor the row threads' stores leave the pipes idle.
     auto finish = [&]() {
       // Accumulator columns 32 at a time (rows = keys: dV, then dK), the pieces dealt to the column
-      // groups.  A thread holds 64 bytes of a row; 16 rows at a time are turned in the warp's
-      // kilobyte, so that 4 lanes store 64 consecutive bytes.  What the first branch left in the
-      // rows comes in the same way, and is added before the one rounding.
-      constexpr int kPieces = C::kAccCols / 32;
+      // groups.  A thread holds 64 bytes of a row; they are turned in the warp's staging rows, so
+      // that 4 lanes store 64 consecutive bytes.  What the first branch left in the rows comes in
+      // the same way, and is added before the one rounding.
+      constexpr int kPieces = C::kAccCols / 32, kPass = 32 / C::kStageRows, kPer = C::kStageRows / 8;
       const int prow = lane >> 2, pc = lane & 3;
       auto turned = [&](int r) { return stage + r * 64 + ((pc ^ ((r >> 1) & 3)) << 4); };
-      auto own = [&](int x8) { return stage + (lane & 15) * 64 + ((x8 ^ ((lane >> 1) & 3)) << 4); };
-      auto out_of = [&](int piece, __nv_bfloat16** out, int64_t* tok_stride) {
-        const int o = piece / (D / 32);
-        const int64_t* st = KEYS ? p.ks : p.qs;
-        *out = (__nv_bfloat16*)(KEYS ? (o == 0 ? p.dv : p.dk) : p.dq) + done_b * st[0] + done_hr * st[1] +
-               32 * (piece % (D / 32)) + 8 * pc;
-        *tok_stride = st[2];
+      auto own = [&](int x8) {
+        return stage + (lane & (C::kStageRows - 1)) * 64 + ((x8 ^ ((lane >> 1) & 3)) << 4);
+      };
+      const int64_t* st = KEYS ? p.ks : p.qs;
+      const int64_t head = done_b * st[0] + done_hr * st[1] + 8 * pc;
+      int64_t off[4];                       // this lane's rows prow, prow + 8, ...
+      bool have[4];
+#pragma unroll
+      for (int y = 0; y < 4; ++y) {
+        off[y] = head + (int64_t)__shfl_sync(0xffffffffu, done_tok, 8 * y + prow) * st[2];
+        have[y] = done_r0 + quad * 32 + 8 * y + prow < p.n;
+      }
+      auto out_of = [&](int piece) {
+        return (__nv_bfloat16*)(!KEYS ? p.dq : piece < D / 32 ? p.dv : p.dk) + 32 * (piece % (D / 32));
       };
       uint4 old[4];
       auto load_old = [&](int piece) {
-        __nv_bfloat16* out;
-        int64_t ts;
-        out_of(piece, &out, &ts);
+        const __nv_bfloat16* out = out_of(piece);
 #pragma unroll
         for (int y = 0; y < 4; ++y) {
-          const int64_t tk = __shfl_sync(0xffffffffu, done_tok, 8 * y + prow);
           old[y] = make_uint4(0u, 0u, 0u, 0u);
-          if (done_r0 + quad * 32 + 8 * y + prow < p.n) old[y] = *reinterpret_cast<const uint4*>(out + tk * ts);
+          if (have[y]) old[y] = *reinterpret_cast<const uint4*>(out + off[y]);
         }
       };
       if (cg < kPieces && p.accumulate) load_old(cg);
@@ -480,9 +518,7 @@ bwd_tc_kernel(const __grid_constant__ BwdTcParams p, const __grid_constant__ CUt
       tc_fence_after();
 #pragma unroll 1
       for (int piece = cg; piece < kPieces; piece += 4) {
-        __nv_bfloat16* out;
-        int64_t ts;
-        out_of(piece, &out, &ts);
+        __nv_bfloat16* out = out_of(piece);
         uint32_t acc[32];
         tmem_ld32(trow + C::kColAcc + ab * C::kAccCols + 32 * piece, acc);
         tmem_wait_ld();
@@ -490,13 +526,13 @@ bwd_tc_kernel(const __grid_constant__ BwdTcParams p, const __grid_constant__ CUt
         if (p.accumulate) {
           if (piece != cg) load_old(piece);
 #pragma unroll
-          for (int hf = 0; hf < 2; ++hf) {
+          for (int hf = 0; hf < kPass; ++hf) {
             __syncwarp();
 #pragma unroll
-            for (int y = 0; y < 2; ++y)
-              sts128(turned(8 * y + prow), reinterpret_cast<const uint32_t(&)[4]>(old[2 * hf + y]));
+            for (int y = 0; y < kPer; ++y)
+              sts128(turned(8 * y + prow), reinterpret_cast<const uint32_t(&)[4]>(old[kPer * hf + y]));
             __syncwarp();
-            if ((lane >> 4) == hf) {
+            if (kPass == 1 || (lane >> 4) == hf) {
 #pragma unroll
               for (int x8 = 0; x8 < 4; ++x8) {
                 uint32_t v[4];
@@ -504,38 +540,37 @@ bwd_tc_kernel(const __grid_constant__ BwdTcParams p, const __grid_constant__ CUt
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
                   const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&v[c]));
-                  acc[8 * x8 + 2 * c] = __float_as_uint(__uint_as_float(acc[8 * x8 + 2 * c]) + f.x);
-                  acc[8 * x8 + 2 * c + 1] = __float_as_uint(__uint_as_float(acc[8 * x8 + 2 * c + 1]) + f.y);
+                  const float2 sum = __fadd2_rn(f, make_float2(__uint_as_float(acc[8 * x8 + 2 * c]),
+                                                               __uint_as_float(acc[8 * x8 + 2 * c + 1])));
+                  acc[8 * x8 + 2 * c] = __float_as_uint(sum.x);
+                  acc[8 * x8 + 2 * c + 1] = __float_as_uint(sum.y);
                 }
               }
             }
           }
         }
+        uint32_t pk[16];
 #pragma unroll
-        for (int hf = 0; hf < 2; ++hf) {
+        for (int c = 0; c < 16; ++c) {
+          const __nv_bfloat162 h2 =
+              __floats2bfloat162_rn(__uint_as_float(acc[2 * c]), __uint_as_float(acc[2 * c + 1]));
+          pk[c] = *reinterpret_cast<const uint32_t*>(&h2);
+        }
+#pragma unroll
+        for (int hf = 0; hf < kPass; ++hf) {
           __syncwarp();
-          if ((lane >> 4) == hf) {
+          if (kPass == 1 || (lane >> 4) == hf) {
 #pragma unroll
-            for (int x8 = 0; x8 < 4; ++x8) {
-              uint32_t v[4];
-#pragma unroll
-              for (int c = 0; c < 4; ++c) {
-                const __nv_bfloat162 h2 = __floats2bfloat162_rn(__uint_as_float(acc[8 * x8 + 2 * c]),
-                                                                __uint_as_float(acc[8 * x8 + 2 * c + 1]));
-                v[c] = *reinterpret_cast<const uint32_t*>(&h2);
-              }
-              sts128(own(x8), v);
-            }
+            for (int x8 = 0; x8 < 4; ++x8)
+              sts128(own(x8), reinterpret_cast<const uint32_t(&)[4]>(pk[4 * x8]));
           }
           __syncwarp();
 #pragma unroll
-          for (int y = 0; y < 2; ++y) {
-            const int r = 16 * hf + 8 * y + prow;
-            const int64_t tk = __shfl_sync(0xffffffffu, done_tok, r);
+          for (int y = 0; y < kPer; ++y) {
             uint32_t v[4];
             lds128(v, turned(8 * y + prow));
-            if (done_r0 + quad * 32 + r < p.n)
-              *reinterpret_cast<uint4*>(out + tk * ts) = make_uint4(v[0], v[1], v[2], v[3]);
+            if (have[kPer * hf + y])
+              *reinterpret_cast<uint4*>(out + off[kPer * hf + y]) = make_uint4(v[0], v[1], v[2], v[3]);
           }
         }
       }
@@ -543,15 +578,25 @@ bwd_tc_kernel(const __grid_constant__ BwdTcParams p, const __grid_constant__ CUt
     };
     RowItem nxt{};
     int w_item = blockIdx.x;
-    if (w_item < total) nxt = fetch(w_item);
+    if (w_item < total) nxt = fetch(first_item());
     Item i = nxt.i;
     int rtok = nxt.tok, hq = KEYS ? i.hk * p.G : i.hr, x = 0, j = 0;
     float lse_r = nxt.lse, delta_r = nxt.delta, g = nxt.g;
     while (true) {
       if (w_item < total) {
         const int rslot = i.r0 + row;
+        if (x == 0 && p.accumulate && rslot < p.n) {
+          // the epilogue will add to these rows: start bringing them into L2
+          const int64_t* st = KEYS ? p.ks : p.qs;
+          const int64_t at = i.b * st[0] + i.hr * st[1] + (int64_t)rtok * st[2];
+#pragma unroll
+          for (int piece = cg; piece < C::kAccCols / 32; piece += 4) {
+            const __nv_bfloat16* out = (const __nv_bfloat16*)(!KEYS ? p.dq : piece < D / 32 ? p.dv : p.dk);
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(out + at + 32 * (piece % (D / 32))));
+          }
+        }
         const uint32_t s = u % C::kC1;
-        const float* vec = reinterpret_cast<const float*>(smem + C::kOffVec) + s * 3 * kTile + c0;
+        const float* vec = reinterpret_cast<const float*>(smem + C::kOffVec) + s * C::kVec + c0;
         const int cb = i.cstart + j * kTile;
         if (kVec) ok = mbar_wait(bar(C::kBarVFull + s), (u / C::kC1) & 1u, gave_up, p.status);
         if (ok) ok = mbar_wait(bar(C::kBarSFull), u & 1u, gave_up, p.status);
@@ -579,7 +624,7 @@ bwd_tc_kernel(const __grid_constant__ BwdTcParams p, const __grid_constant__ CUt
         }
         if (TOK) {
           // rows = queries: hide later key tokens; rows = keys: earlier query tokens
-          const int32_t* ct = reinterpret_cast<const int32_t*>(vec + 2 * kTile);
+          const int32_t* ct = reinterpret_cast<const int32_t*>(vec + C::kVecTok);
 #pragma unroll
           for (int y = 0; y < 32; y += 4) {
             const int4 c4 = *reinterpret_cast<const int4*>(ct + y);
@@ -623,7 +668,7 @@ bwd_tc_kernel(const __grid_constant__ BwdTcParams p, const __grid_constant__ CUt
             if (!(seen & (1u << y))) sv[y] = 0u;
         }
         // what the next item's rows need is on its way while this one's last step is worked on
-        if (x + 1 == i.iters && w_item + (int)gridDim.x < total) nxt = fetch(w_item + gridDim.x);
+        if (x + 1 == i.iters && w_item + (int)gridDim.x < total) nxt = fetch(next_item(i));
         // P times the gate for dV, then dP and dS; both go back as bf16 pairs over dP
         const uint32_t xa = trow + C::kColX + 128 * (u % C::kNX) + c0;
         uint32_t pk[KEYS ? 16 : 1];
@@ -635,7 +680,7 @@ bwd_tc_kernel(const __grid_constant__ BwdTcParams p, const __grid_constant__ CUt
                                                             __uint_as_float(sv[2 * y + 1]) * gp);
             pk[y] = *reinterpret_cast<const uint32_t*>(&h2);
           }
-          ok = mbar_wait(bar(C::kBarDpFull), u & 1u, gave_up, p.status);
+          ok = mbar_wait(bar(C::kBarDpFull + (cg >> 1)), u & 1u, gave_up, p.status);
           ok = __all_sync(0xffffffffu, ok);
           if (!ok) break;
           tc_fence_after();
@@ -667,7 +712,7 @@ bwd_tc_kernel(const __grid_constant__ BwdTcParams p, const __grid_constant__ CUt
         }
         tmem_wait_st();
         // (with two dP buffers a quick warp may be here for step u + 1 before a slow one for step u)
-        arrive(C::kBarPReady + u % C::kNX);
+        arrive(C::kBarPReady + (KEYS ? cg >> 1 : (int)(u & 1u)));
         ++u;
       }
       if (x == 0 && it > 0) finish();
@@ -907,9 +952,13 @@ cudaError_t launch_side(const BwdTcParams& p, const CUtensorMap* tm, int sms, cu
   const cudaError_t e =
       cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kBytes);
   if (e != cudaSuccess) return e;
-  const int total = p.B * (KEYS ? p.Hkv : p.Hq) * p.n_tiles;
-  return launch_dependent(kernel, dim3(total < sms ? total : sms), dim3(kThreads), C::kBytes, st, p,
-                          tm[0], tm[1], tm[2], tm[3]);
+  const int H = KEYS ? p.Hkv : p.Hq, total = p.B * H * p.n_tiles, grid = total < sms ? total : sms;
+  BwdTcParams q = p;
+  q.step_r0 = grid % p.n_tiles * kTile;
+  q.step_h = grid / p.n_tiles % H;
+  q.step_b = grid / p.n_tiles / H;
+  q.magic_g = p.G > 1 ? (uint32_t)(((1ull << 32) + p.G - 1) / p.G) : 0u;
+  return launch_dependent(kernel, dim3(grid), dim3(kThreads), C::kBytes, st, q, tm[0], tm[1], tm[2], tm[3]);
 }
 
 template <int D>
