@@ -288,7 +288,8 @@ bwd_tc_kernel(const __grid_constant__ BwdTcParams p, const __grid_constant__ CUt
                         kTile * 4, vb);
           }
           // (d = 64: C2's slot was freed together with C1's)
-          if (D == 128 && u >= (uint32_t)C::kC2)
+          // (from u = 1 on: a parity wait may not pass over a phase unseen)
+          if (D == 128 && u > 0)
             live = KEYS ? mbar_wait(bar(C::kBarDpFull + 1), (u - 1) & 1u, gave_up, p.status)
                         : mbar_wait(bar(C::kBarSFull), (u - 1) & 1u, gave_up, p.status);
           if (!live) break;
