@@ -7,7 +7,7 @@
 //   kDy: dz w             (w read with its rows as the contraction index: N-major operand);
 //                          epilogue adds dout * g and writes dy
 //   kDw: dz^T y           (both operands read with their rows as the contraction index);
-//                          epilogue writes dw
+//                          epilogue writes dw, or fp32 products of parts of the rows
 // A plain kernel per step serves fp32 and sizes the tensor-core path does not take.
 //
 // Every mbarrier wait is bounded; on expiry the CTA records SA_ERR_TIMEOUT in the device
@@ -22,32 +22,39 @@ enum BwdMode { kDz = 0, kDy = 1, kDw = 2, kFwd = 3 };   // kFwd: the forward's s
 constexpr int kT = 128, kBK = 64;                  // output tiles of 128 rows, K chunks of 64
 constexpr int kATileBytes = kT * kBK * 2;          // A of one K chunk, either major: 16 KB
 constexpr int kChunk = 64 * kBK * 2;               // 64 rows x 64 columns: one box of a row-contracted operand
-constexpr int kRingBytes = 12 * kATileBytes;       // 192 KB of operand stages
-// TN: columns of the output tile.  256 halves the operand bytes per flop of the B side and is
-// used when it still leaves at least one tile per SM; 128 otherwise.  A stage holds 64 KB or
-// 48 KB (two K chunks of A + B at TN = 128, one at TN = 256): eight or four products.
-template <int TN> struct Tile {
-  static constexpr int kCps = TN == 128 ? 2 : 1;                 // K chunks per stage
-  static constexpr int kBTileBytes = TN * kBK * 2;
-  static constexpr int kStageBytes = kCps * (kATileBytes + kBTileBytes);
-  static constexpr int kStages = kRingBytes / kStageBytes;       // 3 or 4
+constexpr int kEpiTile = kT * 128;                 // epilogue: 128 rows x 128 bytes, 16 KB
+// Shared memory: the operand ring, then the epilogue's tiles, for each half of the output columns
+// as many as a chunk of 64 columns has inputs (outputs are written in place): kDz y and dout,
+// kFwd y and out, kDy dout * g, kDw a tile for the output alone.
+template <int MODE> struct Epi {
+  static constexpr int kIn = MODE == kDw ? 0 : MODE == kDy ? 1 : 2;
+  static constexpr int kTiles = kIn == 2 ? 2 : 1;                // per half
+  static constexpr int kRingBytes = (kIn == 2 ? 9 : 12) * kATileBytes;
 };
-constexpr int kMaxStages = 4;
-constexpr int kThreadsB = 320;
-constexpr int kOffBars = kRingBytes;
+// TN: columns of the output tile.  256 halves the operand bytes per flop of the B side and is
+// used when it still leaves at least one tile per SM; 128 otherwise.  A stage is one K chunk of
+// A + B, 48 or 32 KB.
+template <int MODE, int TN> struct Tile {
+  static constexpr int kBTileBytes = TN * kBK * 2;
+  static constexpr int kStageBytes = kATileBytes + kBTileBytes;
+  static constexpr int kStages = Epi<MODE>::kRingBytes / kStageBytes;       // 3 to 6
+};
+constexpr int kMaxStages = 6;
+constexpr int kThreadsB = 384;                     // TMA, MMA, eight epilogue warps, two movers
 constexpr int kBarFull = 0, kBarEmpty = kMaxStages, kBarAccFull = 2 * kMaxStages,
-              kBarAccEmpty = 2 * kMaxStages + 2, kNumBars = 2 * kMaxStages + 4;
-constexpr int kOffMisc = kOffBars + kNumBars * 8;
-constexpr int kSmemB = kOffMisc + 16;
+              kBarAccEmpty = kBarAccFull + 2, kBarIn = kBarAccEmpty + 2, kBarOut = kBarIn + 2,
+              kNumBars = kBarOut + 2;
+template <int MODE> struct Smem {
+  static constexpr int kOffEpi = Epi<MODE>::kRingBytes;
+  static constexpr int kOffBars = kOffEpi + 2 * Epi<MODE>::kTiles * kEpiTile;
+  static constexpr int kOffMisc = kOffBars + kNumBars * 8;
+  static constexpr int kBytes = kOffMisc + 16;
+};
 
 struct BwdGateParams {
-  // epilogue operands, all [*, dm] with the given pitches (elements)
-  const __nv_bfloat16 *dout, *y;   // kDz
-  __nv_bfloat16 *dz, *dyd;         // kDz out; kDy reads dyd
-  __nv_bfloat16* out;              // kDy: dy, kDw: dw
-  int64_t ld_y, ld_ws, ld_out;
-  int64_t m_rows, n_cols;          // extent of the product
-  int tiles_m, tiles_n, k_pairs;   // k_pairs: hand-overs per tile (one or two K chunks each)
+  int m_rows, n_cols;              // extent of the product
+  int tiles_m, tiles_n, k_chunks;  // K chunks of 64
+  int splits, per_split;           // kDw: the K chunks go in `splits` parts of `per_split`
   int accum;                       // kFwd: add to what out already holds (second path)
   int* status;
 };
@@ -67,9 +74,13 @@ __host__ __device__ constexpr uint32_t idesc_of(int tn, bool a_mn, bool b_mn) {
 template <int MODE, int TN>
 __global__ void __launch_bounds__(kThreadsB, 1)
 gate_bwd_kernel(const __grid_constant__ BwdGateParams p, const __grid_constant__ CUtensorMap tm_a,
-                const __grid_constant__ CUtensorMap tm_b) {
+                const __grid_constant__ CUtensorMap tm_b, const __grid_constant__ CUtensorMap tm_i0,
+                const __grid_constant__ CUtensorMap tm_i1, const __grid_constant__ CUtensorMap tm_o0,
+                const __grid_constant__ CUtensorMap tm_o1) {
   constexpr bool kAmn = MODE == kDw, kBmn = MODE == kDy || MODE == kDw;
-  using TL = Tile<TN>;
+  using TL = Tile<MODE, TN>;
+  using SM = Smem<MODE>;
+  constexpr int kIn = Epi<MODE>::kIn;
   constexpr int kStages = TL::kStages, kStageBytes = TL::kStageBytes, kTN = TN;
   constexpr int kBlock = 2048 / TN;       // column tiles per block of the tile order
   extern __shared__ __align__(1024) uint8_t smem[];
@@ -79,14 +90,15 @@ gate_bwd_kernel(const __grid_constant__ BwdGateParams p, const __grid_constant__
     if (threadIdx.x == 0) atomicCAS(p.status, SA_OK, SA_ERR_CUDA);
     return;
   }
-  const uint32_t bar0 = sbase + kOffBars;
+  const uint32_t bar0 = sbase + SM::kOffBars;
   auto bar = [&](int i) { return bar0 + 8u * (uint32_t)i; };
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + kOffMisc);
-  volatile int* gave_up = reinterpret_cast<volatile int*>(smem + kOffMisc + 4);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + SM::kOffMisc);
+  volatile int* gave_up = reinterpret_cast<volatile int*>(smem + SM::kOffMisc + 4);
   if (threadIdx.x == 0) {
     *gave_up = 0;
-    note_skip(reinterpret_cast<volatile int*>(smem + kOffMisc + 8), p.status, nullptr);
-    for (int i = 0; i < kNumBars; ++i) mbar_init(bar(i), (i >= kBarAccEmpty) ? 256 : 1);
+    note_skip(reinterpret_cast<volatile int*>(smem + SM::kOffMisc + 8), p.status, nullptr);
+    for (int i = 0; i < kNumBars; ++i) 
+      mbar_init(bar(i), i >= kBarOut ? 128 : i >= kBarIn ? 1 : i >= kBarAccEmpty ? 256 : 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
@@ -98,16 +110,26 @@ gate_bwd_kernel(const __grid_constant__ BwdGateParams p, const __grid_constant__
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  SA_LEAVE_IF_SKIPPED(reinterpret_cast<volatile int*>(smem + kOffMisc + 8), 1, tmem, 512u)
-  const int total = p.tiles_m * p.tiles_n;
+  SA_LEAVE_IF_SKIPPED(reinterpret_cast<volatile int*>(smem + SM::kOffMisc + 8), 1, tmem, 512u)
+  const int tiles = p.tiles_m * p.tiles_n, total = MODE == kDw ? tiles * p.splits : tiles;
   // blocks of 2048 columns, row tile by row tile inside a block (operand slices stay in L2)
-  auto origin = [&](int tile, int* m0, int* n0) {
+  auto origin = [&](int item, int* m0, int* n0) {
+    const int tile = MODE == kDw ? item % tiles : item;
     const int per_block = p.tiles_m * kBlock;
     const int nb = tile / per_block, rem = tile - nb * per_block;
     const int width = min(kBlock, p.tiles_n - nb * kBlock);
     *m0 = (rem / width) * kT;
     *n0 = (nb * kBlock + rem % width) * kTN;
   };
+  // the K chunks of an item: all, or (kDw) those of its part
+  auto chunks = [&](int item, int* first, int* last) {
+    const int part = MODE == kDw ? item / tiles : 0;
+    *first = MODE == kDw ? part * p.per_split : 0;
+    *last = MODE == kDw ? min(*first + p.per_split, p.k_chunks) : p.k_chunks;
+  };
+  // the epilogue's chunks: 128 bytes of output columns, the tile's columns in two halves
+  const bool parts = MODE == kDw && p.splits > 1;
+  const int chunk_cols = parts ? 32 : 64, half_chunks = (kTN / 2) / chunk_cols;
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
@@ -117,29 +139,27 @@ gate_bwd_kernel(const __grid_constant__ BwdGateParams p, const __grid_constant__
       for (int tile = blockIdx.x; tile < total && ok; tile += gridDim.x) {
         int m0, n0;
         origin(tile, &m0, &n0);
-        for (int kp = 0; kp < p.k_pairs && ok; ++kp, ++use) {
+        int kc, k_end;
+        chunks(tile, &kc, &k_end);
+        for (; kc < k_end && ok; ++kc, ++use) {
           const uint32_t s = use % kStages;
           if (use >= (uint32_t)kStages)
             ok = mbar_wait(bar(kBarEmpty + s), (use / kStages - 1) & 1u, gave_up, p.status);
           if (!ok) break;
-          const uint32_t dst = sbase + s * kStageBytes, fb = bar(kBarFull + s);
+          const uint32_t da = sbase + s * kStageBytes, db = da + kATileBytes, fb = bar(kBarFull + s);
           mbar_expect_tx(fb, kStageBytes);
+          const int k0 = kc * kBK;                                      // past the end: zeros
+          if (kAmn) {
 #pragma unroll
-          for (int q = 0; q < TL::kCps; ++q) {
-            const int k0 = (TL::kCps * kp + q) * kBK;                   // past the end: zeros
-            const uint32_t da = dst + q * (kATileBytes + TL::kBTileBytes), db = da + kATileBytes;
-            if (kAmn) {
+            for (int c = 0; c < kT / 64; ++c) tma_load_2d(da + c * kChunk, &tm_a, m0 + 64 * c, k0, fb);
+          } else {
+            tma_load_2d(da, &tm_a, k0, m0, fb);
+          }
+          if (kBmn) {
 #pragma unroll
-              for (int c = 0; c < kT / 64; ++c) tma_load_2d(da + c * kChunk, &tm_a, m0 + 64 * c, k0, fb);
-            } else {
-              tma_load_2d(da, &tm_a, k0, m0, fb);
-            }
-            if (kBmn) {
-#pragma unroll
-              for (int c = 0; c < kTN / 64; ++c) tma_load_2d(db + c * kChunk, &tm_b, n0 + 64 * c, k0, fb);
-            } else {
-              tma_load_2d(db, &tm_b, k0, n0, fb);
-            }
+            for (int c = 0; c < kTN / 64; ++c) tma_load_2d(db + c * kChunk, &tm_b, n0 + 64 * c, k0, fb);
+          } else {
+            tma_load_2d(db, &tm_b, k0, n0, fb);
           }
         }
       }
@@ -170,34 +190,76 @@ gate_bwd_kernel(const __grid_constant__ BwdGateParams p, const __grid_constant__
         if (!ok) break;
         tc_fence_after();
         const uint32_t d = tmem + buf * kTN;
-        for (int kp = 0; kp < p.k_pairs && ok; ++kp, ++use) {
+        int kc, k_end;
+        chunks(tile, &kc, &k_end);
+        for (uint32_t acc = 0; kc < k_end && ok; ++kc, ++use, acc = 1) {
           const uint32_t s = use % kStages;
           ok = mbar_wait(bar(kBarFull + s), (use / kStages) & 1u, gave_up, p.status);
           if (!ok) break;
           tc_fence_after();
-          const uint32_t lo = (sbase + s * kStageBytes) >> 4;
+          const uint32_t la = (sbase + s * kStageBytes) >> 4;
+          const uint64_t a0 = desc64(la | (kAmn ? kLoMN : kLoK), kDescHi);
+          const uint64_t b0 = desc64((la + (kATileBytes >> 4)) | (kBmn ? kLoMN : kLoK), kDescHi);
 #pragma unroll
-          for (int q = 0; q < TL::kCps; ++q) {
-            const uint32_t la = lo + q * ((kATileBytes + TL::kBTileBytes) >> 4);
-            const uint64_t a0 = desc64(la | (kAmn ? kLoMN : kLoK), kDescHi);
-            const uint64_t b0 = desc64((la + (kATileBytes >> 4)) | (kBmn ? kLoMN : kLoK), kDescHi);
-#pragma unroll
-            for (int ks = 0; ks < 4; ++ks)
-              mma_ss(d, a0 + ks * (kAmn ? kStepMN : kStepK), b0 + ks * (kBmn ? kStepMN : kStepK),
-                     idesc, (kp > 0 || q > 0 || ks > 0) ? 1u : 0u);
-          }
+          for (int ks = 0; ks < 4; ++ks)
+            mma_ss(d, a0 + ks * (kAmn ? kStepMN : kStepK), b0 + ks * (kBmn ? kStepMN : kStepK),
+                   idesc, ks > 0 ? 1u : acc);
           tc_commit(bar(kBarEmpty + s));
         }
         if (ok) tc_commit(bar(kBarAccFull + buf));
       }
     }
     __syncwarp();
+  } else if (warp >= 10) {
+    // --------------------------------- movers: the epilogue's tiles of one half of the columns
+    // A thread holds a row, so reading and writing global memory from the registers touches 32
+    // lines per instruction (30000 cycles for a 128 x 256 tile of kDz, whose products take 8200).
+    // TMA brings a chunk of 64 columns x 128 rows of every input into shared memory, the row
+    // threads write the outputs in their place, and TMA takes them out; the next chunk comes as
+    // soon as this one has been read.
+    if (lane == 0) {
+      const int hf = warp - 10;
+      const uint32_t buf0 = sbase + SM::kOffEpi + hf * Epi<MODE>::kTiles * kEpiTile;
+      const uint32_t in_bar = bar(kBarIn + hf), out_bar = bar(kBarOut + hf);
+      const int inputs = MODE == kFwd ? 1 + p.accum : kIn;
+      uint32_t e = 0;
+      bool ok = true;
+      for (int tile = blockIdx.x; tile < total && ok; tile += gridDim.x) {
+        int m0, n0;
+        origin(tile, &m0, &n0);
+        for (int c = 0; c < half_chunks && ok; ++c, ++e) {
+          const int col = n0 + hf * (kTN / 2) + c * chunk_cols;
+          if (col >= p.n_cols) break;
+          if (e) bulk_wait_read();
+          if (kIn) {
+            mbar_expect_tx(in_bar, inputs * kEpiTile);
+            tma_load_2d(buf0, &tm_i0, col, m0, in_bar);
+            if (inputs > 1) tma_load_2d(buf0 + kEpiTile, &tm_i1, col, m0, in_bar);
+          } else {
+            mbar_arrive(in_bar);
+          }
+          ok = mbar_wait(out_bar, e & 1u, gave_up, p.status);
+          if (!ok) break;
+          if (parts) tma_store_3d(&tm_o0, buf0, col, m0, tile / tiles);
+          else tma_store_2d(&tm_o0, buf0, col, m0);
+          if (MODE == kDz) tma_store_2d(&tm_o1, buf0 + kEpiTile, col, m0);
+          bulk_commit();
+        }
+      }
+      if (!ok && kIn)          // the last inputs must land before the shared memory goes away
+        for (int tries = 0; tries < 100000 && !mbar_try(in_bar, e & 1u); ++tries) __nanosleep(100);
+      bulk_wait();
+    }
+    __syncwarp();
   } else {
     // ---------------------------------------------------------- epilogue (warps 2-9)
+    // one row per thread; warps 2-5 take the first half of the tile's columns, 6-9 the other
     const int half = (warp - 2) >> 2;
     const int row = (warp & 3) * 32 + lane;
     const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
-    uint32_t it = 0;
+    const uint32_t own = sbase + SM::kOffEpi + half * Epi<MODE>::kTiles * kEpiTile + row * 128;
+    auto piece = [&](int j) { return own + ((j ^ (row & 7)) << 4); };   // 16 bytes of the row
+    uint32_t it = 0, e = 0;
     bool ok = true;
     for (int tile = blockIdx.x; tile < total; tile += gridDim.x, ++it) {
       const uint32_t buf = it & 1u;
@@ -207,87 +269,81 @@ gate_bwd_kernel(const __grid_constant__ BwdGateParams p, const __grid_constant__
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       tc_fence_after();
-      const int64_t r = (int64_t)m0 + row;
-      const bool row_ok = r < p.m_rows;
 #pragma unroll 1
-      for (int c = (kTN / 64) * half; c < (kTN / 64) * (half + 1); ++c) {
+      for (int c = 0; c < half_chunks; ++c, ++e) {
+        const int col = half * (kTN / 2) + c * chunk_cols;
+        if (n0 + col >= p.n_cols) break;
+        const uint32_t acc_at = tmem + lane_addr + buf * kTN + col;
         uint32_t acc[32];
-        tmem_ld32(tmem + lane_addr + buf * kTN + 32 * c, acc);
+        tmem_ld32(acc_at, acc);
+        ok = mbar_wait(bar(kBarIn + half), e & 1u, gave_up, p.status);
+        ok = __all_sync(0xffffffffu, ok);
         tmem_wait_ld();
-        const int col = n0 + 32 * c;
-        // the epilogue's row reads are requested together, ahead of the stores they may not
-        // pass (the outputs may alias the inputs as far as the compiler knows), so that their
-        // latencies overlap: fy = y (kDz, kFwd) or dout * g (kDy), fo = dout (kDz) or out (kFwd)
-        uint4 fy[4], fo[4];
-        if (MODE != kDw && row_ok && col < p.n_cols) {
+        if (!ok) break;
+        if (parts) {
 #pragma unroll
-          for (int x8 = 0; x8 < 4; ++x8) {
-            const int64_t e = col + 8 * x8;
-            if (MODE == kDy) fy[x8] = *reinterpret_cast<const uint4*>(p.dyd + r * p.ld_ws + e);
-            else fy[x8] = *reinterpret_cast<const uint4*>(p.y + r * p.ld_y + e);
-            if (MODE == kDz || (MODE == kFwd && p.accum))
-              fo[x8] = *reinterpret_cast<const uint4*>((MODE == kDz ? p.dout : p.out) + r * p.ld_out + e);
+          for (int j = 0; j < 8; ++j) {
+            const uint32_t st[4] = {acc[4 * j], acc[4 * j + 1], acc[4 * j + 2], acc[4 * j + 3]};
+            sts128(piece(j), st);
           }
-        }
-        if (row_ok && col < p.n_cols) {
+        } else {
 #pragma unroll
-          for (int x8 = 0; x8 < 4; ++x8) {
-            const int64_t e = col + 8 * x8;
-            float v8[8];
+          for (int s2 = 0; s2 < 2; ++s2) {
+            if (s2) {
+              tmem_ld32(acc_at + 32, acc);
+              tmem_wait_ld();
+            }
 #pragma unroll
-            for (int x = 0; x < 8; ++x) v8[x] = __uint_as_float(acc[8 * x8 + x]);
-            uint4 st;
-            __nv_bfloat162* hs = reinterpret_cast<__nv_bfloat162*>(&st);
-            if (MODE == kDz) {
-              const __nv_bfloat162* hy = reinterpret_cast<const __nv_bfloat162*>(&fy[x8]);
-              const __nv_bfloat162* hd = reinterpret_cast<const __nv_bfloat162*>(&fo[x8]);
-              uint4 st2;
-              __nv_bfloat162* hs2 = reinterpret_cast<__nv_bfloat162*>(&st2);
+            for (int x8 = 0; x8 < 4; ++x8) {
+              const uint32_t at = piece(4 * s2 + x8);
+              float v8[8];
 #pragma unroll
-              for (int x = 0; x < 4; ++x) {
-                const float g0 = logistic(v8[2 * x]), g1 = logistic(v8[2 * x + 1]);
-                const float d0 = __low2float(hd[x]), d1 = __high2float(hd[x]);
-                hs[x] = __floats2bfloat162_rn(d0 * __low2float(hy[x]) * g0 * (1.f - g0),
-                                              d1 * __high2float(hy[x]) * g1 * (1.f - g1));
-                hs2[x] = __floats2bfloat162_rn(d0 * g0, d1 * g1);
-              }
-              *reinterpret_cast<uint4*>(p.dz + r * p.ld_ws + e) = st;
-              *reinterpret_cast<uint4*>(p.dyd + r * p.ld_ws + e) = st2;
-            } else if (MODE == kFwd) {
-              const __nv_bfloat162* hy = reinterpret_cast<const __nv_bfloat162*>(&fy[x8]);
-#pragma unroll
-              for (int x = 0; x < 4; ++x) {
-                v8[2 * x] = logistic(v8[2 * x]) * __low2float(hy[x]);
-                v8[2 * x + 1] = logistic(v8[2 * x + 1]) * __high2float(hy[x]);
-              }
-              uint4* dst = reinterpret_cast<uint4*>(p.out + r * p.ld_out + e);
-              if (p.accum) {
-                const __nv_bfloat162* ho = reinterpret_cast<const __nv_bfloat162*>(&fo[x8]);
+              for (int x = 0; x < 8; ++x) v8[x] = __uint_as_float(acc[8 * x8 + x]);
+              uint32_t f0[4], f1[4], st[4];
+              if (kIn) lds128(f0, at);
+              if (MODE == kDz || (MODE == kFwd && p.accum)) lds128(f1, at + kEpiTile);
+              __nv_bfloat162* hs = reinterpret_cast<__nv_bfloat162*>(st);
+              const __nv_bfloat162* h0 = reinterpret_cast<const __nv_bfloat162*>(f0);
+              const __nv_bfloat162* h1 = reinterpret_cast<const __nv_bfloat162*>(f1);
+              if (MODE == kDz) {
+                uint32_t st2[4];
+                __nv_bfloat162* hs2 = reinterpret_cast<__nv_bfloat162*>(st2);
 #pragma unroll
                 for (int x = 0; x < 4; ++x) {
-                  v8[2 * x] += __low2float(ho[x]);
-                  v8[2 * x + 1] += __high2float(ho[x]);
+                  const float g0 = logistic(v8[2 * x]), g1 = logistic(v8[2 * x + 1]);
+                  const float d0 = __low2float(h1[x]), d1 = __high2float(h1[x]);
+                  hs[x] = __floats2bfloat162_rn(d0 * __low2float(h0[x]) * g0 * (1.f - g0),
+                                                d1 * __high2float(h0[x]) * g1 * (1.f - g1));
+                  hs2[x] = __floats2bfloat162_rn(d0 * g0, d1 * g1);
                 }
-              }
+                sts128(at + kEpiTile, st2);
+              } else {
+                if (MODE == kFwd) {
 #pragma unroll
-              for (int x = 0; x < 4; ++x) hs[x] = __floats2bfloat162_rn(v8[2 * x], v8[2 * x + 1]);
-              *dst = st;
-            } else {
-              if (MODE == kDy) {
-                const __nv_bfloat162* hp = reinterpret_cast<const __nv_bfloat162*>(&fy[x8]);
-#pragma unroll
-                for (int x = 0; x < 4; ++x) {
-                  v8[2 * x] += __low2float(hp[x]);
-                  v8[2 * x + 1] += __high2float(hp[x]);
+                  for (int x = 0; x < 4; ++x) {
+                    v8[2 * x] = logistic(v8[2 * x]) * __low2float(h0[x]);
+                    v8[2 * x + 1] = logistic(v8[2 * x + 1]) * __high2float(h0[x]);
+                  }
                 }
-              }
+                if (MODE == kDy || (MODE == kFwd && p.accum)) {
+                  const __nv_bfloat162* ha = MODE == kDy ? h0 : h1;
 #pragma unroll
-              for (int x = 0; x < 4; ++x) hs[x] = __floats2bfloat162_rn(v8[2 * x], v8[2 * x + 1]);
-              *reinterpret_cast<uint4*>(p.out + r * p.ld_out + e) = st;
+                  for (int x = 0; x < 4; ++x) {
+                    v8[2 * x] += __low2float(ha[x]);
+                    v8[2 * x + 1] += __high2float(ha[x]);
+                  }
+                }
+#pragma unroll
+                for (int x = 0; x < 4; ++x) hs[x] = __floats2bfloat162_rn(v8[2 * x], v8[2 * x + 1]);
+              }
+              sts128(at, st);
             }
           }
         }
+        fence_proxy_async();
+        mbar_arrive(bar(kBarOut + half));
       }
+      if (!ok) break;
       tc_fence_before();
       mbar_arrive(bar(kBarAccEmpty + buf));
     }
@@ -300,6 +356,25 @@ gate_bwd_kernel(const __grid_constant__ BwdGateParams p, const __grid_constant__
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u)
                  : "memory");
   }
+}
+
+// dw = the sum of its parts, added in their order; 8 columns per thread.
+__global__ void dw_sum_kernel(const float4* __restrict__ part, int splits, int64_t eights,
+                              uint4* __restrict__ dw) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= eights) return;
+  float4 a = part[2 * i], b = part[2 * i + 1];
+#pragma unroll 4
+  for (int s = 1; s < splits; ++s) {
+    const float4 c = part[2 * (s * eights + i)], d = part[2 * (s * eights + i) + 1];
+    a.x += c.x; a.y += c.y; a.z += c.z; a.w += c.w;
+    b.x += d.x; b.y += d.y; b.z += d.z; b.w += d.w;
+  }
+  uint4 st;
+  __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(&st);
+  h[0] = __floats2bfloat162_rn(a.x, a.y); h[1] = __floats2bfloat162_rn(a.z, a.w);
+  h[2] = __floats2bfloat162_rn(b.x, b.y); h[3] = __floats2bfloat162_rn(b.z, b.w);
+  dw[i] = st;
 }
 
 // ------------------------------------------------- plain kernels (fp32, other sizes)
@@ -352,21 +427,52 @@ bool wide_tiles(int64_t m_rows, int64_t n_cols, int sms) {
   return ((m_rows + kT - 1) / kT) * ((n_cols + 255) / 256) >= 2 * (int64_t)sms;
 }
 
+struct Maps { CUtensorMap a, b, i0, i1, o0, o1; };
+
 template <int MODE, int TN>
-cudaError_t launch_mode(BwdGateParams p, const CUtensorMap& a, const CUtensorMap& b, int64_t k,
-                        int sms, cudaStream_t st) {
-  p.tiles_m = (int)((p.m_rows + kT - 1) / kT);
-  p.tiles_n = (int)((p.n_cols + TN - 1) / TN);
-  const int per = Tile<TN>::kCps * kBK;
-  p.k_pairs = (int)((k + per - 1) / per);
+cudaError_t launch_mode(BwdGateParams p, const Maps& m, int64_t k, int sms, cudaStream_t st) {
+  p.tiles_m = (p.m_rows + kT - 1) / kT;
+  p.tiles_n = (p.n_cols + TN - 1) / TN;
+  p.k_chunks = (int)((k + kBK - 1) / kBK);
+  if (p.splits < 1) p.splits = 1;
+  p.per_split = (p.k_chunks + p.splits - 1) / p.splits;
   cudaError_t e = cudaFuncSetAttribute(gate_bwd_kernel<MODE, TN>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemB);
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       Smem<MODE>::kBytes);
   if (e != cudaSuccess) return e;
-  const int64_t total = (int64_t)p.tiles_m * p.tiles_n;
+  const int64_t total = (int64_t)p.tiles_m * p.tiles_n * p.splits;
   const unsigned grid = (unsigned)(total < sms ? total : sms);
-  gate_bwd_kernel<MODE, TN><<<grid, kThreadsB, kSmemB, st>>>(p, a, b);
+  gate_bwd_kernel<MODE, TN><<<grid, kThreadsB, Smem<MODE>::kBytes, st>>>(p, m.a, m.b, m.i0, m.i1,
+                                                                        m.o0, m.o1);
   bump_launches();
   return cudaGetLastError();
+}
+
+// dw contracts over all rows and has few tiles (64 of 128 x 128 at dm = 1024, 148 SMs), so the rows
+// go in parts, whose fp32 products dw_sum_kernel adds up.  Tile width and number of parts: the
+// cheapest by the cycles that a K chunk (512 or 300, by tile width), an item's start and end (3000)
+// and the parts' way through memory (8 bytes per element, 3000 bytes a cycle; 4000 for the launch)
+// take.  The parts use the half of the workspace that bf16 dz and dout * g leave, so they are at
+// most rows / dm.
+// 32768 rows, dm = 1024, nine parts of 128 x 256 tiles: 60 us and 7 us for the sum; the whole
+// backward of one path 332 -> 246 us, with the epilogue's tiles by TMA (dm = 512: 224 -> 103).
+struct DwPlan { int tn, splits; };
+DwPlan plan_dw(int64_t rows, int dm, int sms) {
+  const int64_t kc = (rows + kBK - 1) / kBK;
+  DwPlan best{128, 1};
+  double least = 1e300;
+  for (int tn = 128; tn <= 256; tn += 128) {
+    const int64_t tiles = (int64_t)((dm + kT - 1) / kT) * ((dm + tn - 1) / tn);
+    for (int64_t s = 1; s <= 64 && s <= kc && (s == 1 || s * dm <= rows); ++s) {
+      const int64_t per = (kc + s - 1) / s;
+      if ((kc + per - 1) / per != s) continue;          // an empty part
+      const double waves = (double)((tiles * s + sms - 1) / sms);
+      const double cost = waves * (per * (tn == 256 ? 512. : 300.) + 3000.) +
+                          (s > 1 ? 4000. + s * (double)dm * dm * 8. / 3000. : 0.);
+      if (cost < least) { least = cost; best = {tn, (int)s}; }
+    }
+  }
+  return best;
 }
 
 }  // namespace
@@ -382,18 +488,19 @@ bool gate_forward_wide(int64_t rows, int dm, const void* y_sa, const void* y_swa
   for (int x = 0; x < (y_swa ? 2 : 1); ++x) {
     const void* y = x ? y_swa : y_sa;
     const void* w = x ? w_swa : w_sa;
-    CUtensorMap y_k, w_k;
-    if (!make_map(&y_k, y, rows, dm, ld_y, 128) || !make_map(&w_k, w, dm, dm, dm, 256)) {
+    Maps m;
+    if (!make_map(&m.a, y, rows, dm, ld_y, 128) || !make_map(&m.b, w, dm, dm, dm, 256) ||
+        !make_map(&m.o0, out, rows, dm, ld_out, 128)) {
       *err = cudaErrorUnknown;
       return true;
     }
+    m.i0 = m.a;
+    m.i1 = m.o1 = m.o0;
     BwdGateParams p{};
     p.status = status;
-    p.y = (const __nv_bfloat16*)y; p.ld_y = ld_y;
-    p.out = (__nv_bfloat16*)out; p.ld_out = ld_out;
-    p.m_rows = rows; p.n_cols = dm;
+    p.m_rows = (int)rows; p.n_cols = dm;
     p.accum = x;
-    *err = launch_mode<kFwd, 256>(p, y_k, w_k, dm, sms, st);
+    *err = launch_mode<kFwd, 256>(p, m, dm, sms, st);
     if (*err != cudaSuccess) return true;
   }
   return true;
@@ -439,33 +546,46 @@ extern "C" sa_status sa_gate_projection_backward(
     if (tc) {
       __nv_bfloat16* dz = (__nv_bfloat16*)ws;
       __nv_bfloat16* dyd = dz + rows * (int64_t)dm;
-      const bool wide_r = wide_tiles(rows, dm, sms), wide_w = wide_tiles(dm, dm, sms);
-      CUtensorMap y_k, w_k, dz_k, w_mn, dz_mn, y_mn;
+      float* part = (float*)(dyd + rows * (int64_t)dm);
+      const bool wide = wide_tiles(rows, dm, sms);
+      const DwPlan dwp = plan_dw(rows, dm, sms);
+      CUtensorMap y_k, w_k, dz_k, w_mn, dz_mn, y_mn, dout_k, dyd_k, dy_k, dw_o;
       if (!make_map(&y_k, y, rows, dm, ld_y, 128) ||
-          !make_map(&w_k, w, dm, dm, dm, wide_r ? 256 : 128) ||
+          !make_map(&w_k, w, dm, dm, dm, wide ? 256 : 128) ||
           !make_map(&dz_k, dz, rows, dm, dm, 128) || !make_map(&w_mn, w, dm, dm, dm, 64) ||
-          !make_map(&dz_mn, dz, rows, dm, dm, 64) || !make_map(&y_mn, y, rows, dm, ld_y, 64))
+          !make_map(&dz_mn, dz, rows, dm, dm, 64) || !make_map(&y_mn, y, rows, dm, ld_y, 64) ||
+          !make_map(&dout_k, dout, rows, dm, ld_dout, 128) ||
+          !make_map(&dyd_k, dyd, rows, dm, dm, 128) || !make_map(&dy_k, dy, rows, dm, ld_dy, 128) ||
+          !(dwp.splits > 1 ? make_map_f32(&dw_o, part, dwp.splits, dm, dm)
+                           : make_map(&dw_o, dw, dm, dm, dm, 128)))
         return SA_ERR_CUDA;
       BwdGateParams p{};
       p.status = status;
-      p.dz = dz; p.dyd = dyd; p.ld_ws = dm; p.ld_y = ld_y;
       // z = y w^T; epilogue: dz, dout * g
-      p.dout = (const __nv_bfloat16*)dout; p.y = (const __nv_bfloat16*)y; p.ld_out = ld_dout;
-      p.m_rows = rows; p.n_cols = dm;
-      if ((wide_r ? launch_mode<kDz, 256>(p, y_k, w_k, dm, sms, st)
-                  : launch_mode<kDz, 128>(p, y_k, w_k, dm, sms, st)) != cudaSuccess)
+      p.m_rows = (int)rows; p.n_cols = dm;
+      Maps m{y_k, w_k, y_k, dout_k, dz_k, dyd_k};
+      if ((wide ? launch_mode<kDz, 256>(p, m, dm, sms, st)
+                : launch_mode<kDz, 128>(p, m, dm, sms, st)) != cudaSuccess)
         return SA_ERR_CUDA;
       // dy = dz w + dout * g
-      p.out = (__nv_bfloat16*)dy; p.ld_out = ld_dy;
-      if ((wide_r ? launch_mode<kDy, 256>(p, dz_k, w_mn, dm, sms, st)
-                  : launch_mode<kDy, 128>(p, dz_k, w_mn, dm, sms, st)) != cudaSuccess)
+      m = Maps{dz_k, w_mn, dyd_k, dyd_k, dy_k, dy_k};
+      if ((wide ? launch_mode<kDy, 256>(p, m, dm, sms, st)
+                : launch_mode<kDy, 128>(p, m, dm, sms, st)) != cudaSuccess)
         return SA_ERR_CUDA;
       // dw = dz^T y
-      p.out = (__nv_bfloat16*)dw; p.ld_out = dm;
-      p.m_rows = dm; p.n_cols = dm;
-      if ((wide_w ? launch_mode<kDw, 256>(p, dz_mn, y_mn, rows, sms, st)
-                  : launch_mode<kDw, 128>(p, dz_mn, y_mn, rows, sms, st)) != cudaSuccess)
+      p.m_rows = dm;
+      p.splits = dwp.splits;
+      m = Maps{dz_mn, y_mn, y_mn, y_mn, dw_o, dw_o};
+      if ((dwp.tn == 256 ? launch_mode<kDw, 256>(p, m, rows, sms, st)
+                         : launch_mode<kDw, 128>(p, m, rows, sms, st)) != cudaSuccess)
         return SA_ERR_CUDA;
+      if (dwp.splits > 1) {
+        const int64_t eights = (int64_t)dm * dm / 8;
+        dw_sum_kernel<<<(unsigned)((eights + 255) / 256), 256, 0, st>>>(
+            (const float4*)part, dwp.splits, eights, (uint4*)dw);
+        bump_launches();
+        if (cudaGetLastError() != cudaSuccess) return SA_ERR_CUDA;
+      }
     } else {
       float* dz = (float*)ws;
       float* dyd = dz + rows * (int64_t)dm;
