@@ -17,7 +17,8 @@
 namespace sa {
 namespace {
 
-enum BwdMode { kDz = 0, kDy = 1, kDw = 2, kFwd = 3 };   // kFwd: the forward's sigmoid(y w^T) * y
+// kFwd: the forward's sigmoid(y w^T) * y; kFwdAdd: the same added to what out already holds
+enum BwdMode { kDz = 0, kDy = 1, kDw = 2, kFwd = 3, kFwdAdd = 4 };
 
 constexpr int kT = 128, kBK = 64;                  // output tiles of 128 rows, K chunks of 64
 constexpr int kATileBytes = kT * kBK * 2;          // A of one K chunk, either major: 16 KB
@@ -25,9 +26,9 @@ constexpr int kChunk = 64 * kBK * 2;               // 64 rows x 64 columns: one 
 constexpr int kEpiTile = kT * 128;                 // epilogue: 128 rows x 128 bytes, 16 KB
 // Shared memory: the operand ring, then the epilogue's tiles, for each half of the output columns
 // as many as a chunk of 64 columns has inputs (outputs are written in place): kDz y and dout,
-// kFwd y and out, kDy dout * g, kDw a tile for the output alone.
+// kFwd y, kFwdAdd y and out, kDy dout * g, kDw a tile for the output alone.
 template <int MODE> struct Epi {
-  static constexpr int kIn = MODE == kDw ? 0 : MODE == kDy ? 1 : 2;
+  static constexpr int kIn = MODE == kDw ? 0 : MODE == kDy || MODE == kFwd ? 1 : 2;
   static constexpr int kTiles = kIn == 2 ? 2 : 1;                // per half
   static constexpr int kRingBytes = (kIn == 2 ? 9 : 12) * kATileBytes;
 };
@@ -55,7 +56,6 @@ struct BwdGateParams {
   int m_rows, n_cols;              // extent of the product
   int tiles_m, tiles_n, k_chunks;  // K chunks of 64
   int splits, per_split;           // kDw: the K chunks go in `splits` parts of `per_split`
-  int accum;                       // kFwd: add to what out already holds (second path)
   int* status;
 };
 
@@ -221,7 +221,6 @@ gate_bwd_kernel(const __grid_constant__ BwdGateParams p, const __grid_constant__
       const int hf = warp - 10;
       const uint32_t buf0 = sbase + SM::kOffEpi + hf * Epi<MODE>::kTiles * kEpiTile;
       const uint32_t in_bar = bar(kBarIn + hf), out_bar = bar(kBarOut + hf);
-      const int inputs = MODE == kFwd ? 1 + p.accum : kIn;
       uint32_t e = 0;
       bool ok = true;
       for (int tile = blockIdx.x; tile < total && ok; tile += gridDim.x) {
@@ -232,9 +231,9 @@ gate_bwd_kernel(const __grid_constant__ BwdGateParams p, const __grid_constant__
           if (col >= p.n_cols) break;
           if (e) bulk_wait_read();
           if (kIn) {
-            mbar_expect_tx(in_bar, inputs * kEpiTile);
+            mbar_expect_tx(in_bar, kIn * kEpiTile);
             tma_load_2d(buf0, &tm_i0, col, m0, in_bar);
-            if (inputs > 1) tma_load_2d(buf0 + kEpiTile, &tm_i1, col, m0, in_bar);
+            if (kIn > 1) tma_load_2d(buf0 + kEpiTile, &tm_i1, col, m0, in_bar);
           } else {
             mbar_arrive(in_bar);
           }
@@ -301,7 +300,7 @@ gate_bwd_kernel(const __grid_constant__ BwdGateParams p, const __grid_constant__
               for (int x = 0; x < 8; ++x) v8[x] = __uint_as_float(acc[8 * x8 + x]);
               uint32_t f0[4], f1[4], st[4];
               if (kIn) lds128(f0, at);
-              if (MODE == kDz || (MODE == kFwd && p.accum)) lds128(f1, at + kEpiTile);
+              if (kIn > 1) lds128(f1, at + kEpiTile);
               __nv_bfloat162* hs = reinterpret_cast<__nv_bfloat162*>(st);
               const __nv_bfloat162* h0 = reinterpret_cast<const __nv_bfloat162*>(f0);
               const __nv_bfloat162* h1 = reinterpret_cast<const __nv_bfloat162*>(f1);
@@ -318,14 +317,14 @@ gate_bwd_kernel(const __grid_constant__ BwdGateParams p, const __grid_constant__
                 }
                 sts128(at + kEpiTile, st2);
               } else {
-                if (MODE == kFwd) {
+                if (MODE == kFwd || MODE == kFwdAdd) {
 #pragma unroll
                   for (int x = 0; x < 4; ++x) {
                     v8[2 * x] = logistic(v8[2 * x]) * __low2float(h0[x]);
                     v8[2 * x + 1] = logistic(v8[2 * x + 1]) * __high2float(h0[x]);
                   }
                 }
-                if (MODE == kDy || (MODE == kFwd && p.accum)) {
+                if (MODE == kDy || MODE == kFwdAdd) {
                   const __nv_bfloat162* ha = MODE == kDy ? h0 : h1;
 #pragma unroll
                   for (int x = 0; x < 4; ++x) {
@@ -499,8 +498,8 @@ bool gate_forward_wide(int64_t rows, int dm, const void* y_sa, const void* y_swa
     BwdGateParams p{};
     p.status = status;
     p.m_rows = (int)rows; p.n_cols = dm;
-    p.accum = x;
-    *err = launch_mode<kFwd, 256>(p, m, dm, sms, st);
+    *err = x ? launch_mode<kFwdAdd, 256>(p, m, dm, sms, st)
+             : launch_mode<kFwd, 256>(p, m, dm, sms, st);
     if (*err != cudaSuccess) return true;
   }
   return true;
@@ -547,7 +546,11 @@ extern "C" sa_status sa_gate_projection_backward(
       __nv_bfloat16* dz = (__nv_bfloat16*)ws;
       __nv_bfloat16* dyd = dz + rows * (int64_t)dm;
       float* part = (float*)(dyd + rows * (int64_t)dm);
-      const bool wide = wide_tiles(rows, dm, sms);
+      // 128 x 256 tiles when their waves take less time than those of 128 x 128: a wide tile's
+      // K chunk takes 512 cycles, a narrow one's 300 (64 columns of operands per product more)
+      const int64_t tm = (rows + kT - 1) / kT;
+      const bool wide = (tm * ((dm + 255) / 256) + sms - 1) / sms * 512 <=
+                        (tm * ((dm + 127) / 128) + sms - 1) / sms * 300;
       const DwPlan dwp = plan_dw(rows, dm, sms);
       CUtensorMap y_k, w_k, dz_k, w_mn, dz_mn, y_mn, dout_k, dyd_k, dy_k, dw_o;
       if (!make_map(&y_k, y, rows, dm, ld_y, 128) ||
