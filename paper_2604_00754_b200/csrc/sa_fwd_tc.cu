@@ -765,15 +765,20 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
             lo = max(lo, -kv);
             hi = min(hi, p.n - 1 - kv);
           }
-          if (hi < lo) { lo = 1 << 30; hi = lo; }
-          const uint32_t span = (uint32_t)(hi - lo);
+          // as one bit per column: a bit test and a select per score, where comparing the column
+          // with both ends took a subtraction more (one-sided branch, 8 x 12 heads of 64, n = 4096,
+          // w = 128: 86 -> 77 us; 2 x 16 heads of 128, w = 256: 56 -> 51, its SA branch 83 -> 79)
 #pragma unroll
-          for (int c = 0; c < kHalf; c += 4) {
-            token_mask(c);
-            if ((uint32_t)(c - lo) > span) sr[c] = 0xff800000u;
-            if ((uint32_t)(c + 1 - lo) > span) sr[c + 1] = 0xff800000u;
-            if ((uint32_t)(c + 2 - lo) > span) sr[c + 2] = 0xff800000u;
-            if ((uint32_t)(c + 3 - lo) > span) sr[c + 3] = 0xff800000u;
+          for (int c0 = 0; c0 < kHalf; c0 += 32) {
+            const int a = max(lo - c0, 0), e = min(hi - c0, 31);
+            const uint32_t seen = e < a ? 0u : (0xffffffffu >> (31 - e)) & (0xffffffffu << a);
+#pragma unroll
+            for (int c = c0; c < c0 + 32; c += 4) {
+              token_mask(c);
+#pragma unroll
+              for (int x = c; x < c + 4; ++x)
+                if (!(seen & (1u << (x - c0)))) sr[x] = 0xff800000u;
+            }
           }
         }
         float mx0 = __uint_as_float(sr[0]), mx1 = __uint_as_float(sr[1]);
