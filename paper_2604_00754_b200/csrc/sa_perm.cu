@@ -143,7 +143,8 @@ __global__ void rank_kernel(const uint64_t* __restrict__ bkeys, const int32_t* _
 // against 12.4 us, n = 4096 x 8 sequences 7.7 against 13.0, n = 8192 10.1 against 15.2, n = 16384
 // 14.0 against 16.5 (with eight CTAs of 4096 tokens, n = 32768: 22.0 against 16.1).
 // An owner has room for cap entries; its expected share is n / C with a standard deviation
-// below sqrt(n / C), and cap leaves 10 of those.  If a share is larger all the same, every CTA
+// below sqrt(n / C), and cap leaves 10 of those (an eighth of the share, 3 of them at 512 tokens,
+// was passed by one call in twelve with 8 sequences of 4096, at 760 us instead of 8).  If a share is larger all the same, every CTA
 // ranks its own tokens by comparing with every key of the sequence: slow, and still exact.
 constexpr int kClusterThreads = 1024;
 constexpr int kShareMax = 2048;                                   // tokens per CTA
@@ -161,7 +162,9 @@ __host__ inline ClusterPlan cluster_plan(int n) {
   const int share = (n + (1 << p.log2_c) - 1) >> p.log2_c;
   p.bits = 0;
   while (p.bits < 10 && (share >> (p.bits + 3)) > 0) ++p.bits;    // about 8 keys per bucket
-  p.cap = p.log2_c ? share + share / 8 : share;
+  int sd = 1;
+  while (sd * sd < share) ++sd;
+  p.cap = p.log2_c ? share + 10 * sd : share;
   p.threads = share >= kClusterThreads ? kClusterThreads : (share + 31) / 32 * 32;
   if (p.threads < 64) p.threads = 64;
   p.cap = (p.cap + 3) / 4 * 4;
