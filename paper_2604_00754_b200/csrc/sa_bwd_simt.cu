@@ -67,6 +67,8 @@ __global__ void __launch_bounds__(kWarps * 32) bwd_delta_kernel(const BwdArgs a)
   const int hq = blockIdx.y, b = blockIdx.z;
   const int64_t base = b * a.qs[0] + hq * a.qs[1];
   const int r0 = blockIdx.x * kDeltaRowsPerBlock + warp * 4 + sub;
+  grid_dependency_wait();
+  grid_dependents_launch();
   float part[2] = {0.f, 0.f};
   float dot[2][kDeltaRowsPerBlock / 32];
 #pragma unroll
@@ -112,6 +114,7 @@ __global__ void __launch_bounds__(128) dgate_kernel(const BwdArgs a) {
   __shared__ float wsum[4];
   const int hq = blockIdx.x, x = blockIdx.y;
   grid_dependency_wait();
+  grid_dependents_launch();
   float s = 0.f;
   for (int i = threadIdx.x; i < a.B * a.chunks; i += 128)
     s += a.partials[(((size_t)x * a.B + i / a.chunks) * a.Hq + hq) * a.chunks + i % a.chunks];
@@ -300,6 +303,8 @@ template <int NCG>
 __global__ void __launch_bounds__(kTileThreads)
 bwd_tile_kernel(const BwdArgs a, int x0, int nb, int heads, bool split) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  grid_dependency_wait();
+  grid_dependents_launch();
   if (a.abort_flag && *a.abort_flag) return;
   const int b = blockIdx.z, G = a.Hq / a.Hkv;
   const size_t rows_q = (size_t)a.B * a.Hq * a.n * a.d;
@@ -326,6 +331,8 @@ __global__ void __launch_bounds__(256) reduce_kernel(const BwdArgs a) {
   const int G = a.Hq / a.Hkv, q4 = a.d / 4;
   const size_t nq = (size_t)a.B * a.Hq * a.n * q4, nk = nq / G;
   size_t i = (size_t)blockIdx.x * 256 + threadIdx.x;
+  grid_dependency_wait();
+  grid_dependents_launch();
   if (i >= nq + 2 * nk) return;
   const int which = i < nq ? 0 : (i < nq + nk ? 1 : 2);
   i -= which == 0 ? 0 : (which == 1 ? nq : nq + nk);
@@ -354,18 +361,19 @@ cudaError_t launch_tiles(const BwdArgs& a, cudaStream_t st) {
   if (e != cudaSuccess) return e;
   const unsigned tiles = (a.n + kRows - 1) / kRows;
   if (split_tiles(a.B, a.Hkv, a.n)) {
-    bwd_tile_kernel<NCG><<<dim3(tiles, 2 * a.Hq * a.nbranch, a.B), kTileThreads, smem, st>>>(
-        a, 0, a.nbranch, 1, true);
+    e = launch_dependent(bwd_tile_kernel<NCG>, dim3(tiles, 2 * a.Hq * a.nbranch, a.B),
+                         dim3(kTileThreads), smem, st, a, 0, a.nbranch, 1, true);
+    if (e != cudaSuccess) return e;
     const size_t items = ((size_t)a.Hq + 2 * a.Hkv) * a.B * a.n * (a.d / 4);
-    reduce_kernel<<<(unsigned)((items + 255) / 256), 256, 0, st>>>(a);
     bump_launches(2);
-  } else {
-    for (int x = 0; x < a.nbranch; ++x)
-      bwd_tile_kernel<NCG><<<dim3(tiles, a.Hq + a.Hkv, a.B), kTileThreads, smem, st>>>(
-          a, x, 1, a.Hq / a.Hkv, false);
-    bump_launches(a.nbranch);
+    return launch_dependent(reduce_kernel, dim3((unsigned)((items + 255) / 256)), dim3(256), 0, st, a);
   }
-  return cudaGetLastError();
+  for (int x = 0; x < a.nbranch && e == cudaSuccess; ++x) {
+    e = launch_dependent(bwd_tile_kernel<NCG>, dim3(tiles, a.Hq + a.Hkv, a.B), dim3(kTileThreads),
+                         smem, st, a, x, 1, a.Hq / a.Hkv, false);
+    bump_launches();
+  }
+  return e;
 }
 
 template <typename T>
@@ -539,7 +547,9 @@ cudaError_t launch_all(BwdArgs a, cudaStream_t st) {
     e = launch_bwd_tc(a, st);
     return e != cudaSuccess ? e : launch_dgate(a, st);
   }
-  bwd_delta_kernel<T><<<dim3(a.chunks, a.Hq, a.B), kWarps * 32, 0, st>>>(a);
+  if ((e = launch_dependent(bwd_delta_kernel<T>, dim3(a.chunks, a.Hq, a.B), dim3(kWarps * 32), 0, st,
+                            a)) != cudaSuccess)
+    return e;
   bump_launches();
   if ((e = launch_dgate(a, st)) != cudaSuccess) return e;
   if constexpr (std::is_same<T, float>::value) {

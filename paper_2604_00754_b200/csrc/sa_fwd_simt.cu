@@ -25,6 +25,8 @@ __global__ void __launch_bounds__(kTileThreads) fwd_tile_kernel(const FwdArgs a)
   const int tx = lane & 15, half = lane >> 4;         // key / column index, row group of the warp
   const int row0 = warp * 8 + half * 4;               // this thread's four rows
   const int hq = blockIdx.y, b = blockIdx.z, s0 = blockIdx.x * kRows;
+  grid_dependency_wait();
+  grid_dependents_launch();
   if (a.abort_flag && *a.abort_flag) return;          // an earlier check rejected perm/inv
   const int hk = hq / (a.Hq / a.Hkv), d = a.d;
   const int32_t* perm = a.swa ? nullptr : a.perm + (size_t)b * a.n;
@@ -161,9 +163,8 @@ cudaError_t go(const FwdArgs& a, cudaStream_t st) {
   const int smem = sm.rows_bytes() + 4 * sm.col_bytes() + kTileThreads / 32 * kCols * 8 * 4;
   cudaError_t e = allow_smem((const void*)fwd_tile_kernel<T, NCG>, smem);
   if (e != cudaSuccess) return e;
-  fwd_tile_kernel<T, NCG>
-      <<<dim3((a.n + kRows - 1) / kRows, a.Hq, a.B), kTileThreads, smem, st>>>(a);
-  return cudaSuccess;
+  return launch_dependent(fwd_tile_kernel<T, NCG>, dim3((a.n + kRows - 1) / kRows, a.Hq, a.B),
+                          dim3(kTileThreads), smem, st, a);
 }
 
 template <typename T>

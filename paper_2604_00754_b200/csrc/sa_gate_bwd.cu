@@ -96,6 +96,7 @@ gate_bwd_kernel(const __grid_constant__ BwdGateParams p, const __grid_constant__
   volatile int* gave_up = reinterpret_cast<volatile int*>(smem + SM::kOffMisc + 4);
   if (threadIdx.x == 0) {
     *gave_up = 0;
+    grid_dependency_wait();                   // what earlier launches wrote may be read from here on
     note_skip(reinterpret_cast<volatile int*>(smem + SM::kOffMisc + 8), p.status, nullptr);
     for (int i = 0; i < kNumBars; ++i) 
       mbar_init(bar(i), i >= kBarOut ? 128 : i >= kBarIn ? 1 : i >= kBarAccEmpty ? 256 : 1);
@@ -109,6 +110,7 @@ gate_bwd_kernel(const __grid_constant__ BwdGateParams p, const __grid_constant__
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  grid_dependents_launch();
   const uint32_t tmem = *tmem_slot;
   SA_LEAVE_IF_SKIPPED(reinterpret_cast<volatile int*>(smem + SM::kOffMisc + 8), 1, tmem, 512u)
   const int tiles = p.tiles_m * p.tiles_n, total = MODE == kDw ? tiles * p.splits : tiles;
@@ -361,6 +363,8 @@ gate_bwd_kernel(const __grid_constant__ BwdGateParams p, const __grid_constant__
 __global__ void dw_sum_kernel(const float4* __restrict__ part, int splits, int64_t eights,
                               uint4* __restrict__ dw) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  grid_dependency_wait();
+  grid_dependents_launch();
   if (i >= eights) return;
   float4 a = part[2 * i], b = part[2 * i + 1];
 #pragma unroll 4
@@ -441,10 +445,9 @@ cudaError_t launch_mode(BwdGateParams p, const Maps& m, int64_t k, int sms, cuda
   if (e != cudaSuccess) return e;
   const int64_t total = (int64_t)p.tiles_m * p.tiles_n * p.splits;
   const unsigned grid = (unsigned)(total < sms ? total : sms);
-  gate_bwd_kernel<MODE, TN><<<grid, kThreadsB, Smem<MODE>::kBytes, st>>>(p, m.a, m.b, m.i0, m.i1,
-                                                                        m.o0, m.o1);
   bump_launches();
-  return cudaGetLastError();
+  return launch_dependent(gate_bwd_kernel<MODE, TN>, dim3(grid), dim3(kThreadsB), Smem<MODE>::kBytes,
+                          st, p, m.a, m.b, m.i0, m.i1, m.o0, m.o1);
 }
 
 // dw contracts over all rows and has few tiles (64 of 128 x 128 at dm = 1024, 148 SMs), so the rows
@@ -584,10 +587,10 @@ extern "C" sa_status sa_gate_projection_backward(
         return SA_ERR_CUDA;
       if (dwp.splits > 1) {
         const int64_t eights = (int64_t)dm * dm / 8;
-        dw_sum_kernel<<<(unsigned)((eights + 255) / 256), 256, 0, st>>>(
-            (const float4*)part, dwp.splits, eights, (uint4*)dw);
         bump_launches();
-        if (cudaGetLastError() != cudaSuccess) return SA_ERR_CUDA;
+        if (launch_dependent(dw_sum_kernel, dim3((unsigned)((eights + 255) / 256)), dim3(256), 0, st,
+                             (const float4*)part, dwp.splits, eights, (uint4*)dw) != cudaSuccess)
+          return SA_ERR_CUDA;
       }
     } else {
       float* dz = (float*)ws;

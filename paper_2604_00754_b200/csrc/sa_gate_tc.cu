@@ -70,6 +70,7 @@ gate_tc_kernel(const __grid_constant__ GateParams p, const __grid_constant__ CUt
 
   if (threadIdx.x == 0) {
     *gave_up = 0;
+    grid_dependency_wait();                   // what earlier launches wrote may be read from here on
     note_skip(reinterpret_cast<volatile int*>(smem + kOffMisc + 8), p.status, nullptr);
     for (int i = 0; i < kNumBars; ++i)
       mbar_init(bar(i), (i >= kBarAccEmpty) ? 256 : 1);
@@ -83,6 +84,7 @@ gate_tc_kernel(const __grid_constant__ GateParams p, const __grid_constant__ CUt
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  grid_dependents_launch();
   const uint32_t tmem = *tmem_slot;
   SA_LEAVE_IF_SKIPPED(reinterpret_cast<volatile int*>(smem + kOffMisc + 8), 1, tmem, 512u)
   const int total = p.tiles_m * p.tiles_n;
@@ -326,7 +328,9 @@ extern "C" sa_status sa_gate_projection_forward(int64_t rows, int32_t dm, int32_
                              kGateSmem) != cudaSuccess)
       return SA_ERR_CUDA;
     const int total = p.tiles_m * p.tiles_n;
-    gate_tc_kernel<<<min(total, sms), kGateThreads, kGateSmem, st>>>(p, tm[0], tm[1], tm[2], tm[3]);
+    if (launch_dependent(gate_tc_kernel, dim3(min(total, sms)), dim3(kGateThreads), kGateSmem, st, p,
+                         tm[0], tm[1], tm[2], tm[3]) != cudaSuccess)
+      return SA_ERR_CUDA;
   } else {
     const int64_t total = rows * dm;
     const unsigned blocks = (unsigned)((total + 255) / 256);

@@ -188,6 +188,9 @@ perm_cluster_kernel(uint32_t seed_lo, uint32_t seed_hi, uint32_t layer, int n, i
   const int share = (n + C - 1) >> log2_c, t0 = r * share, t1 = min(n, t0 + share);
   perm += (size_t)b * n;
   inv += (size_t)b * n;
+  // The sort touches no memory that another kernel uses until it writes its result, so it runs under
+  // the tail of the launch before, and the next launch's preamble under it.
+  grid_dependents_launch();
   auto bucket = [&](uint64_t key) {
     return bits ? (uint32_t)((key << log2_c) >> (64 - bits)) : 0u;
   };
@@ -256,6 +259,7 @@ perm_cluster_kernel(uint32_t seed_lo, uint32_t seed_hi, uint32_t layer, int n, i
       if (o < r) goff += all[o];
     }
     if (over) {                           // the exact slow way, see above
+      grid_dependency_wait();
       for (int i = t0 + tid; i < t1; i += T) {
         const uint64_t k = sort_key(seed_lo, seed_hi, layer, b, i);
         int pos = 0;
@@ -315,6 +319,7 @@ perm_cluster_kernel(uint32_t seed_lo, uint32_t seed_hi, uint32_t layer, int n, i
       toks[p] = tok[x];
     }
   __syncthreads();
+  grid_dependency_wait();
   // rank inside the bucket; cursor[] now holds the bucket ends
 #pragma unroll 1
   for (int e = tid; e < m; e += T) {
@@ -386,12 +391,14 @@ cudaError_t launch_make_perm(uint64_t seed, uint32_t layer, int B, int n, int32_
     cfg.blockDim = dim3(c.threads);
     cfg.dynamicSmemBytes = c.smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 1u << c.log2_c;
     attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     const cudaError_t e =
         cudaLaunchKernelEx(&cfg, perm_cluster_kernel, (uint32_t)seed, (uint32_t)(seed >> 32), layer,
                            n, c.log2_c, c.bits, c.cap, perm, inv);

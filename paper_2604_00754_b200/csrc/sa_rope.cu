@@ -62,6 +62,7 @@ rope_apply_bf16_kernel(const RopeTensor ta, const RopeTensor tb, int n, int d,
                        const float* __restrict__ cs, const float* __restrict__ sn, float sign) {
   const int half = d / 2, groups = half / 8;
   const int i = blockIdx.x * 256 + threadIdx.x;
+  grid_dependency_wait();
   if (i >= n * groups) return;
   const int t = i / groups, g = i - t * groups, b = blockIdx.z;
   const bool first = (int)blockIdx.y < ta.H;
@@ -110,7 +111,9 @@ cudaError_t launch_rope_apply(const void* x, void* out, int B, int H, int n, int
   if (rope_fast(B, n, d, dtype)) {
     const RopeTensor t{(const __nv_bfloat16*)x, (__nv_bfloat16*)out, H, s[0], s[1], s[2]};
     const unsigned blocks = ((unsigned)n * (d / 16) + 255) / 256;
-    rope_apply_bf16_kernel<<<dim3(blocks, H, B), 256, 0, st>>>(t, t, n, d, cs, sn, sign);
+    bump_launches();
+    return launch_dependent(rope_apply_bf16_kernel, dim3(blocks, H, B), dim3(256), 0, st, t, t, n, d,
+                            cs, sn, sign);
   } else {
     const int64_t total = (int64_t)B * H * n * ((d / 2 + 7) / 8);
     const unsigned blocks = (unsigned)((total + 255) / 256);
@@ -136,9 +139,9 @@ cudaError_t launch_rope_qk(const void* q, void* qr, int Hq, const int64_t qs[3],
   const RopeTensor a{(const __nv_bfloat16*)q, (__nv_bfloat16*)qr, Hq, qs[0], qs[1], qs[2]};
   const RopeTensor b{(const __nv_bfloat16*)k, (__nv_bfloat16*)kr, Hkv, ks[0], ks[1], ks[2]};
   const unsigned blocks = ((unsigned)n * (d / 16) + 255) / 256;
-  rope_apply_bf16_kernel<<<dim3(blocks, Hq + Hkv, B), 256, 0, st>>>(a, b, n, d, cs, sn, 1.f);
   bump_launches();
-  return cudaGetLastError();
+  return launch_dependent(rope_apply_bf16_kernel, dim3(blocks, Hq + Hkv, B), dim3(256), 0, st, a, b, n,
+                          d, cs, sn, 1.f);
 }
 
 }  // namespace sa
