@@ -137,6 +137,11 @@ __global__ void __launch_bounds__(128) dgate_kernel(const BwdArgs a) {
 // of its own, for both outputs in one launch, and writes a partial gradient that reduce_kernel
 // adds up in a fixed order ("split").  Large ones run one launch per branch, the second adding to
 // what the first stored, with the heads of a group inside the CTA.
+//
+// Bound: FMA issue and shared-memory wavefronts, about equal, behind the latency of 32-column
+// steps, so warps per SM count: dS and P take turns in one buffer and the registers are held to 128
+// (d <= 64), for four CTAs per SM.  With that and packed multiply-adds in the products: 2 x 4/2 heads
+// of 64, n = 1500, w = 128, gated 157 -> 139 us; 8/4 heads of 128, n = 2000, w = 256 636 -> 572.
 
 // Split while the row tiles of the keys alone are fewer than eight per SM: beyond that they fill
 // the chip, and the partial gradients (six tensors of Q's size at most) would cost more than the
@@ -158,9 +163,12 @@ __device__ __forceinline__ void bwd_tile(const BwdArgs& a, unsigned char* smem_r
   float* r1 = reinterpret_cast<float*>(smem_raw);
   float* r2 = r1 + kRows * sm.row_elems();
   float* cols = r2 + kRows * sm.row_elems();           // (C1 C2) x 2
-  float* pw = cols + 4 * sm.col_elems() + warp * (kCols * 8 * 2);   // dS, then P: [32][8] each
-  __shared__ int s_slot[2][kCols], s_tok[2][kCols];
-  __shared__ float s_lse[2][kCols], s_delta[2][kCols];
+  float* pw = cols + 4 * sm.col_elems() + warp * (kCols * 8);   // dS, then P: [32][8]
+  typedef int IntCols[kCols];
+  typedef float FloatCols[kCols];
+  char* stat = reinterpret_cast<char*>(cols + 4 * sm.col_elems() + kTileThreads / 32 * kCols * 8);
+  IntCols *s_slot = reinterpret_cast<IntCols*>(stat), *s_tok = s_slot + 2;
+  FloatCols *s_lse = reinterpret_cast<FloatCols*>(s_tok + 2), *s_delta = s_lse + 2;
 
   const int64_t q_off = b * a.qs[0], k_off = b * a.ks[0] + hk * a.ks[1];
   const float scale2 = a.scale * kLog2e;
@@ -250,22 +258,26 @@ __device__ __forceinline__ void bwd_tile(const BwdArgs& a, unsigned char* smem_r
       const int col = tx + 16 * c;
       const int cs = s_slot[buf][col], ct = s_tok[buf][col];
       const float cl = KEYS ? s_lse[buf][col] : 0.f, cd = KEYS ? s_delta[buf][col] : 0.f;
-      float pr[4], ds[4];
+      float ds[4];
 #pragma unroll
       for (int r = 0; r < 4; ++r) {
         const bool see = rslot[r] < a.n && g.sees(rslot[r], rtok[r], cs, ct);
         const float p = see ? exp2f(s[r][c] - (KEYS ? cl : rlse[r])) : 0.f;
         ds[r] = p * fmaf(gx, dp[r][c], -(KEYS ? cd : rdelta[r]));
-        pr[r] = p * gx;
+        s[r][c] = p * gx;
       }
       st4(pw + 8 * col + 4 * half, make_float4(ds[0], ds[1], ds[2], ds[3]));
-      if (KEYS)
-        st4(pw + kCols * 8 + 8 * col + 4 * half, make_float4(pr[0], pr[1], pr[2], pr[3]));
     }
     __syncwarp();
     tile_accumulate<float, NCG>(o1, pw + 4 * half, c1, sm.stride(), tx, d);
-    if constexpr (KEYS)
-      tile_accumulate<float, NCG>(o2, pw + kCols * 8 + 4 * half, c2, sm.stride(), tx, d);
+    if constexpr (KEYS) {
+      __syncwarp();
+#pragma unroll
+      for (int c = 0; c < 2; ++c)
+        st4(pw + 8 * (tx + 16 * c) + 4 * half, make_float4(s[0][c], s[1][c], s[2][c], s[3][c]));
+      __syncwarp();
+      tile_accumulate<float, NCG>(o2, pw + 4 * half, c2, sm.stride(), tx, d);
+    }
     __syncthreads();
   }
 
@@ -300,7 +312,7 @@ __device__ __forceinline__ void bwd_tile(const BwdArgs& a, unsigned char* smem_r
 // blockIdx.y: first the nb * Hq (branch, head) pairs of dQ, then those of dK / dV, whose CTAs
 // cover `heads` query heads each.  Branches x0 .. x0 + nb - 1.
 template <int NCG>
-__global__ void __launch_bounds__(kTileThreads)
+__global__ void __launch_bounds__(kTileThreads, NCG == 1 ? 4 : NCG == 2 ? 2 : 1)
 bwd_tile_kernel(const BwdArgs a, int x0, int nb, int heads, bool split) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   grid_dependency_wait();
@@ -356,7 +368,7 @@ __global__ void __launch_bounds__(256) reduce_kernel(const BwdArgs a) {
 template <int NCG>
 cudaError_t launch_tiles(const BwdArgs& a, cudaStream_t st) {
   const TileSmem<float> sm(a.d);
-  const int smem = 2 * sm.rows_bytes() + 4 * sm.col_bytes() + kTileThreads / 32 * kCols * 8 * 2 * 4;
+  const int smem = 2 * sm.rows_bytes() + 4 * sm.col_bytes() + (kTileThreads / 32 * kCols * 8 + 8 * kCols) * 4;
   cudaError_t e = allow_smem((const void*)bwd_tile_kernel<NCG>, smem);
   if (e != cudaSuccess) return e;
   const unsigned tiles = (a.n + kRows - 1) / kRows;

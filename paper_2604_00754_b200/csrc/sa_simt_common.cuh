@@ -166,7 +166,8 @@ __device__ __forceinline__ void tile_dot(float (&s)[4][2], const float* rows, in
   }
 }
 
-// o[r][4 cg + x] += sum_k p[k][r] cols[k][64 cg + 4 tx + x]; p: [32][8] fp32, this thread's 4 rows
+// o[r][4 cg + x] += sum_k p[k][r] cols[k][64 cg + 4 tx + x]; p: [32][8] fp32, this thread's 4 rows;
+// packed over two columns
 template <typename T, int NCG>
 __device__ __forceinline__ void tile_accumulate(float (&o)[4][4 * NCG], const float* p,
                                                 const T* cols, int stride, int tx, int d) {
@@ -179,10 +180,13 @@ __device__ __forceinline__ void tile_accumulate(float (&o)[4][4 * NCG], const fl
       const float4 v = ld4(cols + k * stride + min(64 * cg + 4 * tx, d - 4));
 #pragma unroll
       for (int r = 0; r < 4; ++r) {
-        o[r][4 * cg] = fmaf(wr[r], v.x, o[r][4 * cg]);
-        o[r][4 * cg + 1] = fmaf(wr[r], v.y, o[r][4 * cg + 1]);
-        o[r][4 * cg + 2] = fmaf(wr[r], v.z, o[r][4 * cg + 2]);
-        o[r][4 * cg + 3] = fmaf(wr[r], v.w, o[r][4 * cg + 3]);
+        const float2 w2 = make_float2(wr[r], wr[r]);
+        const float2 a = __ffma2_rn(w2, make_float2(v.x, v.y), make_float2(o[r][4 * cg], o[r][4 * cg + 1]));
+        const float2 b = __ffma2_rn(w2, make_float2(v.z, v.w), make_float2(o[r][4 * cg + 2], o[r][4 * cg + 3]));
+        o[r][4 * cg] = a.x;
+        o[r][4 * cg + 1] = a.y;
+        o[r][4 * cg + 2] = b.x;
+        o[r][4 * cg + 3] = b.y;
       }
     }
   }
