@@ -1,0 +1,73 @@
+"""Edges of the tensor-core attention kernels (128-row tiles, 64- or 128-key blocks, persistent
+CTAs that run one launch into the next) and of the projection gates' split dW, bf16, against the
+float64 oracle."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2604_00754_b200 import binding as sa
+from paper_2604_00754_b200.workloads import CAUSAL, LINEAR_WINDOW, SWA_ONE_SIDED, as_f64
+
+pytestmark = pytest.mark.gpu
+
+ONE = CAUSAL | SWA_ONE_SIDED
+
+# n around a row tile; windows that end on and around 32 columns (one mask word), a 64-key and a
+# 128-key block; one, two and three column tiles per row tile; every query head of a group; the
+# band around the whole sequence; and more items than SMs, so that CTAs take several (3 * 8 * 8)
+CASES = [
+    (1, 2, 1, 127, 64, 31, ONE), (1, 2, 2, 128, 64, 33, CAUSAL), (1, 3, 1, 129, 128, 32, ONE),
+    (2, 2, 1, 255, 128, 64, 0), (1, 4, 4, 256, 64, 65, CAUSAL | LINEAR_WINDOW),
+    (1, 4, 2, 257, 128, 127, ONE), (1, 2, 1, 384, 64, 128, ONE), (1, 4, 1, 385, 128, 129, ONE),
+    (1, 2, 1, 300, 64, 299, CAUSAL), (1, 2, 2, 300, 128, 600, ONE),
+    (3, 8, 8, 900, 64, 96, ONE), (3, 16, 8, 900, 128, 200, ONE | LINEAR_WINDOW),
+]
+
+
+# bf16 inputs, probabilities and results with fp32 sums: 2e-2 of the largest value, as for the
+# other bf16 comparisons; 1e-5 for values that cancel to zero
+def _close(got, want, name):
+    err = np.abs(as_f64(got) - want).max()
+    assert err <= 2e-2 * np.abs(want).max() + 1e-5, (name, float(err))
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,n,d,w,flags", CASES)
+def test_gated_pass_at_tile_edges(B, Hq, Hkv, n, d, w, flags):
+    g = torch.Generator().manual_seed(n + w)
+    mk = lambda h: torch.randn(B, h, n, d, generator=g).bfloat16()
+    q, k, v, dy = mk(Hq), mk(Hkv), mk(Hkv), mk(Hq)
+    lg = torch.randn(2, Hq, generator=g)
+    perm, inv = sa.sa_make_perm(n, w, B, n)
+    dev = [t.cuda() for t in (q, k, v)]
+    runs = []
+    for _ in range(2):
+        out = sa.sa_swa_gated_forward(*dev, perm, inv, lg.cuda(), w, flags, save_for_bwd=True)
+        runs.append(tuple(out) + tuple(sa.sa_backward(*dev, perm, inv, lg.cuda(), *out[1:], dy.cuda(),
+                                                      w, flags)))
+    assert sa.sa_read_status() == 0
+    for a, b in zip(*runs):                         # no atomics: bit for bit the same
+        assert torch.equal(a, b)
+    args = [as_f64(t) for t in (q, k, v)] + [perm.cpu().numpy(), inv.cpu().numpy(), lg.double().numpy()]
+    want = tuple(oracle.gated_forward(*args, w, flags)) + tuple(oracle.backward(*args, as_f64(dy), w, flags))
+    for got, ref, name in zip(runs[0], want, ("y", "y_sa", "y_swa", "lse_sa", "lse_swa", "dq", "dk", "dv",
+                                              "dgate")):
+        if name.startswith("lse"):                  # a sum of bf16 products in the exponent
+            assert np.abs(as_f64(got) - ref).max() <= 2e-2, name
+        else:
+            _close(got, ref, name)
+
+
+# dW in parts of the rows: as many as rows / dm allows (64 rows are one contraction step), ragged
+# rows and columns, one part; 18900 x 256 runs the 128 x 256 tiles with several items per CTA
+@pytest.mark.parametrize("rows,dm", [(64, 64), (129, 64), (700, 192), (1300, 320), (4100, 128), (18900, 256)])
+def test_projection_gate_backward_in_parts(rows, dm):
+    g = torch.Generator().manual_seed(rows + dm)
+    y, dout = (torch.randn(rows, dm, generator=g).bfloat16() for _ in range(2))
+    w = (torch.randn(dm, dm, generator=g) * dm ** -0.5).bfloat16()
+    runs = [sa.sa_gate_projection_backward(dout.cuda(), y.cuda(), w.cuda()) for _ in range(2)]
+    assert sa.sa_read_status() == 0
+    want = oracle.gate_projection_backward(dout.double().numpy(), y.double().numpy(), w.double().numpy())
+    for got, again, ref, name in zip(*runs, want, ("dy", "dw")):
+        assert torch.equal(got, again)
+        _close(got, ref, name)
