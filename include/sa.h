@@ -171,7 +171,8 @@ sa_status sa_swa_gated_forward(const sa_problem* p, const void* q, const void* k
  * shared by all ranges; every range is one sa_swa_gated_forward call, so the result has
  * the bits of that call.
  *   ws: DEVICE workspace of sa_host_forward_ws_bytes(p) bytes, 256-byte aligned, owned by the
- *       caller (device copies of q, k, v, y, the permutation and its scratch).  No device memory is allocated; the first call on a device creates the
+ *       caller (device copies of q, k, v, y, one branch output, the permutation and its
+ *       scratch).  No device memory is allocated; the first call on a device creates the
  *       three streams and the events of the pipeline and keeps them.
  *   stream: the call is ordered after what `stream` has queued, and `stream` waits for the
  *       last copy out, so the caller synchronises (or times) on `stream` alone.  y must not

@@ -79,7 +79,7 @@ Pipe* pipe_for_current_device() {
 size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 
 struct Carve {
-  size_t q, k, v, y, gate, perm, inv, perm_ws, total;
+  size_t q, k, v, y, scratch, gate, perm, inv, perm_ws, total;
 };
 
 bool carve(const sa_problem* p, Carve* c) {
@@ -92,6 +92,7 @@ bool carve(const sa_problem* p, Carve* c) {
   c->k = o; o += align256(kb);
   c->v = o; o += align256(kb);
   c->y = o; o += align256(qb);
+  c->scratch = o; o += align256(qb);
   // the logits as they come ([2, Hq]), then one contiguous [2, heads] block per piece
   c->gate = o; o += 2 * align256((size_t)2 * p->Hq * sizeof(float));
   c->perm = o; o += align256((size_t)p->B * p->n * sizeof(int32_t));
@@ -207,7 +208,8 @@ sa_status sa_swa_gated_forward_host(const sa_problem* p, const void* q, const vo
     const size_t qoff = (size_t)g.qa * head_bytes, koff = (size_t)g.ka * head_bytes;
     st = sa_swa_gated_forward(&gp, dq + qoff, dk + koff, dv + koff, dperm, dinv,
                               dgate + gate_at[i], dyv + qoff, nullptr, nullptr, nullptr, nullptr,
-                              nullptr, 0, (sa_stream_t)pipe->s_run);
+                              base + c.scratch, (size_t)(c.gate - c.scratch),
+                              (sa_stream_t)pipe->s_run);
     chk(cudaEventRecord(pipe->ev_done[i], pipe->s_run));
   }
 
