@@ -163,11 +163,12 @@ sa_status sa_swa_gated_forward(const sa_problem* p, const void* q, const void* k
 /* sa_make_perm + sa_swa_gated_forward (Alg. 1 line 1, Alg. 2, Eq. 5) for tensors that live in
  * HOST memory: q, k, v, y are host pointers to contiguous [B,H,n,d] tensors of p->dtype
  * (p's stride fields are ignored), gate_logits a host pointer to fp32 [2,Hq]; pinned memory
- * lets the copies overlap the kernels, pageable memory works but serialises.  The KV heads
- * travel through the GPU in n_groups contiguous ranges (the first and the last range, when
- * they hold one KV head, in q_parts ranges of its query heads if those divide evenly: the
- * ends of the pipeline are what cannot overlap), on three internal streams: copy in,
- * compute, copy out.  The permutation is drawn from (seed, layer) as in sa_make_perm and
+ * lets the copies overlap the kernels, pageable memory works but serialises.  The work
+ * travels through the GPU in about n_groups pieces, none smaller than 2 MB: ranges of
+ * sequences first, then contiguous ranges of their KV heads (the first and the last range of
+ * heads, when they hold one KV head, in q_parts ranges of its query heads if those divide
+ * evenly and still fill the GPU: the ends of the pipeline are what cannot overlap), on three
+ * internal streams: copy in, compute, copy out.  The permutation is drawn from (seed, layer) as in sa_make_perm and
  * shared by all ranges; every range is one sa_swa_gated_forward call, so the result has
  * the bits of that call.
  *   ws: DEVICE workspace of sa_host_forward_ws_bytes(p) bytes, 256-byte aligned, owned by the

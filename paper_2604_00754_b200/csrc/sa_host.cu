@@ -8,6 +8,7 @@
 // every piece is computed by the same entry points a device-resident caller uses, on strided
 // views of whole-size device buffers carved out of the caller's workspace.  The permutation is
 // drawn once per call and shared by all pieces.
+#include <initializer_list>
 #include <mutex>
 
 #include "sa_common.cuh"
@@ -17,7 +18,7 @@ namespace {
 
 constexpr int kMaxPieces = 256;
 
-struct Piece { int ka, kb, qa, qb, with_kv; };
+struct Piece { int ka, kb, qa, qb, with_kv, b0, b1; };
 
 // KV heads in at most n_groups contiguous ranges.  The first and the last range, when they hold
 // one KV head, are cut further into q_parts ranges of query heads if those divide evenly (only
@@ -37,12 +38,35 @@ int plan(int Hq, int Hkv, int n_groups, int q_parts, Piece* out, int max_out) {
       const int step = G / q_parts;
       for (int j = 0; j < q_parts; ++j) {
         if (cnt >= max_out) return -1;
-        out[cnt++] = Piece{a, b, a * G + j * step, a * G + (j + 1) * step, j == 0};
+        out[cnt++] = Piece{a, b, a * G + j * step, a * G + (j + 1) * step, j == 0, 0, 0};
       }
     } else {
       if (cnt >= max_out) return -1;
-      out[cnt++] = Piece{a, b, a * G, b * G, 1};
+      out[cnt++] = Piece{a, b, a * G, b * G, 1, 0, 0};
     }
+  }
+  return cnt;
+}
+
+// The same for B sequences: the sequences are divided first, into at most n_groups or `most` ranges (whole
+// sequences are one block of memory, so a piece is one copy per tensor where a range of heads is one
+// per tensor and sequence), then the heads of each range until there are about n_groups pieces.
+// Only the last range's ends are cut by query heads.  With heads alone, 8 sequences of one head
+// (n = 3248, d = 64) were a single piece whose copies and kernels followed one another (580 -> 410 us); 16 x 12 heads of
+// 64, n = 700: 2880 -> 1280 us, 2 x 32/8 heads of 128, n = 3727: 2680 -> 2150.
+int plan_batch(int most, int B, int Hq, int Hkv, int n_groups, int q_parts, Piece* out, int max_out) {
+  n_groups = n_groups < 1 ? 1 : n_groups;
+  const int parts = most < n_groups ? most : n_groups;
+  int cnt = 0;
+  for (int i = 0; i < parts; ++i) {
+    const int got = plan(Hq, Hkv, n_groups / parts, i == parts - 1 ? q_parts : 1, out + cnt,
+                         max_out - cnt);
+    if (got < 0) return -1;
+    for (int j = 0; j < got; ++j) {
+      out[cnt + j].b0 = (int)((int64_t)i * B / parts);
+      out[cnt + j].b1 = (int)((int64_t)(i + 1) * B / parts);
+    }
+    cnt += got;
   }
   return cnt;
 }
@@ -138,7 +162,22 @@ sa_status sa_swa_gated_forward_host(const sa_problem* p, const void* q, const vo
   if (!carve(p, &c)) return SA_ERR_INVALID_ARG;
   if (ws_bytes < c.total) return SA_ERR_WORKSPACE;
   Piece pieces[kMaxPieces];
-  const int cnt = plan(p->Hq, p->Hkv, n_groups, q_parts, pieces, kMaxPieces);
+  // a range's permutation may have to move to an aligned place in the scratch: one range if that is
+  // too small (rows of a few bytes)
+  const size_t per_seq = 2 * align256((size_t)p->n * sizeof(int32_t));
+  const int ranged = per_seq * p->B <= c.gate - c.scratch ? p->B : 1;
+  // a piece costs the host about 40 us of calls, as long as 2 MB take over PCIe: none smaller
+  const size_t in = c.y - c.q;
+  if ((size_t)n_groups > (in >> 21)) {
+    n_groups = in >> 21 ? (int)(in >> 21) : 1;
+    q_parts = 1;
+  }
+  // half of a group's query heads that leave SMs idle (an item is two tiles of 128 rows) take the
+  // kernels as long as the whole group: 32/8 heads, n = 8192: 2440 -> 2370 us uncut
+  if (q_parts > 1 &&
+      (int64_t)(p->Hq / p->Hkv / q_parts) * ((p->n + 127) / 128) < 2 * 148)
+    q_parts = 1;
+  const int cnt = plan_batch(ranged, p->B, p->Hq, p->Hkv, n_groups, q_parts, pieces, kMaxPieces);
   if (cnt < 1) return SA_ERR_INVALID_ARG;
   // device-side problem: contiguous [B,H,n,d] buffers, whatever the strides field says
   sa_problem dp = *p;
@@ -172,22 +211,23 @@ sa_status sa_swa_gated_forward_host(const sa_problem* p, const void* q, const vo
   // the heads of each piece; the [2, heads] block of a piece is cut out on the compute stream
   chk(cudaMemcpyAsync(dgate_all, gate_logits, (size_t)2 * p->Hq * sizeof(float),
                       cudaMemcpyHostToDevice, pipe->s_in));
-  size_t gate_off = 0;
-  size_t gate_at[kMaxPieces];
+  // heads [a, b) of a piece's sequences, out of H heads per sequence: one block where the piece has
+  // all heads, else one per sequence
+  auto copy_heads = [&](const Piece& g, int H, int a, int e, char* dst, const char* src,
+                        cudaMemcpyKind kind, cudaStream_t st) {
+    const int step = e - a == H ? g.b1 - g.b0 : 1;
+    for (int b = g.b0; b < g.b1; b += step) {
+      const size_t off = ((size_t)b * H + a) * head_bytes;
+      chk(cudaMemcpyAsync(dst + off, src + off, (size_t)step * (e - a) * head_bytes, kind, st));
+    }
+  };
   for (int i = 0; i < cnt && ok; ++i) {
     const Piece& g = pieces[i];
-    const int hq = g.qb - g.qa;
-    gate_at[i] = gate_off;
-    gate_off += (size_t)2 * hq;
-    for (int b = 0; b < p->B; ++b) {   // one contiguous block per sequence and tensor
-      if (g.with_kv) {
-        const size_t off = ((size_t)b * p->Hkv + g.ka) * head_bytes, len = (size_t)(g.kb - g.ka) * head_bytes;
-        chk(cudaMemcpyAsync(dk + off, (const char*)k + off, len, cudaMemcpyHostToDevice, pipe->s_in));
-        chk(cudaMemcpyAsync(dv + off, (const char*)v + off, len, cudaMemcpyHostToDevice, pipe->s_in));
-      }
-      const size_t off = ((size_t)b * p->Hq + g.qa) * head_bytes, len = (size_t)hq * head_bytes;
-      chk(cudaMemcpyAsync(dq + off, (const char*)q + off, len, cudaMemcpyHostToDevice, pipe->s_in));
+    if (g.with_kv) {
+      copy_heads(g, p->Hkv, g.ka, g.kb, dk, (const char*)k, cudaMemcpyHostToDevice, pipe->s_in);
+      copy_heads(g, p->Hkv, g.ka, g.kb, dv, (const char*)v, cudaMemcpyHostToDevice, pipe->s_in);
     }
+    copy_heads(g, p->Hq, g.qa, g.qb, dq, (const char*)q, cudaMemcpyHostToDevice, pipe->s_in);
     chk(cudaEventRecord(pipe->ev_in[i], pipe->s_in));
   }
 
@@ -196,20 +236,42 @@ sa_status sa_swa_gated_forward_host(const sa_problem* p, const void* q, const vo
   if (ok)
     st = sa_make_perm(seed, layer, p->B, p->n, dperm, dinv, base + c.perm_ws,
                       make_perm_ws_bytes(p->B, p->n), (sa_stream_t)pipe->s_run);
+  const int32_t *rperm = dperm, *rinv = dinv;     // of the range at hand
+  int range_at = 0;
+  size_t spare = c.scratch;
   for (int i = 0; i < cnt && ok && st == SA_OK; ++i) {
     const Piece& g = pieces[i];
+    if (g.b0 != range_at) {
+      // the kernels' entry points take index lists that start on 16 bytes
+      const size_t at = (size_t)g.b0 * p->n, len = (size_t)(g.b1 - g.b0) * p->n * sizeof(int32_t);
+      range_at = g.b0;
+      rperm = dperm + at;
+      rinv = dinv + at;
+      if (at % 4 != 0) {
+        for (const int32_t** list : {&rperm, &rinv}) {
+          chk(cudaMemcpyAsync(base + spare, *list, len, cudaMemcpyDeviceToDevice, pipe->s_run));
+          *list = (const int32_t*)(base + spare);
+          spare += align256(len);
+        }
+      }
+    }
     chk(cudaStreamWaitEvent(pipe->s_run, pipe->ev_in[i], 0));
-    chk(cudaMemcpy2DAsync(dgate + gate_at[i], (size_t)(g.qb - g.qa) * sizeof(float), dgate_all + g.qa,
-                          (size_t)p->Hq * sizeof(float), (size_t)(g.qb - g.qa) * sizeof(float), 2,
-                          cudaMemcpyDeviceToDevice, pipe->s_run));
+    const int hq = g.qb - g.qa;
+    float* gates = dgate_all;
+    if (hq < p->Hq) {                       // each range of query heads has its own place
+      gates = dgate + 2 * g.qa;
+      chk(cudaMemcpy2DAsync(gates, (size_t)hq * sizeof(float), dgate_all + g.qa,
+                            (size_t)p->Hq * sizeof(float), (size_t)hq * sizeof(float), 2,
+                            cudaMemcpyDeviceToDevice, pipe->s_run));
+    }
     sa_problem gp = dp;                     // a view of the whole-size buffers: same strides
-    gp.Hq = g.qb - g.qa;
+    gp.B = g.b1 - g.b0;
+    gp.Hq = hq;
     gp.Hkv = g.kb - g.ka;
-    const size_t qoff = (size_t)g.qa * head_bytes, koff = (size_t)g.ka * head_bytes;
-    st = sa_swa_gated_forward(&gp, dq + qoff, dk + koff, dv + koff, dperm, dinv,
-                              dgate + gate_at[i], dyv + qoff, nullptr, nullptr, nullptr, nullptr,
-                              base + c.scratch, (size_t)(c.gate - c.scratch),
-                              (sa_stream_t)pipe->s_run);
+    const size_t qoff = ((size_t)g.b0 * p->Hq + g.qa) * head_bytes;
+    const size_t koff = ((size_t)g.b0 * p->Hkv + g.ka) * head_bytes;
+    st = sa_swa_gated_forward(&gp, dq + qoff, dk + koff, dv + koff, rperm, rinv, gates, dyv + qoff,
+                              nullptr, nullptr, nullptr, nullptr, nullptr, 0, (sa_stream_t)pipe->s_run);
     chk(cudaEventRecord(pipe->ev_done[i], pipe->s_run));
   }
 
@@ -217,10 +279,7 @@ sa_status sa_swa_gated_forward_host(const sa_problem* p, const void* q, const vo
   for (int i = 0; i < cnt && ok && st == SA_OK; ++i) {
     const Piece& g = pieces[i];
     chk(cudaStreamWaitEvent(pipe->s_out, pipe->ev_done[i], 0));
-    for (int b = 0; b < p->B; ++b) {
-      const size_t off = ((size_t)b * p->Hq + g.qa) * head_bytes, len = (size_t)(g.qb - g.qa) * head_bytes;
-      chk(cudaMemcpyAsync((char*)y + off, dyv + off, len, cudaMemcpyDeviceToHost, pipe->s_out));
-    }
+    copy_heads(g, p->Hq, g.qa, g.qb, (char*)y, dyv, cudaMemcpyDeviceToHost, pipe->s_out);
   }
   // the caller's stream resumes when all three streams are done (also after an error, so
   // that nothing of this call is still in flight when the caller goes on)

@@ -71,3 +71,21 @@ def test_projection_gate_backward_in_parts(rows, dm):
     for got, again, ref, name in zip(*runs, want, ("dy", "dw")):
         assert torch.equal(got, again)
         _close(got, ref, name)
+
+
+# pieces of whole sequences, of one head range per sequence range, and of several; odd lengths, so
+# that a range's index lists start off 16 bytes
+@pytest.mark.parametrize("B,Hq,Hkv,n", [(5, 8, 2, 1001), (3, 16, 4, 1003), (2, 16, 8, 1501), (9, 2, 2, 2002)])
+def test_host_pieces_of_a_batch(B, Hq, Hkv, n):
+    from paper_2604_00754_b200.host import HostForward
+    g = torch.Generator().manual_seed(n)
+    q, k, v = (torch.randn(B, h, n, 64, generator=g).bfloat16().pin_memory() for h in (Hq, Hkv, Hkv))
+    lg = torch.randn(2, Hq, generator=g).pin_memory()
+    y = torch.empty_like(q).pin_memory()
+    HostForward(B, Hq, Hkv, n, 64, 96).forward(q, k, v, lg, y, seed=7, layer=1)
+    torch.cuda.synchronize()
+    perm, inv = sa.sa_make_perm(7, 1, B, n)
+    want = sa.sa_swa_gated_forward(q.cuda(), k.cuda(), v.cuda(), perm, inv, lg.cuda(), 96, ONE)
+    want = want[0] if isinstance(want, (tuple, list)) else want
+    assert torch.equal(y, want.cpu())
+    assert sa.sa_read_status() == 0
