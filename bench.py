@@ -189,9 +189,8 @@ def main():
                     help="force the score-block width of the tensor-core kernels (test hook of "
                          "the library; 0 = the library's own choice)")
     ap.add_argument("--gated-form", default="warps", choices=["warps", "epilogue"],
-                    help="where the local branch's launch applies the gates: in its two idle warps "
-                         "(scratch for the SA rows given: the default) or in the row threads' "
-                         "epilogue (no scratch)")
+                    help="warps: the call is given scratch (accepted and not used); epilogue: none. "
+                         "The gates are applied in the local branch's epilogue either way")
     ap.add_argument("--no-extras", action="store_true",
                     help="skip the side measurements (SWA, backward, e2e, CPU oracle)")
     args = ap.parse_args()
@@ -317,9 +316,7 @@ def main():
         "data": "synthetic", "config": workload_config(c), "clocks": clocks,
         "gpu_launches": int(launches),
         "roofline": {"kernel": "fused SA forward (gather, QK^T, softmax, PV, scatter); the gates are applied "
-                               + ("by two idle warps of the local branch's launch"
-                                  if args.gated_form == "warps"
-                                  else "in the epilogue of the local branch's launch"),
+                               "in the epilogue of the local branch's launch",
                      "bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                      "frac": achieved / peak,
                      "peak_kind": "%s bf16 %s" % (pk["source"], "sustained" if sustained else "burst"),

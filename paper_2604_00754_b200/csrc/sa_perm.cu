@@ -56,6 +56,7 @@ __device__ __forceinline__ uint32_t bucket_of(uint64_t key, int bits) {
 __global__ void keys_kernel(uint32_t seed_lo, uint32_t seed_hi, uint32_t layer, int n, int bits,
                             uint64_t* __restrict__ keys, uint32_t* __restrict__ counts) {
   const int b = blockIdx.y;
+  grid_dependents_launch();
   uint32_t* cb = counts + ((size_t)b << bits);
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const uint64_t key = sort_key(seed_lo, seed_hi, layer, b, i);
@@ -69,6 +70,8 @@ __global__ void keys_kernel(uint32_t seed_lo, uint32_t seed_hi, uint32_t layer, 
 __global__ void __launch_bounds__(kThreadsPerBlock)
 scan_kernel(uint32_t* __restrict__ counts, uint32_t* __restrict__ cursor, int nbuckets) {
   __shared__ uint32_t part[kThreadsPerBlock];
+  grid_dependency_wait();
+  grid_dependents_launch();
   uint32_t* c = counts + (size_t)blockIdx.x * nbuckets;
   uint32_t* cur = cursor + (size_t)blockIdx.x * nbuckets;
   const int per = (nbuckets + kThreadsPerBlock - 1) / kThreadsPerBlock;
@@ -97,6 +100,8 @@ __global__ void scatter_kernel(const uint64_t* __restrict__ keys, uint32_t* __re
                                uint64_t* __restrict__ bkeys, int32_t* __restrict__ btoks, int n,
                                int bits) {
   const int b = blockIdx.y;
+  grid_dependency_wait();
+  grid_dependents_launch();
   uint32_t* cur = cursor + ((size_t)b << bits);
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const uint64_t key = keys[(size_t)b * n + i];
@@ -112,6 +117,8 @@ __global__ void rank_kernel(const uint64_t* __restrict__ bkeys, const int32_t* _
                             const uint32_t* __restrict__ starts, int32_t* __restrict__ perm,
                             int32_t* __restrict__ inv, int n, int bits) {
   const int b = blockIdx.y;
+  grid_dependency_wait();
+  grid_dependents_launch();
   const uint64_t* kb = bkeys + (size_t)b * n;
   const int32_t* tb = btoks + (size_t)b * n;
   const uint32_t* st = starts + ((size_t)b << bits);
@@ -421,9 +428,14 @@ cudaError_t launch_make_perm(uint64_t seed, uint32_t layer, int B, int n, int32_
   const int kb = min((n + kThreadsPerBlock - 1) / kThreadsPerBlock, 1024);
   keys_kernel<<<dim3(kb, B), kThreadsPerBlock, 0, st>>>((uint32_t)seed, (uint32_t)(seed >> 32),
                                                         layer, n, bits, keys, counts);
-  scan_kernel<<<B, kThreadsPerBlock, 0, st>>>(counts, cursor, 1 << bits);
-  scatter_kernel<<<dim3(kb, B), kThreadsPerBlock, 0, st>>>(keys, cursor, bkeys, btoks, n, bits);
-  rank_kernel<<<dim3(kb, B), kThreadsPerBlock, 0, st>>>(bkeys, btoks, counts, perm, inv, n, bits);
+  e = launch_dependent(scan_kernel, dim3(B), dim3(kThreadsPerBlock), 0, st, counts, cursor, 1 << bits);
+  if (e == cudaSuccess)
+    e = launch_dependent(scatter_kernel, dim3(kb, B), dim3(kThreadsPerBlock), 0, st, keys, cursor, bkeys,
+                         btoks, n, bits);
+  if (e == cudaSuccess)
+    e = launch_dependent(rank_kernel, dim3(kb, B), dim3(kThreadsPerBlock), 0, st, bkeys, btoks, counts,
+                         perm, inv, n, bits);
+  if (e != cudaSuccess) return e;
   bump_launches(4);
   return cudaGetLastError();
 }
