@@ -1002,12 +1002,23 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
 
 // ---------------------------------------------------------------------------- host
 
-// Score-block width.  Narrow windows skip more with 64-key blocks; from w = 256 on the
-// 128-key block wins (half as many products, commits and softmax rounds per key).  The
-// test hook sa_debug_set(SA_DEBUG_SCORE_BLOCK, 64 | 128) overrides the choice.
-bool key_block_128(int w) {
+// Score-block width.  64-key blocks skip more of a window's ends and let a tile's products and row
+// work interleave; 128-key blocks take half as many products, commits and softmax rounds per key.
+// Measured, us with 64 / 128:
+//   tiles by TMA, d = 64 (two issuing threads hide the commits): 64 at every width (8 x 12 heads,
+//     n = 4096: w = 33 65 / 79, w = 384 116 / 124; 4 x 12 heads, w = 1600 159 / 181);
+//   tiles by TMA, d = 128 (one issuing thread): 128 at every width (32/8 heads, n = 8192: w = 33
+//     57.4 / 56.6, w = 128 65 / 57, w = 1024 204 / 150);
+//   gathered: 64 up to w = 320 (2 x 16 heads of 128, n = 4096: w = 64 58.5 / 62.2, w = 160 72.0 / 75.8,
+//     w = 320 88.0 / 89.9; 16/4 heads of 64, n = 16384: w = 320 102 / 112), 128 from there (32/8 heads of
+//     128, n = 8192: w = 384 133 / 127, w = 1024 244 / 216).  With no more than one item per SM only a
+//     block's latency counts, and 128 is better from w = 129 (32/8 heads of 128, n = 700, w = 256,
+//     gated: 37.4 / 36.0).
+// The test hook sa_debug_set(SA_DEBUG_SCORE_BLOCK, 64 | 128) overrides the choice.
+bool key_block_128(int w, int d, bool tma_tiles, bool one_item) {
   const int forced = debug_option(SA_DEBUG_SCORE_BLOCK);
-  return forced ? forced == 128 : w > 128;
+  if (forced) return forced == 128;
+  return tma_tiles ? d == 128 : w > (one_item ? 128 : 320);
 }
 
 // sa_debug_set(SA_DEBUG_SWA_TILE_LOADS, 0) keeps the cp.async gather for the one-sided SWA
@@ -1056,7 +1067,6 @@ cudaError_t launch_fwd_tc(const FwdArgs& a, cudaStream_t st) {
     if (e != cudaSuccess) return e;
   }
   const unsigned grid = (unsigned)min(p.total_items, sm_count[dev]);
-  const bool wide = key_block_128(a.w);
   const bool combine = a.gate_logits && a.y_other;
   // gates only with the other branch's rows; branch rows of their own only where gates are applied
   if ((a.gate_logits && !a.y_other) || (a.y_branch && !combine) || !a.y) return cudaErrorInvalidValue;
@@ -1074,6 +1084,7 @@ cudaError_t launch_fwd_tc(const FwdArgs& a, cudaStream_t st) {
     if (err != cudaSuccess) return err;
     return launch_dependent(kernel, dim3(grid), dim3(kThreads), smem, st, p, tm_q, tm_k, tm_v);
   };
+  const bool wide = key_block_128(a.w, a.d, natural, p.total_items <= sm_count[dev]);
   // instantiation by (head dimension, score-block width, source of the tiles, rotation, combine)
   auto pick = [&](auto d_c, auto kb_c) {
     constexpr int DD = decltype(d_c)::value, KK = decltype(kb_c)::value;
