@@ -305,7 +305,7 @@ uint64_t sa_launch_count(void);
 
 /* Test hooks.  The library reads no environment variable; these process-wide switches exist
  * so that tests can run every kernel variant on one input.  The paper has no counterpart.
- *   SA_DEBUG_SCORE_BLOCK      0 = choose by w (default), 64 or 128 = force that score-block
+ *   SA_DEBUG_SCORE_BLOCK      0 = choose (default), 64 or 128 = force that score-block
  *                             width in the tensor-core forward
  *   SA_DEBUG_SWA_TILE_LOADS   1 = one-sided SWA branch loads whole tiles by TMA when the layout
  *                             allows (default), 0 = always gather rows
