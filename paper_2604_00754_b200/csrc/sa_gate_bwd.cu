@@ -425,9 +425,24 @@ __global__ void dw_simt_kernel(int64_t rows, int dm, const float* __restrict__ d
 
 // ------------------------------------------------------------------------------ host
 
-// Wide (128 x 256) tiles when they still give every SM at least two tiles.
-bool wide_tiles(int64_t m_rows, int64_t n_cols, int sms) {
-  return ((m_rows + kT - 1) / kT) * ((n_cols + 255) / 256) >= 2 * (int64_t)sms;
+// 128 x 256 tiles take less time than 128 x 128 by their waves: a wide tile's K chunk takes 512
+// cycles, a narrow one's 300 (64 columns of operands per product more).
+bool wide_waves(int64_t rows, int dm, int sms) {
+  const int64_t tm = (rows + kT - 1) / kT;
+  return (tm * ((dm + 255) / 256) + sms - 1) / sms * 512 <=
+         (tm * ((dm + 127) / 128) + sms - 1) / sms * 300;
+}
+
+// Forward: the wide kernel, one launch per path, or (false) the fused 128 x 128 one.  One path: from
+// half a wide tile per SM on (8000 x 1024: 25.9 -> 19.9 us, 1300 x 2048: 23.0 -> 18.5, 9000 x 768: 19.8
+// -> 17.2; even at 5000 x 512, 80 tiles: 13.3 -> 12.7).  Two paths: the fused kernel writes the result
+// once and reads nothing back, so the wide one needs the better waves and the long contraction of
+// dm >= 1024 (4000 x 2048: 79 -> 70, 2000 x 4096: 155 -> 138, 8000 x 1024: 43.4 -> 41.5; but 18000 x 512:
+// 29.6 -> 32.0), or two tiles per SM (32768 x 1024: 170 -> 162).
+bool forward_wide(int64_t rows, int dm, bool dual, int sms) {
+  const int64_t tiles = ((rows + kT - 1) / kT) * ((dm + 255) / 256);
+  if (!dual) return 2 * tiles >= sms;
+  return tiles >= 2 * (int64_t)sms || (dm >= 1024 && wide_waves(rows, dm, sms));
 }
 
 struct Maps { CUtensorMap a, b, i0, i1, o0, o1; };
@@ -486,7 +501,7 @@ bool gate_forward_wide(int64_t rows, int dm, const void* y_sa, const void* y_swa
                        const void* w_sa, const void* w_swa, void* out, int64_t ld_out,
                        int* status, int sms, cudaStream_t st, cudaError_t* err) {
   *err = cudaSuccess;
-  if (!wide_tiles(rows, dm, sms)) return false;
+  if (!forward_wide(rows, dm, y_swa != nullptr, sms)) return false;
   for (int x = 0; x < (y_swa ? 2 : 1); ++x) {
     const void* y = x ? y_swa : y_sa;
     const void* w = x ? w_swa : w_sa;
@@ -549,11 +564,7 @@ extern "C" sa_status sa_gate_projection_backward(
       __nv_bfloat16* dz = (__nv_bfloat16*)ws;
       __nv_bfloat16* dyd = dz + rows * (int64_t)dm;
       float* part = (float*)(dyd + rows * (int64_t)dm);
-      // 128 x 256 tiles when their waves take less time than those of 128 x 128: a wide tile's
-      // K chunk takes 512 cycles, a narrow one's 300 (64 columns of operands per product more)
-      const int64_t tm = (rows + kT - 1) / kT;
-      const bool wide = (tm * ((dm + 255) / 256) + sms - 1) / sms * 512 <=
-                        (tm * ((dm + 127) / 128) + sms - 1) / sms * 300;
+      const bool wide = wide_waves(rows, dm, sms);
       const DwPlan dwp = plan_dw(rows, dm, sms);
       CUtensorMap y_k, w_k, dz_k, w_mn, dz_mn, y_mn, dout_k, dyd_k, dy_k, dw_o;
       if (!make_map(&y_k, y, rows, dm, ld_y, 128) ||

@@ -89,3 +89,18 @@ def test_host_pieces_of_a_batch(B, Hq, Hkv, n):
     want = want[0] if isinstance(want, (tuple, list)) else want
     assert torch.equal(y, want.cpu())
     assert sa.sa_read_status() == 0
+
+
+# the forward's choice of tiles at its lines.  One path: 74 wide tiles (half of 148), 73 x 128 rows and
+# one more at dm = 256.  Two paths: 296 wide tiles at dm = 256; at dm = 1024 18 and 19 row tiles, where the
+# 128 x 128 tiles go from one round of 148 SMs (144) to two (152)
+@pytest.mark.parametrize("rows,dm,dual", [(9344, 256, False), (9345, 256, False), (37889, 256, True),
+                                          (2304, 1024, True), (2305, 1024, True)])
+def test_projection_gate_forward_tile_choice(rows, dm, dual):
+    g = torch.Generator().manual_seed(rows)
+    ya, yb = (torch.randn(rows, dm, generator=g).bfloat16() for _ in range(2))
+    wa, wb = ((torch.randn(dm, dm, generator=g) * dm ** -0.5).bfloat16() for _ in range(2))
+    args = (ya, wa, yb, wb) if dual else (ya, wa)
+    out = sa.sa_gate_projection_forward(*(t.cuda() for t in args))
+    assert sa.sa_read_status() == 0
+    _close(out, oracle.gate_projection(*(t.double().numpy() for t in args)), "out")
