@@ -426,11 +426,11 @@ __global__ void dw_simt_kernel(int64_t rows, int dm, const float* __restrict__ d
 // ------------------------------------------------------------------------------ host
 
 // 128 x 256 tiles take less time than 128 x 128 by their waves: a wide tile's K chunk takes 512
-// cycles, a narrow one's 300 (64 columns of operands per product more).
-bool wide_waves(int64_t rows, int dm, int sms) {
+// cycles, a narrow one's `narrow` (about 300, with 64 columns of operands per product more).
+bool wide_waves(int64_t rows, int dm, int sms, int narrow) {
   const int64_t tm = (rows + kT - 1) / kT;
   return (tm * ((dm + 255) / 256) + sms - 1) / sms * 512 <=
-         (tm * ((dm + 127) / 128) + sms - 1) / sms * 300;
+         (tm * ((dm + 127) / 128) + sms - 1) / sms * narrow;
 }
 
 // Forward: the wide kernel, one launch per path, or (false) the fused 128 x 128 one.  One path: from
@@ -442,7 +442,7 @@ bool wide_waves(int64_t rows, int dm, int sms) {
 bool forward_wide(int64_t rows, int dm, bool dual, int sms) {
   const int64_t tiles = ((rows + kT - 1) / kT) * ((dm + 255) / 256);
   if (!dual) return 2 * tiles >= sms;
-  return tiles >= 2 * (int64_t)sms || (dm >= 1024 && wide_waves(rows, dm, sms));
+  return tiles >= 2 * (int64_t)sms || (dm >= 1024 && wide_waves(rows, dm, sms, 300));
 }
 
 struct Maps { CUtensorMap a, b, i0, i1, o0, o1; };
@@ -564,7 +564,9 @@ extern "C" sa_status sa_gate_projection_backward(
       __nv_bfloat16* dz = (__nv_bfloat16*)ws;
       __nv_bfloat16* dyd = dz + rows * (int64_t)dm;
       float* part = (float*)(dyd + rows * (int64_t)dm);
-      const bool wide = wide_waves(rows, dm, sms);
+      // (with a long contraction the narrow tiles' operand stream counts for more: 2500 x 2048, two
+      // rounds of wide tiles against three, 92 -> 84 us; but 12000 x 512 49 -> 52)
+      const bool wide = wide_waves(rows, dm, sms, dm >= 1024 ? 350 : 300);
       const DwPlan dwp = plan_dw(rows, dm, sms);
       CUtensorMap y_k, w_k, dz_k, w_mn, dz_mn, y_mn, dout_k, dyd_k, dy_k, dw_o;
       if (!make_map(&y_k, y, rows, dm, ld_y, 128) ||
