@@ -69,17 +69,21 @@ at::Tensor fresh(at::IntArrayRef sizes, at::ScalarType type, c10::Device dev) {
   if (!dev.is_cuda()) return at::empty(sizes, at::TensorOptions().dtype(type).device(dev));
   return at::detail::empty_cuda(sizes, type, dev, std::nullopt);
 }
-// A tensor with the shape, strides and type of `t`.
-at::Tensor fresh_like(const at::Tensor& t) {
-  if (t.is_cuda() && t.is_non_overlapping_and_dense())
-    return at::detail::empty_strided_cuda(t.sizes(), t.strides(), t.scalar_type(), t.device());
-  return at::empty_like(t);
-}
-
 void same_layout(const at::Tensor& ref, const at::Tensor* t) {
   if (t && (t->sizes() != ref.sizes() || t->strides() != ref.strides() ||
             t->scalar_type() != ref.scalar_type()))
     raise(PyExc_ValueError, "tensor does not share the layout of its reference tensor");
+}
+
+// A tensor with the shape, strides and type of `t`.  A slice of a larger tensor or an expanded one
+// has strides that a fresh tensor cannot have: the kernels, which are told one set of strides for
+// both, would write outside it.
+at::Tensor fresh_like(const at::Tensor& t) {
+  if (t.is_cuda() && t.is_non_overlapping_and_dense())
+    return at::detail::empty_strided_cuda(t.sizes(), t.strides(), t.scalar_type(), t.device());
+  const at::Tensor r = at::empty_like(t);
+  same_layout(t, &r);
+  return r;
 }
 
 sa_problem problem(const at::Tensor& q, const at::Tensor& k, PyObject* w, uint32_t flags,
