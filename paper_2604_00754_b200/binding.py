@@ -337,6 +337,7 @@ def sa_swa_gated_forward_rope(q, k, v, perm, inv, rope_cos, rope_sin, gate_logit
         for name in ("lse_sa", "lse_swa"):
             out[name] = torch.empty(q.shape[:3], dtype=torch.float32, device=q.device)
     y = torch.empty_like(q)
+    _same_layout(q, y)
     p = make_problem(q, k, w, flags, scale)
     ws = _workspace(sa_workspace_bytes(p, OP_FORWARD_ROPE), q.device, None)
     _check(lib.sa_swa_gated_forward_rope(

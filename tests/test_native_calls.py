@@ -19,7 +19,8 @@ def _expanded():
 
 
 @pytest.mark.parametrize("make", [_packed, _expanded])
-@pytest.mark.parametrize("call", ["forward", "gated", "gated_saving", "backward_q", "backward_k"])
+@pytest.mark.parametrize("call", ["forward", "gated", "gated_saving", "backward_q", "backward_k",
+                                  "rope", "gated_rope"])
 def test_outputs_that_cannot_have_the_layout_are_refused(make, call):
     perm = torch.arange(n, dtype=torch.int32).expand(B, n).contiguous()
     odd, plain = make(), torch.zeros(B, H, n, d).bfloat16()
@@ -31,6 +32,10 @@ def test_outputs_that_cannot_have_the_layout_are_refused(make, call):
         elif call.startswith("gated"):
             sa.sa_swa_gated_forward(odd, plain, plain, perm, perm, lg, w,
                                     save_for_bwd=call == "gated_saving")
+        elif call == "rope":
+            sa.sa_forward_rope(odd, plain, plain, perm, perm, lse, lse, w)
+        elif call == "gated_rope":
+            sa.sa_swa_gated_forward_rope(odd, plain, plain, perm, perm, lse, lse, lg, w)
         else:
             q, k = (odd, plain) if call == "backward_q" else (plain, odd)
             sa.sa_backward(q, k, k, perm, perm, lg, q, q, lse, lse, q, w)
