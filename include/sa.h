@@ -257,8 +257,10 @@ sa_status sa_coverage(int32_t L, int32_t n, int32_t w, uint32_t flags, const int
  * when given the strides of a [B,n,Hq,d] tensor).  w_sa, w_swa: device, [dm, dm] row-major
  * (out_features x in_features, a bias-free linear layer), same dtype.  y_swa == NULL selects
  * the single-path gate (w_swa ignored).  Products accumulate in fp32; the logistic and the
- * combination are fp32, rounded once to the run dtype.  dtype SA_BF16 with dm a multiple of
- * 64 and 16-byte aligned rows runs on the tensor cores; every other case on a plain kernel.
+ * combination are fp32, rounded once to the run dtype (but bf16 with two paths and at least two
+ * 128 x 256 tiles of out per SM: the first path is rounded before the second is added to it).
+ * dtype SA_BF16 with dm a multiple of 64 and 16-byte aligned rows runs on the tensor cores;
+ * every other case on a plain kernel.
  * Nothing is allocated; inputs are not modified; out may not alias an input.
  * Errors: SA_ERR_INVALID_ARG (null pointer, rows < 1, dm < 1, ld < dm), SA_ERR_CUDA. */
 sa_status sa_gate_projection_forward(int64_t rows, int32_t dm, int32_t dtype, const void* y_sa,

@@ -435,14 +435,13 @@ bool wide_waves(int64_t rows, int dm, int sms, int narrow) {
 
 // Forward: the wide kernel, one launch per path, or (false) the fused 128 x 128 one.  One path: from
 // half a wide tile per SM on (8000 x 1024: 25.9 -> 19.9 us, 1300 x 2048: 23.0 -> 18.5, 9000 x 768: 19.8
-// -> 17.2; even at 5000 x 512, 80 tiles: 13.3 -> 12.7).  Two paths: the fused kernel writes the result
-// once and reads nothing back, so the wide one needs the better waves and the long contraction of
-// dm >= 1024 (4000 x 2048: 79 -> 70, 2000 x 4096: 155 -> 138, 8000 x 1024: 43.4 -> 41.5; but 18000 x 512:
-// 29.6 -> 32.0), or two tiles per SM (32768 x 1024: 170 -> 162).
+// -> 17.2; even at 5000 x 512, 80 tiles: 13.3 -> 12.7).  Two paths: the fused kernel adds them in fp32
+// and rounds once, the wide one rounds the first path before the second launch adds to it (2-norm of
+// the error 2.03e-3 of the result's against 1.66e-3), so it serves only from two tiles per SM
+// (32768 x 1024: 170 -> 162 us), although it would be faster at some smaller sizes (2000 x 4096: 155 -> 138).
 bool forward_wide(int64_t rows, int dm, bool dual, int sms) {
   const int64_t tiles = ((rows + kT - 1) / kT) * ((dm + 255) / 256);
-  if (!dual) return 2 * tiles >= sms;
-  return tiles >= 2 * (int64_t)sms || (dm >= 1024 && wide_waves(rows, dm, sms, 300));
+  return dual ? tiles >= 2 * (int64_t)sms : 2 * tiles >= sms;
 }
 
 struct Maps { CUtensorMap a, b, i0, i1, o0, o1; };

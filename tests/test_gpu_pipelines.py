@@ -92,8 +92,7 @@ def test_host_pieces_of_a_batch(B, Hq, Hkv, n):
 
 
 # the forward's choice of tiles at its lines.  One path: 74 wide tiles (half of 148), 73 x 128 rows and
-# one more at dm = 256.  Two paths: 296 wide tiles at dm = 256; at dm = 1024 18 and 19 row tiles, where the
-# 128 x 128 tiles go from one round of 148 SMs (144) to two (152)
+# one more at dm = 256.  Two paths: 296 wide tiles at dm = 256, and sizes below them at dm = 1024
 @pytest.mark.parametrize("rows,dm,dual", [(9344, 256, False), (9345, 256, False), (37889, 256, True),
                                           (2304, 1024, True), (2305, 1024, True)])
 def test_projection_gate_forward_tile_choice(rows, dm, dual):
@@ -104,3 +103,19 @@ def test_projection_gate_forward_tile_choice(rows, dm, dual):
     out = sa.sa_gate_projection_forward(*(t.cuda() for t in args))
     assert sa.sa_read_status() == 0
     _close(out, oracle.gate_projection(*(t.double().numpy() for t in args)), "out")
+
+
+# Two paths below two wide tiles per SM: one launch, both products added in fp32 and rounded once.
+# Half a unit in the last place of bf16 for the rounding, and for each path its value times 2^-11: the
+# logistic is half a hardware tanh, whose relative error is 2^-11, and the rest is for the fp32 sums.
+@pytest.mark.parametrize("rows,dm", [(2305, 1024), (1200, 2048), (640, 4096)])
+def test_two_gate_paths_are_rounded_once(rows, dm):
+    g = torch.Generator().manual_seed(rows)
+    ya, yb = (torch.randn(rows, dm, generator=g).bfloat16() for _ in range(2))
+    wa, wb = ((torch.randn(dm, dm, generator=g) * dm ** -0.5).bfloat16() for _ in range(2))
+    out = sa.sa_gate_projection_forward(ya.cuda(), wa.cuda(), yb.cuda(), wb.cuda())
+    assert sa.sa_read_status() == 0
+    want = oracle.gate_projection(*(t.double().numpy() for t in (ya, wa, yb, wb)))
+    half_ulp = np.exp2(np.floor(np.log2(np.abs(want) + 1e-30)) - 8)
+    bound = half_ulp + 2.0 ** -11 * (as_f64(ya.abs()) + as_f64(yb.abs()))
+    assert (np.abs(as_f64(out) - want) <= bound).all()
