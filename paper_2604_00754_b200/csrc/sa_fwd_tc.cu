@@ -1002,23 +1002,28 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
 
 // ---------------------------------------------------------------------------- host
 
-// Score-block width.  64-key blocks skip more of a window's ends and let a tile's products and row
-// work interleave; 128-key blocks take half as many products, commits and softmax rounds per key.
-// Measured, us with 64 / 128:
-//   tiles by TMA, d = 64 (two issuing threads hide the commits): 64 at every width (8 x 12 heads,
-//     n = 4096: w = 33 65 / 79, w = 384 116 / 124; 4 x 12 heads, w = 1600 159 / 181);
-//   tiles by TMA, d = 128 (one issuing thread): 128 at every width (32/8 heads, n = 8192: w = 33
-//     57.4 / 56.6, w = 128 65 / 57, w = 1024 204 / 150);
-//   gathered: 64 up to w = 320 (2 x 16 heads of 128, n = 4096: w = 64 58.5 / 62.2, w = 160 72.0 / 75.8,
-//     w = 320 88.0 / 89.9; 16/4 heads of 64, n = 16384: w = 320 102 / 112), 128 from there (32/8 heads of
-//     128, n = 8192: w = 384 133 / 127, w = 1024 244 / 216).  With no more than one item per SM only a
-//     block's latency counts, and 128 is better from w = 129 (32/8 heads of 128, n = 700, w = 256,
-//     gated: 37.4 / 36.0).
+// Score-block width: 128 keys from w = 129 on, and at every width where d = 128 tiles come by TMA.
+// 64-key blocks skip more of a window's ends and let a tile's products and row work interleave; 128-key
+// blocks take half as many products, commits and softmax rounds per key.  The first block of a row
+// also sets the maximum that P is rounded under: of 128 keys it is more often the row's own, and its
+// probability then exactly 1.  Error of y against float64, 64 / 128 keys: 2.152e-3 / 2.111e-3 (2 x 16
+// heads of 128, n = 2048, w = 256), 2.172e-3 / 2.143e-3 (16/4 heads of 64, w = 320), TMA tiles 2.171e-3 /
+// 2.154e-3 (16 heads of 64, w = 256).  Times, us with 64 / 128:
+//   gathered: 8/2 heads of 128, n = 4096: w = 129 16.5 / 15.2, w = 256 20.0 / 18.4; 2 x 16 heads of 128,
+//     n = 4096: w = 64 58.5 / 62.2, w = 160 72.0 / 75.8, w = 320 88.0 / 89.9; 32/8 heads of 128, n = 8192:
+//     w = 384 133 / 127, w = 1024 244 / 216;
+//   tiles by TMA, d = 128 (one issuing thread, 32/8 heads, n = 8192): w = 33 57.4 / 56.6, w = 128 65 / 57,
+//     w = 1024 204 / 150;
+//   tiles by TMA, d = 64 (two issuing threads hide the commits): 8 x 12 heads, n = 4096: w = 33 65 / 79,
+//     w = 384 116 / 124.
+// So between w = 129 and 320, and at d = 64 by TMA, the line is drawn by the error, not by the time.
+// It depends on nothing that a part of a batch or of the heads changes: a sequence has the same bits
+// alone, in a batch and in a piece of the host pipeline.
 // The test hook sa_debug_set(SA_DEBUG_SCORE_BLOCK, 64 | 128) overrides the choice.
-bool key_block_128(int w, int d, bool tma_tiles, bool one_item) {
+bool key_block_128(int w, int d, bool tma_tiles) {
   const int forced = debug_option(SA_DEBUG_SCORE_BLOCK);
   if (forced) return forced == 128;
-  return tma_tiles ? d == 128 : w > (one_item ? 128 : 320);
+  return w > 128 || (tma_tiles && d == 128);
 }
 
 // sa_debug_set(SA_DEBUG_SWA_TILE_LOADS, 0) keeps the cp.async gather for the one-sided SWA
@@ -1084,7 +1089,7 @@ cudaError_t launch_fwd_tc(const FwdArgs& a, cudaStream_t st) {
     if (err != cudaSuccess) return err;
     return launch_dependent(kernel, dim3(grid), dim3(kThreads), smem, st, p, tm_q, tm_k, tm_v);
   };
-  const bool wide = key_block_128(a.w, a.d, natural, p.total_items <= sm_count[dev]);
+  const bool wide = key_block_128(a.w, a.d, natural);
   // instantiation by (head dimension, score-block width, source of the tiles, rotation, combine)
   auto pick = [&](auto d_c, auto kb_c) {
     constexpr int DD = decltype(d_c)::value, KK = decltype(kb_c)::value;

@@ -91,6 +91,37 @@ def test_host_pieces_of_a_batch(B, Hq, Hkv, n):
     assert sa.sa_read_status() == 0
 
 
+# A sequence's result does not depend on what else is in the call: alone (at most one item per SM) and
+# in a batch (several), or in a piece of the host pipeline, it has the same bits.
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("w", [128, 129, 256, 320])
+def test_bits_of_a_sequence_alone_and_in_a_batch(w, d):
+    g = torch.Generator().manual_seed(w)
+    q, k, v = (torch.randn(8, h, 600, d, generator=g).bfloat16().cuda() for h in (16, 8, 8))
+    lg = torch.randn(2, 16, generator=g).cuda()
+    perm, inv = sa.sa_make_perm(3, 1, 8, 600)
+    whole = sa.sa_swa_gated_forward(q, k, v, perm, inv, lg, w, save_for_bwd=True)
+    part = [t[2:3].contiguous() for t in (q, k, v, perm, inv)]
+    for a, b in zip(whole, sa.sa_swa_gated_forward(*part, lg, w, save_for_bwd=True)):
+        assert torch.equal(a[2:3], b)
+    assert sa.sa_read_status() == 0
+
+
+@pytest.mark.parametrize("w", [129, 256, 320])
+def test_host_pieces_have_the_bits_of_the_whole(w):
+    from paper_2604_00754_b200.host import HostForward
+    g = torch.Generator().manual_seed(w)
+    q, k, v = (torch.randn(1, h, 2048, 128, generator=g).bfloat16().pin_memory() for h in (32, 8, 8))
+    lg = torch.randn(2, 32, generator=g).pin_memory()
+    y = torch.empty_like(q).pin_memory()
+    HostForward(1, 32, 8, 2048, 128, w).forward(q, k, v, lg, y, seed=7, layer=1)
+    torch.cuda.synchronize()
+    perm, inv = sa.sa_make_perm(7, 1, 1, 2048)
+    want = sa.sa_swa_gated_forward(q.cuda(), k.cuda(), v.cuda(), perm, inv, lg.cuda(), w, ONE)
+    assert torch.equal(y, want.cpu())
+    assert sa.sa_read_status() == 0
+
+
 # the forward's choice of tiles at its lines.  One path: 74 wide tiles (half of 148), 73 x 128 rows and
 # one more at dm = 256.  Two paths: 296 wide tiles at dm = 256, and sizes below them at dm = 1024
 @pytest.mark.parametrize("rows,dm,dual", [(9344, 256, False), (9345, 256, False), (37889, 256, True),
