@@ -150,8 +150,10 @@ bool split_tiles(int B, int Hkv, int n) {
   return (int64_t)B * Hkv * ((n + kRows - 1) / kRows) < 8 * 148;
 }
 
-template <bool KEYS, int NCG>
-__device__ __forceinline__ void bwd_tile(const BwdArgs& a, unsigned char* smem_raw, int b, int x,
+// Without SEEN nothing is stored and false returned where a sum of this CTA ended in a NaN: see
+// tile_accumulate_seen.
+template <bool KEYS, int NCG, bool SEEN>
+__device__ __forceinline__ bool bwd_tile(const BwdArgs& a, unsigned char* smem_raw, int b, int x,
                                          int hfirst, int heads, float* out1, float* out2,
                                          bool split) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -269,16 +271,26 @@ __device__ __forceinline__ void bwd_tile(const BwdArgs& a, unsigned char* smem_r
       st4(pw + 8 * col + 4 * half, make_float4(ds[0], ds[1], ds[2], ds[3]));
     }
     __syncwarp();
-    tile_accumulate<float, NCG>(o1, pw + 4 * half, c1, sm.stride(), tx, d);
+    auto seen = [&](int r, int k) {
+      return rslot[r] < a.n && g.sees(rslot[r], rtok[r], s_slot[buf][k], s_tok[buf][k]);
+    };
+    if constexpr (SEEN) tile_accumulate_seen<float, NCG>(o1, pw + 4 * half, c1, sm.stride(), tx, d, seen);
+    else tile_accumulate<float, NCG>(o1, pw + 4 * half, c1, sm.stride(), tx, d);
     if constexpr (KEYS) {
       __syncwarp();
 #pragma unroll
       for (int c = 0; c < 2; ++c)
         st4(pw + 8 * (tx + 16 * c) + 4 * half, make_float4(s[0][c], s[1][c], s[2][c], s[3][c]));
       __syncwarp();
-      tile_accumulate<float, NCG>(o2, pw + 4 * half, c2, sm.stride(), tx, d);
+      if constexpr (SEEN) tile_accumulate_seen<float, NCG>(o2, pw + 4 * half, c2, sm.stride(), tx, d, seen);
+      else tile_accumulate<float, NCG>(o2, pw + 4 * half, c2, sm.stride(), tx, d);
     }
     __syncthreads();
+  }
+  if constexpr (!SEEN) {
+    bool nan = any_nan(o1);
+    if constexpr (KEYS) nan |= any_nan(o2);
+    if (__syncthreads_or(nan)) return false;
   }
 
 #pragma unroll
@@ -307,13 +319,20 @@ __device__ __forceinline__ void bwd_tile(const BwdArgs& a, unsigned char* smem_r
       }
     }
   }
+  return true;
+}
+
+template <bool KEYS, int NCG>
+__device__ __noinline__ void bwd_tile_seen(const BwdArgs& a, unsigned char* smem_raw, int b, int x,
+                                           int hfirst, int heads, float* out1, float* out2, bool split) {
+  bwd_tile<KEYS, NCG, true>(a, smem_raw, b, x, hfirst, heads, out1, out2, split);
 }
 
 // blockIdx.y: first the nb * Hq (branch, head) pairs of dQ, then those of dK / dV, whose CTAs
 // cover `heads` query heads each.  Branches x0 .. x0 + nb - 1.
 template <int NCG>
 __global__ void __launch_bounds__(kTileThreads, NCG == 1 ? 4 : NCG == 2 ? 2 : 1)
-bwd_tile_kernel(const BwdArgs a, int x0, int nb, int heads, bool split) {
+bwd_tile_kernel(const __grid_constant__ BwdArgs a, int x0, int nb, int heads, bool split) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   grid_dependency_wait();
   grid_dependents_launch();
@@ -325,7 +344,8 @@ bwd_tile_kernel(const BwdArgs a, int x0, int nb, int heads, bool split) {
     const int hq = y % a.Hq, x = x0 + y / a.Hq;
     float* out = split ? a.parts + x * rows_q + ((size_t)b * a.Hq + hq) * a.n * a.d
                        : (float*)a.dq + b * a.qs[0] + hq * a.qs[1];
-    bwd_tile<false, NCG>(a, smem_raw, b, x, hq, 1, out, nullptr, split);
+    if (!bwd_tile<false, NCG, false>(a, smem_raw, b, x, hq, 1, out, nullptr, split))
+      bwd_tile_seen<false, NCG>(a, smem_raw, b, x, hq, 1, out, nullptr, split);
   } else {
     y -= nb * a.Hq;
     const int groups = a.Hq / heads, h0 = (y % groups) * heads, x = x0 + y / groups, hk = h0 / G;
@@ -333,8 +353,10 @@ bwd_tile_kernel(const BwdArgs a, int x0, int nb, int heads, bool split) {
     // partial (x, h0 % G): [B,Hkv,n,d] each; dK's first, dV's 2 * rows_q further on
     float* part = a.parts + 2 * rows_q + (size_t)(x * G + h0 % G) * (rows_q / G) +
                   ((size_t)b * a.Hkv + hk) * a.n * a.d;
-    bwd_tile<true, NCG>(a, smem_raw, b, x, h0, heads, split ? part : (float*)a.dk + off,
-                        split ? part + 2 * rows_q : (float*)a.dv + off, split);
+    float* dk = split ? part : (float*)a.dk + off;
+    float* dv = split ? part + 2 * rows_q : (float*)a.dv + off;
+    if (!bwd_tile<true, NCG, false>(a, smem_raw, b, x, h0, heads, dk, dv, split))
+      bwd_tile_seen<true, NCG>(a, smem_raw, b, x, h0, heads, dk, dv, split);
   }
 }
 

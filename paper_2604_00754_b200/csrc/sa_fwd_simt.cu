@@ -17,17 +17,17 @@
 namespace sa {
 namespace {
 
-// NCG: groups of 64 output columns (d <= 64 * NCG)
-template <typename T, int NCG>
-__global__ void __launch_bounds__(kTileThreads) fwd_tile_kernel(const FwdArgs a) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
+typedef int IntCols[kCols];
+
+// NCG: groups of 64 output columns (d <= 64 * NCG).  Without SEEN nothing is stored and false returned
+// where a sum of this CTA ended in a NaN: see tile_accumulate_seen.
+template <typename T, int NCG, bool SEEN>
+__device__ __forceinline__ bool fwd_tile(const FwdArgs& a, unsigned char* smem_raw, IntCols* s_slot,
+                                         IntCols* s_tok) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int tx = lane & 15, half = lane >> 4;         // key / column index, row group of the warp
   const int row0 = warp * 8 + half * 4;               // this thread's four rows
   const int hq = blockIdx.y, b = blockIdx.z, s0 = blockIdx.x * kRows;
-  grid_dependency_wait();
-  grid_dependents_launch();
-  if (a.abort_flag && *a.abort_flag) return;          // an earlier check rejected perm/inv
   const int hk = hq / (a.Hq / a.Hkv), d = a.d;
   const int32_t* perm = a.swa ? nullptr : a.perm + (size_t)b * a.n;
   const TileSmem<T> sm(d);
@@ -35,7 +35,6 @@ __global__ void __launch_bounds__(kTileThreads) fwd_tile_kernel(const FwdArgs a)
   T* kv = reinterpret_cast<T*>(smem_raw + sm.rows_bytes());       // K0 V0 K1 V1
   float* ps = reinterpret_cast<float*>(smem_raw + sm.rows_bytes() + 4 * sm.col_bytes());
   float* pw = ps + warp * (kCols * 8);                // this warp's probabilities [key][8 rows]
-  __shared__ int s_slot[2][kCols], s_tok[2][kCols];
 
   const T* kbase = (const T*)a.k + b * a.ks[0] + hk * a.ks[1];
   const T* vbase = (const T*)a.v + b * a.ks[0] + hk * a.ks[1];
@@ -114,9 +113,15 @@ __global__ void __launch_bounds__(kTileThreads) fwd_tile_kernel(const FwdArgs a)
       *reinterpret_cast<float4*>(pw + (tx + 16 * c) * 8 + 4 * half) =
           make_float4(s[0][c], s[1][c], s[2][c], s[3][c]);
     __syncwarp();
-    tile_accumulate<T, NCG>(o, pw + 4 * half, vs_, sm.stride(), tx, d);
+    if constexpr (SEEN)
+      tile_accumulate_seen<T, NCG>(o, pw + 4 * half, vs_, sm.stride(), tx, d, [&](int r, int k) {
+        return g.sees(qslot[r], qtok[r], s_slot[buf][k], s_tok[buf][k]);
+      });
+    else
+      tile_accumulate<T, NCG>(o, pw + 4 * half, vs_, sm.stride(), tx, d);
     __syncthreads();                                  // the buffer may be refilled now
   }
+  if (!SEEN && __syncthreads_or(any_nan(o))) return false;
 
   float g_this = 1.f, g_other = 0.f;
   if (a.gate_logits) {
@@ -155,6 +160,24 @@ __global__ void __launch_bounds__(kTileThreads) fwd_tile_kernel(const FwdArgs a)
     if (a.lse && tx == 0)
       a.lse[((size_t)b * a.Hq + hq) * a.n + qtok[r]] = (m[r] + log2f(l[r])) * kLn2;
   }
+  return true;
+}
+
+template <typename T, int NCG>
+__device__ __noinline__ void fwd_tile_seen(const FwdArgs& a, unsigned char* smem_raw, IntCols* s_slot,
+                                           IntCols* s_tok) {
+  fwd_tile<T, NCG, true>(a, smem_raw, s_slot, s_tok);
+}
+
+template <typename T, int NCG>
+__global__ void __launch_bounds__(kTileThreads) fwd_tile_kernel(const __grid_constant__ FwdArgs a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ int s_slot[2][kCols], s_tok[2][kCols];
+  grid_dependency_wait();
+  grid_dependents_launch();
+  if (a.abort_flag && *a.abort_flag) return;          // an earlier check rejected perm/inv
+  if (!fwd_tile<T, NCG, false>(a, smem_raw, s_slot, s_tok))
+    fwd_tile_seen<T, NCG>(a, smem_raw, s_slot, s_tok);
 }
 
 template <typename T, int NCG>

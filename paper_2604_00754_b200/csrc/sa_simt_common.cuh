@@ -192,6 +192,41 @@ __device__ __forceinline__ void tile_accumulate(float (&o)[4][4 * NCG], const fl
   }
 }
 
+// The same, leaving out the pairs that sees(r, k) hides: their weight is 0, and 0 times an infinity or
+// a NaN would reach rows that do not see that column.  One select per pair more than the tile needs
+// otherwise, so a tile's walk is repeated with it only where the plain sums ended in a NaN.
+template <typename T, int NCG, typename F>
+__device__ __forceinline__ void tile_accumulate_seen(float (&o)[4][4 * NCG], const float* p,
+                                                     const T* cols, int stride, int tx, int d, F&& sees) {
+#pragma unroll 1
+  for (int k = 0; k < kCols; ++k) {
+    const float4 w = ld4(p + 8 * k);
+    const float wr[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+    for (int cg = 0; cg < NCG; ++cg) {
+      const float4 v = ld4(cols + k * stride + min(64 * cg + 4 * tx, d - 4));
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        if (!sees(r, k)) continue;
+        o[r][4 * cg] = fmaf(wr[r], v.x, o[r][4 * cg]);
+        o[r][4 * cg + 1] = fmaf(wr[r], v.y, o[r][4 * cg + 1]);
+        o[r][4 * cg + 2] = fmaf(wr[r], v.z, o[r][4 * cg + 2]);
+        o[r][4 * cg + 3] = fmaf(wr[r], v.w, o[r][4 * cg + 3]);
+      }
+    }
+  }
+}
+
+template <int N>
+__device__ __forceinline__ bool any_nan(const float (&o)[4][N]) {
+  bool nan = false;
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int c = 0; c < N; ++c) nan |= isnan(o[r][c]);
+  return nan;
+}
+
 // Dynamic shared memory above 48 KB has to be asked for.
 inline cudaError_t allow_smem(const void* kernel, int bytes) {
   if (bytes <= 48 * 1024) return cudaSuccess;

@@ -44,6 +44,40 @@ def test_fp32_tiles(B, Hq, Hkv, n, d, w, flags):
     assert sa.sa_read_status() == 0
 
 
+# An infinity or a NaN reaches the rows and columns that its token meets and no others, although the
+# tiles hold pairs that do not see each other.  Finite where the oracle is, to the tolerances above
+# (bf16: 2e-2 of the largest finite value); the rest is not finite.
+@pytest.mark.parametrize("B,Hq,Hkv,n,d,dtype,flags", [
+    (1, 2, 1, 300, 64, torch.float32, CAUSAL | SWA_ONE_SIDED),
+    (1, 2, 2, 301, 128, torch.float32, 0),
+    (8, 8, 4, 1185, 16, torch.float32, CAUSAL | LINEAR_WINDOW),     # gradients not split
+    (1, 4, 2, 300, 72, torch.bfloat16, CAUSAL | SWA_ONE_SIDED),
+])
+def test_not_finite_values_stay_with_the_pairs_that_see_them(B, Hq, Hkv, n, d, dtype, flags):
+    g = torch.Generator().manual_seed(n)
+    mk = lambda h: torch.randn(B, h, n, d, generator=g).to(dtype)
+    q, k, v, dy = mk(Hq), mk(Hkv), mk(Hkv), mk(Hq)
+    v[:, :, 150, d // 2] = float("inf")
+    k[:, :, 40] = float("nan")
+    q[:, :, 250, 0] = float("nan")
+    dy[:, :, 200, d - 1] = -float("inf")
+    lg, w = torch.randn(2, Hq, generator=g), 9
+    perm, inv = sa.sa_make_perm(n, 1, B, n)
+    dev = [t.cuda() for t in (q, k, v)]
+    out = sa.sa_swa_gated_forward(*dev, perm, inv, lg.cuda(), w, flags, save_for_bwd=True)
+    grads = sa.sa_backward(*dev, perm, inv, lg.cuda(), *out[1:], dy.cuda(), w, flags)
+    assert sa.sa_read_status() == 0
+    args = [as_f64(t) for t in (q, k, v)] + [perm.cpu().numpy(), inv.cpu().numpy(), lg.double().numpy()]
+    want = tuple(oracle.gated_forward(*args, w, flags))[:3] + \
+        tuple(oracle.backward(*args, as_f64(dy), w, flags))[:3]
+    for got, ref, name in zip(out[:3] + tuple(grads[:3]), want, ("y", "y_sa", "y_swa", "dq", "dk", "dv")):
+        got, finite = as_f64(got), np.isfinite(ref)
+        assert finite.mean() > 0.4 and not finite.all(), name
+        assert np.array_equal(np.isfinite(got), finite), name
+        err, top = np.abs(got[finite] - ref[finite]).max(), np.abs(ref[finite]).max()
+        assert err <= (1e-4 * max(1.0, top) if dtype == torch.float32 else 2e-2 * top), name
+
+
 # one CTA up to 1024 tokens, clusters of 2, 4 and 8 up to 16384, global memory beyond
 @pytest.mark.parametrize("B,n", [(2, 33), (1, 1024), (2, 1025), (1, 2049), (3, 4097), (2, 8191),
                                  (1, 16384), (1, 16385)])
