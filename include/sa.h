@@ -164,13 +164,13 @@ sa_status sa_swa_gated_forward(const sa_problem* p, const void* q, const void* k
  * HOST memory: q, k, v, y are host pointers to contiguous [B,H,n,d] tensors of p->dtype
  * (p's stride fields are ignored), gate_logits a host pointer to fp32 [2,Hq]; pinned memory
  * lets the copies overlap the kernels, pageable memory works but serialises.  The work
- * travels through the GPU in about n_groups pieces, none smaller than 2 MB: ranges of
- * sequences first, then contiguous ranges of their KV heads (the first and the last range of
- * heads, when they hold one KV head, in q_parts ranges of its query heads if those divide
- * evenly and still fill the GPU: the ends of the pipeline are what cannot overlap), on three
- * internal streams: copy in, compute, copy out.  The permutation is drawn from (seed, layer) as in sa_make_perm and
- * shared by all ranges; every range is one sa_swa_gated_forward call, so the result has
- * the bits of that call.
+ * travels through the GPU in at most n_groups pieces (below 1 means 1; 256 are the most), none
+ * smaller than 2 MB: ranges of sequences first, then contiguous ranges of their KV heads.  The
+ * first and the last range of heads, when they hold one KV head, go in q_parts ranges of its
+ * query heads if those divide evenly and still fill the GPU: the ends of the pipeline are what
+ * cannot overlap.  There are three internal streams: copy in, compute, copy out.  The permutation
+ * is drawn from (seed, layer) as in sa_make_perm and shared by all ranges; every range is one
+ * sa_swa_gated_forward call, and the result has the bits of that call on the whole problem.
  *   ws: DEVICE workspace of sa_host_forward_ws_bytes(p) bytes, 256-byte aligned, owned by the
  *       caller (device copies of q, k, v, y, one branch output, the permutation and its
  *       scratch).  No device memory is allocated; the first call on a device creates the
@@ -185,9 +185,15 @@ sa_status sa_swa_gated_forward_host(const sa_problem* p, const void* q, const vo
                                     uint64_t seed, uint32_t layer, int32_t n_groups,
                                     int32_t q_parts, void* ws, size_t ws_bytes,
                                     sa_stream_t stream);
-/* The head ranges sa_swa_gated_forward_host uses, for inspection (host only, no GPU needed):
- * writes up to max_pieces rows of (kv_begin, kv_end, q_begin, q_end, carries_kv) and returns
- * their number, or -1 for bad head counts or too small an array. */
+/* The pieces sa_swa_gated_forward_host makes of a problem, in order, for inspection (host only, no
+ * GPU needed): writes up to max_pieces rows of (kv_begin, kv_end, q_begin, q_end, carries_kv,
+ * sequence_begin, sequence_end) and returns their number, or -1 for a bad problem or too small an
+ * array. */
+int32_t sa_host_forward_pieces(const sa_problem* p, int32_t n_groups, int32_t q_parts,
+                               int32_t* pieces, int32_t max_pieces);
+/* The division of the heads of one sequence alone, which the pieces of large problems follow (no
+ * least size, every cut by query heads that divides evenly): rows of (kv_begin, kv_end, q_begin,
+ * q_end, carries_kv); returns as above, -1 also for bad head counts. */
 int32_t sa_host_forward_plan(int32_t Hq, int32_t Hkv, int32_t n_groups, int32_t q_parts,
                              int32_t* pieces, int32_t max_pieces);
 

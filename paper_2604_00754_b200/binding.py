@@ -32,6 +32,7 @@ EXPORTS = [
     "sa_gate_projection_forward", "sa_gate_projection_backward",
     "sa_gate_projection_backward_ws_bytes", "sa_debug_set", "sa_debug_wait_timeout",
     "sa_swa_gated_forward_host", "sa_host_forward_ws_bytes", "sa_host_forward_plan",
+    "sa_host_forward_pieces",
     "sa_rope_table", "sa_rope_apply", "sa_forward_rope", "sa_swa_gated_forward_rope",
 ]
 OP_FORWARD_ROPE = 7
@@ -111,6 +112,8 @@ def load_library(path: Optional[str] = None) -> ctypes.CDLL:
     lib.sa_host_forward_ws_bytes.restype = sz
     lib.sa_host_forward_plan.argtypes = [i32, i32, i32, i32, vp, i32]
     lib.sa_host_forward_plan.restype = i32
+    lib.sa_host_forward_pieces.argtypes = [pp, i32, i32, vp, i32]
+    lib.sa_host_forward_pieces.restype = i32
     lib.sa_swa_gated_forward_host.argtypes = [pp, vp, vp, vp, vp, vp, u64, u32, i32, i32, vp, sz, vp]
     lib.sa_swa_gated_forward_host.restype = ctypes.c_int
     lib.sa_rope_table.argtypes = [i32, i32, ctypes.c_double, vp, vp, vp]
@@ -450,12 +453,25 @@ def sa_gate_projection_backward(dout, y_sa, w_sa, y_swa=None, w_swa=None, ws=Non
 
 
 def host_forward_plan(Hq: int, Hkv: int, n_groups: int, q_parts: int):
-    """Head ranges of the host-memory forward: (kv_begin, kv_end, q_begin, q_end, carries_kv)."""
+    """Head ranges of one sequence alone: (kv_begin, kv_end, q_begin, q_end, carries_kv)."""
     buf = (ctypes.c_int32 * (5 * 256))()
     cnt = int(load_library().sa_host_forward_plan(Hq, Hkv, n_groups, q_parts, buf, 256))
     if cnt < 0:
         raise ValueError("Hq must be a positive multiple of Hkv")
     return [tuple(buf[5 * i + j] for j in range(4)) + (bool(buf[5 * i + 4]),) for i in range(cnt)]
+
+
+def host_forward_pieces(B, Hq, Hkv, n, d, dtype=BF16, n_groups=8, q_parts=2):
+    """What sa_swa_gated_forward_host makes of a problem: (kv_begin, kv_end, q_begin, q_end,
+    carries_kv, sequence_begin, sequence_end) per piece, in order."""
+    host_forward_plan(Hq, Hkv, n_groups, q_parts)      # raises for bad head counts
+    p = SaProblem(B=B, Hq=Hq, Hkv=Hkv, n=n, d=d, w=1, dtype=dtype)
+    buf = (ctypes.c_int32 * (7 * 256))()
+    cnt = int(load_library().sa_host_forward_pieces(ctypes.byref(p), n_groups, q_parts, buf, 256))
+    if cnt < 0:
+        raise SaError(1, "sa_host_forward_pieces")
+    rows = [tuple(buf[7 * i:7 * i + 7]) for i in range(cnt)]
+    return [r[:4] + (bool(r[4]),) + r[5:] for r in rows]
 
 
 def host_forward_ws_bytes(B, Hq, Hkv, n, d, dtype=BF16) -> int:

@@ -17,6 +17,7 @@ namespace sa {
 namespace {
 
 constexpr int kMaxPieces = 256;
+constexpr int kPlanSms = 148;       // SMs of the GPU planned for: a plan is the same without one at hand
 
 struct Piece { int ka, kb, qa, qb, with_kv, b0, b1; };
 
@@ -71,6 +72,37 @@ int plan_batch(int most, int B, int Hq, int Hkv, int n_groups, int q_parts, Piec
   return cnt;
 }
 
+// Input bytes on the device (q, k, v, each rounded up to 256 bytes).
+size_t align256(size_t x) { return (x + 255) / 256 * 256; }
+size_t tensor_bytes(const sa_problem* p, int heads) {
+  return align256((size_t)p->B * heads * p->n * p->d * (p->dtype == SA_BF16 ? 2 : 4));
+}
+
+// The pieces of one call; -1 for what plan() refuses for the heads alone.  Any number of groups that
+// it takes for the heads is taken for a batch too: below 1 means 1, and more pieces than there are
+// events are not made.
+int plan_call(const sa_problem* p, int n_groups, int q_parts, Piece* out) {
+  if (plan(p->Hq, p->Hkv, n_groups, q_parts, out, kMaxPieces) < 1) return -1;
+  n_groups = n_groups < 1 ? 1 : (n_groups > kMaxPieces ? kMaxPieces : n_groups);
+  // a range's permutation may have to move to an aligned place in the scratch, which is as large as Q:
+  // one range if that is too small (rows of a few bytes)
+  const size_t per_seq = 2 * align256((size_t)p->n * sizeof(int32_t));
+  const int ranged = per_seq * p->B <= tensor_bytes(p, p->Hq) ? p->B : 1;
+  // a piece costs the host about 40 us of calls, as long as 2 MB take over PCIe: none smaller
+  const size_t most = (tensor_bytes(p, p->Hq) + 2 * tensor_bytes(p, p->Hkv)) >> 21;
+  if ((size_t)n_groups > most) {
+    n_groups = most ? (int)most : 1;
+    q_parts = 1;
+  }
+  // half of a group's query heads that leave SMs idle (an item is two tiles of 128 rows) take the
+  // kernels as long as the whole group: 32/8 heads, n = 8192: 2440 -> 2370 us uncut
+  if (q_parts > 1 &&
+      (int64_t)(p->Hq / p->Hkv / q_parts) * ((p->n + 127) / 128) < 2 * kPlanSms)
+    q_parts = 1;
+  const int cnt = plan_batch(ranged, p->B, p->Hq, p->Hkv, n_groups, q_parts, out, kMaxPieces);
+  return cnt > 0 ? cnt : plan_batch(ranged, p->B, p->Hq, p->Hkv, n_groups, 1, out, kMaxPieces);
+}
+
 // Streams and events of the pipeline, created at the first call on a device and kept.
 struct Pipe {
   bool ready = false;
@@ -100,23 +132,19 @@ Pipe* pipe_for_current_device() {
   return &p;
 }
 
-size_t align256(size_t x) { return (x + 255) / 256 * 256; }
-
 struct Carve {
   size_t q, k, v, y, scratch, gate, perm, inv, perm_ws, total;
 };
 
 bool carve(const sa_problem* p, Carve* c) {
   if (!p || p->B < 1 || p->Hq < 1 || p->Hkv < 1 || p->n < 1 || p->d < 1) return false;
-  const size_t es = p->dtype == SA_BF16 ? 2 : 4;
-  const size_t qb = (size_t)p->B * p->Hq * p->n * p->d * es;
-  const size_t kb = (size_t)p->B * p->Hkv * p->n * p->d * es;
+  const size_t qb = tensor_bytes(p, p->Hq), kb = tensor_bytes(p, p->Hkv);
   size_t o = 0;
-  c->q = o; o += align256(qb);
-  c->k = o; o += align256(kb);
-  c->v = o; o += align256(kb);
-  c->y = o; o += align256(qb);
-  c->scratch = o; o += align256(qb);
+  c->q = o; o += qb;
+  c->k = o; o += kb;
+  c->v = o; o += kb;
+  c->y = o; o += qb;
+  c->scratch = o; o += qb;
   // the logits as they come ([2, Hq]), then one contiguous [2, heads] block per piece
   c->gate = o; o += 2 * align256((size_t)2 * p->Hq * sizeof(float));
   c->perm = o; o += align256((size_t)p->B * p->n * sizeof(int32_t));
@@ -146,6 +174,21 @@ int32_t sa_host_forward_plan(int32_t Hq, int32_t Hkv, int32_t n_groups, int32_t 
   return cnt;
 }
 
+int32_t sa_host_forward_pieces(const sa_problem* p, int32_t n_groups, int32_t q_parts,
+                               int32_t* pieces, int32_t max_pieces) {
+  Carve c;
+  Piece tmp[kMaxPieces];
+  if (!pieces || !carve(p, &c)) return -1;
+  const int cnt = plan_call(p, n_groups, q_parts, tmp);
+  if (cnt < 0 || cnt > max_pieces) return -1;
+  for (int i = 0; i < cnt; ++i) {
+    const Piece& g = tmp[i];
+    const int row[7] = {g.ka, g.kb, g.qa, g.qb, g.with_kv, g.b0, g.b1};
+    for (int x = 0; x < 7; ++x) pieces[7 * i + x] = row[x];
+  }
+  return cnt;
+}
+
 size_t sa_host_forward_ws_bytes(const sa_problem* p) {
   Carve c;
   return carve(p, &c) ? c.total : (size_t)-1;
@@ -162,22 +205,7 @@ sa_status sa_swa_gated_forward_host(const sa_problem* p, const void* q, const vo
   if (!carve(p, &c)) return SA_ERR_INVALID_ARG;
   if (ws_bytes < c.total) return SA_ERR_WORKSPACE;
   Piece pieces[kMaxPieces];
-  // a range's permutation may have to move to an aligned place in the scratch: one range if that is
-  // too small (rows of a few bytes)
-  const size_t per_seq = 2 * align256((size_t)p->n * sizeof(int32_t));
-  const int ranged = per_seq * p->B <= c.gate - c.scratch ? p->B : 1;
-  // a piece costs the host about 40 us of calls, as long as 2 MB take over PCIe: none smaller
-  const size_t in = c.y - c.q;
-  if ((size_t)n_groups > (in >> 21)) {
-    n_groups = in >> 21 ? (int)(in >> 21) : 1;
-    q_parts = 1;
-  }
-  // half of a group's query heads that leave SMs idle (an item is two tiles of 128 rows) take the
-  // kernels as long as the whole group: 32/8 heads, n = 8192: 2440 -> 2370 us uncut
-  if (q_parts > 1 &&
-      (int64_t)(p->Hq / p->Hkv / q_parts) * ((p->n + 127) / 128) < 2 * 148)
-    q_parts = 1;
-  const int cnt = plan_batch(ranged, p->B, p->Hq, p->Hkv, n_groups, q_parts, pieces, kMaxPieces);
+  const int cnt = plan_call(p, n_groups, q_parts, pieces);
   if (cnt < 1) return SA_ERR_INVALID_ARG;
   // device-side problem: contiguous [B,H,n,d] buffers, whatever the strides field says
   sa_problem dp = *p;

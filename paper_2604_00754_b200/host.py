@@ -1,8 +1,8 @@
 """Gated SA + SWA forward for tensors that live in host memory.
 
 A thin holder of the device workspace around the C entry point ``sa_swa_gated_forward_host``,
-which owns the pipeline: the KV heads (and the query heads that share them) travel through the
-GPU in pieces on three streams (copy in, compute, copy out), the permutation of Section 3.1 is
+which owns the pipeline: ranges of the sequences and of their KV heads (with the query heads that
+share them) travel through the GPU in pieces on three streams (copy in, compute, copy out), the permutation of Section 3.1 is
 drawn once per call and shared by all pieces.  Nothing of the path runs here.
 """
 from typing import Optional
@@ -24,8 +24,8 @@ class HostForward:
         self.shape = (B, Hq, Hkv, n, d)
         self.w, self.flags, self.dtype = w, flags, dtype
         self.n_groups, self.q_parts = n_groups, q_parts
-        self.pieces = sa.host_forward_plan(Hq, Hkv, n_groups, q_parts)
         code = sa.BF16 if dtype == torch.bfloat16 else sa.F32
+        self.pieces = sa.host_forward_pieces(B, Hq, Hkv, n, d, code, n_groups, q_parts)
         self.ws = torch.empty(sa.host_forward_ws_bytes(B, Hq, Hkv, n, d, code), dtype=torch.uint8,
                               device=self.device)
 

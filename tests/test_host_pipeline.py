@@ -56,6 +56,44 @@ def test_host_forward_rejects_bad_arguments_before_any_cuda_call():
     assert lib.sa_swa_gated_forward_host(*args(fake, need - 1)) == 3
 
 
+# what the call makes of a problem: every head of every sequence once, K and V with the first piece that
+# reads them; many sequences with many groups, none, and more than there are events for
+@pytest.mark.parametrize("B,Hq,Hkv,n,d,n_groups,q_parts", [
+    (300, 8, 8, 683, 64, 300, 2), (300, 8, 8, 683, 64, 1000, 1), (16, 64, 32, 4096, 128, 512, 2),
+    (1, 8, 1, 9600, 64, 1, 2), (1, 16, 2, 38000, 64, 256, 8), (8, 8, 2, 4096, 64, 0, 2),
+    (8, 8, 2, 4096, 64, -1, 2), (300, 2, 2, 20000, 64, -5, 1),
+])
+def test_pieces_cover_every_head_of_every_sequence_once(B, Hq, Hkv, n, d, n_groups, q_parts):
+    pieces = sab.host_forward_pieces(B, Hq, Hkv, n, d, sab.BF16, n_groups, q_parts)
+    assert 1 <= len(pieces) <= 256
+    if q_parts == 1:
+        assert len(pieces) <= max(1, n_groups)
+    q_seen, kv_seen = set(), set()
+    for ka, kb, qa, qb, with_kv, b0, b1 in pieces:
+        G = Hq // Hkv
+        assert ka * G <= qa < qb <= kb * G and b0 < b1
+        if with_kv:
+            new = {(b, h) for b in range(b0, b1) for h in range(ka, kb)}
+            assert not new & kv_seen
+            kv_seen |= new
+        assert all((b, h) in kv_seen for b in range(b0, b1) for h in range(ka, kb))
+        new = {(b, h) for b in range(b0, b1) for h in range(qa, qb)}
+        assert not new & q_seen
+        q_seen |= new
+    assert len(q_seen) == B * Hq and len(kv_seen) == B * Hkv
+    if n_groups < 1 and q_parts == 1:
+        assert len(pieces) == 1
+
+
+def test_what_the_heads_alone_refuse_stays_refused():
+    with pytest.raises(ValueError):
+        sab.host_forward_pieces(1, 300, 300, 64, 64, n_groups=300)      # more pieces than 256
+    with pytest.raises(ValueError):
+        sab.host_forward_pieces(1, 10, 4, 64, 64)
+    with pytest.raises(sab.SaError):
+        sab.host_forward_pieces(0, 8, 4, 64, 64)
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("n_groups,q_parts", [(1, 1), (3, 2), (4, 2), (4, 1)])
 def test_pipelined_forward_equals_single_call(n_groups, q_parts):
@@ -82,4 +120,25 @@ def test_pipelined_forward_equals_single_call(n_groups, q_parts):
     torch.cuda.synchronize()
     perm, inv = sa.sa_make_perm(5, 3, B, n)
     ref = sa.sa_swa_gated_forward(q.cuda(), k.cuda(), v.cuda(), perm, inv, lg.cuda(), w, ws=scratch)
+    assert torch.equal(hy, ref.cpu())
+
+
+# more groups than events, and none: two launches per piece and one for the permutation
+@pytest.mark.gpu
+@pytest.mark.parametrize("B,n,n_groups", [(300, 683, 300), (4, 2100, -1)])
+def test_any_number_of_groups(B, n, n_groups):
+    from paper_2604_00754_b200 import binding as sa
+    g = torch.Generator(device="cuda").manual_seed(n)
+    dev = [torch.randn(B, 8, n, 64, generator=g, device="cuda").bfloat16() for _ in range(3)]
+    lg = torch.randn(2, 8, generator=g, device="cuda")
+    q, k, v, hlg = (torch.empty(t.shape, dtype=t.dtype, pin_memory=True).copy_(t) for t in dev + [lg])
+    hy = torch.empty(q.shape, dtype=q.dtype, pin_memory=True)
+    hf = host.HostForward(B, 8, 8, n, 64, 32, n_groups=n_groups)
+    launches = sa.launch_count()
+    hf.forward(q, k, v, hlg, hy, seed=5, layer=2)
+    assert sa.launch_count() - launches == 1 + 2 * len(hf.pieces)
+    torch.cuda.synchronize()
+    perm, inv = sa.sa_make_perm(5, 2, B, n)
+    ref = sa.sa_swa_gated_forward(*dev, perm, inv, lg, 32)
+    assert sa.sa_read_status() == 0
     assert torch.equal(hy, ref.cpu())
