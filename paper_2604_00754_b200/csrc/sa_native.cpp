@@ -36,6 +36,16 @@ void check(int status, const char* where) {
   throw Raised{};
 }
 
+// The C call, with its arguments in hand, without the interpreter's lock: a launch waits for room
+// where the device's queue is full, and other threads go on meanwhile.
+template <typename... P, typename... A>
+int unlocked(sa_status (*call)(P...), A... args) {
+  PyThreadState* state = PyEval_SaveThread();
+  const int status = call(static_cast<P>(args)...);
+  PyEval_RestoreThread(state);
+  return status;
+}
+
 const at::Tensor& tensor(PyObject* o) {
   if (!THPVariable_Check(o)) raise(PyExc_TypeError, "expected a tensor");
   return THPVariable_Unpack(o);
@@ -167,7 +177,7 @@ PyObject* make_perm(PyObject* const* a) {
   at::Tensor own;
   const at::Tensor* ws = tensor_or_null(a[6]);
   if (!ws) ws = &(own = fresh({(int64_t)need}, at::kByte, dev));
-  check(sa_make_perm(integer_mask(a[0]), (uint32_t)integer(a[1]), p.B, p.n, (int32_t*)ptr(perm),
+  check(unlocked(sa_make_perm, integer_mask(a[0]), (uint32_t)integer(a[1]), p.B, p.n, (int32_t*)ptr(perm),
                      (int32_t*)ptr(inv), ptr(*ws), (size_t)ws->numel(), stream()),
         "sa_make_perm");
   return tuple({perm.result(), inv.result()});
@@ -183,7 +193,7 @@ PyObject* forward(PyObject* const* a) {
   const bool has_lse = a[10] != Py_None || truth(a[9]);
   Out lse;
   if (has_lse) lse = output(a[10], [&] { return rows_f32(q); });
-  check(sa_forward(&p, ptr(q), ptr(k), ptr(v), (const int32_t*)ptr(tensor(a[3])),
+  check(unlocked(sa_forward, &p, ptr(q), ptr(k), ptr(v), (const int32_t*)ptr(tensor(a[3])),
                    (const int32_t*)ptr(tensor(a[4])), ptr(y), has_lse ? (float*)ptr(lse) : nullptr,
                    nullptr, 0, stream()),
         "sa_forward");
@@ -209,7 +219,7 @@ PyObject* gated_forward(PyObject* const* a) {
   auto at_or_null = [](const Out& o) { return o.t || o.own.defined() ? ptr(o) : nullptr; };
   const sa_problem p = problem(q, k, a[6], flags, a[8]);
   const at::Tensor* ws = tensor_or_null(a[15]);
-  check(sa_swa_gated_forward(&p, ptr(q), ptr(k), ptr(v), (const int32_t*)ptr(tensor(a[3])),
+  check(unlocked(sa_swa_gated_forward, &p, ptr(q), ptr(k), ptr(v), (const int32_t*)ptr(tensor(a[3])),
                              (const int32_t*)ptr(tensor(a[4])), (const float*)ptr(tensor(a[5])),
                              ptr(y), at_or_null(branch[0]), at_or_null(branch[1]),
                              (float*)at_or_null(lse[0]), (float*)at_or_null(lse[1]), ptr(ws),
@@ -243,7 +253,7 @@ PyObject* backward(PyObject* const* a) {
   at::Tensor own;
   const at::Tensor* ws = tensor_or_null(a[14]);
   if (!ws) ws = &(own = fresh({(int64_t)ws_bytes(p, SA_OP_BACKWARD)}, at::kByte, q.device()));
-  check(sa_backward(&p, ptr(q), ptr(k), ptr(v), (const int32_t*)ptr(tensor(a[3])),
+  check(unlocked(sa_backward, &p, ptr(q), ptr(k), ptr(v), (const int32_t*)ptr(tensor(a[3])),
                     (const int32_t*)ptr(tensor(a[4])), (const float*)ptr(gate), ptr(y_sa),
                     ptr(y_swa), (const float*)ptr(tensor(a[8])), (const float*)ptr(lse_swa),
                     ptr(dy), ptr(dq), ptr(dk), ptr(dv), gate ? (float*)ptr(dgate) : nullptr,

@@ -39,3 +39,45 @@ def test_outputs_that_cannot_have_the_layout_are_refused(make, call):
         else:
             q, k = (odd, plain) if call == "backward_q" else (plain, odd)
             sa.sa_backward(q, k, k, perm, perm, lg, q, q, lse, lse, q, w)
+
+
+# A launch waits where the device's queue is full (behind a kernel that runs for half a second here):
+# the other threads of the interpreter go on meanwhile.
+@pytest.mark.gpu
+@pytest.mark.parametrize("call", ["make_perm", "forward", "gated", "backward"])
+def test_a_waiting_launch_does_not_stop_other_threads(call):
+    import threading
+    import time
+    q, y = (torch.zeros(1, 1, 64, 64, device="cuda").bfloat16() for _ in range(2))
+    perm, inv = sa.sa_make_perm(1, 0, 1, 64)
+    ws = torch.empty(1 << 20, dtype=torch.uint8, device="cuda")
+    lg, lse = torch.zeros(2, 1, device="cuda"), torch.zeros(1, 1, 64, device="cuda")
+    dgate = torch.empty_like(lg)
+    grads = dict(dq=torch.empty_like(q), dk=torch.empty_like(q), dv=torch.empty_like(q), dgate=dgate)
+    one = {"make_perm": lambda: sa.sa_make_perm(1, 0, 1, 64, perm=perm, inv=inv, ws=ws),
+           "forward": lambda: sa.sa_forward(q, q, q, perm, inv, 8, y=y),
+           "gated": lambda: sa.sa_swa_gated_forward(q, q, q, perm, inv, lg, 8, out=dict(y=y)),
+           "backward": lambda: sa.sa_backward(q, q, q, perm, inv, lg, y, y, lse, lse, q, 8, ws=ws,
+                                              out=grads)}[call]
+    one()
+    torch.cuda.synchronize()
+    took = []
+
+    def enqueue():
+        t0 = time.perf_counter()
+        for _ in range(3000):
+            one()
+        took.append(time.perf_counter() - t0)
+
+    torch.cuda._sleep(1000000000)
+    thread, gap = threading.Thread(target=enqueue), 0.0
+    last = time.perf_counter()
+    thread.start()
+    while thread.is_alive():
+        time.sleep(0.001)
+        now = time.perf_counter()
+        gap, last = max(gap, now - last), now
+    thread.join()
+    torch.cuda.synchronize()
+    assert sa.sa_read_status() == 0
+    assert took[0] > 0.3 and gap < 0.15, (took[0], gap)
