@@ -62,9 +62,16 @@ unsigned long long integer_mask(PyObject* o) {        // as int(o), modulo 2^64
   return v;
 }
 long long integer(PyObject* o) { return (long long)integer_mask(o); }
-double real(PyObject* o) {
-  const double v = PyFloat_AsDouble(o);
-  if (v == -1.0 && PyErr_Occurred()) throw Raised{};
+int64_t size(PyObject* o) {                           // a tensor's extent: whole numbers only
+  const Py_ssize_t v = PyNumber_AsSsize_t(o, PyExc_OverflowError);
+  if (v == -1 && PyErr_Occurred()) throw Raised{};
+  return v;
+}
+double real(PyObject* o) {                            // as float(o)
+  PyObject* f = PyFloat_CheckExact(o) ? o : PyNumber_Float(o);
+  if (!f) throw Raised{};
+  const double v = PyFloat_AS_DOUBLE(f);
+  if (f != o) Py_DECREF(f);
   return v;
 }
 bool truth(PyObject* o) {
@@ -165,7 +172,7 @@ at::Tensor rows_f32(const at::Tensor& q) {
 
 // make_perm(seed, layer, B, n, perm, inv, ws): perm or inv None: made on the current device
 PyObject* make_perm(PyObject* const* a) {
-  const int64_t B = integer(a[2]), n = integer(a[3]);
+  const int64_t B = size(a[2]), n = size(a[3]);
   const c10::Device dev = a[4] != Py_None ? tensor(a[4]).device()
                                           : c10::Device(c10::kCUDA, c10::cuda::current_device());
   auto make = [&] { return fresh({B, n}, at::kInt, dev); };

@@ -41,6 +41,25 @@ def test_outputs_that_cannot_have_the_layout_are_refused(make, call):
             sa.sa_backward(q, k, k, perm, perm, lg, q, q, lse, lse, q, w)
 
 
+# Numbers are taken as the Python calls took them: whole extents, and whatever float() takes.
+@pytest.mark.parametrize("B, n", [(2.0, 16), (2, 16.5), ("2", 16)])
+def test_extents_are_whole_numbers(B, n):
+    perm, ws = torch.zeros(2, 16, dtype=torch.int32), torch.zeros(1 << 16, dtype=torch.uint8)
+    with pytest.raises(TypeError):
+        sa.sa_make_perm(1, 0, B, n, perm=perm, inv=perm.clone(), ws=ws)
+
+
+@pytest.mark.gpu
+def test_scale_is_what_float_takes():
+    q = torch.randn(1, 1, 64, 64, device="cuda").bfloat16()
+    perm, inv = sa.sa_make_perm(1, 0, 1, 64)
+    want = sa.sa_forward(q, q, q, perm, inv, 8, scale=0.25)
+    for scale in ("0.25", torch.tensor(0.25), 1 / 4):
+        assert torch.equal(sa.sa_forward(q, q, q, perm, inv, 8, scale=scale), want)
+    with pytest.raises(TypeError):
+        sa.sa_forward(q, q, q, perm, inv, 8, scale=None)
+
+
 # A launch waits where the device's queue is full (behind a kernel that runs for half a second here):
 # the other threads of the interpreter go on meanwhile.
 @pytest.mark.gpu
