@@ -133,21 +133,35 @@ __global__ void __launch_bounds__(128) dgate_kernel(const BwdArgs a) {
 // the forward (sa_fwd_simt.cu).  Rows = queries: R = (Q, dY), columns (K, V), output dQ.  Rows =
 // keys: R = (K, V), columns (Q, dY) of every query head the CTA covers, outputs dK and dV.
 //
-// Small problems have too few row tiles for the SMs, so there each (branch, query head) gets CTAs
-// of its own, for both outputs in one launch, and writes a partial gradient that reduce_kernel
-// adds up in a fixed order ("split").  Large ones run one launch per branch, the second adding to
-// what the first stored, with the heads of a group inside the CTA.
+// Small problems have too few row tiles for the SMs, so there each branch, and with grouped heads each
+// of `parts` shares of a group's query heads, gets CTAs of its own, for all outputs in one launch, and
+// writes a partial gradient that reduce_kernel adds up in a fixed order ("split").  Large ones run one
+// launch per branch, the second adding to what the first stored, with the heads of a group inside the
+// CTA.
 //
 // Bound: FMA issue and shared-memory wavefronts, about equal, behind the latency of 32-column
 // steps, so warps per SM count: dS and P take turns in one buffer and the registers are held to 128
 // (d <= 64), for four CTAs per SM.  With that and packed multiply-adds in the products: 2 x 4/2 heads
 // of 64, n = 1500, w = 128, gated 157 -> 139 us; 8/4 heads of 128, n = 2000, w = 256 636 -> 572.
 
-// Split while the row tiles of the keys alone are fewer than eight per SM: beyond that they fill
-// the chip, and the partial gradients (six tensors of Q's size at most) would cost more than the
-// tail they save.
-bool split_tiles(int B, int Hkv, int n) {
-  return (int64_t)B * Hkv * ((n + kRows - 1) / kRows) < 8 * 148;
+// Split (number of parts of a group's query heads; 0: not split) while the row tiles of the keys are
+// fewer than eight per SM, in so many parts that they are not.  us, split / not: 2 x 4/2 heads of 64,
+// n = 1500 (1.3 per SM) 139 / 186; 32/8 heads of 128, n = 512 (0.9) 538 / 864, n = 2000 (3.4) 2151 / 2309;
+// 2 x 8 heads of 128, n = 1800 (6.2) 995 / 1048, n = 2000 (6.8) 685 / 717; 16 heads of 64, n = 2000 (6.8)
+// 332 / 337.
+// The partial gradients are two tensors of Q's size, and four of K's per part.  One part per query head
+// would make them six of Q's and be slower: 64/1 heads of 128, n = 8000 (eight parts for 64) 9834 / 10302
+// us, n = 16000 (four) 19547 / 20627; 64/8 heads, n = 4096 (two for eight) 5126 / 5304.
+// A constant for the SMs: the size of the workspace may not depend on the device that happens to be
+// current.
+constexpr int kPlanSms = 148;
+int split_parts(int B, int Hq, int Hkv, int n) {
+  const int64_t tiles = (int64_t)B * Hkv * ((n + kRows - 1) / kRows), enough = 8 * kPlanSms;
+  if (tiles >= enough) return 0;
+  const int G = Hq / Hkv;
+  for (int p = 1; p < G; ++p)
+    if (G % p == 0 && tiles * p >= enough) return p;
+  return G;
 }
 
 // Without SEEN nothing is stored and false returned where a sum of this CTA ended in a NaN: see
@@ -322,21 +336,13 @@ __device__ __forceinline__ bool bwd_tile(const BwdArgs& a, unsigned char* smem_r
   return true;
 }
 
-template <bool KEYS, int NCG>
-__device__ __noinline__ void bwd_tile_seen(const BwdArgs& a, unsigned char* smem_raw, int b, int x,
-                                           int hfirst, int heads, float* out1, float* out2, bool split) {
-  bwd_tile<KEYS, NCG, true>(a, smem_raw, b, x, hfirst, heads, out1, out2, split);
-}
-
-// blockIdx.y: first the nb * Hq (branch, head) pairs of dQ, then those of dK / dV, whose CTAs
-// cover `heads` query heads each.  Branches x0 .. x0 + nb - 1.
-template <int NCG>
-__global__ void __launch_bounds__(kTileThreads, NCG == 1 ? 4 : NCG == 2 ? 2 : 1)
-bwd_tile_kernel(const __grid_constant__ BwdArgs a, int x0, int nb, int heads, bool split) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  grid_dependency_wait();
-  grid_dependents_launch();
-  if (a.abort_flag && *a.abort_flag) return;
+// The tile of this CTA.  blockIdx.y: first the nb * Hq (branch, head) pairs of dQ, then those of dK /
+// dV, whose CTAs cover `heads` query heads of a group each.  Branches x0 .. x0 + nb - 1.  heads and the
+// place of dV's partials come as parameters: worked out here, they would take registers from the walk
+// (one head of 64, n = 700: 33.7 -> 35.9 us).
+template <int NCG, bool SEEN>
+__device__ __forceinline__ bool bwd_block(const BwdArgs& a, unsigned char* smem_raw, int x0, int nb,
+                                          int heads, bool split, size_t dv_at) {
   const int b = blockIdx.z, G = a.Hq / a.Hkv;
   const size_t rows_q = (size_t)a.B * a.Hq * a.n * a.d;
   int y = blockIdx.y;
@@ -344,24 +350,37 @@ bwd_tile_kernel(const __grid_constant__ BwdArgs a, int x0, int nb, int heads, bo
     const int hq = y % a.Hq, x = x0 + y / a.Hq;
     float* out = split ? a.parts + x * rows_q + ((size_t)b * a.Hq + hq) * a.n * a.d
                        : (float*)a.dq + b * a.qs[0] + hq * a.qs[1];
-    if (!bwd_tile<false, NCG, false>(a, smem_raw, b, x, hq, 1, out, nullptr, split))
-      bwd_tile_seen<false, NCG>(a, smem_raw, b, x, hq, 1, out, nullptr, split);
-  } else {
-    y -= nb * a.Hq;
-    const int groups = a.Hq / heads, h0 = (y % groups) * heads, x = x0 + y / groups, hk = h0 / G;
-    const int64_t off = b * a.ks[0] + hk * a.ks[1];
-    // partial (x, h0 % G): [B,Hkv,n,d] each; dK's first, dV's 2 * rows_q further on
-    float* part = a.parts + 2 * rows_q + (size_t)(x * G + h0 % G) * (rows_q / G) +
-                  ((size_t)b * a.Hkv + hk) * a.n * a.d;
-    float* dk = split ? part : (float*)a.dk + off;
-    float* dv = split ? part + 2 * rows_q : (float*)a.dv + off;
-    if (!bwd_tile<true, NCG, false>(a, smem_raw, b, x, h0, heads, dk, dv, split))
-      bwd_tile_seen<true, NCG>(a, smem_raw, b, x, h0, heads, dk, dv, split);
+    return bwd_tile<false, NCG, SEEN>(a, smem_raw, b, x, hq, 1, out, nullptr, split);
   }
+  y -= nb * a.Hq;
+  const int groups = a.Hq / heads, h0 = (y % groups) * heads, x = x0 + y / groups, hk = h0 / G;
+  const int64_t off = b * a.ks[0] + hk * a.ks[1];
+  // partial (x, part of the group): [B,Hkv,n,d] each; dK's first, dV's dv_at further on
+  float* part = a.parts + 2 * rows_q + (size_t)((x * G + h0 % G) / heads) * (rows_q / G) +
+                ((size_t)b * a.Hkv + hk) * a.n * a.d;
+  return bwd_tile<true, NCG, SEEN>(a, smem_raw, b, x, h0, heads, split ? part : (float*)a.dk + off,
+                                   split ? part + dv_at : (float*)a.dv + off, split);
+}
+
+template <int NCG>
+__global__ void __launch_bounds__(kTileThreads, NCG == 1 ? 4 : NCG == 2 ? 2 : 1)
+bwd_tile_kernel(const __grid_constant__ BwdArgs a, int x0, int nb, int heads, bool split, size_t dv_at) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  unsigned char* smem = smem_raw;
+  grid_dependency_wait();
+  grid_dependents_launch();
+  if (a.abort_flag && *a.abort_flag) return;
+  if (bwd_block<NCG, false>(a, smem, x0, nb, heads, split, dv_at)) return;
+  // Nothing of the first walk is to be kept in registers for this one.  Measured on 1 x 1 head of 64,
+  // n = 700 / 2 x 4/2 heads of 64, n = 1500 / 8/2 heads of 128, n = 1000, us: without it 33.6 / 138.4 /
+  // 128.6, like this 33.9 / 137.1 / 130.6, with the second walk as a function 36.3 / 140.4 / 133.6, as
+  // another turn of the first 36.1 / 139.0 / 131.4.
+  asm volatile("" : "+r"(x0), "+r"(nb), "+r"(heads), "+l"(smem));
+  bwd_block<NCG, true>(a, smem, x0, nb, heads, split, dv_at);
 }
 
 // dq, dk, dv from the partial gradients of the split form, 16 bytes per thread.
-__global__ void __launch_bounds__(256) reduce_kernel(const BwdArgs a) {
+__global__ void __launch_bounds__(256) reduce_kernel(const BwdArgs a, int parts) {
   const int G = a.Hq / a.Hkv, q4 = a.d / 4;
   const size_t nq = (size_t)a.B * a.Hq * a.n * q4, nk = nq / G;
   size_t i = (size_t)blockIdx.x * 256 + threadIdx.x;
@@ -371,9 +390,9 @@ __global__ void __launch_bounds__(256) reduce_kernel(const BwdArgs a) {
   const int which = i < nq ? 0 : (i < nq + nk ? 1 : 2);
   i -= which == 0 ? 0 : (which == 1 ? nq : nq + nk);
   const float4* p = reinterpret_cast<const float4*>(a.parts) +
-                    (which == 0 ? i : 2 * nq * which + i);
+                    (which == 0 ? i : 2 * nq + (which - 1) * 2 * parts * nk + i);
   const size_t step = which ? nk : nq;
-  const int terms = which ? a.nbranch * G : a.nbranch;
+  const int terms = which ? a.nbranch * parts : a.nbranch;
   float4 s = p[0];
   for (int t = 1; t < terms; ++t) {
     const float4 v = p[t * step];
@@ -394,17 +413,19 @@ cudaError_t launch_tiles(const BwdArgs& a, cudaStream_t st) {
   cudaError_t e = allow_smem((const void*)bwd_tile_kernel<NCG>, smem);
   if (e != cudaSuccess) return e;
   const unsigned tiles = (a.n + kRows - 1) / kRows;
-  if (split_tiles(a.B, a.Hkv, a.n)) {
-    e = launch_dependent(bwd_tile_kernel<NCG>, dim3(tiles, 2 * a.Hq * a.nbranch, a.B),
-                         dim3(kTileThreads), smem, st, a, 0, a.nbranch, 1, true);
+  const int G = a.Hq / a.Hkv;
+  if (const int parts = split_parts(a.B, a.Hq, a.Hkv, a.n)) {
+    e = launch_dependent(bwd_tile_kernel<NCG>, dim3(tiles, a.nbranch * (a.Hq + a.Hkv * parts), a.B),
+                         dim3(kTileThreads), smem, st, a, 0, a.nbranch, G / parts, true,
+                         (size_t)2 * parts * a.B * a.Hkv * a.n * a.d);
     if (e != cudaSuccess) return e;
     const size_t items = ((size_t)a.Hq + 2 * a.Hkv) * a.B * a.n * (a.d / 4);
     bump_launches(2);
-    return launch_dependent(reduce_kernel, dim3((unsigned)((items + 255) / 256)), dim3(256), 0, st, a);
+    return launch_dependent(reduce_kernel, dim3((unsigned)((items + 255) / 256)), dim3(256), 0, st, a, parts);
   }
   for (int x = 0; x < a.nbranch && e == cudaSuccess; ++x) {
     e = launch_dependent(bwd_tile_kernel<NCG>, dim3(tiles, a.Hq + a.Hkv, a.B), dim3(kTileThreads),
-                         smem, st, a, x, 1, a.Hq / a.Hkv, false);
+                         smem, st, a, x, 1, G, false, (size_t)0);
     bump_launches();
   }
   return e;
@@ -607,7 +628,9 @@ size_t bwd_ws_bytes(int B, int Hq, int Hkv, int n, int d, int w, int dtype, int*
   size_t bytes = align_up((size_t)2 * B * Hq * n * sizeof(float), 256) +
                  align_up((size_t)2 * B * Hq * chunks * sizeof(float), 256);
   if (parts_at) *parts_at = bytes;
-  if (dtype == SA_F32 && split_tiles(B, Hkv, n)) bytes += (size_t)6 * B * Hq * n * d * sizeof(float);
+  if (dtype == SA_F32)
+    if (const int parts = split_parts(B, Hq, Hkv, n))
+      bytes += ((size_t)2 * Hq + (size_t)4 * Hkv * parts) * B * n * d * sizeof(float);
   if (dtype == SA_BF16) {      // room for either way: the tensor cores' kernels carve their own
     const size_t tc = tc_backward_ws_bytes(B, Hq, Hkv, n, d, w);
     bytes = tc > bytes ? tc : bytes;

@@ -21,6 +21,8 @@ pytestmark = pytest.mark.gpu
     (1, 4, 2, 129, 136, 128, CAUSAL | LINEAR_WINDOW),
     (1, 2, 1, 65, 256, 64, CAUSAL | SWA_ONE_SIDED),
     (8, 8, 4, 1185, 16, 3, CAUSAL | SWA_ONE_SIDED),     # 32 * 38 key tiles: not split
+    (1, 8, 1, 9473, 8, 9, CAUSAL | SWA_ONE_SIDED),      # 297: a group's heads in four parts
+    (1, 6, 1, 12641, 8, 7, 0),                          # 396: in three
 ])
 def test_fp32_tiles(B, Hq, Hkv, n, d, w, flags):
     g = torch.Generator().manual_seed(n + d)

@@ -46,6 +46,16 @@ def test_contiguous_strides_and_workspace_sizes():
         sa.sa_workspace_bytes(p, 99)
 
 
+# The partial gradients of the fp32 backward: two tensors of Q's size and four of K's per part of a
+# group's heads, in no more parts than fill the GPU; none where the keys' rows alone fill it.
+@pytest.mark.parametrize("Hq,Hkv,n,most", [(64, 1, 38000, 0), (64, 1, 16000, 2.3), (64, 1, 2000, 4.0),
+                                           (4, 2, 1500, 6), (12, 12, 500, 6)])
+def test_backward_workspace_fp32(Hq, Hkv, n, most):
+    p = problem(B=1, Hq=Hq, Hkv=Hkv, n=n, d=128, w=128, dtype=sa.F32)
+    rows = 2 * Hq * n * 4 + 2 * Hq * ((n + 63) // 64) * 4 + 1024      # Delta and its partial sums
+    assert sa.sa_workspace_bytes(p, sa.OP_BACKWARD) <= rows + most * Hq * n * 128 * 4
+
+
 FAKE = ctypes.c_void_p(0x1000)      # aligned, never dereferenced: every case fails before a launch
 ODD = ctypes.c_void_p(0x1004)
 
