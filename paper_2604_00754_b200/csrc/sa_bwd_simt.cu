@@ -336,16 +336,16 @@ __device__ __forceinline__ bool bwd_tile(const BwdArgs& a, unsigned char* smem_r
   return true;
 }
 
-// The tile of this CTA.  blockIdx.y: first the nb * Hq (branch, head) pairs of dQ, then those of dK /
+// The tile of this CTA.  y0 + blockIdx.y: first the nb * Hq (branch, head) pairs of dQ, then those of dK /
 // dV, whose CTAs cover `heads` query heads of a group each.  Branches x0 .. x0 + nb - 1.  heads and the
 // place of dV's partials come as parameters: worked out here, they would take registers from the walk
 // (one head of 64, n = 700: 33.7 -> 35.9 us).
 template <int NCG, bool SEEN>
-__device__ __forceinline__ bool bwd_block(const BwdArgs& a, unsigned char* smem_raw, int x0, int nb,
-                                          int heads, bool split, size_t dv_at) {
+__device__ __forceinline__ bool bwd_block(const BwdArgs& a, unsigned char* smem_raw, int y0, int x0,
+                                          int nb, int heads, bool split, size_t dv_at) {
   const int b = blockIdx.z, G = a.Hq / a.Hkv;
   const size_t rows_q = (size_t)a.B * a.Hq * a.n * a.d;
-  int y = blockIdx.y;
+  int y = y0 + blockIdx.y;
   if (y < nb * a.Hq) {
     const int hq = y % a.Hq, x = x0 + y / a.Hq;
     float* out = split ? a.parts + x * rows_q + ((size_t)b * a.Hq + hq) * a.n * a.d
@@ -364,19 +364,20 @@ __device__ __forceinline__ bool bwd_block(const BwdArgs& a, unsigned char* smem_
 
 template <int NCG>
 __global__ void __launch_bounds__(kTileThreads, NCG == 1 ? 4 : NCG == 2 ? 2 : 1)
-bwd_tile_kernel(const __grid_constant__ BwdArgs a, int x0, int nb, int heads, bool split, size_t dv_at) {
+bwd_tile_kernel(const __grid_constant__ BwdArgs a, int y0, int x0, int nb, int heads, bool split,
+                size_t dv_at) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   unsigned char* smem = smem_raw;
   grid_dependency_wait();
   grid_dependents_launch();
   if (a.abort_flag && *a.abort_flag) return;
-  if (bwd_block<NCG, false>(a, smem, x0, nb, heads, split, dv_at)) return;
+  if (bwd_block<NCG, false>(a, smem, y0, x0, nb, heads, split, dv_at)) return;
   // Nothing of the first walk is to be kept in registers for this one.  Measured on 1 x 1 head of 64,
   // n = 700 / 2 x 4/2 heads of 64, n = 1500 / 8/2 heads of 128, n = 1000, us: without it 33.6 / 138.4 /
   // 128.6, like this 33.9 / 137.1 / 130.6, with the second walk as a function 36.3 / 140.4 / 133.6, as
   // another turn of the first 36.1 / 139.0 / 131.4.
   asm volatile("" : "+r"(x0), "+r"(nb), "+r"(heads), "+l"(smem));
-  bwd_block<NCG, true>(a, smem, x0, nb, heads, split, dv_at);
+  bwd_block<NCG, true>(a, smem, y0, x0, nb, heads, split, dv_at);
 }
 
 // dq, dk, dv from the partial gradients of the split form, 16 bytes per thread.
@@ -413,21 +414,24 @@ cudaError_t launch_tiles(const BwdArgs& a, cudaStream_t st) {
   cudaError_t e = allow_smem((const void*)bwd_tile_kernel<NCG>, smem);
   if (e != cudaSuccess) return e;
   const unsigned tiles = (a.n + kRows - 1) / kRows;
-  const int G = a.Hq / a.Hkv;
-  if (const int parts = split_parts(a.B, a.Hq, a.Hkv, a.n)) {
-    e = launch_dependent(bwd_tile_kernel<NCG>, dim3(tiles, a.nbranch * (a.Hq + a.Hkv * parts), a.B),
-                         dim3(kTileThreads), smem, st, a, 0, a.nbranch, G / parts, true,
-                         (size_t)2 * parts * a.B * a.Hkv * a.n * a.d);
+  const int G = a.Hq / a.Hkv, parts = split_parts(a.B, a.Hq, a.Hkv, a.n);
+  // `blocks` of the grid's second dimension, in launches of as many as it can have
+  auto walk = [&](int x0, int nb, int heads, bool split, size_t dv_at) {
+    const int blocks = nb * (a.Hq + a.Hq / heads), most = 65535;
+    for (int y0 = 0; y0 < blocks && e == cudaSuccess; y0 += most) {
+      e = launch_dependent(bwd_tile_kernel<NCG>, dim3(tiles, min(blocks - y0, most), a.B),
+                           dim3(kTileThreads), smem, st, a, y0, x0, nb, heads, split, dv_at);
+      bump_launches();
+    }
+  };
+  if (parts) {
+    walk(0, a.nbranch, G / parts, true, (size_t)2 * parts * a.B * a.Hkv * a.n * a.d);
     if (e != cudaSuccess) return e;
     const size_t items = ((size_t)a.Hq + 2 * a.Hkv) * a.B * a.n * (a.d / 4);
-    bump_launches(2);
+    bump_launches();
     return launch_dependent(reduce_kernel, dim3((unsigned)((items + 255) / 256)), dim3(256), 0, st, a, parts);
   }
-  for (int x = 0; x < a.nbranch && e == cudaSuccess; ++x) {
-    e = launch_dependent(bwd_tile_kernel<NCG>, dim3(tiles, a.Hq + a.Hkv, a.B), dim3(kTileThreads),
-                         smem, st, a, x, 1, G, false, (size_t)0);
-    bump_launches();
-  }
+  for (int x = 0; x < a.nbranch && e == cudaSuccess; ++x) walk(x, 1, G, false, 0);
   return e;
 }
 

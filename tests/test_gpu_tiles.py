@@ -46,6 +46,24 @@ def test_fp32_tiles(B, Hq, Hkv, n, d, w, flags):
     assert sa.sa_read_status() == 0
 
 
+# More (branch, head) pairs than a grid's second dimension has: split (two parts per group, 84000) and
+# not (80000 per branch)
+@pytest.mark.parametrize("Hq,Hkv,n", [(40000, 1000, 32), (40000, 40000, 8)])
+def test_fp32_backward_of_many_heads(Hq, Hkv, n):
+    g = torch.Generator().manual_seed(n)
+    mk = lambda h: torch.randn(1, h, n, 8, generator=g)
+    q, k, v, dy = mk(Hq), mk(Hkv), mk(Hkv), mk(Hq)
+    lg, w, flags = torch.randn(2, Hq, generator=g), 5, CAUSAL | SWA_ONE_SIDED
+    perm, inv = sa.sa_make_perm(n, 3, 1, n)
+    dev = [t.cuda() for t in (q, k, v)]
+    out = sa.sa_swa_gated_forward(*dev, perm, inv, lg.cuda(), w, flags, save_for_bwd=True)
+    grads = sa.sa_backward(*dev, perm, inv, lg.cuda(), *out[1:], dy.cuda(), w, flags)
+    assert sa.sa_read_status() == 0
+    args = [as_f64(t) for t in (q, k, v)] + [perm.cpu().numpy(), inv.cpu().numpy(), lg.double().numpy()]
+    for got, want in zip(grads, oracle.backward(*args, as_f64(dy), w, flags)):
+        assert np.abs(as_f64(got) - want).max() <= 1e-4 * max(1.0, np.abs(want).max())
+
+
 # An infinity or a NaN reaches the rows and columns that its token meets and no others, although the
 # tiles hold pairs that do not see each other.  Finite where the oracle is, to the tolerances above
 # (bf16: 2e-2 of the largest finite value); the rest is not finite.
