@@ -381,7 +381,8 @@ sa_status sa_coverage(int32_t L, int32_t n, int32_t w, uint32_t flags, const int
 }
 
 sa_status sa_read_status(sa_stream_t stream) {
-  if (cudaStreamSynchronize((cudaStream_t)stream) != cudaSuccess) return SA_ERR_CUDA;
+  const cudaError_t e = cudaStreamSynchronize((cudaStream_t)stream);
+  if (e != cudaSuccess) return from_cuda(reported(e));
   int* p = status_ptr();
   if (!p) return SA_ERR_CUDA;
   int host = 0;

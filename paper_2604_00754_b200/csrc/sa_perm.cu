@@ -409,7 +409,7 @@ cudaError_t launch_make_perm(uint64_t seed, uint32_t layer, int B, int n, int32_
     const cudaError_t e =
         cudaLaunchKernelEx(&cfg, perm_cluster_kernel, (uint32_t)seed, (uint32_t)(seed >> 32), layer,
                            n, c.log2_c, c.bits, c.cap, perm, inv);
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess) return reported(e);
     bump_launches();
     return cudaGetLastError();
   }

@@ -100,3 +100,40 @@ def test_a_waiting_launch_does_not_stop_other_threads(call):
     torch.cuda.synchronize()
     assert sa.sa_read_status() == 0
     assert took[0] > 0.3 and gap < 0.15, (took[0], gap)
+
+
+# A launch that fails (here into a graph capture that a synchronisation has spoiled) is told by its own
+# call and not once more by the next one.  In a process of its own: torch keeps the spoiled capture.
+SPOILED = """
+import sys, torch
+sys.path.insert(0, sys.argv[1])
+from paper_2604_00754_b200 import binding as sa
+lib = sa.load_library()
+t = [torch.empty(64, dtype=torch.int32, device="cuda") for _ in range(2)]
+ws = torch.empty(1 << 16, dtype=torch.uint8, device="cuda")
+draw = lambda s: lib.sa_make_perm(1, 0, 1, 64, t[0].data_ptr(), t[1].data_ptr(), ws.data_ptr(),
+                                  ws.numel(), s.cuda_stream)
+side, main = torch.cuda.Stream(), torch.cuda.current_stream()
+assert draw(main) == 0
+torch.cuda.synchronize()
+with torch.cuda.stream(side):
+    graph = torch.cuda.CUDAGraph()
+    graph.capture_begin()
+    codes = [lib.sa_read_status(side.cuda_stream), draw(side)]
+    try:
+        graph.capture_end()
+    except RuntimeError:
+        pass
+codes.append(draw(main))
+print(codes, lib.sa_read_status(main.cuda_stream))
+"""
+
+
+@pytest.mark.gpu
+def test_a_failed_launch_is_told_once():
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    out = subprocess.run([sys.executable, "-c", SPOILED, root], capture_output=True, text=True, timeout=300)
+    assert out.stdout.strip().endswith("[4, 4, 0] 0"), out.stdout + out.stderr
