@@ -94,11 +94,18 @@ def test_what_the_heads_alone_refuse_stays_refused():
         sab.host_forward_pieces(0, 8, 4, 64, 64)
 
 
+# Input enough for the pieces asked for (2 MB each): two sequences, then ranges of their heads; heads
+# alone; and the first and last KV head cut by query heads, whose later part finds K and V on the GPU
+# (half of 8 heads' 75 row tiles each still fill it).
 @pytest.mark.gpu
-@pytest.mark.parametrize("n_groups,q_parts", [(1, 1), (3, 2), (4, 2), (4, 1)])
-def test_pipelined_forward_equals_single_call(n_groups, q_parts):
+@pytest.mark.parametrize("B,Hq,Hkv,n,n_groups,q_parts,pieces", [
+    (2, 8, 4, 2100, 1, 1, 1), (2, 8, 4, 2100, 3, 2, 2), (2, 8, 4, 2100, 4, 2, 4), (2, 8, 4, 2100, 4, 1, 4),
+    (1, 8, 4, 4200, 3, 2, 3), (1, 8, 4, 4200, 4, 1, 4),
+    (1, 8, 1, 9600, 1, 2, 2), (1, 16, 2, 9600, 2, 2, 4), (1, 8, 1, 9600, 1, 4, 1),
+])
+def test_pipelined_forward_equals_single_call(B, Hq, Hkv, n, n_groups, q_parts, pieces):
     from paper_2604_00754_b200 import binding as sa
-    B, Hq, Hkv, n, d, w = 2, 8, 4, 1000, 64, 256
+    d, w = 64, 256
     g = torch.Generator().manual_seed(11)
     q = torch.randn(B, Hq, n, d, generator=g).bfloat16().pin_memory()
     k = torch.randn(B, Hkv, n, d, generator=g).bfloat16().pin_memory()
@@ -106,21 +113,17 @@ def test_pipelined_forward_equals_single_call(n_groups, q_parts):
     lg = torch.randn(2, Hq, generator=g).pin_memory()
     hy = torch.empty_like(q).pin_memory()
     hf = host.HostForward(B, Hq, Hkv, n, d, w, n_groups=n_groups, q_parts=q_parts)
-    hf.forward(q, k, v, lg, hy, seed=5, layer=2)
-    torch.cuda.synchronize()
-    perm, inv = sa.sa_make_perm(5, 2, B, n)
-    # the pipeline hands the library scratch, so its gates are applied by the idle-warp
-    # kernel: the single call does the same (the fused epilogue rounds differently)
-    scratch = torch.empty(hy.numel() * hy.element_size(), dtype=torch.uint8, device="cuda")
-    ref = sa.sa_swa_gated_forward(q.cuda(), k.cuda(), v.cuda(), perm, inv, lg.cuda(), w, ws=scratch)
-    assert sa.sa_read_status() == 0
-    assert torch.equal(hy, ref.cpu())
-    # a second call with another layer index draws another permutation
-    hf.forward(q, k, v, lg, hy, seed=5, layer=3)
-    torch.cuda.synchronize()
-    perm, inv = sa.sa_make_perm(5, 3, B, n)
-    ref = sa.sa_swa_gated_forward(q.cuda(), k.cuda(), v.cuda(), perm, inv, lg.cuda(), w, ws=scratch)
-    assert torch.equal(hy, ref.cpu())
+    assert len(hf.pieces) == pieces
+    dev = [t.cuda() for t in (q, k, v)]
+    for layer in (2, 3):                   # another layer index draws another permutation
+        launches = sa.launch_count()
+        hf.forward(q, k, v, lg, hy, seed=5, layer=layer)
+        assert sa.launch_count() - launches == 1 + 2 * pieces
+        torch.cuda.synchronize()
+        perm, inv = sa.sa_make_perm(5, layer, B, n)
+        ref = sa.sa_swa_gated_forward(*dev, perm, inv, lg.cuda(), w)
+        assert sa.sa_read_status() == 0
+        assert torch.equal(hy, ref.cpu())
 
 
 # more groups than events, and none: two launches per piece and one for the permutation
