@@ -188,9 +188,6 @@ def main():
     ap.add_argument("--score-block", type=int, default=0, choices=[0, 64, 128],
                     help="force the score-block width of the tensor-core kernels (test hook of "
                          "the library; 0 = the library's own choice)")
-    ap.add_argument("--gated-form", default="warps", choices=["warps", "epilogue"],
-                    help="warps: the call is given scratch (accepted and not used); epilogue: none. "
-                         "The gates are applied in the local branch's epilogue either way")
     ap.add_argument("--no-extras", action="store_true",
                     help="skip the side measurements (SWA, backward, e2e, CPU oracle)")
     args = ap.parse_args()
@@ -231,10 +228,6 @@ def main():
     prob = sa.SaProblem(B=c.B, n=c.n)
     ws = torch.empty(sa.sa_workspace_bytes(prob, sa.OP_MAKE_PERM), dtype=torch.uint8, device="cuda")
     out = {"y": y}
-    # scratch for the SA branch's rows: the local branch's launch then combines with its idle warps
-    gws = torch.empty(sa.sa_workspace_bytes(sa.make_problem(q, k, c.w, c.flags),
-                                            sa.OP_GATED_FORWARD_SCRATCH),
-                      dtype=torch.uint8, device="cuda")
     torch.cuda.synchronize()
 
     if args.leg == "backward":
@@ -255,8 +248,7 @@ def main():
 
     def step():
         sa.sa_make_perm(cr.seed, layer[0], c.B, c.n, perm=perm, inv=inv, ws=ws)
-        sa.sa_swa_gated_forward(q, k, v, perm, inv, lg, c.w, c.flags, out=out,
-                                ws=gws if args.gated_form == "warps" else None)
+        sa.sa_swa_gated_forward(q, k, v, perm, inv, lg, c.w, c.flags, out=out)
         layer[0] += 1
 
     def barrier():
@@ -302,11 +294,11 @@ def main():
     flops_branch = 4.0 * c.B * c.Hq * c.n * c.w * c.d
     achieved = flops_branch / (sa_kernel_ms * 1e-3) / 1e12
     # DRAM bytes of one SA-branch launch: dram__bytes_read.sum + dram__bytes_write.sum of one ncu
-    # capture of this kernel on this shape at n = 8192 (100.9 MB + 26.5 MB; the counter summary
+    # capture of this kernel on this shape at n = 8192 (100.8 MB + 33.1 MB; the counter summary
     # is under profiles/), scaled by n because every tensor grows in proportion to it.
     traffic = None
     if (c.B, c.Hq, c.Hkv, c.d, c.w) == (1, 32, 8, 128, 1024):
-        traffic = 127443200.0 * c.n / 8192
+        traffic = 133836288.0 * c.n / 8192
     sustained = args.steps * ms_per_step > 1500.0
     peak = pk["bf16_tflops_sustained"] if sustained else pk["bf16_tflops"]
     line = {
