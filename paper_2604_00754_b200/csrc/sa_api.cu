@@ -214,9 +214,9 @@ sa_status sa_swa_gated_forward(const sa_problem* p, const void* q, const void* k
   if ((s = maybe_validate(p, perm, inv, st)) != SA_OK) return s;
   // Two launches.  The SA branch first: its ungated rows land in y_sa, else in y itself.  The
   // local branch then owns each output row exactly once: its epilogue reads the matching SA row
-  // (the tensor-core kernel in coalesced pieces), applies both gates and writes y.  (Reading the
-  // scattered rows of the local branch from the SA branch's epilogue, the other possible order,
-  // costs more than a third launch would.)
+  // (the tensor-core kernel in coalesced pieces), applies both gates and writes y.  (In the other order
+  // the rows of the local branch would be read scattered from the SA branch's epilogue, and that branch
+  // could not start before the local one is complete.)
   (void)ws_bytes;
   void* sa_rows = y_sa ? y_sa : y;
   FwdArgs a = fwd_args(p, q, k, v, false);

@@ -36,9 +36,9 @@
 //
 // Bound: the tensor pipe (128-cycle-per-16-columns products in four groups, and ~180 cycles per
 // commit) where windows are wide, HBM and the item's fixed latencies where they are narrow.
-// Measured against the gathering, one-item-per-CTA kernels before (whole gated backward):
-// 32/8 heads of 128, n = 10007, w = 1024: 2166 -> 1664 us; 8 x 12 heads of 64, n = 4096, w = 128:
-// 687 -> 561 us; SA alone, 16 x 16 heads of 64, n = 2048, w = 256: 810 -> 491 us.
+// Whole backward, us, gathering kernels with one item per CTA before / now: 32/8 heads of 128, n = 10007,
+// w = 1024, gated 2166 / 1440; 8 x 12 heads of 64, n = 4096, w = 128, gated 687 / 515; SA alone, 16 x 16
+// heads of 64, n = 2048, w = 256 810 / 479.
 //
 // Every mbarrier wait is bounded; on expiry the CTA records SA_ERR_TIMEOUT in the device status
 // word, stops issuing work, drains what it started and returns.

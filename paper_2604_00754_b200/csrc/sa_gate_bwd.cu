@@ -32,9 +32,9 @@ template <int MODE> struct Epi {
   static constexpr int kTiles = kIn == 2 ? 2 : 1;                // per half
   static constexpr int kRingBytes = (kIn == 2 ? 9 : 12) * kATileBytes;
 };
-// TN: columns of the output tile.  256 halves the operand bytes per flop of the B side and is
-// used when it still leaves at least one tile per SM; 128 otherwise.  A stage is one K chunk of
-// A + B, 48 or 32 KB.
+// TN: columns of the output tile.  256 halves the operand bytes per flop of the B side; which of the
+// two a product takes is decided by forward_wide, wide_waves and plan_dw below.  A stage is one K chunk
+// of A + B, 48 or 32 KB.
 template <int MODE, int TN> struct Tile {
   static constexpr int kBTileBytes = TN * kBK * 2;
   static constexpr int kStageBytes = kATileBytes + kBTileBytes;
@@ -494,8 +494,8 @@ DwPlan plan_dw(int64_t rows, int dm, int sms) {
 }  // namespace
 
 // Forward of one or two paths with 128 x 256 tiles, one launch per path (the second adds to
-// the first's rounded result); false when the product is too small for wide tiles to fill
-// the GPU, and the caller's fused kernel should run instead.
+// the first's rounded result); false where forward_wide says so, and the caller's fused kernel
+// should run instead.
 bool gate_forward_wide(int64_t rows, int dm, const void* y_sa, const void* y_swa, int64_t ld_y,
                        const void* w_sa, const void* w_swa, void* out, int64_t ld_out,
                        int* status, int sms, cudaStream_t st, cudaError_t* err) {
@@ -563,8 +563,10 @@ extern "C" sa_status sa_gate_projection_backward(
       __nv_bfloat16* dz = (__nv_bfloat16*)ws;
       __nv_bfloat16* dyd = dz + rows * (int64_t)dm;
       float* part = (float*)(dyd + rows * (int64_t)dm);
-      // (with a long contraction the narrow tiles' operand stream counts for more: 2500 x 2048, two
-      // rounds of wide tiles against three, 92 -> 84 us; but 12000 x 512 49 -> 52)
+      // (With a long contraction the narrow tiles' operand stream counts for more.  Both widths at 67
+      // sizes, 300 ... 20000 rows x 512 ... 4096: the one taken is the faster at all but four, where they
+      // are within 4 %.  The lines between: 8000 x 768 57.7 us wide / 55.6, 12000 x 512 51.1 / 47.0, but
+      // 5000 x 1024 61.5 / 63.3, 2500 x 2048 85.0 / 92.8, 1500 x 4096 175 / 179.)
       const bool wide = wide_waves(rows, dm, sms, dm >= 1024 ? 350 : 300);
       const DwPlan dwp = plan_dw(rows, dm, sms);
       CUtensorMap y_k, w_k, dz_k, w_mn, dz_mn, y_mn, dout_k, dyd_k, dy_k, dw_o;

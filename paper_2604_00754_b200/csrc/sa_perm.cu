@@ -146,9 +146,10 @@ __global__ void rank_kernel(const uint64_t* __restrict__ bkeys, const int32_t* _
 // its share of the tokens (in registers), sends every (key, token) to its owner's shared memory
 // (places reserved with one remote atomic per CTA pair), and the owner sorts what arrived into
 // buckets and ranks it there.  Bound: latency (launch, two cluster barriers, a handful of block
-// barriers).  Measured back to back (one launch against the four and a memset): n = 256 2.8
-// against 12.4 us, n = 4096 x 8 sequences 7.7 against 13.0, n = 8192 10.1 against 15.2, n = 16384
-// 14.0 against 16.5 (with eight CTAs of 4096 tokens, n = 32768: 22.0 against 16.1).
+// barriers).  Back to back, before launches started under one another (one launch against the four and
+// a memset): n = 256 2.8 against 12.4 us, n = 4096 x 8 sequences 7.7 against 13.0, n = 8192 10.1 against
+// 15.2, n = 16384 14.0 against 16.5 (with eight CTAs of 4096 tokens, n = 32768: 22.0 against 16.1).  Now,
+// overlapping: n = 8192 3.3, n = 16384 4.4, and the four launches at n = 32768 18.4.
 // An owner has room for cap entries; its expected share is n / C with a standard deviation
 // below sqrt(n / C), and cap leaves 10 of those (an eighth of the share, 3 of them at 512 tokens,
 // was passed by one call in twelve with 8 sequences of 4096, at 760 us instead of 8).  If a share is larger all the same, every CTA
