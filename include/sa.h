@@ -77,7 +77,8 @@ typedef enum {
   SA_OP_BACKWARD = 4,
   SA_OP_COVERAGE = 5,
   SA_OP_GATED_FORWARD_SCRATCH = 6, /* accepted by sa_swa_gated_forward, see there           */
-  SA_OP_FORWARD_ROPE = 7           /* sa_forward_rope / sa_swa_gated_forward_rope           */
+  SA_OP_FORWARD_ROPE = 7,          /* sa_forward_rope / sa_swa_gated_forward_rope           */
+  SA_OP_KEY_LISTS = 8              /* sa_forward_lists / sa_swa_gated_forward_lists         */
 } sa_op;
 
 typedef struct {
@@ -159,6 +160,20 @@ sa_status sa_swa_gated_forward(const sa_problem* p, const void* q, const void* k
                                const float* gate_logits, void* y, void* y_sa, void* y_swa,
                                float* lse_sa, float* lse_swa, void* ws, size_t ws_bytes,
                                sa_stream_t stream);
+
+/* sa_forward and sa_swa_gated_forward with scratch of sa_workspace_bytes(.., SA_OP_KEY_LISTS) bytes (0
+ * for problems that have no use for it; 16-byte aligned; with less, or NULL, they are the calls above).
+ * Causal bf16 problems with wide windows then walk their keys in token order: one launch more, which
+ * writes per 256 or 512 slots the tokens of their window in order and per query tile and 128 keys what
+ * each row sees, and an SA branch that passes over most of what causality hides.  Same result up to
+ * the order of summation. */
+sa_status sa_forward_lists(const sa_problem* p, const void* q, const void* k, const void* v,
+                           const int32_t* perm, const int32_t* inv, void* y, float* lse, void* ws,
+                           size_t ws_bytes, sa_stream_t stream);
+sa_status sa_swa_gated_forward_lists(const sa_problem* p, const void* q, const void* k, const void* v,
+                                     const int32_t* perm, const int32_t* inv, const float* gate_logits,
+                                     void* y, void* y_sa, void* y_swa, float* lse_sa, float* lse_swa,
+                                     void* ws, size_t ws_bytes, sa_stream_t stream);
 
 /* sa_make_perm + sa_swa_gated_forward (Alg. 1 line 1, Alg. 2, Eq. 5) for tensors that live in
  * HOST memory: q, k, v, y are host pointers to contiguous [B,H,n,d] tensors of p->dtype

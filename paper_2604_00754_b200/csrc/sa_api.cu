@@ -98,8 +98,12 @@ FwdArgs fwd_args(const sa_problem* p, const void* q, const void* k, const void* 
 cudaError_t run_forward(const FwdArgs& a, int dtype, cudaStream_t st) {
   const bool prof = !a.swa && g_prof_start && g_prof_stop;
   if (prof) cudaEventRecord(g_prof_start, st);
-  const cudaError_t e = tc_forward_supported(a, dtype) ? launch_fwd_tc(a, st)
-                                                       : launch_fwd_simt(a, dtype, st);
+  OrderGeom g;
+  cudaError_t e = cudaSuccess;
+  if (a.lists && !a.lists_ready && tc_forward_ordered(a, dtype, &g))
+    e = launch_order(a.perm, a.B, a.n, a.w, a.flags, g, order_view(a.lists, a.B, g), a.abort_flag, st);
+  if (e == cudaSuccess)
+    e = tc_forward_supported(a, dtype) ? launch_fwd_tc(a, st) : launch_fwd_simt(a, dtype, st);
   if (prof) cudaEventRecord(g_prof_stop, st);
   return e;
 }
@@ -112,7 +116,68 @@ sa_status maybe_validate(const sa_problem* p, const int32_t* perm, const int32_t
   return from_cuda(launch_validate_perm(perm, inv, p->B, p->n, st));
 }
 
+// Scratch for the key lists, where there is enough of it.
+void* list_room(const sa_problem* p, void* lists, size_t bytes) {
+  const size_t need = key_list_bytes(p);
+  return need && lists && aligned16(lists) && bytes >= need ? lists : nullptr;
+}
+
+sa_status forward(const sa_problem* p, const void* q, const void* k, const void* v,
+                  const int32_t* perm, const int32_t* inv, void* y, float* lse, void* lists,
+                  size_t lists_bytes, cudaStream_t st) {
+  sa_status s = check_problem(p);
+  if (s != SA_OK) return s;
+  if (!good_ptr(q) || !good_ptr(k) || !good_ptr(v) || !good_ptr(perm) || !good_ptr(inv) ||
+      !good_ptr(y) || (lse && !aligned16(lse)))
+    return SA_ERR_INVALID_ARG;
+  if ((s = maybe_validate(p, perm, inv, st)) != SA_OK) return s;
+  FwdArgs a = fwd_args(p, q, k, v, false);
+  a.perm = perm; a.inv = inv; a.y = y; a.lse = lse;
+  a.lists = list_room(p, lists, lists_bytes);
+  return from_cuda(run_forward(a, p->dtype, st));
+}
+
 }  // namespace
+
+size_t key_list_bytes(const sa_problem* p) {
+  OrderGeom g;
+  FwdArgs a = fwd_args(p, p, p, p, false);            // pointers unused by the test
+  return tc_forward_ordered(a, p->dtype, &g) ? order_bytes(p->B, g) : 0;
+}
+
+sa_status gated_forward(const sa_problem* p, const void* q, const void* k, const void* v,
+                        const int32_t* perm, const int32_t* inv, const float* gate_logits, void* y,
+                        void* y_sa, void* y_swa, float* lse_sa, float* lse_swa, void* lists,
+                        size_t lists_bytes, bool lists_ready, cudaStream_t st) {
+  sa_status s = check_problem(p);
+  if (s != SA_OK) return s;
+  if (!good_ptr(q) || !good_ptr(k) || !good_ptr(v) || !good_ptr(perm) || !good_ptr(inv) ||
+      !good_ptr(y) || !gate_logits)
+    return SA_ERR_INVALID_ARG;
+  if ((y_sa && !aligned16(y_sa)) || (y_swa && !aligned16(y_swa)) ||
+      (lse_sa && !aligned16(lse_sa)) || (lse_swa && !aligned16(lse_swa)))
+    return SA_ERR_INVALID_ARG;
+  if ((p->flags & SA_SAVE_FOR_BWD) && (!y_sa || !y_swa || !lse_sa || !lse_swa))
+    return SA_ERR_INVALID_ARG;
+  if ((s = maybe_validate(p, perm, inv, st)) != SA_OK) return s;
+  // Two launches.  The SA branch first: its ungated rows land in y_sa, else in y itself.  The
+  // local branch then owns each output row exactly once: its epilogue reads the matching SA row
+  // (the tensor-core kernel in coalesced pieces), applies both gates and writes y.  (In the other order
+  // the rows of the local branch would be read scattered from the SA branch's epilogue, and that branch
+  // could not start before the local one is complete.)
+  void* sa_rows = y_sa ? y_sa : y;
+  FwdArgs a = fwd_args(p, q, k, v, false);
+  a.perm = perm; a.inv = inv; a.y = sa_rows; a.lse = lse_sa;
+  a.lists = list_room(p, lists, lists_bytes);
+  a.lists_ready = lists_ready;
+  cudaError_t e = run_forward(a, p->dtype, st);
+  if (e != cudaSuccess) return SA_ERR_CUDA;
+  FwdArgs b = fwd_args(p, q, k, v, true);
+  b.y = y; b.y_branch = y_swa; b.lse = lse_swa;
+  b.y_other = sa_rows; b.gate_logits = gate_logits;
+  return from_cuda(run_forward(b, p->dtype, st));
+}
+
 }  // namespace sa
 
 using namespace sa;
@@ -150,8 +215,10 @@ size_t sa_workspace_bytes(const sa_problem* p, int op) {
                           nullptr);
     case SA_OP_FORWARD_ROPE: {
       if (check_problem(p) != SA_OK || p->d % 2 != 0) return (size_t)-1;
-      return rope_bytes(p);
+      return rope_bytes(p) + key_list_bytes(p);
     }
+    case SA_OP_KEY_LISTS:
+      return check_problem(p) == SA_OK ? key_list_bytes(p) : (size_t)-1;
     default:
       return (size_t)-1;
   }
@@ -170,16 +237,13 @@ sa_status sa_forward(const sa_problem* p, const void* q, const void* k, const vo
                      const int32_t* perm, const int32_t* inv, void* y, float* lse, void* ws,
                      size_t ws_bytes, sa_stream_t stream) {
   (void)ws; (void)ws_bytes;
-  sa_status s = check_problem(p);
-  if (s != SA_OK) return s;
-  if (!good_ptr(q) || !good_ptr(k) || !good_ptr(v) || !good_ptr(perm) || !good_ptr(inv) ||
-      !good_ptr(y) || (lse && !aligned16(lse)))
-    return SA_ERR_INVALID_ARG;
-  cudaStream_t st = (cudaStream_t)stream;
-  if ((s = maybe_validate(p, perm, inv, st)) != SA_OK) return s;
-  FwdArgs a = fwd_args(p, q, k, v, false);
-  a.perm = perm; a.inv = inv; a.y = y; a.lse = lse;
-  return from_cuda(run_forward(a, p->dtype, st));
+  return forward(p, q, k, v, perm, inv, y, lse, nullptr, 0, (cudaStream_t)stream);
+}
+
+sa_status sa_forward_lists(const sa_problem* p, const void* q, const void* k, const void* v,
+                           const int32_t* perm, const int32_t* inv, void* y, float* lse, void* ws,
+                           size_t ws_bytes, sa_stream_t stream) {
+  return forward(p, q, k, v, perm, inv, y, lse, ws, ws_bytes, (cudaStream_t)stream);
 }
 
 sa_status sa_swa_forward(const sa_problem* p, const void* q, const void* k, const void* v,
@@ -199,34 +263,18 @@ sa_status sa_swa_gated_forward(const sa_problem* p, const void* q, const void* k
                                const float* gate_logits, void* y, void* y_sa, void* y_swa,
                                float* lse_sa, float* lse_swa, void* ws, size_t ws_bytes,
                                sa_stream_t stream) {
-  sa_status s = check_problem(p);
-  if (s != SA_OK) return s;
-  if (!good_ptr(q) || !good_ptr(k) || !good_ptr(v) || !good_ptr(perm) || !good_ptr(inv) ||
-      !good_ptr(y) || !gate_logits)
-    return SA_ERR_INVALID_ARG;
   if (ws && !aligned16(ws)) return SA_ERR_INVALID_ARG;
-  if ((y_sa && !aligned16(y_sa)) || (y_swa && !aligned16(y_swa)) ||
-      (lse_sa && !aligned16(lse_sa)) || (lse_swa && !aligned16(lse_swa)))
-    return SA_ERR_INVALID_ARG;
-  if ((p->flags & SA_SAVE_FOR_BWD) && (!y_sa || !y_swa || !lse_sa || !lse_swa))
-    return SA_ERR_INVALID_ARG;
-  cudaStream_t st = (cudaStream_t)stream;
-  if ((s = maybe_validate(p, perm, inv, st)) != SA_OK) return s;
-  // Two launches.  The SA branch first: its ungated rows land in y_sa, else in y itself.  The
-  // local branch then owns each output row exactly once: its epilogue reads the matching SA row
-  // (the tensor-core kernel in coalesced pieces), applies both gates and writes y.  (In the other order
-  // the rows of the local branch would be read scattered from the SA branch's epilogue, and that branch
-  // could not start before the local one is complete.)
   (void)ws_bytes;
-  void* sa_rows = y_sa ? y_sa : y;
-  FwdArgs a = fwd_args(p, q, k, v, false);
-  a.perm = perm; a.inv = inv; a.y = sa_rows; a.lse = lse_sa;
-  cudaError_t e = run_forward(a, p->dtype, st);
-  if (e != cudaSuccess) return SA_ERR_CUDA;
-  FwdArgs b = fwd_args(p, q, k, v, true);
-  b.y = y; b.y_branch = y_swa; b.lse = lse_swa;
-  b.y_other = sa_rows; b.gate_logits = gate_logits;
-  return from_cuda(run_forward(b, p->dtype, st));
+  return gated_forward(p, q, k, v, perm, inv, gate_logits, y, y_sa, y_swa, lse_sa, lse_swa, nullptr, 0,
+                       false, (cudaStream_t)stream);
+}
+
+sa_status sa_swa_gated_forward_lists(const sa_problem* p, const void* q, const void* k, const void* v,
+                                     const int32_t* perm, const int32_t* inv, const float* gate_logits,
+                                     void* y, void* y_sa, void* y_swa, float* lse_sa, float* lse_swa,
+                                     void* ws, size_t ws_bytes, sa_stream_t stream) {
+  return gated_forward(p, q, k, v, perm, inv, gate_logits, y, y_sa, y_swa, lse_sa, lse_swa, ws, ws_bytes,
+                       false, (cudaStream_t)stream);
 }
 
 sa_status sa_rope_apply(const sa_problem* p, int32_t kv, const void* x, const float* rope_cos,
@@ -256,6 +304,12 @@ sa_status rope_prepass(const sa_problem* p, const void*& q, const void*& k, cons
   return SA_OK;
 }
 
+// Key lists behind the rotated copies, where the workspace has room for both.
+void* rope_lists(const sa_problem* p, void* ws, size_t ws_bytes) {
+  const size_t at = rope_bytes(p);
+  return ws && ws_bytes > at ? list_room(p, (char*)ws + at, ws_bytes - at) : nullptr;
+}
+
 // Rotation inside the gather or as a pass of its own?  A K row is gathered, and would be turned,
 // once per query tile that meets it, at ~45 instructions per 16 bytes; the pass turns it once, at
 // HBM speed (32/8 heads of 128, n = 8192, w = 1024: 840 us against 12 + 230 us).  In the gather
@@ -265,7 +319,7 @@ bool rope_in_gather(const sa_problem* p, bool one_launch, const void* ws, size_t
   FwdArgs probe = fwd_args(p, p, p, p, false);        // pointers unused by the support test
   if (!tc_forward_supported(probe, p->dtype)) return false;
   if (!ws || !aligned16(ws) || ws_bytes < rope_bytes(p)) return true;
-  return one_launch && (int64_t)p->B * p->Hq * p->n * p->d < (8 << 20);
+  return one_launch && (int64_t)p->B * p->Hq * p->n * p->d < (8 << 20) && !rope_lists(p, (void*)ws, ws_bytes);
 }
 }  // namespace
 
@@ -288,6 +342,7 @@ sa_status sa_forward_rope(const sa_problem* p, const void* q, const void* k, con
     a.rope_cos = rope_cos; a.rope_sin = rope_sin;
   } else {
     if ((s = rope_prepass(p, a.q, a.k, rope_cos, rope_sin, ws, ws_bytes, st)) != SA_OK) return s;
+    a.lists = rope_lists(p, ws, ws_bytes);
   }
   return from_cuda(run_forward(a, p->dtype, st));
 }
@@ -320,6 +375,7 @@ sa_status sa_swa_gated_forward_rope(const sa_problem* p, const void* q, const vo
   FwdArgs a = fwd_args(p, q, k, v, false);
   a.perm = perm; a.inv = inv; a.y = sa_rows; a.lse = lse_sa;
   if (in_gather) { a.rope_cos = rope_cos; a.rope_sin = rope_sin; }
+  else a.lists = rope_lists(p, ws, ws_bytes);
   if (run_forward(a, p->dtype, st) != cudaSuccess) return SA_ERR_CUDA;
   FwdArgs b = fwd_args(p, q, k, v, true);
   b.y = y; b.y_branch = y_swa; b.lse = lse_swa;

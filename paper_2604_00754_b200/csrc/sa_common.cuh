@@ -158,6 +158,8 @@ struct FwdArgs {
   float scale;
   int64_t qs[3], ks[3];
   bool swa;
+  void* lists;            // nullable: room for token-ordered key lists (order_bytes of the problem's geometry)
+  bool lists_ready;       // an earlier call made them from the same permutation
   const int* abort_flag;  // nullable: kernels return at once when it reads non-zero
 };
 
@@ -181,6 +183,15 @@ struct BwdArgs {
   int nbranch;
   const int* abort_flag;  // nullable: kernels return at once when it reads non-zero
 };
+
+// sa_swa_gated_forward with room for the SA branch's key lists, made by this call or (ready) by an
+// earlier one with the same permutation, n, w and flags.
+sa_status gated_forward(const sa_problem* p, const void* q, const void* k, const void* v,
+                        const int32_t* perm, const int32_t* inv, const float* gate_logits, void* y,
+                        void* y_sa, void* y_swa, float* lse_sa, float* lse_swa, void* lists,
+                        size_t lists_bytes, bool lists_ready, cudaStream_t st);
+// Bytes of those lists; 0 where the branch does without.
+size_t key_list_bytes(const sa_problem* p);
 
 // Launchers (each returns cudaGetLastError() of its launches).
 cudaError_t launch_make_perm(uint64_t seed, uint32_t layer, int B, int n, int32_t* perm,

@@ -31,6 +31,7 @@
 
 #include "sa_fwd_tc.cuh"
 #include "sa_gemm_common.cuh"
+#include "sa_order.cuh"
 #include "sa_tc_common.cuh"
 
 namespace sa {
@@ -39,7 +40,7 @@ namespace {
 constexpr int kTile = 128;           // query rows per tile and keys per K/V tile
 constexpr uint32_t kTmemCols = 512;
 
-enum Src { kGather = 0, kNatural = 1 };
+enum Src { kGather = 0, kNatural = 1, kOrdered = 2 };
 // Who does what.  At d = 64 each query tile has an issuing thread of its own: a tcgen05.commit holds
 // its thread up for some 180 cycles, which the other tile's products fill (8 x 12 heads of 64,
 // n = 4096, w = 128: SWA 114 -> 88 us, SA 144 -> 129; 256 heads of 64, n = 2048, w = 256: 165 -> 143
@@ -67,6 +68,8 @@ struct TcParams {
   int items_per_kv;           // work items per (b, hk)
   int total_items;
   float scale2;               // softmax scale * log2(e)
+  OrderView order;            // kOrdered: what sa_order.cu made
+  OrderGeom og;
   int64_t qs[3];              // element strides of q / y / y_branch / y_other: batch, head, token
   int64_t ks[3];              // element strides of k / v
 };
@@ -79,6 +82,7 @@ struct Geo {
   int valid[2];     // tile exists
   int kstart;       // virtual slot of the first key of K/V tile 0
   int T;            // K/V tiles in the stream
+  int Tt[2];        // kOrdered: those that each query tile meets, the first of the stream
 };
 
 // Score blocks whose first key kv lies in [*lo, *hi] are wholly inside the window of every query
@@ -152,6 +156,41 @@ __device__ __forceinline__ Geo make_geo(const TcParams& p, int item, int hk) {
     kend = qlast + p.h;
   }
   g.T = (kend - g.kstart + kTile) / kTile;
+  return g;
+}
+
+// kOrdered: the query tiles of an item.  Those that meet the most blocks come first, class by class, so
+// that the classes fall evenly on the CTAs and the last round is of the shortest.
+__device__ __forceinline__ void ordered_tiles(const TcParams& p, int item, int hk, int (&tile)[2],
+                                              int (&hq)[2]) {
+  const int per_unit = p.pair_heads ? 1 : 2, units = p.og.slots / (kTile * per_unit);
+  const int full = p.n_tiles / (units * per_unit);                   // groups with all their tiles
+  const int heads = p.pair_heads ? p.G / 2 : p.G;
+  const int x = item / heads, hh = item - x * heads;
+  int unit = x;
+  if (x < full * units) {
+    const int cls = x / full;
+    unit = (x - cls * full) * units + units - 1 - cls;
+  }
+  tile[0] = unit * per_unit;
+  tile[1] = tile[0] + per_unit - 1;
+  hq[0] = hk * p.G + (p.pair_heads ? 2 * hh : hh);
+  hq[1] = hq[0] + (p.pair_heads ? 1 : 0);
+}
+
+// kOrdered: q0 are places in the tokens of the query tiles, keys count from the start of the group's list.
+__device__ __forceinline__ Geo ordered_geo(const TcParams& p, int item, int hk, int b) {
+  Geo g;
+  int tile[2];
+  ordered_tiles(p, item, hk, tile, g.hq);
+#pragma unroll
+  for (int t = 0; t < 2; ++t) {
+    g.q0[t] = tile[t] * kTile;
+    g.valid[t] = tile[t] < p.n_tiles;
+    g.Tt[t] = g.valid[t] ? __ldcg(p.order.tiles + (size_t)b * p.n_tiles + tile[t]) : 0;
+  }
+  g.kstart = 0;
+  g.T = max(g.Tt[0], g.Tt[1]);
   return g;
 }
 
@@ -238,6 +277,16 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
   constexpr int kIssuers = issuers(D);
   constexpr int kMmaWarp = kRowWarps, kLoadWarp = kRowWarps + kIssuers;
   constexpr int kGWarps = 4 - kIssuers;      // the loading warps, when rows are gathered
+  constexpr bool kRows = SRC != kNatural;    // tiles are gathered row by row
+  static_assert(SRC != kOrdered || (KB == 128 && !ROPE && !COMBINE), "ordered lists");
+  auto geo_of = [&](int item, int hk, int b) {
+    if constexpr (SRC == kOrdered) return ordered_geo(p, item, hk, b);
+    else return make_geo(p, item, hk);
+  };
+  auto active_of = [&](const Geo& g, int t, int H, int shift, int* first, int* last) {
+    if constexpr (SRC == kOrdered) { *first = 0; *last = (t ? g.Tt[1] : g.Tt[0]) - 1; }
+    else active_halves(p, t ? g.q0[1] : g.q0[0], t ? g.valid[1] : g.valid[0], g.kstart, H, shift, first, last);
+  };
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
   const uint32_t sbase = smem_u32(smem);
@@ -261,7 +310,7 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
     for (int i = 0; i < C::kNumBars; ++i) {
       int count = 1;
       if (i >= C::kBarPReady && i < C::kBarPvDone) count = kTile;
-      if ((i < C::kBarQEmpty || (i >= C::kBarSlotFull && i < C::kBarFree)) && SRC == kGather)
+      if ((i < C::kBarQEmpty || (i >= C::kBarSlotFull && i < C::kBarFree)) && kRows)
         count = 32 * kGWarps;
       if ((i >= C::kBarQEmpty && i < C::kBarSlotFull) || (i >= C::kBarFree && i < C::kBarTokFull))
         count = kIssuers;
@@ -368,7 +417,7 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
           landed(C::kBarQFull + q_armed % C::kQBufs, (q_armed / C::kQBufs) & 1u);
       }
     }
-  } else if (SRC == kGather && warp >= kLoadWarp) {
+  } else if (kRows && warp >= kLoadWarp) {
     // ------------------------------------------------------------------ gather producers
     // Each 16-byte piece of a row goes from global memory to its swizzled place in shared
     // memory with cp.async; one warp instruction moves kRpi whole rows.
@@ -493,17 +542,23 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
     for (int w_item = blockIdx.x; w_item < p.total_items && live; w_item += gridDim.x, ++it) {
       const int item = w_item % p.items_per_kv, bh = w_item / p.items_per_kv;
       const int hk = bh % p.Hkv, b = bh / p.Hkv;
-      const Geo g = make_geo(p, item, hk);
+      const Geo g = geo_of(item, hk, b);
       const int32_t* perm = p.perm ? p.perm + (size_t)b * p.n : nullptr;
+      const int32_t* list = nullptr;           // kOrdered: the group's keys
+      if constexpr (SRC == kOrdered) {
+        perm = p.order.q + (size_t)b * p.n_tiles * kTile;
+        list = p.order.k + ((size_t)b * p.og.groups + g.q0[0] / p.og.slots) * p.og.pitch;
+      }
       const uint32_t q_bar = bar(C::kBarQFull + it % C::kQBufs);
       const uint32_t q_dst = sbase + C::kOffQ + 2 * (it % C::kQBufs) * C::kTileBytes;
       auto q_tok = [&](int t, int r) {
-        const int slot = min((t ? g.q0[1] : g.q0[0]) + r, p.n - 1);
+        const int slot = min((t ? g.q0[1] : g.q0[0]) + r, (SRC == kOrdered ? p.n_tiles * kTile : p.n) - 1);
         return perm ? perm[slot] : slot;
       };
       const __nv_bfloat16* kb = kg + b * p.ks[0] + hk * p.ks[1];
       const __nv_bfloat16* vb = vg + b * p.ks[0] + hk * p.ks[1];
       auto key_tok = [&](int j, int r) {
+        if constexpr (SRC == kOrdered) return list[j * kTile + r];
         const int slot = actual_slot(p, g.kstart + j * kTile + r);
         return perm ? perm[slot] : slot;
       };
@@ -518,7 +573,7 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
         ktok[ptid] = tk0;
         if (ptid + kPt < kTile) ktok[ptid + kPt] = tk1;
         if (group_sync_stop()) { live = false; break; }
-        if (ptid == 0) mbar_arrive(bar(C::kBarTokFull + gt % C::kTok));
+        if (SRC == kGather && ptid == 0) mbar_arrive(bar(C::kBarTokFull + gt % C::kTok));
         const uint32_t k_dst = sbase + C::kOffRing + 2 * pr * C::kTileBytes;
         const uint32_t k_bar = bar(C::kBarSlotFull + 2 * pr);
         auto tok_of = [&](int r) { return ktok[r]; };
@@ -618,16 +673,14 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
       };
       for (int w_item = blockIdx.x; w_item < p.total_items && ok; w_item += gridDim.x, ++it) {
         const int item = w_item % p.items_per_kv, bh = w_item / p.items_per_kv;
-        const Geo g = make_geo(p, item, bh % p.Hkv);
+        const Geo g = geo_of(item, bh % p.Hkv, bh / p.Hkv);
         const int H = NB * g.T;         // score blocks of this item
         // half-steps [first, last] that each query tile takes part in (a contiguous range)
         int first[kN], last[kN];
         uint32_t started[kN] = {};
 #pragma unroll
         for (int x = 0; x < kN; ++x) {
-          const int t = tb + x;
-          active_halves(p, t ? g.q0[1] : g.q0[0], t ? g.valid[1] : g.valid[0], g.kstart, H, kShift,
-                        &first[x], &last[x]);
+          active_of(g, tb + x, H, kShift, &first[x], &last[x]);
         }
         const uint32_t qb = it % C::kQBufs;
         q_item = qb * (2 * C::kTileBytes >> 4);
@@ -864,20 +917,28 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
       int q0, hq, kstart, first, last, in_lo, in_hi;
       const uint32_t gt0 = gt;
       {
-        const Geo g = make_geo(p, item, bh % p.Hkv);
+        const Geo g = geo_of(item, bh % p.Hkv, b);
         q0 = t ? g.q0[1] : g.q0[0];
         hq = t ? g.hq[1] : g.hq[0];
         kstart = g.kstart;
         gt += g.T;
-        active_halves(p, q0, t ? g.valid[1] : g.valid[0], kstart, NB * g.T, kShift, &first, &last);
+        active_of(g, t, NB * g.T, kShift, &first, &last);
       }
       const int this_tok = next_tok;
       next_tok = token_of(w_item + gridDim.x);
       if (first > last) continue;           // no such tile
-      inner_range(p, q0, kHalf, &in_lo, &in_hi);
+      if (SRC != kOrdered) inner_range(p, q0, kHalf, &in_lo, &in_hi);
       const int qv = q0 + row;
       const bool row_valid = qv < p.n;
-      const int q_tok = SRC == kGather && p.perm ? this_tok : row_valid ? qv : 0;
+      int q_tok = SRC == kGather && p.perm ? this_tok : row_valid ? qv : 0;
+      const uint4* bits = nullptr;            // kOrdered: what this row sees, block by block
+      uint4 seen_next = make_uint4(0u, 0u, 0u, 0u);
+      if constexpr (SRC == kOrdered) {
+        const size_t place = (size_t)b * p.n_tiles * kTile + qv;
+        q_tok = __ldcg(p.order.q + place);
+        bits = p.order.bits + (place - row) * p.og.blocks + row;
+        seen_next = __ldcg(bits);
+      }
       const int qcmp = (p.causal && !p.one_sided) ? q_tok : 0x7fffffff;
       if (COMBINE && row_valid) {
         // the epilogue will read the other branch's row: start bringing it into L2 now
@@ -895,7 +956,7 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
         const int hb = h & (NB - 1);
         const uint32_t tg = gt0 + (h >> (NB - 1));
         // the token list belongs to the whole 128-key tile: wait for it at its first half only
-        if (SRC != kNatural && (hb == 0 || h == first))
+        if (SRC == kGather && (hb == 0 || h == first))
           ok = mbar_wait(bar(C::kBarTokFull + tg % C::kTok), (tg / C::kTok) & 1u, gave_up, p.status);
         if (ok)
           ok = mbar_wait(bar(C::kBarSFull + 2 * t + hb), (hb ? s_cnt1 : s_cnt0) & 1u, gave_up,
@@ -910,13 +971,13 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
         uint32_t sr[kHalf];
         // Gathered branch: 32 columns are masked while the next 32 are on their way (SA, 32/8 heads of
         // 128, n = 10007, w = 1024: 277 -> 273 us).  The other, with next to no masks, takes all at once.
-        constexpr int kFirst = SRC == kGather ? 32 : kHalf;
+        constexpr int kFirst = kRows ? 32 : kHalf;
 #pragma unroll
         for (int c = 0; c < kFirst / 32; ++c)
           tmem_ld32(sh_addr + 32 * c, reinterpret_cast<uint32_t(&)[32]>(sr[32 * c]));
         tmem_wait_ld();
         auto next32 = [&](int c) {
-          if (SRC == kGather) {
+          if (kRows) {
             if (c > 0) tmem_wait_ld();
             if (c + 32 < kHalf)
               tmem_ld32(sh_addr + c + 32, reinterpret_cast<uint32_t(&)[32]>(sr[(c + 32) % kHalf]));
@@ -936,7 +997,18 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
         // plain SWA: keys wholly before the queries need no causal test (no wrap inside)
         const bool tokens_matter =
             p.causal && !p.one_sided && !(p.swa && kv >= 0 && kv + kHalf - 1 <= q0);
-        if (kv >= in_lo && kv <= in_hi) {
+        if constexpr (SRC == kOrdered) {
+          const uint4 seen4 = seen_next;
+          if (h < last) seen_next = __ldcg(bits + (size_t)(h + 1) * kTile);
+          const uint32_t seen[4] = {seen4.x, seen4.y, seen4.z, seen4.w};
+#pragma unroll
+          for (int c0 = 0; c0 < kHalf; c0 += 32) {
+            next32(c0);
+#pragma unroll
+            for (int c = 0; c < 32; ++c)
+              if (!(seen[c0 / 32] & (1u << ((c & 1) * 16 + c / 2)))) sr[c0 + c] = 0xff800000u;
+          }
+        } else if (kv >= in_lo && kv <= in_hi) {
           if (tokens_matter) {
 #pragma unroll
             for (int c0 = 0; c0 < kHalf; c0 += 32) {
@@ -1112,6 +1184,11 @@ bool tc_forward_supported(const FwdArgs& a, int dtype) {
   return true;
 }
 
+bool tc_forward_ordered(const FwdArgs& a, int dtype, OrderGeom* g) {
+  return !a.swa && !a.rope_cos && tc_forward_supported(a, dtype) &&
+         debug_option(SA_DEBUG_SCORE_BLOCK) != 64 && order_geom(a.n, a.d, a.w, a.flags, g);
+}
+
 cudaError_t launch_fwd_tc(const FwdArgs& a, cudaStream_t st) {
   TcParams p{};
   p.q = a.q; p.k = a.k; p.v = a.v;
@@ -1132,6 +1209,13 @@ cudaError_t launch_fwd_tc(const FwdArgs& a, cudaStream_t st) {
   p.items_per_kv = p.pair_heads ? p.n_tiles * (p.G / 2) : ((p.n_tiles + 1) / 2) * p.G;
   p.scale2 = a.scale * kLog2e;
   for (int i = 0; i < 3; ++i) { p.qs[i] = a.qs[i]; p.ks[i] = a.ks[i]; }
+  const bool ordered = a.lists && tc_forward_ordered(a, SA_BF16, &p.og);
+  if (ordered) {
+    const int per_group = p.og.slots / kTile, full = p.n_tiles / per_group;
+    if (!p.pair_heads)
+      p.items_per_kv = (full * (per_group / 2) + (p.n_tiles - full * per_group + 1) / 2) * p.G;
+    p.order = order_view(a.lists, a.B, p.og);
+  }
   p.total_items = a.B * a.Hkv * p.items_per_kv;
 
   static int sm_count[64] = {0};
@@ -1161,6 +1245,13 @@ cudaError_t launch_fwd_tc(const FwdArgs& a, cudaStream_t st) {
     return launch_dependent(kernel, dim3(grid), dim3(kThreads), smem, st, p, tm_q, tm_k, tm_v);
   };
   const bool wide = key_block_128(a.w, a.d, natural);
+  if (ordered) {
+    e = a.d == 128 ? go(fwd_tc_kernel<128, 128, kOrdered>, Cfg<128>::kBytes)
+                   : go(fwd_tc_kernel<64, 128, kOrdered>, Cfg<64>::kBytes);
+    if (e != cudaSuccess) return e;
+    bump_launches();
+    return cudaGetLastError();
+  }
   // instantiation by (head dimension, score-block width, source of the tiles, rotation, combine)
   auto pick = [&](auto d_c, auto kb_c) {
     constexpr int DD = decltype(d_c)::value, KK = decltype(kb_c)::value;

@@ -134,6 +134,7 @@ Pipe* pipe_for_current_device() {
 
 struct Carve {
   size_t q, k, v, y, scratch, gate, perm, inv, perm_ws, total;
+  size_t lists, list_bytes, with_lists;   // key lists of the SA branch; bytes with room for them
 };
 
 bool carve(const sa_problem* p, Carve* c) {
@@ -151,6 +152,16 @@ bool carve(const sa_problem* p, Carve* c) {
   c->inv = o; o += align256((size_t)p->B * p->n * sizeof(int32_t));
   c->perm_ws = o; o += align256(make_perm_ws_bytes(p->B, p->n));
   c->total = o;
+  // The key lists of all sequences go behind the copies of index lists that some ranges need in the scratch
+  // (at most one of each per sequence), or behind everything where that is too small.
+  sa_problem dp = *p;
+  sa_problem_set_contiguous(&dp);
+  const size_t lb = sa_workspace_bytes(&dp, SA_OP_KEY_LISTS);
+  c->list_bytes = lb == (size_t)-1 ? 0 : lb;
+  const size_t copies = 2 * (size_t)p->B * align256((size_t)p->n * sizeof(int32_t));
+  const bool fits = copies + c->list_bytes <= qb;
+  c->lists = fits ? c->scratch + copies : o;
+  c->with_lists = fits ? o : o + c->list_bytes;
   return true;
 }
 
@@ -191,7 +202,7 @@ int32_t sa_host_forward_pieces(const sa_problem* p, int32_t n_groups, int32_t q_
 
 size_t sa_host_forward_ws_bytes(const sa_problem* p) {
   Carve c;
-  return carve(p, &c) ? c.total : (size_t)-1;
+  return carve(p, &c) ? c.with_lists : (size_t)-1;
 }
 
 sa_status sa_swa_gated_forward_host(const sa_problem* p, const void* q, const void* k,
@@ -264,7 +275,10 @@ sa_status sa_swa_gated_forward_host(const sa_problem* p, const void* q, const vo
   if (ok)
     st = sa_make_perm(seed, layer, p->B, p->n, dperm, dinv, base + c.perm_ws,
                       make_perm_ws_bytes(p->B, p->n), (sa_stream_t)pipe->s_run);
+  // the SA branch's key lists are made once per range of sequences, by its first piece
+  void* lists = c.list_bytes && ws_bytes >= c.with_lists ? base + c.lists : nullptr;
   const int32_t *rperm = dperm, *rinv = dinv;     // of the range at hand
+  bool lists_ready = false;
   int range_at = 0;
   size_t spare = c.scratch;
   for (int i = 0; i < cnt && ok && st == SA_OK; ++i) {
@@ -273,6 +287,7 @@ sa_status sa_swa_gated_forward_host(const sa_problem* p, const void* q, const vo
       // the kernels' entry points take index lists that start on 16 bytes
       const size_t at = (size_t)g.b0 * p->n, len = (size_t)(g.b1 - g.b0) * p->n * sizeof(int32_t);
       range_at = g.b0;
+      lists_ready = false;
       rperm = dperm + at;
       rinv = dinv + at;
       if (at % 4 != 0) {
@@ -298,8 +313,9 @@ sa_status sa_swa_gated_forward_host(const sa_problem* p, const void* q, const vo
     gp.Hkv = g.kb - g.ka;
     const size_t qoff = ((size_t)g.b0 * p->Hq + g.qa) * head_bytes;
     const size_t koff = ((size_t)g.b0 * p->Hkv + g.ka) * head_bytes;
-    st = sa_swa_gated_forward(&gp, dq + qoff, dk + koff, dv + koff, rperm, rinv, gates, dyv + qoff,
-                              nullptr, nullptr, nullptr, nullptr, nullptr, 0, (sa_stream_t)pipe->s_run);
+    st = gated_forward(&gp, dq + qoff, dk + koff, dv + koff, rperm, rinv, gates, dyv + qoff, nullptr, nullptr,
+                       nullptr, nullptr, lists, lists ? c.list_bytes : 0, lists_ready, pipe->s_run);
+    lists_ready = lists != nullptr;
     chk(cudaEventRecord(pipe->ev_done[i], pipe->s_run));
   }
 

@@ -133,6 +133,20 @@ size_t ws_bytes(const sa_problem& p, int op) {
   return n;
 }
 
+// Scratch for the SA branch's key lists, from the allocator's pool of the current stream; undefined
+// where the problem has no use for any.
+at::Tensor key_lists(const sa_problem& p, c10::Device dev) {
+  const size_t n = sa_workspace_bytes(&p, SA_OP_KEY_LISTS);
+  if (n == 0 || n == (size_t)-1) return at::Tensor();
+  try {
+    return fresh({(int64_t)n}, at::kByte, dev);
+  } catch (const c10::OutOfMemoryError&) {          // the call works without
+    return at::Tensor();
+  }
+}
+void* ptr_or_null(const at::Tensor& t) { return t.defined() ? t.data_ptr() : nullptr; }
+size_t bytes_of(const at::Tensor& t) { return t.defined() ? (size_t)t.numel() : 0; }
+
 PyObject* wrap(at::Tensor t) { return THPVariable_Wrap(std::move(t)); }
 PyObject* pass(PyObject* o) {
   Py_INCREF(o);
@@ -200,9 +214,10 @@ PyObject* forward(PyObject* const* a) {
   const bool has_lse = a[10] != Py_None || truth(a[9]);
   Out lse;
   if (has_lse) lse = output(a[10], [&] { return rows_f32(q); });
-  check(unlocked(sa_forward, &p, ptr(q), ptr(k), ptr(v), (const int32_t*)ptr(tensor(a[3])),
+  at::Tensor lists = key_lists(p, q.device());
+  check(unlocked(sa_forward_lists, &p, ptr(q), ptr(k), ptr(v), (const int32_t*)ptr(tensor(a[3])),
                    (const int32_t*)ptr(tensor(a[4])), ptr(y), has_lse ? (float*)ptr(lse) : nullptr,
-                   nullptr, 0, stream()),
+                   ptr_or_null(lists), bytes_of(lists), stream()),
         "sa_forward");
   return has_lse ? tuple({y.result(), lse.result()}) : y.result();
 }
@@ -226,11 +241,13 @@ PyObject* gated_forward(PyObject* const* a) {
   auto at_or_null = [](const Out& o) { return o.t || o.own.defined() ? ptr(o) : nullptr; };
   const sa_problem p = problem(q, k, a[6], flags, a[8]);
   const at::Tensor* ws = tensor_or_null(a[15]);
-  check(unlocked(sa_swa_gated_forward, &p, ptr(q), ptr(k), ptr(v), (const int32_t*)ptr(tensor(a[3])),
+  if (ws && ((uintptr_t)ptr(ws) & 15u)) check(SA_ERR_INVALID_ARG, "sa_swa_gated_forward");
+  at::Tensor lists = key_lists(p, q.device());
+  check(unlocked(sa_swa_gated_forward_lists, &p, ptr(q), ptr(k), ptr(v), (const int32_t*)ptr(tensor(a[3])),
                              (const int32_t*)ptr(tensor(a[4])), (const float*)ptr(tensor(a[5])),
                              ptr(y), at_or_null(branch[0]), at_or_null(branch[1]),
-                             (float*)at_or_null(lse[0]), (float*)at_or_null(lse[1]), ptr(ws),
-                             ws ? (size_t)ws->numel() : 0, stream()),
+                             (float*)at_or_null(lse[0]), (float*)at_or_null(lse[1]), ptr_or_null(lists),
+                             bytes_of(lists), stream()),
         "sa_swa_gated_forward");
   if (!save) return y.result();
   return tuple({y.result(), branch[0].result(), branch[1].result(), lse[0].result(),

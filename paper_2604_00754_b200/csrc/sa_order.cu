@@ -1,0 +1,235 @@
+// Key lists of the causal SA branch: per group of consecutive slots, the union of its queries' windows
+// in token order.
+//
+// Causality is in token order and the window in slot order, so a tile of 128 consecutive slots meets
+// every key of its window although half of the pairs are hidden.  Here a group of 256 or 512 slots is
+// dealt to its query tiles by token: tile i holds the i-th 128 of the group's tokens.  The keys of the
+// group's window, in token order, are one list for all its tiles, and a tile stops at the last token
+// it holds: with w = 1024 two tiles meet 5.3 and 10 blocks of 128 keys where they met 9 each, with
+// w = 2048 four tiles 3.6 to 20 (12.8 on the average) where they met 17.  What a row sees of a block is
+// one bit per key, worked out here once for all heads.
+#include "sa_order.cuh"
+
+namespace sa {
+namespace {
+
+constexpr int kThreads = 512, kBuckets = 1024;
+
+struct OrderParams {
+  const int32_t* perm;
+  int32_t *q, *k, *tiles;
+  uint4* bits;
+  const int* abort_flag;
+  int n, h, linear;
+  OrderGeom g;
+  uint32_t bucket_mul;          // bucket of a token: umulhi(token, bucket_mul) < kBuckets
+};
+
+size_t shared_bytes(int span) {
+  const size_t l = ((size_t)span + 7) / 8 * 8;
+  return l * 12 + kBuckets * 4;
+}
+
+// One CTA per query tile; the tiles of a group each sort the group's keys (a few microseconds that
+// run side by side), and each works out its own bits.  Sort: counts per bucket of tokens, a place per
+// key, and the rank inside the bucket by counting; any contents give the unique order.
+__global__ void __launch_bounds__(kThreads) order_kernel(const __grid_constant__ OrderParams p) {
+  extern __shared__ __align__(16) uint8_t smem[];
+  __shared__ uint32_t part[kThreads / 32];
+  __shared__ int q_pos[kOrderTile], q_off[kOrderTile], skip;
+  constexpr uint32_t kGuard = 0x8000u;            // set in the sorted offsets (all below 2^15)
+  const OrderGeom& g = p.g;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int b = blockIdx.y, tile = blockIdx.x, per_group = g.slots / kOrderTile;
+  const int group = tile / per_group, part_of = tile % per_group;
+  const int s0 = group * g.slots, slots = min(g.slots, p.n - s0), span = slots + 2 * p.h;
+  const int cap = (g.span + 7) / 8 * 8;
+  int32_t* tok = reinterpret_cast<int32_t*>(smem);
+  int32_t* tok2 = tok + cap;
+  uint16_t* off = reinterpret_cast<uint16_t*>(tok2 + cap);
+  uint16_t* off2 = off + cap;
+  uint32_t* start = reinterpret_cast<uint32_t*>(off2 + cap);
+
+  for (int i = tid; i < kBuckets; i += kThreads) start[i] = 0u;
+  grid_dependency_wait();
+  grid_dependents_launch();
+  if (tid == 0) skip = p.abort_flag && *(volatile const int*)p.abort_flag;
+  __syncthreads();
+  if (skip) return;                                    // an earlier check rejected perm/inv
+  const int32_t* perm = p.perm + (size_t)b * p.n;
+  auto bucket_of = [&](int32_t t) { return min(__umulhi((uint32_t)t, p.bucket_mul), kBuckets - 1u); };
+  // a token of -1: outside the sequence (linear windows)
+  for (int o = tid; o < span; o += kThreads) {
+    int s = s0 - p.h + o;
+    int32_t t = -1;
+    if (!p.linear) { s = s < 0 ? s + p.n : s >= p.n ? s - p.n : s; }
+    if (s >= 0 && s < p.n) t = perm[s];
+    tok[o] = t;
+    if (t >= 0) off[o] = (uint16_t)atomicAdd(&start[bucket_of(t)], 1u);
+  }
+  __syncthreads();
+  // exclusive scan over the block: `mine` per thread; returns the sum of those before it
+  auto scan = [&](uint32_t mine, uint32_t* total) {
+    uint32_t x = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    if (lane == 31) part[warp] = x;
+    __syncthreads();
+    uint32_t before = 0, sum = 0;
+#pragma unroll
+    for (int w = 0; w < kThreads / 32; ++w) {
+      if (w < warp) before += part[w];
+      sum += part[w];
+    }
+    __syncthreads();
+    *total = sum;
+    return before + x - mine;
+  };
+  uint32_t keys;
+  {
+    constexpr int kPer = kBuckets / kThreads;
+    uint32_t c[kPer], mine = 0;
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) { c[i] = start[kPer * tid + i]; mine += c[i]; }
+    uint32_t at = scan(mine, &keys);
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) { start[kPer * tid + i] = at; at += c[i]; }
+  }
+  __syncthreads();
+  for (int o = tid; o < span; o += kThreads) {
+    const int32_t t = tok[o];
+    if (t < 0) continue;
+    const uint32_t at = start[bucket_of(t)] + off[o];
+    tok2[at] = t;
+    off2[at] = (uint16_t)o;
+  }
+  __syncthreads();
+  for (int x = tid; x < (int)keys; x += kThreads) {
+    const int32_t t = tok2[x];
+    const uint16_t o = off2[x];
+    const uint32_t bk = bucket_of(t), lo = start[bk], hi = bk + 1 < kBuckets ? start[bk + 1] : keys;
+    uint32_t rank = lo;
+    for (uint32_t y = lo; y < hi; ++y) {
+      const int32_t u = tok2[y];
+      rank += u < t || (u == t && off2[y] < o);
+    }
+    tok[rank] = t;
+    off[rank] = (uint16_t)(o | kGuard);
+  }
+  if (tid < kOrderTile) q_pos[tid] = -1;
+  __syncthreads();
+  // this tile's queries: the 128 that follow 128 * part_of of the group's in token order
+  const int rows = min(kOrderTile, slots - part_of * kOrderTile);
+  int32_t* q_out = p.q + ((size_t)b * g.tiles + tile) * kOrderTile;
+  {
+    const int per = ((int)keys + kThreads - 1) / kThreads, x0 = tid * per, x1 = min(x0 + per, (int)keys);
+    auto query = [&](int x) { return (int)(off[x] ^ kGuard) - p.h; };     // in [0, slots): a query of the group
+    uint32_t mine = 0, all;
+    for (int x = x0; x < x1; ++x) mine += (uint32_t)query(x) < (uint32_t)slots;
+    int r = (int)scan(mine, &all) - part_of * kOrderTile;
+    for (int x = x0; x < x1; ++x)
+      if ((uint32_t)query(x) < (uint32_t)slots) {
+        if (r >= 0 && r < kOrderTile) {
+          q_pos[r] = x;
+          q_off[r] = query(x);
+          q_out[r] = tok[x];
+        }
+        ++r;
+      }
+  }
+  __syncthreads();
+  const int end = max(q_pos[rows - 1], 0), blocks = end / kOrderTile + 1;
+  if (tid >= rows && tid < kOrderTile) q_out[tid] = tok[end];      // rows that do not exist
+  if (tid == 0) p.tiles[(size_t)b * g.tiles + tile] = blocks;
+  if (part_of * kOrderTile + rows == slots) {                    // the last tile meets the whole list
+    int32_t* k_out = p.k + ((size_t)b * g.groups + group) * g.pitch;
+    for (int x = tid; x < blocks * kOrderTile; x += kThreads) k_out[x] = tok[min(x, (int)keys - 1)];
+  }
+  // A key's bit: it is in the row's window (its offset in [q, q + 2 h]) and not after the row's token
+  // (its place in the list is not after the row's own).  Two offsets at a time: with the guard bits
+  // set a subtraction of both halves borrows nothing across, and leaves the bit where the offset is
+  // not below the bound.
+  uint4* bits = p.bits + ((size_t)b * g.tiles + tile) * g.blocks * kOrderTile;
+  for (int task = warp; task < 4 * blocks; task += kThreads / 32) {
+    const int j = task >> 2, r = (task & 3) * 32 + lane;
+    const int pos = q_pos[r], qo = pos < 0 ? 0 : q_off[r];
+    const int last = __reduce_max_sync(0xffffffffu, pos);
+    const uint32_t from = qo * 0x10001u, past = (uint32_t)(qo + 2 * p.h + 1) * 0x10001u;
+    uint32_t word[4];
+#pragma unroll
+    for (int y = 0; y < 4; ++y) {
+      const int x0 = kOrderTile * j + 32 * y;
+      word[y] = 0u;
+      if (x0 > last) continue;
+      uint32_t v = 0;
+#pragma unroll
+      for (int c = 0; c < 32; c += 8) {
+        const uint4 o8 = *reinterpret_cast<const uint4*>(off + x0 + c);
+        const uint32_t o[4] = {o8.x, o8.y, o8.z, o8.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) v = (v >> 1) | ((o[e] - from) & ~(o[e] - past) & 0x80008000u);
+      }
+      const int upto = min(max(pos + 1 - x0, 0), 32), even = (upto + 1) >> 1, odd = upto >> 1;
+      word[y] = v & (((1u << even) - 1u) | (((1u << odd) - 1u) << 16));
+    }
+    bits[(size_t)j * kOrderTile + r] = make_uint4(word[0], word[1], word[2], word[3]);
+  }
+}
+
+size_t up(size_t x) { return (x + 255) / 256 * 256; }
+
+}  // namespace
+
+bool order_geom(int n, int d, int w, uint32_t flags, OrderGeom* g) {
+  const MaskGeom m = make_geom(n, w, flags, false);
+  if (!m.causal || w < 1024 || n < 32768 || (d != 64 && d != 128)) return false;
+  g->slots = w <= 1280 ? 256 : 512;
+  if ((int64_t)g->slots + 2ll * m.h > n || (int64_t)g->slots + 2ll * m.h > 8192) return false;
+  g->span = g->slots + 2 * m.h;
+  g->groups = (n + g->slots - 1) / g->slots;
+  g->tiles = (n + kOrderTile - 1) / kOrderTile;
+  g->blocks = (g->span + kOrderTile - 1) / kOrderTile;
+  g->pitch = g->blocks * kOrderTile;
+  return true;
+}
+
+size_t order_bytes(int B, const OrderGeom& g) {
+  return up((size_t)B * g.tiles * kOrderTile * 4) + up((size_t)B * g.groups * g.pitch * 4) +
+         up((size_t)B * g.tiles * 4) + up((size_t)B * g.tiles * g.blocks * kOrderTile * 16);
+}
+
+OrderView order_view(void* ws, int B, const OrderGeom& g) {
+  OrderView v;
+  char* at = (char*)ws;
+  v.q = (int32_t*)at;
+  at += up((size_t)B * g.tiles * kOrderTile * 4);
+  v.k = (int32_t*)at;
+  at += up((size_t)B * g.groups * g.pitch * 4);
+  v.tiles = (int32_t*)at;
+  at += up((size_t)B * g.tiles * 4);
+  v.bits = (uint4*)at;
+  return v;
+}
+
+cudaError_t launch_order(const int32_t* perm, int B, int n, int w, uint32_t flags, const OrderGeom& g,
+                         const OrderView& v, const int* abort_flag, cudaStream_t st) {
+  const MaskGeom m = make_geom(n, w, flags, false);
+  OrderParams p{};
+  p.perm = perm;
+  p.q = v.q; p.k = v.k; p.tiles = v.tiles; p.bits = v.bits;
+  p.abort_flag = abort_flag;
+  p.n = n; p.h = m.h; p.linear = m.linear;
+  p.g = g;
+  p.bucket_mul = (uint32_t)(((uint64_t)kBuckets << 32) / (uint64_t)n);     // n > kBuckets: fits
+  const size_t smem = shared_bytes(g.span);
+  const cudaError_t e =
+      cudaFuncSetAttribute(order_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return reported(e);
+  bump_launches();
+  return launch_dependent(order_kernel, dim3(g.tiles, B), dim3(kThreads), smem, st, p);
+}
+
+}  // namespace sa
