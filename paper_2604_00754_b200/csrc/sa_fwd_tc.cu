@@ -50,6 +50,19 @@ enum Src { kGather = 0, kNatural = 1, kOrdered = 2 };
 constexpr int kRowWarps = 8, kThreads = 32 * (kRowWarps + 4);
 __host__ __device__ constexpr int issuers(int d) { return d == 64 ? 2 : 1; }
 
+// Division of numbers below 2^31 by one known at the launch: a multiplication and a shift, where the
+// division proper costs every warp some twenty instructions, five times per item.
+struct FastDiv {
+  uint32_t mul = 0;
+  int shift = 0;
+  FastDiv() = default;
+  explicit FastDiv(uint32_t d) {
+    while ((1ull << shift) < d) ++shift;
+    mul = (uint32_t)((((1ull << shift) - d) << 32) / d + 1);
+  }
+  __device__ __forceinline__ int of(int x) const { return (int)((__umulhi((uint32_t)x, mul) + (uint32_t)x) >> shift); }
+};
+
 struct TcParams {
   const void *q, *k, *v;
   const int32_t* perm;        // null for the SWA branch
@@ -67,6 +80,7 @@ struct TcParams {
   int n_tiles;                // slot tiles of 128
   int items_per_kv;           // work items per (b, hk)
   int total_items;
+  FastDiv by_items, by_kv, by_inner, by_full;   // items_per_kv, Hkv; make_geo / ordered_tiles
   float scale2;               // softmax scale * log2(e)
   OrderView order;            // kOrdered: what sa_order.cu made
   OrderGeom og;
@@ -75,6 +89,14 @@ struct TcParams {
 };
 
 // ------------------------------------------------------------------------- geometry
+
+// Work item -> item of a KV head, KV head, sequence.
+struct Place { int item, hk, b; };
+
+__device__ __forceinline__ Place place_of(const TcParams& p, int w_item) {
+  const int bh = p.by_items.of(w_item), b = p.by_kv.of(bh);
+  return {w_item - bh * p.items_per_kv, bh - b * p.Hkv, b};
+}
 
 struct Geo {
   int q0[2];        // first slot of each query tile
@@ -125,14 +147,14 @@ __device__ __forceinline__ Geo make_geo(const TcParams& p, int item, int hk) {
   Geo g;
   if (p.pair_heads) {
     const int pairs = p.G / 2;
-    const int tile = item / pairs, pr = item % pairs;
+    const int tile = p.by_inner.of(item), pr = item - tile * pairs;
     g.q0[0] = g.q0[1] = tile * kTile;
     g.hq[0] = hk * p.G + 2 * pr;
     g.hq[1] = g.hq[0] + 1;
     g.valid[0] = g.valid[1] = 1;
   } else {
     const int tpairs = (p.n_tiles + 1) / 2;
-    const int tp = item % tpairs, hh = item / tpairs;
+    const int hh = p.by_inner.of(item), tp = item - hh * tpairs;
     g.q0[0] = 2 * tp * kTile;
     g.q0[1] = g.q0[0] + kTile;
     g.hq[0] = g.hq[1] = hk * p.G + hh;
@@ -166,10 +188,10 @@ __device__ __forceinline__ void ordered_tiles(const TcParams& p, int item, int h
   const int per_unit = p.pair_heads ? 1 : 2, units = p.og.slots / (kTile * per_unit);
   const int full = p.n_tiles / (units * per_unit);                   // groups with all their tiles
   const int heads = p.pair_heads ? p.G / 2 : p.G;
-  const int x = item / heads, hh = item - x * heads;
+  const int x = p.by_inner.of(item), hh = item - x * heads;
   int unit = x;
   if (x < full * units) {
-    const int cls = x / full;
+    const int cls = p.by_full.of(x);
     unit = (x - cls * full) * units + units - 1 - cls;
   }
   tile[0] = unit * per_unit;
@@ -366,8 +388,8 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
         return mbar_wait(bar(C::kBarFree + e % C::kEvents), (e / C::kEvents) & 1u, gave_up, p.status);
       };
       for (int w_item = blockIdx.x; w_item < p.total_items && live; w_item += gridDim.x, ++it) {
-        const int item = w_item % p.items_per_kv, bh = w_item / p.items_per_kv;
-        const int hk = bh % p.Hkv, b = bh / p.Hkv;
+        const Place at = place_of(p, w_item);
+        const int item = at.item, hk = at.hk, b = at.b;
         const Geo g = make_geo(p, item, hk);
         for (int j = 0; j < g.T; ++j, ++gt) {
           const uint32_t pr = gt % C::kRing;
@@ -540,8 +562,8 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
 
     bool live = true;
     for (int w_item = blockIdx.x; w_item < p.total_items && live; w_item += gridDim.x, ++it) {
-      const int item = w_item % p.items_per_kv, bh = w_item / p.items_per_kv;
-      const int hk = bh % p.Hkv, b = bh / p.Hkv;
+      const Place at = place_of(p, w_item);
+      const int item = at.item, hk = at.hk, b = at.b;
       const Geo g = geo_of(item, hk, b);
       const int32_t* perm = p.perm ? p.perm + (size_t)b * p.n : nullptr;
       const int32_t* list = nullptr;           // kOrdered: the group's keys
@@ -672,8 +694,8 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
         if (NB == 2) tc_commit(bar(C::kBarPvDone + t));
       };
       for (int w_item = blockIdx.x; w_item < p.total_items && ok; w_item += gridDim.x, ++it) {
-        const int item = w_item % p.items_per_kv, bh = w_item / p.items_per_kv;
-        const Geo g = geo_of(item, bh % p.Hkv, bh / p.Hkv);
+        const Place at = place_of(p, w_item);
+        const Geo g = geo_of(at.item, at.hk, at.b);
         const int H = NB * g.T;         // score blocks of this item
         // half-steps [first, last] that each query tile takes part in (a contiguous range)
         int first[kN], last[kN];
@@ -745,9 +767,6 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
     bool ok = true;
 
     // ------------------------------------------------------------------- epilogue
-    // It runs behind the softmax of the next item's first block: the registers of the scores are free,
-    // the last P V is over, and while O goes out the tensor core has this block's P V and the next
-    // scores to do.  What it needs until then waits in the warp's staging rows.
     // A thread holds a row, so storing from the registers would touch 32 lines per instruction
     // (4000 cycles per item).  Each warp turns 32 rows x 64 columns at a time in 4 KB of shared
     // memory (16-byte pieces, swizzled by the row number): 8 lanes then store 128 consecutive
@@ -786,21 +805,11 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
     auto take = [&](Done* it, uint32_t (&out)[D / 2]) {
       {
         // (opaque: nothing of the epilogue is worked out ahead and kept across the softmax)
-        uint32_t rec[4];
         it->stage = stage;
         it->lane = lane;
         asm volatile("" : "+r"(it->lane));
         it->prow = it->lane >> 3;
         it->pc = it->lane & 7;
-        lds128(rec, stage + it->lane * 128);
-        it->m = __uint_as_float(rec[0]);
-        it->l = __uint_as_float(rec[1]);
-        it->tok = (int)rec[2];
-        it->hq = (int)rec[3];
-        lds128(rec, stage + it->lane * 128 + 16);
-        it->b = (int)rec[0];
-        it->q0 = (int)rec[1];
-        __syncwarp();
       }
       it->g_this = 1.f;
       it->g_other = 0.f;
@@ -900,24 +909,23 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
       if (p.lse && it.q0 + row < p.n)
         p.lse[((size_t)it.b * p.Hq + it.hq) * p.n + it.tok] = (it.m * p.scale2 + log2f(it.l)) * kLn2;
     };
-    bool pending = false;
     // gathered branch: an item's tokens are fetched while the one before is worked on
     auto token_of = [&](int w_item) {
       if (SRC != kGather || !p.perm || w_item >= p.total_items) return 0;
-      const int bh = w_item / p.items_per_kv;
-      const Geo g = make_geo(p, w_item % p.items_per_kv, bh % p.Hkv);
+      const Place at = place_of(p, w_item);
+      const Geo g = make_geo(p, at.item, at.hk);
       const int slot = (t ? g.q0[1] : g.q0[0]) + row;
-      return slot < p.n ? p.perm[(size_t)(bh / p.Hkv) * p.n + slot] : 0;
+      return slot < p.n ? p.perm[(size_t)at.b * p.n + slot] : 0;
     };
     int next_tok = token_of(blockIdx.x);
 
     for (int w_item = blockIdx.x; w_item < p.total_items && ok; w_item += gridDim.x) {
-      const int item = w_item % p.items_per_kv, bh = w_item / p.items_per_kv;
-      const int b = bh / p.Hkv;
+      const Place at = place_of(p, w_item);
+      const int b = at.b;
       int q0, hq, kstart, first, last, in_lo, in_hi;
       const uint32_t gt0 = gt;
       {
-        const Geo g = geo_of(item, bh % p.Hkv, b);
+        const Geo g = geo_of(at.item, at.hk, b);
         q0 = t ? g.q0[1] : g.q0[0];
         hq = t ? g.hq[1] : g.hq[0];
         kstart = g.kstart;
@@ -1101,34 +1109,24 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
         }
         l += lsum.x + lsum.y;
         tmem_wait_st();
-        if (pending) {
-          uint32_t out[D / 2];
-          Done it;
-          if (!take(&it, out)) break;
-          tc_fence_before();
-          mbar_arrive(bar(C::kBarPReady + 2 * t + hb));
-          put(it, out);
-          pending = false;
-        } else {
-          tc_fence_before();
-          mbar_arrive(bar(C::kBarPReady + 2 * t + hb));
-        }
+        tc_fence_before();
+        mbar_arrive(bar(C::kBarPReady + 2 * t + hb));
         ++pv_cnt;                           // the issuer answers every arrive with one P V
       }
       if (!ok) break;
 
-      // the next item's first P V overwrites O: it is let start once O has been taken
-      pending = true;
-      uint32_t rec[4] = {__float_as_uint(m), __float_as_uint(l), (uint32_t)q_tok, (uint32_t)hq};
-      sts128(stage + lane * 128, rec);
-      rec[0] = (uint32_t)b;
-      rec[1] = (uint32_t)q0;
-      sts128(stage + lane * 128 + 16, rec);
-    }
-    if (ok && pending) {
-      uint32_t out[D / 2];
       Done it;
-      if (take(&it, out)) put(it, out);
+      it.m = m;
+      it.l = l;
+      it.tok = q_tok;
+      it.hq = hq;
+      it.b = b;
+      it.q0 = q0;
+      uint32_t out[D / 2];
+      if (!take(&it, out)) break;
+      put(it, out);
+      // the next item's first P V overwrites O: order these reads before the arrive that lets it start
+      tc_fence_before();
     }
   }
 
@@ -1217,6 +1215,10 @@ cudaError_t launch_fwd_tc(const FwdArgs& a, cudaStream_t st) {
     p.order = order_view(a.lists, a.B, p.og);
   }
   p.total_items = a.B * a.Hkv * p.items_per_kv;
+  p.by_items = FastDiv(p.items_per_kv);
+  p.by_kv = FastDiv(a.Hkv);
+  p.by_inner = FastDiv(p.pair_heads ? p.G / 2 : ordered ? p.G : (p.n_tiles + 1) / 2);
+  p.by_full = FastDiv(ordered ? max(p.n_tiles / (p.og.slots / kTile), 1) : 1);
 
   static int sm_count[64] = {0};
   int dev = 0;
