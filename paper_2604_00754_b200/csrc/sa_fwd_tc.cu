@@ -787,6 +787,7 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
         return stage + (4 * i + prow) * 128 + ((pc ^ (prow + (i & 1) * 4)) << 4);
       }
     };
+    using Others = uint4[COMBINE ? D / 64 : 1][kPieces];   // the other branch's rows, as they are moved
     auto at_row = [&](const Done& it, int i) {
       return it.b * p.qs[0] + it.hq * p.qs[1] + it.pc * 8 +
              (int64_t)__shfl_sync(0xffffffffu, it.tok, 4 * i + it.prow) * p.qs[2];
@@ -802,7 +803,7 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
       }
     };
     // O of the item before, normalised and rounded, two columns a word
-    auto take = [&](Done* it, uint32_t (&out)[D / 2]) {
+    auto take = [&](Done* it, uint32_t (&out)[D / 2], Others& oth) {
       {
         // (opaque: nothing of the epilogue is worked out ahead and kept across the softmax)
         it->stage = stage;
@@ -820,12 +821,18 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
         it->g_other = p.swa ? s_sa : s_swa;
       }
       if (kLateWait) grid_dependency_wait();
+      if constexpr (COMBINE) {
+#pragma unroll
+        for (int hf = 0; hf < D / 64; ++hf) load_other(*it, hf, oth[hf]);
+      }
+      ok = mbar_wait(bar(C::kBarODone + t), o_cnt & 1u, gave_up, p.status);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) return false;
+      ++o_cnt;
+      tc_fence_after();
       const bool mix = COMBINE && !p.y_branch;   // the gates act on unrounded local rows:
       if constexpr (COMBINE) {                   // the other row goes to the row's thread
         if (mix) {
-          uint4 oth[D / 64][kPieces];
-#pragma unroll
-          for (int hf = 0; hf < D / 64; ++hf) load_other(*it, hf, oth[hf]);
 #pragma unroll
           for (int hf = 0; hf < D / 64; ++hf) {
 #pragma unroll
@@ -842,11 +849,6 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
           for (int x = 0; x < D / 2; ++x) out[x] = 0u;
         }
       }
-      ok = mbar_wait(bar(C::kBarODone + t), o_cnt & 1u, gave_up, p.status);
-      ok = __all_sync(0xffffffffu, ok);
-      if (!ok) return false;
-      ++o_cnt;
-      tc_fence_after();
       const float inv_l = 1.f / it->l;
 #pragma unroll
       for (int c = 0; c < D; c += 32) {
@@ -868,12 +870,9 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
       return true;
     };
     // the rows taken go out
-    auto put = [&](const Done& it, uint32_t (&out)[D / 2]) {
+    auto put = [&](const Done& it, uint32_t (&out)[D / 2], const Others& oth) {
 #pragma unroll
       for (int hf = 0; hf < D / 64; ++hf) {
-        uint4 oth[COMBINE ? kPieces : 1] = {};
-        if constexpr (COMBINE)
-          if (p.y_branch) load_other(it, hf, oth);
 #pragma unroll
         for (int x = 0; x < kPieces; ++x)
           sts128(it.piece(x), reinterpret_cast<const uint32_t(&)[4]>(out[32 * hf + 4 * x]));
@@ -888,7 +887,7 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
               // both branches as they are stored, and as the backward pass will read them
               if (have(it, i))
                 *reinterpret_cast<uint4*>((__nv_bfloat16*)p.y_branch + e) = make_uint4(v[0], v[1], v[2], v[3]);
-              const __nv_bfloat162* ho = reinterpret_cast<const __nv_bfloat162*>(&oth[i]);
+              const __nv_bfloat162* ho = reinterpret_cast<const __nv_bfloat162*>(&oth[hf][i]);
 #pragma unroll
               for (int c = 0; c < 4; ++c) {
                 const float2 w = __bfloat1622float2(ho[c]);
@@ -902,23 +901,13 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
           if (have(it, i))
             *reinterpret_cast<uint4*>((__nv_bfloat16*)p.y + e) = make_uint4(v[0], v[1], v[2], v[3]);
         }
-        // y may be the buffer the other branch's rows sit in: these columns are read before the
-        // same columns are written, and nobody else touches them
+        // y may be the buffer the other branch's rows sit in: they are read before they are written,
+        // and nobody else touches them
         __syncwarp();
       }
       if (p.lse && it.q0 + row < p.n)
         p.lse[((size_t)it.b * p.Hq + it.hq) * p.n + it.tok] = (it.m * p.scale2 + log2f(it.l)) * kLn2;
     };
-    // gathered branch: an item's tokens are fetched while the one before is worked on
-    auto token_of = [&](int w_item) {
-      if (SRC != kGather || !p.perm || w_item >= p.total_items) return 0;
-      const Place at = place_of(p, w_item);
-      const Geo g = make_geo(p, at.item, at.hk);
-      const int slot = (t ? g.q0[1] : g.q0[0]) + row;
-      return slot < p.n ? p.perm[(size_t)at.b * p.n + slot] : 0;
-    };
-    int next_tok = token_of(blockIdx.x);
-
     for (int w_item = blockIdx.x; w_item < p.total_items && ok; w_item += gridDim.x) {
       const Place at = place_of(p, w_item);
       const int b = at.b;
@@ -932,13 +921,12 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
         gt += g.T;
         active_of(g, t, NB * g.T, kShift, &first, &last);
       }
-      const int this_tok = next_tok;
-      next_tok = token_of(w_item + gridDim.x);
       if (first > last) continue;           // no such tile
       if (SRC != kOrdered) inner_range(p, q0, kHalf, &in_lo, &in_hi);
       const int qv = q0 + row;
       const bool row_valid = qv < p.n;
-      int q_tok = SRC == kGather && p.perm ? this_tok : row_valid ? qv : 0;
+      int q_tok = 0;
+      if (SRC != kOrdered && row_valid) q_tok = p.perm ? p.perm[(size_t)b * p.n + qv] : qv;
       const uint4* bits = nullptr;            // kOrdered: what this row sees, block by block
       uint4 seen_next = make_uint4(0u, 0u, 0u, 0u);
       if constexpr (SRC == kOrdered) {
@@ -1007,7 +995,6 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
             p.causal && !p.one_sided && !(p.swa && kv >= 0 && kv + kHalf - 1 <= q0);
         if constexpr (SRC == kOrdered) {
           const uint4 seen4 = seen_next;
-          if (h < last) seen_next = __ldcg(bits + (size_t)(h + 1) * kTile);
           const uint32_t seen[4] = {seen4.x, seen4.y, seen4.z, seen4.w};
 #pragma unroll
           for (int c0 = 0; c0 < kHalf; c0 += 32) {
@@ -1111,6 +1098,10 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
         tmem_wait_st();
         tc_fence_before();
         mbar_arrive(bar(C::kBarPReady + 2 * t + hb));
+        // (here, where the warp would wait: the gathering warps keep the load unit's queue full, and a
+        // warp that joins it between its mask and its exponentials holds its tile up)
+        if constexpr (SRC == kOrdered)
+          if (h < last) seen_next = __ldcg(bits + (size_t)(h + 1) * kTile);
         ++pv_cnt;                           // the issuer answers every arrive with one P V
       }
       if (!ok) break;
@@ -1123,8 +1114,9 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
       it.b = b;
       it.q0 = q0;
       uint32_t out[D / 2];
-      if (!take(&it, out)) break;
-      put(it, out);
+      Others oth;
+      if (!take(&it, out, oth)) break;
+      put(it, out, oth);
       // the next item's first P V overwrites O: order these reads before the arrive that lets it start
       tc_fence_before();
     }
