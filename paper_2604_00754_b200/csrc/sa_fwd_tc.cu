@@ -766,148 +766,6 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
     uint32_t s_cnt0 = 0, s_cnt1 = 0, o_cnt = 0, pv_cnt = 0, gt = 0;
     bool ok = true;
 
-    // ------------------------------------------------------------------- epilogue
-    // A thread holds a row, so storing from the registers would touch 32 lines per instruction
-    // (4000 cycles per item).  Each warp turns 32 rows x 64 columns at a time in 4 KB of shared
-    // memory (16-byte pieces, swizzled by the row number): 8 lanes then store 128 consecutive
-    // bytes of a row, 4 rows per instruction.  The other branch's rows come in the same way.
-    // Measured with the ring of the loads (8 x 12 heads of 64, n = 4096, w = 128, gated):
-    // 346 -> 307 us; 32/8 heads of 128, n = 32768, w = 1024: 1711 -> 1605.
-    constexpr int kPieces = 8;                       // 16-byte pieces of 64 columns = row groups
-    const uint32_t stage = sbase + C::kOffStage + warp * 4096;
-    struct Done {
-      float m, l, g_this, g_other;
-      int tok, hq, b, q0;
-      uint32_t stage;
-      int lane, prow, pc;                            // it moves piece pc of rows prow, prow + 4, ...
-      __device__ __forceinline__ uint32_t piece(int x) const {    // of this lane's row
-        return stage + lane * 128 + ((x ^ (lane & 7)) << 4);
-      }
-      __device__ __forceinline__ uint32_t turned(int i) const {   // its piece of row 4 i + prow
-        return stage + (4 * i + prow) * 128 + ((pc ^ (prow + (i & 1) * 4)) << 4);
-      }
-    };
-    using Others = uint4[COMBINE ? D / 64 : 1][kPieces];   // the other branch's rows, as they are moved
-    auto at_row = [&](const Done& it, int i) {
-      return it.b * p.qs[0] + it.hq * p.qs[1] + it.pc * 8 +
-             (int64_t)__shfl_sync(0xffffffffu, it.tok, 4 * i + it.prow) * p.qs[2];
-    };
-    auto have = [&](const Done& it, int i) { return it.q0 + quad * 32 + 4 * i + it.prow < p.n; };
-    auto load_other = [&](const Done& it, int hf, uint4 (&oth)[kPieces]) {
-#pragma unroll
-      for (int i = 0; i < kPieces; ++i) {
-        oth[i] = make_uint4(0u, 0u, 0u, 0u);
-        const int64_t at = at_row(it, i);
-        if (have(it, i))
-          oth[i] = __ldcg(reinterpret_cast<const uint4*>((const __nv_bfloat16*)p.y_other + at + 64 * hf));
-      }
-    };
-    // O of the item before, normalised and rounded, two columns a word
-    auto take = [&](Done* it, uint32_t (&out)[D / 2], Others& oth) {
-      {
-        // (opaque: nothing of the epilogue is worked out ahead and kept across the softmax)
-        it->stage = stage;
-        it->lane = lane;
-        asm volatile("" : "+r"(it->lane));
-        it->prow = it->lane >> 3;
-        it->pc = it->lane & 7;
-      }
-      it->g_this = 1.f;
-      it->g_other = 0.f;
-      if (COMBINE) {
-        const float s_sa = 1.f / (1.f + __expf(-p.gate_logits[it->hq]));
-        const float s_swa = 1.f / (1.f + __expf(-p.gate_logits[p.Hq + it->hq]));
-        it->g_this = p.swa ? s_swa : s_sa;
-        it->g_other = p.swa ? s_sa : s_swa;
-      }
-      if (kLateWait) grid_dependency_wait();
-      if constexpr (COMBINE) {
-#pragma unroll
-        for (int hf = 0; hf < D / 64; ++hf) load_other(*it, hf, oth[hf]);
-      }
-      ok = mbar_wait(bar(C::kBarODone + t), o_cnt & 1u, gave_up, p.status);
-      ok = __all_sync(0xffffffffu, ok);
-      if (!ok) return false;
-      ++o_cnt;
-      tc_fence_after();
-      const bool mix = COMBINE && !p.y_branch;   // the gates act on unrounded local rows:
-      if constexpr (COMBINE) {                   // the other row goes to the row's thread
-        if (mix) {
-#pragma unroll
-          for (int hf = 0; hf < D / 64; ++hf) {
-#pragma unroll
-            for (int i = 0; i < kPieces; ++i)
-              sts128(it->turned(i), reinterpret_cast<uint32_t(&)[4]>(oth[hf][i]));
-            __syncwarp();
-#pragma unroll
-            for (int x = 0; x < kPieces; ++x)
-              lds128(reinterpret_cast<uint32_t(&)[4]>(out[32 * hf + 4 * x]), it->piece(x));
-            __syncwarp();
-          }
-        } else {                                 // (never left undefined: they would count as live before)
-#pragma unroll
-          for (int x = 0; x < D / 2; ++x) out[x] = 0u;
-        }
-      }
-      const float inv_l = 1.f / it->l;
-#pragma unroll
-      for (int c = 0; c < D; c += 32) {
-        uint32_t raw[32];
-        tmem_ld32(o_addr + c, raw);
-        tmem_wait_ld();
-#pragma unroll
-        for (int x = 0; x < 16; ++x) {
-          float2 o = make_float2(__uint_as_float(raw[2 * x]) * inv_l, __uint_as_float(raw[2 * x + 1]) * inv_l);
-          if (COMBINE && mix) {
-            const float2 w = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&out[c / 2 + x]));
-            o.x = fmaf(it->g_other, w.x, o.x * it->g_this);
-            o.y = fmaf(it->g_other, w.y, o.y * it->g_this);
-          }
-          const __nv_bfloat162 h2 = __floats2bfloat162_rn(o.x, o.y);
-          out[c / 2 + x] = *reinterpret_cast<const uint32_t*>(&h2);
-        }
-      }
-      return true;
-    };
-    // the rows taken go out
-    auto put = [&](const Done& it, uint32_t (&out)[D / 2], const Others& oth) {
-#pragma unroll
-      for (int hf = 0; hf < D / 64; ++hf) {
-#pragma unroll
-        for (int x = 0; x < kPieces; ++x)
-          sts128(it.piece(x), reinterpret_cast<const uint32_t(&)[4]>(out[32 * hf + 4 * x]));
-        __syncwarp();
-#pragma unroll
-        for (int i = 0; i < kPieces; ++i) {
-          uint32_t v[4];
-          lds128(v, it.turned(i));
-          const int64_t e = at_row(it, i) + 64 * hf;
-          if constexpr (COMBINE) {
-            if (p.y_branch) {
-              // both branches as they are stored, and as the backward pass will read them
-              if (have(it, i))
-                *reinterpret_cast<uint4*>((__nv_bfloat16*)p.y_branch + e) = make_uint4(v[0], v[1], v[2], v[3]);
-              const __nv_bfloat162* ho = reinterpret_cast<const __nv_bfloat162*>(&oth[hf][i]);
-#pragma unroll
-              for (int c = 0; c < 4; ++c) {
-                const float2 w = __bfloat1622float2(ho[c]);
-                const float2 u = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&v[c]));
-                const __nv_bfloat162 h2 = __floats2bfloat162_rn(fmaf(it.g_other, w.x, u.x * it.g_this),
-                                                                fmaf(it.g_other, w.y, u.y * it.g_this));
-                v[c] = *reinterpret_cast<const uint32_t*>(&h2);
-              }
-            }
-          }
-          if (have(it, i))
-            *reinterpret_cast<uint4*>((__nv_bfloat16*)p.y + e) = make_uint4(v[0], v[1], v[2], v[3]);
-        }
-        // y may be the buffer the other branch's rows sit in: they are read before they are written,
-        // and nobody else touches them
-        __syncwarp();
-      }
-      if (p.lse && it.q0 + row < p.n)
-        p.lse[((size_t)it.b * p.Hq + it.hq) * p.n + it.tok] = (it.m * p.scale2 + log2f(it.l)) * kLn2;
-    };
     for (int w_item = blockIdx.x; w_item < p.total_items && ok; w_item += gridDim.x) {
       const Place at = place_of(p, w_item);
       const int b = at.b;
@@ -1001,7 +859,7 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
             next32(c0);
 #pragma unroll
             for (int c = 0; c < 32; ++c)
-              if (!(seen[c0 / 32] & (1u << ((c & 1) * 16 + c / 2)))) sr[c0 + c] = 0xff800000u;
+              if (!(seen[c0 / 32] & (1u << c))) sr[c0 + c] = 0xff800000u;
           }
         } else if (kv >= in_lo && kv <= in_hi) {
           if (tokens_matter) {
@@ -1106,18 +964,125 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
       }
       if (!ok) break;
 
-      Done it;
-      it.m = m;
-      it.l = l;
-      it.tok = q_tok;
-      it.hq = hq;
-      it.b = b;
-      it.q0 = q0;
-      uint32_t out[D / 2];
-      Others oth;
-      if (!take(&it, out, oth)) break;
-      put(it, out, oth);
-      // the next item's first P V overwrites O: order these reads before the arrive that lets it start
+      // ------------------------------------------------------------------- epilogue
+      // A thread holds a row, so storing from the registers would touch 32 lines per instruction
+      // (4000 cycles per item).  Each warp turns 32 rows x 64 columns at a time in 4 KB of shared
+      // memory (16-byte pieces, swizzled by the row number): 8 lanes then store 128 consecutive
+      // bytes of a row, 4 rows per instruction.  The other branch's rows come in the same way.
+      // Measured with the ring of the loads (8 x 12 heads of 64, n = 4096, w = 128, gated):
+      // 346 -> 307 us; 32/8 heads of 128, n = 32768, w = 1024: 1711 -> 1605.
+      constexpr int kPieces = 8;                       // 16-byte pieces of 64 columns = row groups
+      const int prow = lane >> 3, pc = lane & 7;       // piece pc of rows prow, prow + 4, ...
+      const uint32_t stage = sbase + C::kOffStage + warp * 4096;
+      const uint32_t own_row = stage + lane * 128;
+      auto turned = [&](int i) {                       // this lane's piece of row 4 i + prow
+        const int r = 4 * i + prow;
+        return stage + r * 128 + ((pc ^ (r & 7)) << 4);
+      };
+      const int64_t base = b * p.qs[0] + hq * p.qs[1] + pc * 8;
+      int64_t at_row[kPieces];
+      bool have[kPieces];
+#pragma unroll
+      for (int i = 0; i < kPieces; ++i) {
+        at_row[i] = base + (int64_t)__shfl_sync(0xffffffffu, q_tok, 4 * i + prow) * p.qs[2];
+        have[i] = q0 + quad * 32 + 4 * i + prow < p.n;
+      }
+      if (kLateWait) grid_dependency_wait();
+      uint4 oth[COMBINE ? kPieces : 1];
+      auto load_other = [&](int hf) {
+        if constexpr (COMBINE) {
+#pragma unroll
+          for (int i = 0; i < kPieces; ++i) {
+            oth[i] = make_uint4(0u, 0u, 0u, 0u);
+            if (have[i])
+              oth[i] = __ldcg(reinterpret_cast<const uint4*>((const __nv_bfloat16*)p.y_other +
+                                                             at_row[i] + 64 * hf));
+          }
+        }
+      };
+      load_other(0);
+      float g_this = 1.f, g_other = 0.f;
+      if (COMBINE) {
+        const float s_sa = 1.f / (1.f + __expf(-p.gate_logits[hq]));
+        const float s_swa = 1.f / (1.f + __expf(-p.gate_logits[p.Hq + hq]));
+        g_this = p.swa ? s_swa : s_sa;
+        g_other = p.swa ? s_sa : s_swa;
+      }
+
+      ok = mbar_wait(bar(C::kBarODone + t), o_cnt & 1u, gave_up, p.status);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+      ++o_cnt;
+      tc_fence_after();
+      const float inv_l = 1.f / l;
+#pragma unroll
+      for (int hf = 0; hf < D / 64; ++hf) {
+        uint32_t raw[64];
+        tmem_ld32(o_addr + 64 * hf, reinterpret_cast<uint32_t(&)[32]>(raw[0]));
+        tmem_ld32(o_addr + 64 * hf + 32, reinterpret_cast<uint32_t(&)[32]>(raw[32]));
+        if (COMBINE && !p.y_branch) {
+          // the gates act on unrounded local rows: the other row goes to the row's thread
+#pragma unroll
+          for (int i = 0; i < kPieces; ++i) sts128(turned(i), reinterpret_cast<uint32_t(&)[4]>(oth[i]));
+          __syncwarp();
+        }
+        tmem_wait_ld();
+        // piece x of this thread's row: 8 output columns, normalised
+#pragma unroll
+        for (int x = 0; x < kPieces; ++x) {
+          float o[8];
+#pragma unroll
+          for (int c = 0; c < 8; ++c) o[c] = __uint_as_float(raw[8 * x + c]) * inv_l;
+          const uint32_t at = own_row + ((x ^ (lane & 7)) << 4);
+          uint32_t st[4];
+          if (COMBINE && !p.y_branch) {
+            lds128(st, at);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+              const float2 w = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&st[c]));
+              o[2 * c] = fmaf(g_other, w.x, o[2 * c] * g_this);
+              o[2 * c + 1] = fmaf(g_other, w.y, o[2 * c + 1] * g_this);
+            }
+          }
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            const __nv_bfloat162 h2 = __floats2bfloat162_rn(o[2 * c], o[2 * c + 1]);
+            st[c] = *reinterpret_cast<const uint32_t*>(&h2);
+          }
+          sts128(at, st);
+        }
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < kPieces; ++i) {
+          uint32_t v[4];
+          lds128(v, turned(i));
+          const int64_t e = at_row[i] + 64 * hf;
+          if (COMBINE && p.y_branch) {
+            // both branches as they are stored, and as the backward pass will read them
+            if (have[i])
+              *reinterpret_cast<uint4*>((__nv_bfloat16*)p.y_branch + e) = make_uint4(v[0], v[1], v[2], v[3]);
+            const __nv_bfloat162* ho = reinterpret_cast<const __nv_bfloat162*>(&oth[i]);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+              const float2 w = __bfloat1622float2(ho[c]);
+              const float2 u = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&v[c]));
+              const __nv_bfloat162 h2 = __floats2bfloat162_rn(fmaf(g_other, w.x, u.x * g_this),
+                                                              fmaf(g_other, w.y, u.y * g_this));
+              v[c] = *reinterpret_cast<const uint32_t*>(&h2);
+            }
+          }
+          if (have[i])
+            *reinterpret_cast<uint4*>((__nv_bfloat16*)p.y + e) = make_uint4(v[0], v[1], v[2], v[3]);
+        }
+        // y may be the buffer the other branch's rows sit in: these columns are read before the
+        // same columns are written, and nobody else touches them
+        if (hf + 1 < D / 64) load_other(hf + 1);
+        __syncwarp();
+      }
+      if (p.lse && row_valid)
+        p.lse[((size_t)b * p.Hq + hq) * p.n + q_tok] = (m * p.scale2 + log2f(l)) * kLn2;
+      // the next item's first P V overwrites O: order these reads before the arrive that
+      // lets it start
       tc_fence_before();
     }
   }

@@ -172,8 +172,16 @@ __global__ void __launch_bounds__(kThreads) order_kernel(const __grid_constant__
 #pragma unroll
         for (int e = 0; e < 4; ++e) v = (v >> 1) | ((o[e] - from) & ~(o[e] - past) & 0x80008000u);
       }
-      const int upto = min(max(pos + 1 - x0, 0), 32), even = (upto + 1) >> 1, odd = upto >> 1;
-      word[y] = v & (((1u << even) - 1u) | (((1u << odd) - 1u) << 16));
+      // the even keys are in the lower half, the odd in the upper: merge them
+      uint32_t even = v & 0xffffu, odd = v >> 16;
+#pragma unroll
+      for (int e = 8; e > 0; e >>= 1) {
+        const uint32_t keep = e == 8 ? 0x00ff00ffu : e == 4 ? 0x0f0f0f0fu : e == 2 ? 0x33333333u : 0x55555555u;
+        even = (even | (even << e)) & keep;
+        odd = (odd | (odd << e)) & keep;
+      }
+      const int upto = pos - x0;
+      word[y] = upto < 0 ? 0u : (even | (odd << 1)) & (upto >= 31 ? ~0u : (2u << upto) - 1u);
     }
     bits[(size_t)j * kOrderTile + r] = make_uint4(word[0], word[1], word[2], word[3]);
   }

@@ -13,11 +13,9 @@ struct OrderGeom {
   int blocks, pitch;       // most key blocks of a tile; tokens between two groups' lists
 };
 
-// bits: what a row sees of a block, four words of 32 keys; key 2 e of a word is its bit e, key
-// 2 e + 1 its bit 16 + e.
 struct OrderView {
   int32_t *q, *k, *tiles;  // [B, tiles, 128] query tokens; [B, groups, pitch] key tokens; [B, tiles] blocks
-  uint4* bits;             // [B, tiles, blocks, 128]
+  uint4* bits;             // [B, tiles, blocks, 128]: what a row sees of a block, one bit per key
 };
 
 // Whether the SA branch of such a problem walks token-ordered lists, and their geometry.  Depends on
