@@ -481,12 +481,13 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
       const uint32_t ts = (uint32_t)tok_stride * 2u;      // bytes
       const char* src0 = reinterpret_cast<const char*>(base + chunk * 8);
       const uint32_t dst0 = dst_tile + dst_lane + sub * 128;
-      int grp = pw;
-      for (; grp + 3 * kGWarps < kGroups; grp += 4 * kGWarps) {
+      int grp = pw, nth = 0;                       // group, the nth of this warp
+#pragma unroll 1
+      for (; grp + 3 * kGWarps < kGroups; grp += 4 * kGWarps, nth += 4) {
         const uint32_t d = dst0 + grp * (kRpi * 128);
         uint32_t tok[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) tok[k] = (uint32_t)tok_of((grp + kGWarps * k) * kRpi + sub);
+        for (int k = 0; k < 4; ++k) tok[k] = (uint32_t)tok_of((grp + kGWarps * k) * kRpi + sub, nth + k);
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
           const char* src = src0 + (uint64_t)tok[k] * ts;
@@ -494,9 +495,10 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
                        : "memory");
         }
       }
-      for (; grp < kGroups; grp += kGWarps) {
+#pragma unroll 1
+      for (; grp < kGroups; grp += kGWarps, ++nth) {
         const int r = grp * kRpi + sub;
-        const char* src = src0 + (uint64_t)(uint32_t)tok_of(r) * ts;
+        const char* src = src0 + (uint64_t)(uint32_t)tok_of(r, nth) * ts;
         const uint32_t dst = dst_tile + dst_lane + r * 128 + (((chunk & 7) ^ (r & 7)) << 4);
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
       }
@@ -584,6 +586,19 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
         const int slot = actual_slot(p, g.kstart + j * kTile + r);
         return perm ? perm[slot] : slot;
       };
+      // The tokens of a query tile come all at once, at most two per lane: those of the rows that this
+      // warp moves, in its order.  (Fetched group by group, each four groups waited for a load of their
+      // own: six times some 700 cycles per tile, with the tensor core idle.)
+      static_assert((kGroups + kGWarps - 1) / kGWarps * kRpi <= 64, "two tokens per lane");
+      int qt[2];
+      auto fetch_q = [&](int t) {
+#pragma unroll
+        for (int x = 0; x < 2; ++x) {
+          const int e = 32 * x + lane;
+          qt[x] = q_tok(t, min((pw + kGWarps * (e / kRpi)) * kRpi + e % kRpi, kTile - 1));
+        }
+      };
+      fetch_q(0);
       // tokens are fetched one tile ahead of their use
       int tk0 = key_tok(0, ptid), tk1 = ptid + kPt < kTile ? key_tok(0, ptid + kPt) : 0;
       for (int j = 0; j < g.T; ++j, ++gt) {
@@ -598,7 +613,7 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
         if (SRC == kGather && ptid == 0) mbar_arrive(bar(C::kBarTokFull + gt % C::kTok));
         const uint32_t k_dst = sbase + C::kOffRing + 2 * pr * C::kTileBytes;
         const uint32_t k_bar = bar(C::kBarSlotFull + 2 * pr);
-        auto tok_of = [&](int r) { return ktok[r]; };
+        auto tok_of = [&](int r, int = 0) { return ktok[r]; };
         gather(kb, p.ks[2], tok_of, k_dst);
         if (ROPE) commit_group(); else signal(k_bar);
         if (j + 1 < g.T) {
@@ -611,9 +626,14 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
             mbar_wait(bar(C::kBarQEmpty + it % C::kQBufs), (it / C::kQBufs - 1) & 1u, gave_up, p.status);
           if (group_sync_stop()) { live = false; break; }
 #pragma unroll 1
-          for (int t = 0; t < 2; ++t)
+          for (int t = 0; t < 2; ++t) {
+            if (t && !p.pair_heads) fetch_q(1);
             gather(qg + b * p.qs[0] + (t ? g.hq[1] : g.hq[0]) * p.qs[1], p.qs[2],
-                   [&](int r) { return q_tok(t, r); }, q_dst + t * C::kTileBytes);
+                   [&](int, int nth) {
+                     return __shfl_sync(0xffffffffu, nth < 32 / kRpi ? qt[0] : qt[1], (nth * kRpi + sub) & 31);
+                   },
+                   q_dst + t * C::kTileBytes);
+          }
           if (ROPE) commit_group(); else signal(q_bar);
         }
         // ---- V_j
