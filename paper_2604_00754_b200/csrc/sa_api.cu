@@ -118,7 +118,7 @@ sa_status maybe_validate(const sa_problem* p, const int32_t* perm, const int32_t
 
 // Scratch for the key lists, where there is enough of it.
 void* list_room(const sa_problem* p, void* lists, size_t bytes) {
-  const size_t need = key_list_bytes(p);
+  const size_t need = check_problem(p) == SA_OK ? key_list_bytes(p) : 0;
   return need && lists && aligned16(lists) && bytes >= need ? lists : nullptr;
 }
 
@@ -142,13 +142,15 @@ sa_status forward(const sa_problem* p, const void* q, const void* k, const void*
 size_t key_list_bytes(const sa_problem* p) {
   OrderGeom g;
   FwdArgs a = fwd_args(p, p, p, p, false);            // pointers unused by the test
-  return tc_forward_ordered(a, p->dtype, &g) ? order_bytes(p->B, g) : 0;
+  // Only where two heads of a group share an item: two tiles of one head share a stream that ends where
+  // the later one ends, and gain nothing (16 heads of 128, n = 8192, w = 1024: 158 us for 138).
+  return p->Hq / p->Hkv % 2 == 0 && tc_forward_ordered(a, p->dtype, &g) ? order_bytes(p->B, g) : 0;
 }
 
 sa_status gated_forward(const sa_problem* p, const void* q, const void* k, const void* v,
                         const int32_t* perm, const int32_t* inv, const float* gate_logits, void* y,
                         void* y_sa, void* y_swa, float* lse_sa, float* lse_swa, void* lists,
-                        size_t lists_bytes, bool lists_ready, cudaStream_t st) {
+                        bool lists_ready, cudaStream_t st) {
   sa_status s = check_problem(p);
   if (s != SA_OK) return s;
   if (!good_ptr(q) || !good_ptr(k) || !good_ptr(v) || !good_ptr(perm) || !good_ptr(inv) ||
@@ -168,7 +170,7 @@ sa_status gated_forward(const sa_problem* p, const void* q, const void* k, const
   void* sa_rows = y_sa ? y_sa : y;
   FwdArgs a = fwd_args(p, q, k, v, false);
   a.perm = perm; a.inv = inv; a.y = sa_rows; a.lse = lse_sa;
-  a.lists = list_room(p, lists, lists_bytes);
+  a.lists = lists;
   a.lists_ready = lists_ready;
   cudaError_t e = run_forward(a, p->dtype, st);
   if (e != cudaSuccess) return SA_ERR_CUDA;
@@ -265,16 +267,16 @@ sa_status sa_swa_gated_forward(const sa_problem* p, const void* q, const void* k
                                sa_stream_t stream) {
   if (ws && !aligned16(ws)) return SA_ERR_INVALID_ARG;
   (void)ws_bytes;
-  return gated_forward(p, q, k, v, perm, inv, gate_logits, y, y_sa, y_swa, lse_sa, lse_swa, nullptr, 0,
-                       false, (cudaStream_t)stream);
+  return gated_forward(p, q, k, v, perm, inv, gate_logits, y, y_sa, y_swa, lse_sa, lse_swa, nullptr, false,
+                       (cudaStream_t)stream);
 }
 
 sa_status sa_swa_gated_forward_lists(const sa_problem* p, const void* q, const void* k, const void* v,
                                      const int32_t* perm, const int32_t* inv, const float* gate_logits,
                                      void* y, void* y_sa, void* y_swa, float* lse_sa, float* lse_swa,
                                      void* ws, size_t ws_bytes, sa_stream_t stream) {
-  return gated_forward(p, q, k, v, perm, inv, gate_logits, y, y_sa, y_swa, lse_sa, lse_swa, ws, ws_bytes,
-                       false, (cudaStream_t)stream);
+  return gated_forward(p, q, k, v, perm, inv, gate_logits, y, y_sa, y_swa, lse_sa, lse_swa,
+                       list_room(p, ws, ws_bytes), false, (cudaStream_t)stream);
 }
 
 sa_status sa_rope_apply(const sa_problem* p, int32_t kv, const void* x, const float* rope_cos,

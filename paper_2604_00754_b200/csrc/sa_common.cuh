@@ -184,12 +184,12 @@ struct BwdArgs {
   const int* abort_flag;  // nullable: kernels return at once when it reads non-zero
 };
 
-// sa_swa_gated_forward with room for the SA branch's key lists, made by this call or (ready) by an
-// earlier one with the same permutation, n, w and flags.
+// sa_swa_gated_forward with room for the SA branch's key lists (null: without them), made by this call or
+// (ready) by an earlier one with the same permutation, n, w and flags.
 sa_status gated_forward(const sa_problem* p, const void* q, const void* k, const void* v,
                         const int32_t* perm, const int32_t* inv, const float* gate_logits, void* y,
                         void* y_sa, void* y_swa, float* lse_sa, float* lse_swa, void* lists,
-                        size_t lists_bytes, bool lists_ready, cudaStream_t st);
+                        bool lists_ready, cudaStream_t st);
 // Bytes of those lists; 0 where the branch does without.
 size_t key_list_bytes(const sa_problem* p);
 

@@ -356,13 +356,13 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
   SA_LEAVE_IF_SKIPPED(reinterpret_cast<volatile int*>(smem + C::kOffMisc + 8), kMmaWarp, tmem, kTmemCols)
 
   // Registers move from the issuer and producer warps to the row threads, which hold a whole score
-  // row each.  Per lane over the 12 warps: 4 x 56 + 8 x 224 = 2016, all that the launch holds
-  // (12 x 168).  The four warps of a warpgroup must ask for the same count, so the issuing
-  // warps and the producer warps go down together.  With 224 registers the 128 scores and the
-  // packed probabilities of a row thread stay in registers (at 208 they spilled).
-  // With ROPE the producers need room for the rotation: 4 x 72 + 8 x 216 = 2016 again.  (The
-  // sum may never exceed what the launch holds: a warpgroup asking for more waits for ever.)
-  constexpr int kLow = ROPE ? 72 : 56, kHigh = ROPE ? 216 : 224;
+  // row each.  Per lane over the 12 warps: 4 x 56 + 8 x 224 = 4 x 72 + 8 x 216 = 2016, all that the
+  // launch holds (12 x 168).  The four warps of a warpgroup must ask for the same count, so the issuing
+  // warps and the producer warps go down together.  72 where rows are gathered: at 56 the gathering
+  // warps spilled their tokens, and what they reload queues behind their own copies; the row threads
+  // keep their 128 scores at 216 as at 224 (at 208 they spilled).  (The sum may never exceed what the
+  // launch holds: a warpgroup asking for more waits for ever.)
+  constexpr int kLow = kRows ? 72 : 56, kHigh = kRows ? 216 : 224;
   static_assert(4 * kLow + kRowWarps * kHigh == (kRowWarps + 4) * 168, "register split");
   if (warp >= kRowWarps) {
   asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kLow));

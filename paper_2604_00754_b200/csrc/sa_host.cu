@@ -314,7 +314,7 @@ sa_status sa_swa_gated_forward_host(const sa_problem* p, const void* q, const vo
     const size_t qoff = ((size_t)g.b0 * p->Hq + g.qa) * head_bytes;
     const size_t koff = ((size_t)g.b0 * p->Hkv + g.ka) * head_bytes;
     st = gated_forward(&gp, dq + qoff, dk + koff, dv + koff, rperm, rinv, gates, dyv + qoff, nullptr, nullptr,
-                       nullptr, nullptr, lists, lists ? c.list_bytes : 0, lists_ready, pipe->s_run);
+                       nullptr, nullptr, lists, lists_ready, pipe->s_run);
     lists_ready = lists != nullptr;
     chk(cudaEventRecord(pipe->ev_done[i], pipe->s_run));
   }

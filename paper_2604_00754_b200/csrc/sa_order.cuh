@@ -18,8 +18,8 @@ struct OrderView {
   uint4* bits;             // [B, tiles, blocks, 128]: what a row sees of a block, one bit per key
 };
 
-// Whether the SA branch of such a problem walks token-ordered lists, and their geometry.  Depends on
-// nothing that a part of a batch or of the heads changes: a sequence has the same bits in either.
+// Whether the SA branch of such a problem can walk token-ordered lists, and their geometry.  Depends on
+// nothing that a part of a batch or of the KV heads changes: a sequence has the same bits in either.
 bool order_geom(int n, int d, int w, uint32_t flags, OrderGeom* g);
 size_t order_bytes(int B, const OrderGeom& g);
 OrderView order_view(void* ws, int B, const OrderGeom& g);
