@@ -1,0 +1,104 @@
+"""The causal SA branch over token-ordered key lists (wide windows, long sequences, an even number of
+query heads per KV head): rows against the float64 oracle, and against the same kernels without
+lists."""
+import ctypes
+
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2604_00754_b200 import binding as sa
+from paper_2604_00754_b200.workloads import CAUSAL, LINEAR_WINDOW, SWA_ONE_SIDED, as_f64
+
+KEY_LISTS = 8                                      # SA_OP_KEY_LISTS
+
+# groups of 256 and of 512 slots (w from 1281 on); last groups of one slot, of less than a tile, of an
+# odd number of tiles; both head dimensions; windows that wrap and windows that end with the sequence
+CASES = [
+    (1, 2, 1, 32768, 128, 1024, CAUSAL), (1, 4, 2, 32769, 64, 1280, CAUSAL),
+    (2, 2, 1, 32768 + 200, 64, 1025, CAUSAL | LINEAR_WINDOW), (1, 2, 1, 32768 + 300, 128, 1281, CAUSAL),
+    (1, 4, 1, 33000, 128, 2048, CAUSAL | LINEAR_WINDOW), (1, 2, 1, 32768 + 385, 64, 7000, CAUSAL),
+]
+
+
+def problem(Hq, Hkv, n, d, w, flags, B=1, dtype=sa.BF16):
+    p = sa.SaProblem(B=B, Hq=Hq, Hkv=Hkv, n=n, d=d, w=w, dtype=dtype, flags=flags)
+    sa.load_library().sa_problem_set_contiguous(ctypes.byref(p))
+    return p
+
+
+def test_which_problems_use_lists():
+    size = lambda *a, **k: sa.sa_workspace_bytes(problem(*a, **k), KEY_LISTS)
+    assert size(2, 1, 32768, 128, 1024, CAUSAL) > 32768 * 4
+    assert size(4, 2, 32768, 64, 1024, CAUSAL, B=2) == 2 * size(4, 2, 32768, 64, 1024, CAUSAL)
+    assert size(2, 1, 32768, 128, 1024, 0) == 0                        # nothing is hidden by token
+    assert size(2, 2, 32768, 128, 1024, CAUSAL) == 0                   # no two heads share a stream
+    assert size(2, 1, 32768, 128, 1024, CAUSAL, dtype=sa.F32) == 0
+    assert size(2, 1, 32768, 128, 32768, CAUSAL) == 0                  # a group's window over everything
+    assert size(2, 1, 32767, 128, 1024, CAUSAL) == size(2, 1, 32768, 128, 1023, CAUSAL) == 0
+    with pytest.raises(sa.SaError):
+        sa.sa_workspace_bytes(problem(3, 2, 32768, 128, 1024, CAUSAL), KEY_LISTS)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("B,Hq,Hkv,n,d,w,flags", CASES)
+def test_rows_against_the_oracle(B, Hq, Hkv, n, d, w, flags):
+    g = torch.Generator().manual_seed(n + w)
+    q, k, v = (torch.randn(B, h, n, d, generator=g).bfloat16() for h in (Hq, Hkv, Hkv))
+    dev = [t.cuda() for t in (q, k, v)]
+    perm, inv = sa.sa_make_perm(n, w, B, n)
+    y, lse = sa.sa_forward(*dev, perm, inv, w, flags, want_lse=True)
+    again = sa.sa_forward(*dev, perm, inv, w, flags)
+    assert torch.equal(y, again)
+    # the same call without scratch: every block of the window in slot order
+    p = sa.make_problem(dev[0], dev[1], w, flags)
+    plain, plse = torch.empty_like(y), torch.empty_like(lse)
+    at = lambda t: ctypes.c_void_p(t.data_ptr())
+    st = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    assert sa.load_library().sa_forward(ctypes.byref(p), *map(at, dev), at(perm), at(inv), at(plain), at(plse),
+                                        None, 0, st) == 0
+    assert sa.sa_read_status() == 0
+    assert not torch.equal(y, plain)
+    # two roundings of P and one of y on either side, each 2^-9 of a row's largest weight or value at most
+    assert (y.float() - plain.float()).norm() <= 1e-2 * plain.float().norm()
+    assert (lse - plse).abs().max() <= 1e-4            # fp32 sums of the same terms in another order
+    permc, invc = perm.cpu().numpy(), inv.cpu().numpy()
+    rng = np.random.default_rng(0)
+    # random rows, the first and last tokens, and the tokens of the first and last slots (the last group)
+    tokens = np.concatenate([[0, 1, n - 1], permc[-1, :2], permc[-1, -140:]])
+    rows = np.unique(np.concatenate([rng.integers(0, B * Hq * n, 1500), (B * Hq - 1) * n + tokens]))
+    ry, rl = oracle.forward_rows(0, *(as_f64(t) for t in (q, k, v)), permc, invc, w, flags, rows)
+    sel = torch.from_numpy(rows).cuda()
+    assert np.abs(as_f64(y.reshape(-1, d)[sel]) - ry).max() <= 2e-2 * np.abs(ry).max()
+    assert np.abs(as_f64(lse.reshape(-1)[sel]) - rl).max() <= 2e-2
+
+
+# a part of the heads, the rotated call and the host pipeline (whose pieces cut a group's heads) take the
+# same route and give the same bits
+@pytest.mark.gpu
+@pytest.mark.parametrize("w", [1024, 2000])
+def test_bits_of_a_part_and_of_the_host_pipeline(w):
+    from paper_2604_00754_b200.host import HostForward
+    n, d, flags = 33100, 64, CAUSAL | SWA_ONE_SIDED
+    g = torch.Generator().manual_seed(w)
+    q, k, v = (torch.randn(1, h, n, d, generator=g).bfloat16().pin_memory() for h in (4, 2, 2))
+    lg = torch.randn(2, 4, generator=g).pin_memory()
+    dev = [t.cuda() for t in (q, k, v)]
+    perm, inv = sa.sa_make_perm(7, 1, 1, n)
+    whole = sa.sa_swa_gated_forward(*dev, perm, inv, lg.cuda(), w, flags, save_for_bwd=True)
+    part = sa.sa_swa_gated_forward(dev[0][:, 2:], dev[1][:, 1:], dev[2][:, 1:], perm, inv,
+                                   lg[:, 2:].contiguous().cuda(), w, flags, save_for_bwd=True,
+                                   out={x: torch.empty_like(dev[0])[:, 2:] for x in ("y", "y_sa", "y_swa")})
+    for a, b in zip(whole, part):
+        assert torch.equal(a[:, 2:], b)
+    cs, sn = sa.sa_rope_table(n, d, 1e6)
+    turned = sa.sa_rope_apply(dev[0], dev[1], cs, sn), sa.sa_rope_apply(dev[1], dev[0], cs, sn, kv=True)
+    assert torch.equal(sa.sa_forward_rope(*dev, perm, inv, cs, sn, w, CAUSAL),
+                       sa.sa_forward(*turned, dev[2], perm, inv, w, CAUSAL))
+    y = torch.empty_like(q).pin_memory()
+    HostForward(1, 4, 2, n, d, w, flags, q_parts=2).forward(q, k, v, lg, y, seed=7, layer=1)
+    torch.cuda.synchronize()
+    want = sa.sa_swa_gated_forward(*dev, perm, inv, lg.cuda(), w, flags)
+    assert torch.equal(y, want.cpu())
+    assert sa.sa_read_status() == 0
