@@ -134,7 +134,7 @@ sa_status sa_make_perm(uint64_t seed, uint32_t layer, int32_t B, int32_t n, int3
 sa_status sa_make_perm_static(uint64_t seed, uint32_t layer, int32_t B, int32_t n,
                               int32_t* perm, int32_t* inv, sa_stream_t stream);
 
-/* SA forward (Alg. 1; Eq. 1 on the neighbourhood of Eq. 3; mask of App. B).
+/* SA forward (Alg. 1; Eq. 1 on the neighbourhood of Eq. 3; mask of App. B).  See sa_forward_lists.
  * Rows of q/k/v are gathered through perm inside the kernel and rows of y are scattered
  * back; no permuted copy of any tensor is made.  y: out.  lse: out, nullable, the
  * log-sum-exp of each query's visible scaled scores (needed by sa_backward). */
@@ -226,11 +226,12 @@ int32_t sa_host_forward_plan(int32_t Hq, int32_t Hkv, int32_t n_groups, int32_t 
  *   opposite angle (the transpose: maps a gradient with respect to the rotated tensor back).
  * sa_forward_rope / sa_swa_gated_forward_rope: sa_forward / sa_swa_gated_forward on rotated Q
  *   and K.  With a workspace of sa_workspace_bytes(.., SA_OP_FORWARD_ROPE) bytes (copies of Q and
- *   K in their layouts) the rotation is a pass over Q and K in one launch.
+ *   K in their layouts, and the scratch of SA_OP_KEY_LISTS; the copies alone will do) the rotation is a
+ *   pass over Q and K in one launch.
  *   bf16 with d = 64 or 128 also works without a workspace, and for small sa_forward_rope calls
- *   (less than 16 MB of Q) ignores it: the rows are then rotated inside the kernels' row gather,
- *   which is one launch less and turns each K row once per query tile that meets it.  Same
- *   results as sa_rope_apply followed by the plain call.  For the backward pass rotate q and k with
+ *   (less than 16 MB of Q, no key lists) ignores it: the rows are then rotated inside the kernels' row
+ *   gather, which is one launch less and turns each K row once per query tile that meets it.  Same
+ *   results as sa_rope_apply followed by the plain call (by the call with lists where it has them).  For the backward pass rotate q and k with
  *   sa_rope_apply, call sa_backward on them, and turn dq and dk back with inverse = 1.
  * Errors: as the plain calls, plus SA_ERR_INVALID_ARG for null tables or odd d. */
 sa_status sa_rope_table(int32_t n, int32_t d, double base, float* rope_cos, float* rope_sin,

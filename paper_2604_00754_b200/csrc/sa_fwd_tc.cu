@@ -16,6 +16,8 @@
 //             them.  (Copying K and V in slot order first and loading whole tiles by TMA was
 //             built and timed: 875 against 859 us at 32/8 heads, n = 32768, w = 1024.)
 //   kNatural  the one-sided SWA branch, whose rows are consecutive tokens: Q, K, V by TMA.
+//   kOrdered  gathered as well, by the lists of sa_order.cu: the keys of a group of slots in token order,
+//             query tiles by token, and one bit per row and key for the mask.
 //
 // Warp roles (384 threads): warps 0-3 softmax/epilogue of query tile 0, warps 4-7 of query tile
 // 1, warp 8 MMA issuer and TMEM allocator (d = 64: warps 8 and 9, one per tile), then the
@@ -50,8 +52,9 @@ enum Src { kGather = 0, kNatural = 1, kOrdered = 2 };
 constexpr int kRowWarps = 8, kThreads = 32 * (kRowWarps + 4);
 __host__ __device__ constexpr int issuers(int d) { return d == 64 ? 2 : 1; }
 
-// Division of numbers below 2^31 by one known at the launch: a multiplication and a shift, where the
-// division proper costs every warp some twenty instructions, five times per item.
+// Division of numbers below 2^30 by one known at the launch: a multiplication and a shift, where the
+// division proper costs every warp some twenty instructions, five times per item (2 x 16 heads of 128,
+// n = 4096, w = 256 82 -> 75 us, its SWA branch 54 -> 50; 8 x 12 heads of 64, w = 128 132 -> 125 and 77 -> 71).
 struct FastDiv {
   uint32_t mul = 0;
   int shift = 0;
@@ -359,8 +362,9 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
   // row each.  Per lane over the 12 warps: 4 x 56 + 8 x 224 = 4 x 72 + 8 x 216 = 2016, all that the
   // launch holds (12 x 168).  The four warps of a warpgroup must ask for the same count, so the issuing
   // warps and the producer warps go down together.  72 where rows are gathered: at 56 the gathering
-  // warps spilled their tokens, and what they reload queues behind their own copies; the row threads
-  // keep their 128 scores at 216 as at 224 (at 208 they spilled).  (The sum may never exceed what the
+  // warps spilled their tokens, and what they reload queues behind their own copies (SA, 8 x 12 heads of 64,
+  // n = 4096, w = 128 128 -> 105 us; 2 x 16 heads of 128, w = 256 76 -> 71); the row threads keep their
+  // 128 scores at 216 as at 224 (at 208 they spilled).  (The sum may never exceed what the
   // launch holds: a warpgroup asking for more waits for ever.)
   constexpr int kLow = kRows ? 72 : 56, kHigh = kRows ? 216 : 224;
   static_assert(4 * kLow + kRowWarps * kHigh == (kRowWarps + 4) * 168, "register split");
@@ -587,8 +591,9 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
         return perm ? perm[slot] : slot;
       };
       // The tokens of a query tile come all at once, at most two per lane: those of the rows that this
-      // warp moves, in its order.  (Fetched group by group, each four groups waited for a load of their
-      // own: six times some 700 cycles per tile, with the tensor core idle.)
+      // warp moves, in its order.  Fetched group by group, each four groups waited for a load of their
+      // own, six times some 700 cycles per tile with the tensor core idle (SA, 32/8 heads of 128: n = 32768,
+      // w = 1024 833 -> 780 us, over lists 790 -> 629; n = 10007, w = 512 184 -> 166).
       static_assert((kGroups + kGWarps - 1) / kGWarps * kRpi <= 64, "two tokens per lane");
       int qt[2];
       auto fetch_q = [&](int t) {
@@ -976,8 +981,7 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
         tmem_wait_st();
         tc_fence_before();
         mbar_arrive(bar(C::kBarPReady + 2 * t + hb));
-        // (here, where the warp would wait: the gathering warps keep the load unit's queue full, and a
-        // warp that joins it between its mask and its exponentials holds its tile up)
+        // (here, where the warp waits anyway)
         if constexpr (SRC == kOrdered)
           if (h < last) seen_next = __ldcg(bits + (size_t)(h + 1) * kTile);
         ++pv_cnt;                           // the issuer answers every arrive with one P V

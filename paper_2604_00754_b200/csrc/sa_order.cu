@@ -8,6 +8,9 @@
 // it holds: with w = 1024 two tiles meet 5.3 and 10 blocks of 128 keys where they met 9 each, with
 // w = 2048 four tiles 3.6 to 20 (12.8 on the average) where they met 17.  What a row sees of a block is
 // one bit per key, worked out here once for all heads.
+// SA branch of 32/8 heads of 128, n = 32768, w = 1024: 744 us without lists, 618 with them and this launch;
+// of 32/4 heads, n = 131072, w = 2048: 5494 and 4347.  The launch itself takes 15 us at n = 8192 and 19 at
+// 32768: a chain of latencies (tokens, counts, scan, places, ranks, bits) in each CTA.
 #include "sa_order.cuh"
 
 namespace sa {
@@ -193,6 +196,10 @@ size_t up(size_t x) { return (x + 255) / 256 * 256; }
 
 bool order_geom(int n, int d, int w, uint32_t flags, OrderGeom* g) {
   const MaskGeom m = make_geom(n, w, flags, false);
+  // Narrower windows gain little (blocks met on the average, w = 512: 4.7 for 5, w = 768: 6.2 for 7), and in
+  // shorter sequences of few heads the launch costs more than it saves (4/2 heads of 64, w = 1024:
+  // n = 8192 57 us with lists, 36 without; n = 32768 123 and 123).
+  // 256 slots or 512: blocks per tile 7.7 / 7.8 at w = 1024, 10.7 / 10.3 at 1536, 13.7 / 12.8 at 2048.
   if (!m.causal || w < 1024 || n < 32768 || (d != 64 && d != 128)) return false;
   g->slots = w <= 1280 ? 256 : 512;
   if ((int64_t)g->slots + 2ll * m.h > n || (int64_t)g->slots + 2ll * m.h > 8192) return false;
