@@ -317,9 +317,9 @@ sa_status sa_read_status(sa_stream_t stream);
 const char* sa_status_string(sa_status s);
 
 /* Profiling hook.  start/stop are cudaEvent_t handles (host values) or both NULL.  While set,
- * every SA-branch attention kernel launched by sa_forward / sa_swa_gated_forward is bracketed
- * by cudaEventRecord(start) and cudaEventRecord(stop) on the call's stream, so a caller can
- * time that one kernel inside a longer step.  Process-wide; not thread-safe.  The paper has
+ * every SA-branch attention kernel launched by sa_forward / sa_swa_gated_forward, with the launch
+ * that makes its key lists where it has them, is bracketed by cudaEventRecord(start) and
+ * cudaEventRecord(stop) on the call's stream, so a caller can time that branch inside a longer step.  Process-wide; not thread-safe.  The paper has
  * no counterpart: this exists for the roofline measurement only. */
 void sa_set_profile_events(void* start, void* stop);
 
