@@ -34,8 +34,10 @@ EXPORTS = [
     "sa_swa_gated_forward_host", "sa_host_forward_ws_bytes", "sa_host_forward_plan",
     "sa_host_forward_pieces",
     "sa_rope_table", "sa_rope_apply", "sa_forward_rope", "sa_swa_gated_forward_rope",
+    "sa_forward_lists", "sa_swa_gated_forward_lists",
 ]
 OP_FORWARD_ROPE = 7
+OP_KEY_LISTS = 8
 DEBUG_SCORE_BLOCK, DEBUG_SWA_TILE_LOADS, DEBUG_TENSOR_CORES, DEBUG_GATE_WIDE_TILES = range(4)
 
 
@@ -99,6 +101,10 @@ def load_library(path: Optional[str] = None) -> ctypes.CDLL:
                                                 i64, vp, vp, vp, sz, vp]
     lib.sa_gate_projection_backward.restype = ctypes.c_int
     lib.sa_read_status.argtypes = [vp]
+    lib.sa_forward_lists.argtypes = [pp] + [vp] * 7 + [vp, sz, vp]
+    lib.sa_forward_lists.restype = ctypes.c_int
+    lib.sa_swa_gated_forward_lists.argtypes = [pp] + [vp] * 11 + [vp, sz, vp]
+    lib.sa_swa_gated_forward_lists.restype = ctypes.c_int
     for f in ("sa_make_perm", "sa_forward", "sa_swa_forward", "sa_swa_gated_forward",
               "sa_backward", "sa_coverage", "sa_read_status"):
         getattr(lib, f).restype = ctypes.c_int
@@ -359,7 +365,8 @@ def sa_swa_gated_forward(q, k, v, perm, inv, gate_logits, w, flags=CAUSAL | SWA_
 
     ``out`` may hold preallocated tensors under the keys y, y_sa, y_swa, lse_sa, lse_swa.
     ``ws`` (scratch of OP_GATED_FORWARD_SCRATCH bytes) and ``fused_epilogue`` are accepted and
-    change nothing: the gates are applied in the local branch's epilogue.  Two launches."""
+    change nothing: the gates are applied in the local branch's epilogue.  Two launches, three where
+    the SA branch walks key lists."""
     o = out or {}
     return (_nat or load_native()).gated_forward(
         q, k, v, perm, inv, gate_logits, w, flags, scale, save_for_bwd, o.get("y"), o.get("y_sa"),

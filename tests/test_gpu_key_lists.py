@@ -11,8 +11,6 @@ import oracle
 from paper_2604_00754_b200 import binding as sa
 from paper_2604_00754_b200.workloads import CAUSAL, LINEAR_WINDOW, SWA_ONE_SIDED, as_f64
 
-KEY_LISTS = 8                                      # SA_OP_KEY_LISTS
-
 # groups of 256 and of 512 slots (w from 1281 on); last groups of one slot, of less than a tile, of an
 # odd number of tiles; both head dimensions; windows that wrap and windows that end with the sequence
 CASES = [
@@ -29,7 +27,7 @@ def problem(Hq, Hkv, n, d, w, flags, B=1, dtype=sa.BF16):
 
 
 def test_which_problems_use_lists():
-    size = lambda *a, **k: sa.sa_workspace_bytes(problem(*a, **k), KEY_LISTS)
+    size = lambda *a, **k: sa.sa_workspace_bytes(problem(*a, **k), sa.OP_KEY_LISTS)
     assert size(2, 1, 32768, 128, 1024, CAUSAL) > 32768 * 4
     assert size(4, 2, 32768, 64, 1024, CAUSAL, B=2) == 2 * size(4, 2, 32768, 64, 1024, CAUSAL)
     assert size(2, 1, 32768, 128, 1024, 0) == 0                        # nothing is hidden by token
@@ -38,7 +36,7 @@ def test_which_problems_use_lists():
     assert size(2, 1, 32768, 128, 32768, CAUSAL) == 0                  # a group's window over everything
     assert size(2, 1, 32767, 128, 1024, CAUSAL) == size(2, 1, 32768, 128, 1023, CAUSAL) == 0
     with pytest.raises(sa.SaError):
-        sa.sa_workspace_bytes(problem(3, 2, 32768, 128, 1024, CAUSAL), KEY_LISTS)
+        sa.sa_workspace_bytes(problem(3, 2, 32768, 128, 1024, CAUSAL), sa.OP_KEY_LISTS)
 
 
 @pytest.mark.gpu
