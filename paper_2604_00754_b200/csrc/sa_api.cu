@@ -101,7 +101,7 @@ cudaError_t run_forward(const FwdArgs& a, int dtype, cudaStream_t st) {
   OrderGeom g;
   cudaError_t e = cudaSuccess;
   if (a.lists && !a.lists_ready && tc_forward_ordered(a, dtype, &g))
-    e = launch_order(a.perm, a.B, a.n, a.w, a.flags, g, order_view(a.lists, a.B, g), a.abort_flag, st);
+    e = launch_order(a.perm, a.B, a.n, a.w, a.flags, g, order_view(a.lists, a.B, g), st);
   if (e == cudaSuccess)
     e = tc_forward_supported(a, dtype) ? launch_fwd_tc(a, st) : launch_fwd_simt(a, dtype, st);
   if (prof) cudaEventRecord(g_prof_stop, st);

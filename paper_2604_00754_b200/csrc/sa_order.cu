@@ -22,7 +22,6 @@ struct OrderParams {
   const int32_t* perm;
   int32_t *q, *k, *tiles;
   uint4* bits;
-  const int* abort_flag;
   int n, h, linear;
   OrderGeom g;
   uint32_t bucket_mul;          // bucket of a token: umulhi(token, bucket_mul) < kBuckets
@@ -36,10 +35,13 @@ size_t shared_bytes(int span) {
 // One CTA per query tile; the tiles of a group each sort the group's keys (a few microseconds that
 // run side by side), and each works out its own bits.  Sort: counts per bucket of tokens, a place per
 // key, and the rank inside the bucket by counting; any contents give the unique order.
+// Whatever perm holds, a rejected one of SA_VALIDATE_PERM too, everything that the attention launch reads
+// is written and in range: that launch looks at the status word for itself, later, and the word may have
+// been read and cleared in between.
 __global__ void __launch_bounds__(kThreads) order_kernel(const __grid_constant__ OrderParams p) {
   extern __shared__ __align__(16) uint8_t smem[];
   __shared__ uint32_t part[kThreads / 32];
-  __shared__ int q_pos[kOrderTile], q_off[kOrderTile], skip;
+  __shared__ int q_pos[kOrderTile], q_off[kOrderTile];
   constexpr uint32_t kGuard = 0x8000u;            // set in the sorted offsets (all below 2^15)
   const OrderGeom& g = p.g;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -56,17 +58,15 @@ __global__ void __launch_bounds__(kThreads) order_kernel(const __grid_constant__
   for (int i = tid; i < kBuckets; i += kThreads) start[i] = 0u;
   grid_dependency_wait();
   grid_dependents_launch();
-  if (tid == 0) skip = p.abort_flag && *(volatile const int*)p.abort_flag;
   __syncthreads();
-  if (skip) return;                                    // an earlier check rejected perm/inv
   const int32_t* perm = p.perm + (size_t)b * p.n;
   auto bucket_of = [&](int32_t t) { return min(__umulhi((uint32_t)t, p.bucket_mul), kBuckets - 1u); };
-  // a token of -1: outside the sequence (linear windows)
+  // a token of -1: outside the sequence (linear windows); of n and more, or negative: taken for n - 1
   for (int o = tid; o < span; o += kThreads) {
     int s = s0 - p.h + o;
     int32_t t = -1;
     if (!p.linear) { s = s < 0 ? s + p.n : s >= p.n ? s - p.n : s; }
-    if (s >= 0 && s < p.n) t = perm[s];
+    if (s >= 0 && s < p.n) t = (int32_t)min((uint32_t)perm[s], (uint32_t)p.n - 1u);
     tok[o] = t;
     if (t >= 0) off[o] = (uint16_t)atomicAdd(&start[bucket_of(t)], 1u);
   }
@@ -230,12 +230,11 @@ OrderView order_view(void* ws, int B, const OrderGeom& g) {
 }
 
 cudaError_t launch_order(const int32_t* perm, int B, int n, int w, uint32_t flags, const OrderGeom& g,
-                         const OrderView& v, const int* abort_flag, cudaStream_t st) {
+                         const OrderView& v, cudaStream_t st) {
   const MaskGeom m = make_geom(n, w, flags, false);
   OrderParams p{};
   p.perm = perm;
   p.q = v.q; p.k = v.k; p.tiles = v.tiles; p.bits = v.bits;
-  p.abort_flag = abort_flag;
   p.n = n; p.h = m.h; p.linear = m.linear;
   p.g = g;
   p.bucket_mul = (uint32_t)(((uint64_t)kBuckets << 32) / (uint64_t)n);     // n > kBuckets: fits

@@ -24,6 +24,6 @@ bool order_geom(int n, int d, int w, uint32_t flags, OrderGeom* g);
 size_t order_bytes(int B, const OrderGeom& g);
 OrderView order_view(void* ws, int B, const OrderGeom& g);
 cudaError_t launch_order(const int32_t* perm, int B, int n, int w, uint32_t flags, const OrderGeom& g,
-                         const OrderView& v, const int* abort_flag, cudaStream_t st);
+                         const OrderView& v, cudaStream_t st);
 
 }  // namespace sa

@@ -100,3 +100,43 @@ def test_bits_of_a_part_and_of_the_host_pipeline(w):
     want = sa.sa_swa_gated_forward(*dev, perm, inv, lg.cuda(), w, flags)
     assert torch.equal(y, want.cpu())
     assert sa.sa_read_status() == 0
+
+
+# The attention launch looks at the status word for itself, after the launch that makes the lists, and the
+# word may have been read and cleared in between: the lists are written whatever the word says, with tokens
+# that exist whatever the permutation holds.
+@pytest.mark.gpu
+def test_lists_are_written_whatever_the_status_word_says():
+    n, d, w, flags = 33000, 64, 1024, CAUSAL | 16                     # SA_VALIDATE_PERM
+    g = torch.Generator(device="cuda").manual_seed(n)
+    q, k, v = (torch.randn(1, h, n, d, generator=g, device="cuda").bfloat16() for h in (2, 1, 1))
+    perm, inv = sa.sa_make_perm(n, w, 1, n)
+    bad = perm.clone()
+    bad[0, :4] = torch.tensor([n, -1, 2 ** 31 - 1, -2 ** 31])
+    bad[0, 500:700] = bad[0, 700]
+    p = sa.make_problem(q, k, w, flags)
+    size = sa.sa_workspace_bytes(p, sa.OP_KEY_LISTS)
+    at = lambda t: ctypes.c_void_p(t.data_ptr())
+
+    def lists(sigma):
+        ws, y = torch.zeros(size, dtype=torch.uint8, device="cuda"), torch.zeros_like(q)
+        st = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+        assert sa.load_library().sa_forward_lists(ctypes.byref(p), at(q), at(k), at(v), at(sigma), at(inv), at(y),
+                                                  None, at(ws), size, st) == 0
+        return ws, y
+
+    want, y = lists(perm)
+    assert sa.sa_read_status() == 0 and y.any()
+    rejected, y = lists(bad)
+    assert not y.any()                                   # the attention launch left
+    again, y = lists(perm)                               # the word is set still
+    assert not y.any() and torch.equal(again, want)
+    assert sa.sa_read_status() == 5                      # SA_ERR_BAD_PERM
+    tiles, blocks = (n + 127) // 128, (256 + 2 * ((w + 1) // 2 - 1) + 127) // 128
+    groups = (n + 255) // 256
+    up = lambda x: (x + 255) // 256 * 256
+    words = rejected.view(torch.int32)
+    k_end = up(tiles * 512) + up(groups * blocks * 512)
+    assert 0 <= words[:k_end // 4].min() and words[:k_end // 4].max() < n
+    met = words[k_end // 4:k_end // 4 + tiles]
+    assert 1 <= met.min() and met.max() <= blocks
