@@ -465,8 +465,8 @@ def extras(args, c, wl, sa, torch, dev, host, perm, inv, ws, y, pk):
     # copies in, kernels and copies out overlap
     hy = torch.empty_like(host["q"]).pin_memory()
     hg = host["gate_logits"].pin_memory()
-    hws = torch.empty(sa.host_forward_ws_bytes(c.B, c.Hq, c.Hkv, c.n, c.d), dtype=torch.uint8,
-                      device="cuda")
+    hws = torch.empty(sa.host_forward_ws_bytes(c.B, c.Hq, c.Hkv, c.n, c.d, w=c.w, flags=c.flags),
+                      dtype=torch.uint8, device="cuda")
     layer = [1000]
 
     def e2e_step():

@@ -185,10 +185,13 @@ sa_status sa_swa_gated_forward_lists(const sa_problem* p, const void* q, const v
  * query heads if those divide evenly and still fill the GPU: the ends of the pipeline are what
  * cannot overlap.  There are three internal streams: copy in, compute, copy out.  The permutation
  * is drawn from (seed, layer) as in sa_make_perm and shared by all ranges; every range is one
- * sa_swa_gated_forward call, and the result has the bits of that call on the whole problem.
+ * sa_swa_gated_forward_lists call, and the result has the bits of that call on the whole problem
+ * with scratch of SA_OP_KEY_LISTS bytes.
  *   ws: DEVICE workspace of sa_host_forward_ws_bytes(p) bytes, 256-byte aligned, owned by the
  *       caller (device copies of q, k, v, y, one branch output, the permutation and its
- *       scratch).  No device memory is allocated; the first call on a device creates the
+ *       scratch, and the key lists of the SA branch, which depend on w and flags, where they find no room
+ *       within the branch output).  The bytes of the same problem with w = 1 will do: the lists that do
+ *       not fit are then done without, and the bits are those of sa_swa_gated_forward.  No device memory is allocated; the first call on a device creates the
  *       three streams and the events of the pipeline and keeps them.
  *   stream: the call is ordered after what `stream` has queued, and `stream` waits for the
  *       last copy out, so the caller synchronises (or times) on `stream` alone.  y must not

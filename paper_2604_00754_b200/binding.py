@@ -481,8 +481,11 @@ def host_forward_pieces(B, Hq, Hkv, n, d, dtype=BF16, n_groups=8, q_parts=2):
     return [r[:4] + (bool(r[4]),) + r[5:] for r in rows]
 
 
-def host_forward_ws_bytes(B, Hq, Hkv, n, d, dtype=BF16) -> int:
-    p = SaProblem(B=B, Hq=Hq, Hkv=Hkv, n=n, d=d, w=1, dtype=dtype)
+def host_forward_ws_bytes(B, Hq, Hkv, n, d, dtype=BF16, w=1, flags=0) -> int:
+    """Bytes of the device workspace.  ``w`` and ``flags`` of the calls to come make room for the SA
+    branch's key lists where those have none within the rest (few heads, very wide windows); without
+    it such a call goes without lists."""
+    p = SaProblem(B=B, Hq=Hq, Hkv=Hkv, n=n, d=d, w=int(w), dtype=dtype, flags=int(flags))
     r = int(load_library().sa_host_forward_ws_bytes(ctypes.byref(p)))
     if r == ctypes.c_size_t(-1).value:
         raise SaError(1, "sa_host_forward_ws_bytes")
@@ -492,8 +495,9 @@ def host_forward_ws_bytes(B, Hq, Hkv, n, d, dtype=BF16) -> int:
 def sa_swa_gated_forward_host(q, k, v, gate_logits, y, w, flags, seed, layer, ws, n_groups=8,
                               q_parts=2, scale=0.0):
     """Fresh permutation + gated SA+SWA forward on HOST tensors (contiguous [B,H,n,d], pinned
-    for overlap); ws: CUDA uint8 tensor of host_forward_ws_bytes(...).  y (host) is complete
-    once the current stream has been synchronised."""
+    for overlap); ws: CUDA uint8 tensor of host_forward_ws_bytes(.., w, flags).  y (host) is complete
+    once the current stream has been synchronised, with the bits of sa_swa_gated_forward on the whole
+    problem (with a smaller ws that still does: see sa.h)."""
     for t in (q, k, v, y, gate_logits):
         if t.is_cuda or not t.is_contiguous():
             raise ValueError("host tensors must be contiguous CPU tensors")

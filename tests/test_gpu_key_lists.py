@@ -72,8 +72,38 @@ def test_rows_against_the_oracle(B, Hq, Hkv, n, d, w, flags):
     assert np.abs(as_f64(lse.reshape(-1)[sel]) - rl).max() <= 2e-2
 
 
-# a part of the heads, the rotated call and the host pipeline (whose pieces cut a group's heads) take the
-# same route and give the same bits
+# The host pipeline has the bits of the call on the whole problem: lists that do not fit within the scratch
+# it needs otherwise; ranges of sequences, whose lists are made anew from a permutation off 16 bytes; pieces
+# that cut a group to one head, whose items are two tiles of that head (a last group of one and of three tiles)
+@pytest.mark.gpu
+@pytest.mark.parametrize("B,Hq,Hkv,n,w,kind", [
+    (1, 2, 1, 32768, 2048, "outside"), (3, 2, 1, 33001, 2000, "outside"), (2, 4, 2, 33001, 1024, "ranges"),
+    (1, 4, 2, 38001, 1024, "cut"), (1, 4, 2, 38001, 2000, "cut"), (1, 4, 2, 38201, 2000, "cut"),
+])
+def test_bits_of_the_host_pipeline(B, Hq, Hkv, n, w, kind):
+    from paper_2604_00754_b200.host import HostForward
+    flags = CAUSAL | SWA_ONE_SIDED
+    g = torch.Generator().manual_seed(n + w)
+    q, k, v = (torch.randn(B, h, n, 64, generator=g).bfloat16().pin_memory() for h in (Hq, Hkv, Hkv))
+    lg = torch.randn(2, Hq, generator=g).pin_memory()
+    hf = HostForward(B, Hq, Hkv, n, 64, w, flags)
+    if kind == "outside":
+        assert hf.ws.numel() > sa.host_forward_ws_bytes(B, Hq, Hkv, n, 64)
+    if B > 1:
+        assert len({piece[5:] for piece in hf.pieces}) == B
+    if kind == "cut":
+        assert any((piece[3] - piece[2]) % 2 for piece in hf.pieces)
+    y = torch.empty_like(q).pin_memory()
+    for layer in (1, 2):
+        hf.forward(q, k, v, lg, y, seed=7, layer=layer)
+        torch.cuda.synchronize()
+        perm, inv = sa.sa_make_perm(7, layer, B, n)
+        assert torch.equal(y, sa.sa_swa_gated_forward(q.cuda(), k.cuda(), v.cuda(), perm, inv, lg.cuda(), w,
+                                                      flags).cpu())
+    assert sa.sa_read_status() == 0
+
+
+# a part of the heads, the rotated call and the host pipeline take the same route and give the same bits
 @pytest.mark.gpu
 @pytest.mark.parametrize("w", [1024, 2000])
 def test_bits_of_a_part_and_of_the_host_pipeline(w):

@@ -56,6 +56,24 @@ def test_host_forward_rejects_bad_arguments_before_any_cuda_call():
     assert lib.sa_swa_gated_forward_host(*args(fake, need - 1)) == 3
 
 
+# the workspace as the library sizes it for the calls to come: with room of its own for key lists that do
+# not fit beside the rest
+@pytest.mark.parametrize("B,Hq,Hkv,n,d,w,extra", [
+    (1, 2, 1, 32768, 64, 2048, True), (1, 4, 2, 33000, 64, 4000, True), (2, 2, 1, 33001, 64, 2000, True),
+    (1, 4, 2, 33100, 64, 2000, False), (1, 2, 1, 32768, 64, 512, False), (1, 2, 2, 32768, 64, 2048, False),
+])
+def test_workspace_has_room_for_the_key_lists(B, Hq, Hkv, n, d, w, extra):
+    import ctypes
+    p = sab.SaProblem(B=B, Hq=Hq, Hkv=Hkv, n=n, d=d, w=w, dtype=sab.BF16, flags=sab.CAUSAL)
+    sab.load_library().sa_problem_set_contiguous(ctypes.byref(p))
+    need = sab.load_library().sa_host_forward_ws_bytes(ctypes.byref(p))
+    least = sab.host_forward_ws_bytes(B, Hq, Hkv, n, d)
+    assert sab.host_forward_ws_bytes(B, Hq, Hkv, n, d, w=w, flags=sab.CAUSAL) == need
+    assert (need > least) == extra
+    if extra:
+        assert need - least == sab.sa_workspace_bytes(p, sab.OP_KEY_LISTS)
+
+
 # what the call makes of a problem: every head of every sequence once, K and V with the first piece that
 # reads them; many sequences with many groups, none, and more than there are events for
 @pytest.mark.parametrize("B,Hq,Hkv,n,d,n_groups,q_parts", [
