@@ -593,7 +593,11 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
       // The tokens of a query tile come all at once, at most two per lane: those of the rows that this
       // warp moves, in its order.  Fetched group by group, each four groups waited for a load of their
       // own, six times some 700 cycles per tile with the tensor core idle (SA, 32/8 heads of 128: n = 32768,
-      // w = 1024 833 -> 780 us, over lists 790 -> 629; n = 10007, w = 512 184 -> 166).
+      // w = 1024 833 -> 780 us, over lists 790 -> 629; n = 10007, w = 512 184 -> 166).  Not where rows of
+      // d = 128 are turned on the way: with two tokens more to hold, those warps spill 108 bytes for 60
+      // (sa_forward_rope, 8/2 heads, n = 4096, w = 1024 110.7 us for 108.3; d = 64, 64 bytes for 56: 12 heads,
+      // w = 128 76.5 for 78.1).
+      constexpr bool kRowTokens = !(ROPE && D == 128);
       static_assert((kGroups + kGWarps - 1) / kGWarps * kRpi <= 64, "two tokens per lane");
       int qt[2];
       auto fetch_q = [&](int t) {
@@ -603,7 +607,7 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
           qt[x] = q_tok(t, min((pw + kGWarps * (e / kRpi)) * kRpi + e % kRpi, kTile - 1));
         }
       };
-      fetch_q(0);
+      if constexpr (kRowTokens) fetch_q(0);
       // tokens are fetched one tile ahead of their use
       int tk0 = key_tok(0, ptid), tk1 = ptid + kPt < kTile ? key_tok(0, ptid + kPt) : 0;
       for (int j = 0; j < g.T; ++j, ++gt) {
@@ -632,9 +636,10 @@ fwd_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtens
           if (group_sync_stop()) { live = false; break; }
 #pragma unroll 1
           for (int t = 0; t < 2; ++t) {
-            if (t && !p.pair_heads) fetch_q(1);
+            if (kRowTokens && t && !p.pair_heads) fetch_q(1);
             gather(qg + b * p.qs[0] + (t ? g.hq[1] : g.hq[0]) * p.qs[1], p.qs[2],
-                   [&](int, int nth) {
+                   [&](int r, int nth) {
+                     if constexpr (!kRowTokens) return q_tok(t, r);
                      return __shfl_sync(0xffffffffu, nth < 32 / kRpi ? qt[0] : qt[1], (nth * kRpi + sub) & 31);
                    },
                    q_dst + t * C::kTileBytes);
