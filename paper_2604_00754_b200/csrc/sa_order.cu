@@ -16,7 +16,7 @@
 namespace sa {
 namespace {
 
-constexpr int kThreads = 512, kBuckets = 1024;
+constexpr int kThreads = 512, kBuckets = 1024, kDeep = 16;
 
 struct OrderParams {
   const int32_t* perm;
@@ -34,11 +34,19 @@ size_t shared_bytes(int span) {
 
 // One CTA per query tile; the tiles of a group each sort the group's keys (a few microseconds that
 // run side by side), and each works out its own bits.  Sort: counts per bucket of tokens, a place per
-// key, and the rank inside the bucket by counting; any contents give the unique order.
+// key, and the rank inside the bucket by counting; any contents give the unique order.  A random
+// permutation puts up to 8 keys on the average into a bucket.  One that keeps neighbours together (the
+// identity, shuffled blocks) may put the whole window into a few: where some bucket holds more than kDeep
+// keys, each is divided once more, after which sqrt(n / 1024) keys at most share one.  This launch, w = 2048,
+// random / identity / blocks of 256: n = 131072 75 / 70 / 77 us where the second division was missing 74 /
+// 194 / 201; w = 1024, n = 2^20 291 / 287 / 296 and 289 / 2861 / 1184.  16 is where the second division is worth
+// it: with 32 keys to a bucket (identity, n = 32768, w = 1024) 17.5 us with it, 21.9 without.
 // Whatever perm holds, a rejected one of SA_VALIDATE_PERM too, everything that the attention launch reads
 // is written and in range: that launch looks at the status word for itself, later, and the word may have
 // been read and cleared in between.
-__global__ void __launch_bounds__(kThreads) order_kernel(const __grid_constant__ OrderParams p) {
+// 32 registers, four CTAs per SM (with the loops of the second division unrolled, 60 and two: n = 2^20, w = 1024
+// 289 -> 375 us).
+__global__ void __launch_bounds__(kThreads, 4) order_kernel(const __grid_constant__ OrderParams p) {
   extern __shared__ __align__(16) uint8_t smem[];
   __shared__ uint32_t part[kThreads / 32];
   __shared__ int q_pos[kOrderTile], q_off[kOrderTile];
@@ -91,36 +99,99 @@ __global__ void __launch_bounds__(kThreads) order_kernel(const __grid_constant__
     *total = sum;
     return before + x - mine;
   };
-  uint32_t keys;
+  uint32_t keys, most = 0;
   {
     constexpr int kPer = kBuckets / kThreads;
     uint32_t c[kPer], mine = 0;
 #pragma unroll
-    for (int i = 0; i < kPer; ++i) { c[i] = start[kPer * tid + i]; mine += c[i]; }
+    for (int i = 0; i < kPer; ++i) {
+      c[i] = start[kPer * tid + i];
+      mine += c[i];
+      most = max(most, c[i]);
+    }
     uint32_t at = scan(mine, &keys);
 #pragma unroll
     for (int i = 0; i < kPer; ++i) { start[kPer * tid + i] = at; at += c[i]; }
   }
-  __syncthreads();
-  for (int o = tid; o < span; o += kThreads) {
-    const int32_t t = tok[o];
-    if (t < 0) continue;
-    const uint32_t at = start[bucket_of(t)] + off[o];
-    tok2[at] = t;
-    off2[at] = (uint16_t)o;
-  }
-  __syncthreads();
-  for (int x = tid; x < (int)keys; x += kThreads) {
-    const int32_t t = tok2[x];
-    const uint16_t o = off2[x];
-    const uint32_t bk = bucket_of(t), lo = start[bk], hi = bk + 1 < kBuckets ? start[bk + 1] : keys;
-    uint32_t rank = lo;
-    for (uint32_t y = lo; y < hi; ++y) {
-      const int32_t u = tok2[y];
-      rank += u < t || (u == t && off2[y] < o);
+  if (!__syncthreads_or(most > kDeep)) {
+    for (int o = tid; o < span; o += kThreads) {
+      const int32_t t = tok[o];
+      if (t < 0) continue;
+      const uint32_t at = start[bucket_of(t)] + off[o];
+      tok2[at] = t;
+      off2[at] = (uint16_t)o;
     }
-    tok[rank] = t;
-    off[rank] = (uint16_t)(o | kGuard);
+    __syncthreads();
+    for (int x = tid; x < (int)keys; x += kThreads) {
+      const int32_t t = tok2[x];
+      const uint16_t o = off2[x];
+      const uint32_t bk = bucket_of(t), lo = start[bk], hi = bk + 1 < kBuckets ? start[bk + 1] : keys;
+      uint32_t rank = lo;
+      for (uint32_t y = lo; y < hi; ++y) {
+        const int32_t u = tok2[y];
+        rank += u < t || (u == t && off2[y] < o);
+      }
+      tok[rank] = t;
+      off[rank] = (uint16_t)(o | kGuard);
+    }
+  } else {
+    // A bucket of c keys is cut into c of its own, by where a token lies in it; these are counted and scanned
+    // like the first, in the room of tok2, and hold the keys' offsets alone.
+    uint32_t* sub = reinterpret_cast<uint32_t*>(tok2);
+    auto sub_of = [&](int32_t t) {
+      const uint64_t at = (uint64_t)(uint32_t)t * p.bucket_mul;
+      const uint32_t bk = (uint32_t)(at >> 32), lo = start[bk], hi = bk + 1 < kBuckets ? start[bk + 1] : keys;
+      return lo + __umulhi((uint32_t)at, hi - lo);
+    };
+#pragma unroll 1
+    for (int x = tid; x < (int)keys; x += kThreads) sub[x] = 0u;
+    __syncthreads();
+#pragma unroll 1
+    for (int o = tid; o < span; o += kThreads) {
+      const int32_t t = tok[o];
+      if (t >= 0) off[o] = (uint16_t)atomicAdd(&sub[sub_of(t)], 1u);
+    }
+    __syncthreads();
+    {
+      const int per = ((int)keys + kThreads - 1) / kThreads, x0 = tid * per, x1 = min(x0 + per, (int)keys);
+      uint32_t mine = 0, all;
+#pragma unroll 1
+      for (int x = x0; x < x1; ++x) mine += sub[x];
+      uint32_t at = scan(mine, &all);
+#pragma unroll 1
+      for (int x = x0; x < x1; ++x) {
+        const uint32_t c = sub[x];
+        sub[x] = at;
+        at += c;
+      }
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int o = tid; o < span; o += kThreads) {
+      const int32_t t = tok[o];
+      if (t >= 0) off2[sub[sub_of(t)] + off[o]] = (uint16_t)o;
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int x = tid; x < (int)keys; x += kThreads) {
+      const uint16_t o = off2[x];
+      const int32_t t = tok[o];
+      const uint32_t sb = sub_of(t), lo = sub[sb], hi = sb + 1 < keys ? sub[sb + 1] : keys;
+      uint32_t rank = lo;
+#pragma unroll 1
+      for (uint32_t y = lo; y < hi; ++y) {
+        const uint16_t r = off2[y];
+        const int32_t u = tok[r];
+        rank += u < t || (u == t && r < o);
+      }
+      off[rank] = (uint16_t)(o | kGuard);
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int x = tid; x < (int)keys; x += kThreads) tok2[x] = tok[off[x] ^ kGuard];
+    __syncthreads();
+#pragma unroll 1
+    for (int x = tid; x < (int)keys; x += kThreads) tok[x] = tok2[x];
   }
   if (tid < kOrderTile) q_pos[tid] = -1;
   __syncthreads();

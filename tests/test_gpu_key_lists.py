@@ -170,3 +170,66 @@ def test_lists_are_written_whatever_the_status_word_says():
     assert 0 <= words[:k_end // 4].min() and words[:k_end // 4].max() < n
     met = words[k_end // 4:k_end // 4 + tiles]
     assert 1 <= met.min() and met.max() <= blocks
+
+
+def structured(kind, n):
+    i = torch.arange(n, dtype=torch.int64, device="cuda")
+    if kind == "identity":
+        perm = i
+    elif kind == "reversed":
+        perm = n - 1 - i
+    elif kind == "blocks":                              # shuffled blocks of 250 tokens and a ragged one
+        g = torch.Generator(device="cuda").manual_seed(n)
+        first = torch.randperm((n + 249) // 250, generator=g, device="cuda")
+        perm = (first[:, None] * 250 + torch.arange(250, device="cuda")).reshape(-1)
+        perm = perm[perm < n]
+    else:                                               # strides: neighbours are 64 slots apart
+        perm = torch.cat([i[s::64] for s in range(64)])
+    inv = torch.empty_like(perm)
+    inv[perm] = i
+    return perm.int()[None].contiguous(), inv.int()[None].contiguous()
+
+
+# permutations that keep neighbours together, 64 tokens and more to a bucket of the launch that makes the lists
+@pytest.mark.gpu
+@pytest.mark.parametrize("kind", ["identity", "reversed", "blocks", "strides"])
+@pytest.mark.parametrize("n,w,flags", [(65613, 1024, CAUSAL), (65613, 1500, CAUSAL | LINEAR_WINDOW),
+                                       (70001, 7000, CAUSAL)])
+def test_structured_permutations(kind, n, w, flags):
+    g = torch.Generator().manual_seed(n)
+    q, k, v = (torch.randn(1, h, n, 64, generator=g).bfloat16() for h in (2, 1, 1))
+    dev = [t.cuda() for t in (q, k, v)]
+    perm, inv = structured(kind, n)
+    y, lse = sa.sa_forward(*dev, perm, inv, w, flags, want_lse=True)
+    assert sa.sa_read_status() == 0
+    rows = np.unique(np.concatenate([np.random.default_rng(0).integers(0, 2 * n, 600), np.arange(n - 140, n),
+                                     perm[0, -80:].cpu().numpy()]))
+    ry, rl = oracle.forward_rows(0, *(as_f64(t) for t in (q, k, v)), perm.cpu().numpy(), inv.cpu().numpy(), w,
+                                 flags, rows)
+    sel = torch.from_numpy(rows).cuda()
+    assert np.abs(as_f64(y.reshape(-1, 64)[sel]) - ry).max() <= 2e-2 * np.abs(ry).max()
+    assert np.abs(as_f64(lse.reshape(-1)[sel]) - rl).max() <= 2e-2
+
+
+# ... and they take about the time of a random one: 1.6 times as long, and 4.3 times at n = 2^20, where the
+# keys of a bucket were counted through for each of them
+@pytest.mark.gpu
+def test_structured_permutations_are_not_slow():
+    n, w = 1 << 18, 2048
+    g = torch.Generator(device="cuda").manual_seed(n)
+    q, k, v = (torch.randn(1, h, n, 64, generator=g, device="cuda").bfloat16() for h in (2, 1, 1))
+    times = {}
+    for kind in ("random", "identity", "blocks"):
+        perm, inv = sa.sa_make_perm(1, 0, 1, n) if kind == "random" else structured(kind, n)
+        runs = []
+        for _ in range(6):
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            a.record()
+            for _ in range(4):
+                sa.sa_forward(q, k, v, perm, inv, w, CAUSAL)
+            b.record()
+            torch.cuda.synchronize()
+            runs.append(a.elapsed_time(b))
+        times[kind] = min(runs)
+    assert sa.sa_read_status() == 0
+    assert max(times["identity"], times["blocks"]) <= 1.3 * times["random"], times
