@@ -13,6 +13,7 @@ from __future__ import annotations
 import ctypes
 import importlib.util
 import os
+import warnings
 from typing import Optional
 
 import torch
@@ -235,6 +236,22 @@ def _workspace(nbytes: int, device, ws: Optional[torch.Tensor]):
     return torch.empty(max(nbytes, 16), dtype=torch.uint8, device=device)
 
 
+def workspace_with_lists(nbytes: int, without: int, device) -> torch.Tensor:
+    """A workspace with room for key lists; without them, and with a warning, where memory is short."""
+    try:
+        return torch.empty(max(nbytes, 16), dtype=torch.uint8, device=device)
+    except torch.OutOfMemoryError:
+        if nbytes <= without:
+            raise
+    warnings.warn("no memory for the key lists: the call goes without them", RuntimeWarning, stacklevel=3)
+    return torch.empty(max(without, 16), dtype=torch.uint8, device=device)
+
+
+def _rope_workspace(p: SaProblem, device) -> torch.Tensor:
+    nbytes = sa_workspace_bytes(p, OP_FORWARD_ROPE)
+    return workspace_with_lists(nbytes, nbytes - sa_workspace_bytes(p, OP_KEY_LISTS), device)
+
+
 def _same_layout(ref: torch.Tensor, *others):
     for t in others:
         if t is not None and (t.shape != ref.shape or t.stride() != ref.stride()
@@ -274,7 +291,11 @@ def sa_make_perm_static(seed: int, layer: int, B: int, n: int, perm: torch.Tenso
 
 def sa_forward(q, k, v, perm, inv, w, flags=CAUSAL, scale=0.0, y=None, want_lse=False,
                lse=None):
-    """SA forward; returns y (and lse when asked)."""
+    """SA forward; returns y (and lse when asked).
+
+    Takes sa_workspace_bytes(.., OP_KEY_LISTS) bytes of scratch from torch's allocator for the call, where that
+    is not 0 (so a capture of it into a graph has to be torch's); where memory is short it goes without, with a
+    RuntimeWarning: the sums then run in another order."""
     return (_nat or load_native()).forward(q, k, v, perm, inv, w, flags, scale, y, want_lse, lse)
 
 
@@ -326,7 +347,7 @@ def sa_forward_rope(q, k, v, perm, inv, rope_cos, rope_sin, w, flags=CAUSAL, sca
     y = torch.empty_like(q) if y is None else y
     _same_layout(q, y)
     lse = torch.empty(q.shape[:3], dtype=torch.float32, device=q.device) if want_lse else None
-    ws = _workspace(sa_workspace_bytes(p, OP_FORWARD_ROPE), q.device, None)
+    ws = _rope_workspace(p, q.device)
     _check(lib.sa_forward_rope(ctypes.byref(p), _ptr(q), _ptr(k), _ptr(v), _ptr(perm), _ptr(inv),
                                _ptr(rope_cos), _ptr(rope_sin), _ptr(y), _ptr(lse), _ptr(ws),
                                ws.numel(), _stream()), "sa_forward_rope")
@@ -348,7 +369,7 @@ def sa_swa_gated_forward_rope(q, k, v, perm, inv, rope_cos, rope_sin, gate_logit
     y = torch.empty_like(q)
     _same_layout(q, y)
     p = make_problem(q, k, w, flags, scale)
-    ws = _workspace(sa_workspace_bytes(p, OP_FORWARD_ROPE), q.device, None)
+    ws = _rope_workspace(p, q.device)
     _check(lib.sa_swa_gated_forward_rope(
         ctypes.byref(p), _ptr(q), _ptr(k), _ptr(v), _ptr(perm), _ptr(inv), _ptr(rope_cos),
         _ptr(rope_sin), _ptr(gate_logits), _ptr(y), _ptr(out.get("y_sa")), _ptr(out.get("y_swa")),
@@ -366,7 +387,7 @@ def sa_swa_gated_forward(q, k, v, perm, inv, gate_logits, w, flags=CAUSAL | SWA_
     ``out`` may hold preallocated tensors under the keys y, y_sa, y_swa, lse_sa, lse_swa.
     ``ws`` (scratch of OP_GATED_FORWARD_SCRATCH bytes) and ``fused_epilogue`` are accepted and
     change nothing: the gates are applied in the local branch's epilogue.  Two launches, three where
-    the SA branch walks key lists."""
+    the SA branch walks key lists, whose scratch is as in sa_forward."""
     o = out or {}
     return (_nat or load_native()).gated_forward(
         q, k, v, perm, inv, gate_logits, w, flags, scale, save_for_bwd, o.get("y"), o.get("y_sa"),

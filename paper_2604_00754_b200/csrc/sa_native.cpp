@@ -134,13 +134,16 @@ size_t ws_bytes(const sa_problem& p, int op) {
 }
 
 // Scratch for the SA branch's key lists, from the allocator's pool of the current stream; undefined
-// where the problem has no use for any.
+// where the problem has no use for any, and, with a warning (the sums run in another order then), where there
+// is no memory for it.
 at::Tensor key_lists(const sa_problem& p, c10::Device dev) {
   const size_t n = sa_workspace_bytes(&p, SA_OP_KEY_LISTS);
   if (n == 0 || n == (size_t)-1) return at::Tensor();
   try {
     return fresh({(int64_t)n}, at::kByte, dev);
-  } catch (const c10::OutOfMemoryError&) {          // the call works without
+  } catch (const c10::OutOfMemoryError&) {
+    if (PyErr_WarnEx(PyExc_RuntimeWarning, "no memory for the key lists: the call goes without them", 1) < 0)
+      throw Raised{};
     return at::Tensor();
   }
 }

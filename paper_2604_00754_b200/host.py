@@ -26,8 +26,8 @@ class HostForward:
         self.n_groups, self.q_parts = n_groups, q_parts
         code = sa.BF16 if dtype == torch.bfloat16 else sa.F32
         self.pieces = sa.host_forward_pieces(B, Hq, Hkv, n, d, code, n_groups, q_parts)
-        self.ws = torch.empty(sa.host_forward_ws_bytes(B, Hq, Hkv, n, d, code, w, flags),
-                              dtype=torch.uint8, device=self.device)
+        self.ws = sa.workspace_with_lists(sa.host_forward_ws_bytes(B, Hq, Hkv, n, d, code, w, flags),
+                                          sa.host_forward_ws_bytes(B, Hq, Hkv, n, d, code), self.device)
 
     def _elt(self) -> int:
         return 2 if self.dtype == torch.bfloat16 else 4

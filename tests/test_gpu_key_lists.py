@@ -233,3 +233,48 @@ def test_structured_permutations_are_not_slow():
         times[kind] = min(runs)
     assert sa.sa_read_status() == 0
     assert max(times["identity"], times["blocks"]) <= 1.3 * times["random"], times
+
+
+# Without memory for the lists the calls work as they did without them, and say so.
+@pytest.mark.gpu
+def test_calls_go_without_lists_where_memory_is_short():
+    from paper_2604_00754_b200.host import HostForward
+    n, w, flags = 65536, 2048, CAUSAL                   # 22 MB of lists: never within another block
+    g = torch.Generator(device="cuda").manual_seed(n)
+    q, k, v = (torch.randn(1, h, n, 64, generator=g, device="cuda").bfloat16() for h in (2, 1, 1))
+    perm, inv = sa.sa_make_perm(n, w, 1, n)
+    cs, sn = sa.sa_rope_table(n, 64)
+    lg = torch.zeros(2, 2, device="cuda")
+    p = sa.make_problem(q, k, w, flags)
+    at = lambda t: ctypes.c_void_p(t.data_ptr())
+    want, y, y2, out = (torch.empty_like(q) for _ in range(4))
+    st = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    assert sa.load_library().sa_forward(ctypes.byref(p), at(q), at(k), at(v), at(perm), at(inv), at(want), None,
+                                        None, 0, st) == 0
+    copies = sa.sa_workspace_bytes(p, sa.OP_FORWARD_ROPE) - sa.sa_workspace_bytes(p, sa.OP_KEY_LISTS)
+    least = sa.host_forward_ws_bytes(1, 2, 1, n, 64)
+    total = torch.cuda.get_device_properties(0).total_memory
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    short = lambda spare: torch.cuda.set_per_process_memory_fraction(
+        (torch.cuda.memory_reserved() + spare) / total)
+    try:
+        short(0)
+        with pytest.warns(RuntimeWarning, match="key lists"):
+            sa.sa_forward(q, k, v, perm, inv, w, flags, y=y)
+        with pytest.warns(RuntimeWarning, match="key lists"):
+            sa.sa_swa_gated_forward(q, k, v, perm, inv, lg, w, flags | SWA_ONE_SIDED, out={"y": out, "y_sa": y2})
+        torch.cuda.synchronize()
+        assert torch.equal(y, want) and torch.equal(y2, want)
+        torch.cuda.empty_cache()
+        short(copies + 2 * q.numel() + (4 << 20))       # ... and y
+        with pytest.warns(RuntimeWarning, match="key lists"):
+            sa.sa_forward_rope(q, k, v, perm, inv, cs, sn, w, flags)
+        torch.cuda.empty_cache()
+        short(least + (4 << 20))
+        with pytest.warns(RuntimeWarning, match="key lists"):
+            assert HostForward(1, 2, 1, n, 64, w, flags).ws.numel() == least
+    finally:
+        torch.cuda.set_per_process_memory_fraction(1.0)
+    assert not torch.equal(sa.sa_forward(q, k, v, perm, inv, w, flags), y)
+    assert sa.sa_read_status() == 0
