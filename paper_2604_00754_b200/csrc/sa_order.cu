@@ -8,9 +8,12 @@
 // it holds: with w = 1024 two tiles meet 5.3 and 10 blocks of 128 keys where they met 9 each, with
 // w = 2048 four tiles 3.6 to 20 (12.8 on the average) where they met 17.  What a row sees of a block is
 // one bit per key, worked out here once for all heads.
-// SA branch of 32/8 heads of 128, n = 32768, w = 1024: 744 us without lists, 618 with them and this launch;
-// of 32/4 heads, n = 131072, w = 2048: 5494 and 4347.  The launch itself takes 15 us at n = 8192 and 19 at
-// 32768: a chain of latencies (tokens, counts, scan, places, ranks, bits) in each CTA.
+// SA branch of 32/8 heads of 128, n = 32768, w = 1024: 818 us without lists, 674 with them and this launch (calls
+// back to back, one box); of 32/4 heads, n = 131072, w = 2048: 5363 and 4034.  The launch itself takes 17.5 us at
+// n = 32768, w = 1024, 29 at w = 2048, 75 at n = 131072, w = 2048.  Clocks inside it, n = 32768, median of the
+// CTAs from the start, w = 1024 / 2048: tokens counted 1.0 / 1.7 us, sorted 4.1 / 6.9, queries found 6.1 / 9.2,
+// bits written 11.8 / 19.7, those of the longest list 16.4 / 28: the bits bound it (360 instructions per 32 keys
+// and 128 rows, two CTAs on most SMs), then the chain of latencies before them.
 #include "sa_order.cuh"
 
 namespace sa {
@@ -267,13 +270,34 @@ size_t up(size_t x) { return (x + 255) / 256 * 256; }
 
 bool order_geom(int n, int d, int w, uint32_t flags, OrderGeom* g) {
   const MaskGeom m = make_geom(n, w, flags, false);
-  // Narrower windows gain little (blocks met on the average, w = 512: 4.7 for 5, w = 768: 6.2 for 7), and in
-  // shorter sequences of few heads the launch costs more than it saves (4/2 heads of 64, w = 1024:
-  // n = 8192 57 us with lists, 36 without; n = 32768 123 and 123).
+  // Times of the SA branch without lists / with lists and their launch, us (heads of d; n):
+  //                          w = 512      768          1024         2048
+  //   4/2 of 64;    8192      23 / 40      29 / 48      34 / 58      57 / 100
+  //                16384      41 / 56      52 / 69      63 / 84     108 / 144
+  //                32768      76 / 78      98 / 96     121 / 116    210 / 199
+  //   4/1 of 128;  32768      74 / 81      92 / 97     112 / 116    188 / 174
+  //                49152     106 / 112    134 / 135    163 / 160    275 / 239
+  //   8/2 of 128;   8192      41 / 56      51 / 68      60 / 81      99 / 136
+  //                16384      74 / 80      92 / 95     111 / 113    187 / 187
+  //                32768     126 / 130    161 / 156    203 / 193    331 / 298
+  //   32/8 of 128;  8192     128 / 126    162 / 151    195 / 177    334 / 293
+  //                10007     163 / 167    205 / 206    252 / 244    421 / 398
+  //                16384     243 / 228    310 / 278    377 / 328    659 / 530
+  //                32768     490 / 455    637 / 553    818 / 674   1355 / 1030
+  //   2/1 of 64;   32768      41 / 52      52 / 63      64 / 75     108 / 125
+  //                49152      59 / 68      75 / 84      92 / 101    160 / 154
+  //                65536      76 / 80      99 / 98     121 / 117    210 / 182
+  //   2/1 of 128;  32768      41 / 52      50 / 62      60 / 74      99 / 120
+  //                65536      74 / 84      93 / 100    114 / 119    191 / 178
+  // The line is drawn where four query heads break even.  Thirty-two would gain from n = 8192 on, and two lose
+  // up to 22 us, a quarter at most, below n = 65536 (2/1 of 128, w = 1024: 3 % at 131072 still): the launch takes
+  // the same time for any number of heads.  The line is one for all of them because a sequence has the same
+  // bits alone and in a batch, and a KV head the same in any part of the heads (tensor-parallel shards).
   // 256 slots or 512: blocks per tile 7.7 / 7.8 at w = 1024, 10.7 / 10.3 at 1536, 13.7 / 12.8 at 2048.
   if (!m.causal || w < 1024 || n < 32768 || (d != 64 && d != 128)) return false;
   g->slots = w <= 1280 ? 256 : 512;
-  if ((int64_t)g->slots + 2ll * m.h > n || (int64_t)g->slots + 2ll * m.h > 8192) return false;
+  // 16 bits per offset with one to spare, 102 KB of shared memory; and no slot twice, as 8192 < n
+  if ((int64_t)g->slots + 2ll * m.h > 8192) return false;
   g->span = g->slots + 2 * m.h;
   g->groups = (n + g->slots - 1) / g->slots;
   g->tiles = (n + kOrderTile - 1) / kOrderTile;
