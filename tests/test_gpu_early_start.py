@@ -14,6 +14,7 @@ CASES = [
     (4, 12, 12, 1024, 64, 128, torch.bfloat16),    # several
     (1, 4, 1, 17000, 64, 200, torch.bfloat16),     # the permutation's four launches
     (1, 4, 2, 600, 64, 64, torch.float32),
+    (1, 4, 2, 32768 + 200, 64, 1024, torch.bfloat16),    # the SA branch over key lists
 ]
 
 

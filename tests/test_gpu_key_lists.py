@@ -278,3 +278,84 @@ def test_calls_go_without_lists_where_memory_is_short():
         torch.cuda.set_per_process_memory_fraction(1.0)
     assert not torch.equal(sa.sa_forward(q, k, v, perm, inv, w, flags), y)
     assert sa.sa_read_status() == 0
+
+
+def _lists_call(q, k, v, perm, inv, w, flags, ws, size):
+    """The C call with the given scratch (None: the plain one's route)."""
+    p, y = sa.make_problem(q, k, w, flags), torch.empty_like(q)
+    at = lambda t: ctypes.c_void_p(t.data_ptr())
+    st = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    assert sa.load_library().sa_forward_lists(ctypes.byref(p), at(q), at(k), at(v), at(perm), at(inv), at(y), None,
+                                              ws, size, st) == 0
+    return y
+
+
+# token-major tensors, checked permutations and a batch take the lists with the same bits; scratch that is too
+# small, or off 16 bytes, is left alone and the call goes without
+@pytest.mark.gpu
+def test_layouts_checks_and_scratch():
+    n, w = 33000, 1300
+    g = torch.Generator(device="cuda").manual_seed(n)
+    q, k, v = (torch.randn(2, h, n, 64, generator=g, device="cuda").bfloat16() for h in (4, 2, 2))
+    perm, inv = sa.sa_make_perm(n, w, 2, n)
+    y = sa.sa_forward(q, k, v, perm, inv, w, CAUSAL)
+    major = [t.permute(0, 2, 1, 3).contiguous().permute(0, 2, 1, 3) for t in (q, k, v)]
+    assert torch.equal(sa.sa_forward(*major, perm, inv, w, CAUSAL), y)
+    assert torch.equal(sa.sa_forward(q, k, v, perm, inv, w, CAUSAL | 16), y)      # SA_VALIDATE_PERM
+    one = [t[1:2].contiguous() for t in (q, k, v, perm, inv)]
+    assert torch.equal(sa.sa_forward(*one, w, CAUSAL), y[1:2])
+    size = sa.sa_workspace_bytes(sa.make_problem(q, k, w, CAUSAL), sa.OP_KEY_LISTS)
+    ws = torch.zeros(size + 16, dtype=torch.uint8, device="cuda")
+    args = (q, k, v, perm, inv, w, CAUSAL)
+    plain = _lists_call(*args, None, 0)
+    assert not torch.equal(plain, y)
+    assert torch.equal(_lists_call(*args, ctypes.c_void_p(ws.data_ptr()), size - 1), plain)
+    assert torch.equal(_lists_call(*args, ctypes.c_void_p(ws.data_ptr() + 8), size), plain)
+    assert not ws.any()
+    assert torch.equal(_lists_call(*args, ctypes.c_void_p(ws.data_ptr() + 16), size), y)
+    assert sa.sa_read_status() == 0
+
+
+# An infinity or a NaN in V: the rows that see it have it, and no row does outside the groups of 256 slots whose
+# window holds it (hidden pairs within a group's blocks weigh 0, and 0 times it is a NaN).
+@pytest.mark.gpu
+@pytest.mark.parametrize("value", [float("inf"), float("nan")])
+def test_reach_of_what_is_not_finite(value):
+    n, w = 33000, 1024
+    g = torch.Generator(device="cuda").manual_seed(n)
+    q, k, v = (torch.randn(1, h, n, 64, generator=g, device="cuda").bfloat16() for h in (2, 1, 1))
+    perm, inv = sa.sa_make_perm(n, w, 1, n)
+    clean = sa.sa_forward(q, k, v, perm, inv, w, CAUSAL)
+    token = n // 2
+    v[0, 0, token] = value
+    y = sa.sa_forward(q, k, v, perm, inv, w, CAUSAL)
+    assert sa.sa_read_status() == 0
+    slot, h = int(inv[0, token]), (w + 1) // 2 - 1
+    slots = torch.arange(n, device="cuda")
+    away = lambda a, b: torch.minimum((a - b).abs(), n - (a - b).abs())
+    tokens = perm[0].long()
+    sees = (away(slots, slot) <= h) & (tokens >= token)
+    assert sees.sum() > w // 8
+    assert not torch.isfinite(y[0][:, tokens[sees]]).any()
+    first = slots // 256 * 256
+    last = torch.minimum(first + 255, torch.tensor(n - 1, device="cuda"))
+    held = (away(first, slot) <= h) | (away(last, slot) <= h) | ((first <= slot) & (slot <= last))
+    rest = tokens[~held]
+    assert rest.numel() > n // 2 and torch.equal(y[0][:, rest], clean[0][:, rest])
+
+
+# two query heads: rotated Q and K are below the size from which the pass is taken without lists
+@pytest.mark.gpu
+def test_small_rotated_call_takes_the_pass_and_lists():
+    n, d, w = 32768, 64, 1024
+    g = torch.Generator(device="cuda").manual_seed(n)
+    q, k, v = (torch.randn(1, h, n, d, generator=g, device="cuda").bfloat16() for h in (2, 1, 1))
+    assert q.numel() < 8 << 20
+    perm, inv = sa.sa_make_perm(n, w, 1, n)
+    cs, sn = sa.sa_rope_table(n, d, 1e6)
+    turned = sa.sa_rope_apply(q, k, cs, sn), sa.sa_rope_apply(k, q, cs, sn, kv=True)
+    launches = sa.launch_count()
+    y = sa.sa_forward_rope(q, k, v, perm, inv, cs, sn, w, CAUSAL)
+    assert sa.launch_count() - launches == 3
+    assert torch.equal(y, sa.sa_forward(*turned, v, perm, inv, w, CAUSAL))
+    assert sa.sa_read_status() == 0
