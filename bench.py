@@ -293,12 +293,15 @@ def main():
 
     flops_branch = 4.0 * c.B * c.Hq * c.n * c.w * c.d
     achieved = flops_branch / (sa_kernel_ms * 1e-3) / 1e12
-    # DRAM bytes of one SA-branch launch: dram__bytes_read.sum + dram__bytes_write.sum of one ncu
-    # capture of this kernel on this shape at n = 8192 (100.8 MB + 33.1 MB; the counter summary
-    # is under profiles/), scaled by n because every tensor grows in proportion to it.
-    traffic = None
+    # DRAM bytes of the SA branch, dram__bytes_read.sum + dram__bytes_write.sum of ncu captures (the
+    # counter summaries are under profiles/): with key lists both launches at n = 32768 (0.2 MB, 436.8 +
+    # 235.1 MB), without them the one at n = 8192 (100.8 + 33.1 MB); scaled by n because every tensor
+    # grows in proportion to it.
+    traffic = traffic_at = None
     if (c.B, c.Hq, c.Hkv, c.d, c.w) == (1, 32, 8, 128, 1024):
-        traffic = 133836288.0 * c.n / 8192
+        lists = sa.sa_workspace_bytes(sa.make_problem(q, k, c.w, c.flags), sa.OP_KEY_LISTS) > 0
+        traffic_at = 32768 if lists else 8192
+        traffic = (672034560.0 if lists else 133836288.0) * c.n / traffic_at
     sustained = args.steps * ms_per_step > 1500.0
     peak = pk["bf16_tflops_sustained"] if sustained else pk["bf16_tflops"]
     line = {
@@ -314,7 +317,7 @@ def main():
                      "peak_kind": "%s bf16 %s" % (pk["source"], "sustained" if sustained else "burst"),
                      "kernel_ms": sa_kernel_ms, "flops_per_launch": flops_branch,
                      "traffic": traffic,
-                     "traffic_note": "ncu DRAM read+write of one launch at n=8192, scaled by n"},
+                     "traffic_note": "ncu DRAM read+write of the branch at n=%s, scaled by n" % traffic_at},
     }
 
     if rank == 0 and not args.no_extras:
@@ -506,8 +509,8 @@ def extras(args, c, wl, sa, torch, dev, host, perm, inv, ws, y, pk):
         del dyb, sv, bws3, bo
         torch.cuda.empty_cache()
 
-    # rotary position embedding with original positions (Sec. 4.2): rotation inside the gather
-    # of the SA forward against a rotation pass over Q and K followed by the plain forward
+    # rotary position embedding with original positions (Sec. 4.2): the call (which turns Q and K in a
+    # pass of its own at this size), and rotation passes over Q and K followed by the plain forward
     cs, sn = sa.sa_rope_table(c.n, c.d, 1e6)
     qr, kr = torch.empty_like(q), torch.empty_like(k)
     fused_ms = event_ms(lambda: sa.sa_forward_rope(q, k, v, perm, inv, cs, sn, c.w, c.flags, y=y),
@@ -520,7 +523,7 @@ def extras(args, c, wl, sa, torch, dev, host, perm, inv, ws, y, pk):
     unfused_ms = event_ms(unfused, it, 3, torch)
     pass_ms = event_ms(lambda: (sa.sa_rope_apply(q, k, cs, sn, out=qr),
                                 sa.sa_rope_apply(k, q, cs, sn, out=kr, kv=True)), it, 3, torch)
-    res["rope"] = {"sa_fwd_rope_in_gather_ms": fused_ms, "rope_pass_plus_sa_fwd_ms": unfused_ms,
+    res["rope"] = {"sa_forward_rope_ms": fused_ms, "rope_pass_plus_sa_fwd_ms": unfused_ms,
                    "rope_pass_ms": pass_ms, "sa_fwd_ms": sa_ms,
                    "pass_bytes": 2.0 * 2 * (q.numel() + k.numel()),
                    "pass_gbs": 2.0 * 2 * (q.numel() + k.numel()) / (pass_ms * 1e-3) / 1e9}

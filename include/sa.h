@@ -166,7 +166,12 @@ sa_status sa_swa_gated_forward(const sa_problem* p, const void* q, const void* k
  * Causal bf16 problems with wide windows then walk their keys in token order: one launch more, which
  * writes per 256 or 512 slots the tokens of their window in order and per query tile and 128 keys what
  * each row sees, and an SA branch that passes over most of what causality hides.  Same result up to
- * the order of summation. */
+ * the order of summation.  An infinity or a NaN in a row of V makes a NaN of what a tile multiplies by 0
+ * because it is hidden: with lists it reaches no row outside the groups whose window holds that row's
+ * slot, without them none more than w / 2 + 256 slots away.
+ * Bytes: about B n (16 blocks + 4 + 4 window / group) with group = 256 slots for w <= 1280, 512 above,
+ * window = group + w and blocks = window / 128 rounded up: 6.0 MB at n = 32768, w = 1024, 45 MB at
+ * n = 131072, w = 2048, 1.06 GB at n = 2^20, w = 7000. */
 sa_status sa_forward_lists(const sa_problem* p, const void* q, const void* k, const void* v,
                            const int32_t* perm, const int32_t* inv, void* y, float* lse, void* ws,
                            size_t ws_bytes, sa_stream_t stream);

@@ -162,7 +162,7 @@ sa_status gated_forward(const sa_problem* p, const void* q, const void* k, const
   if ((p->flags & SA_SAVE_FOR_BWD) && (!y_sa || !y_swa || !lse_sa || !lse_swa))
     return SA_ERR_INVALID_ARG;
   if ((s = maybe_validate(p, perm, inv, st)) != SA_OK) return s;
-  // Two launches.  The SA branch first: its ungated rows land in y_sa, else in y itself.  The
+  // Two launches, three where key lists are made here.  The SA branch first: its ungated rows land in y_sa, else in y itself.  The
   // local branch then owns each output row exactly once: its epilogue reads the matching SA row
   // (the tensor-core kernel in coalesced pieces), applies both gates and writes y.  (In the other order
   // the rows of the local branch would be read scattered from the SA branch's epilogue, and that branch

@@ -52,7 +52,8 @@ enum Src { kGather = 0, kNatural = 1, kOrdered = 2 };
 constexpr int kRowWarps = 8, kThreads = 32 * (kRowWarps + 4);
 __host__ __device__ constexpr int issuers(int d) { return d == 64 ? 2 : 1; }
 
-// Division of numbers below 2^30 by one known at the launch: a multiplication and a shift, where the
+// Division of numbers below 2^30 by one known at the launch: a multiplication and a shift (Granlund and
+// Montgomery, Division by invariant integers using multiplication, 1994), where the
 // division proper costs every warp some twenty instructions, five times per item (2 x 16 heads of 128,
 // n = 4096, w = 256 82 -> 75 us, its SWA branch 54 -> 50; 8 x 12 heads of 64, w = 128 132 -> 125 and 77 -> 71).
 struct FastDiv {
@@ -184,8 +185,9 @@ __device__ __forceinline__ Geo make_geo(const TcParams& p, int item, int hk) {
   return g;
 }
 
-// kOrdered: the query tiles of an item.  Those that meet the most blocks come first, class by class, so
-// that the classes fall evenly on the CTAs and the last round is of the shortest.
+// kOrdered: the query tiles of an item.  Within a KV head those that meet the most blocks come first, class
+// by class, so that the classes fall evenly on the CTAs; the last rounds of the last KV head are of the
+// shortest.
 __device__ __forceinline__ void ordered_tiles(const TcParams& p, int item, int hk, int (&tile)[2],
                                               int (&hq)[2]) {
   const int per_unit = p.pair_heads ? 1 : 2, units = p.og.slots / (kTile * per_unit);
