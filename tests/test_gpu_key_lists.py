@@ -264,8 +264,6 @@ def test_calls_go_without_lists_where_memory_is_short():
             sa.sa_forward(q, k, v, perm, inv, w, flags, y=y)
         with pytest.warns(RuntimeWarning, match="key lists"):
             sa.sa_swa_gated_forward(q, k, v, perm, inv, lg, w, flags | SWA_ONE_SIDED, out={"y": out, "y_sa": y2})
-        torch.cuda.synchronize()
-        assert torch.equal(y, want) and torch.equal(y2, want)
         torch.cuda.empty_cache()
         short(copies + 2 * q.numel() + (4 << 20))       # ... and y
         with pytest.warns(RuntimeWarning, match="key lists"):
@@ -276,6 +274,7 @@ def test_calls_go_without_lists_where_memory_is_short():
             assert HostForward(1, 2, 1, n, 64, w, flags).ws.numel() == least
     finally:
         torch.cuda.set_per_process_memory_fraction(1.0)
+    assert torch.equal(y, want) and torch.equal(y2, want)
     assert not torch.equal(sa.sa_forward(q, k, v, perm, inv, w, flags), y)
     assert sa.sa_read_status() == 0
 
