@@ -9,7 +9,7 @@
 // w = 2048 four tiles 3.6 to 20 (12.8 on the average) where they met 17.  What a row sees of a block is
 // one bit per key, worked out here once for all heads.
 // SA branch of 32/8 heads of 128, n = 32768, w = 1024: 818 us without lists, 674 with them and this launch (calls
-// back to back, one box); of 32/4 heads, n = 131072, w = 2048: 5363 and 4034.  The launch itself takes 17.5 us at
+// back to back, in turn); of 32/4 heads, n = 131072, w = 2048: 5363 and 4034.  The launch itself takes 17.5 us at
 // n = 32768, w = 1024, 29 at w = 2048, 75 at n = 131072, w = 2048.  Clocks inside it, n = 32768, median of the
 // CTAs from the start, w = 1024 / 2048: tokens counted 1.0 / 1.7 us, sorted 4.1 / 6.9, queries found 6.1 / 9.2,
 // bits written 11.8 / 19.7, those of the longest list 16.4 / 28: the bits bound it (some 360 instructions per 32 keys
